@@ -159,6 +159,9 @@ FP_DEV uint32_t match_bits(uint32_t v, bool valid)
     return peers;
 }
 
+// the line at p on its way to L2
+FP_DEV void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 // volatile load for inter-block flags
 FP_DEV uint32_t ld_volatile(const uint32_t* p) { return *(const volatile uint32_t*)p; }
 

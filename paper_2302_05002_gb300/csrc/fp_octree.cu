@@ -31,16 +31,13 @@
 //   5. the points are scattered stably by leaf id (leaf-grouped output) and,
 //      in fp_subsample, by owner id (final output); owner segments of nodes
 //      above the chunks (the stitch) are re-sorted by original index.
+#include "fp_grid.cuh"
 #include "fp_seg.cuh"
 
 namespace fp {
 
 constexpr int kPieceMax = 1024;                 // largest piece handled in shared memory
 constexpr int kRoundLevels = 3;                 // levels a split round groups the open nodes' records by
-constexpr int kWindow = 1024;                   // pieces starting in one window form a unit
-constexpr int kUnitCap = kPieceMax + kWindow;   // records of one unit
-constexpr int kUnitNT = 512;
-constexpr int kUnitWarps = kUnitNT / 32;
 constexpr uint8_t kInner = 0xFF;                // hierarchy still inner at this level
 constexpr uint8_t kEmpty = 0xFE;
 
@@ -53,9 +50,9 @@ static_assert(sizeof(NodeRec) == 24, "NodeRec layout");
 
 struct Piece {
     uint32_t begin, count;   // record range in the cell-grouped arrays
-    uint8_t q, hier, A, dup; // level, leaf level or kInner, first-min level of its minimum, oversized
+    uint8_t q, hier, A;      // level, leaf level or kInner, first-min level of its minimum
     uint8_t srt;             // its records are in key order down to this level
-    uint8_t pad[3];
+    uint8_t pad[4];
 };
 static_assert(sizeof(Piece) == 16, "Piece layout");
 
@@ -84,15 +81,13 @@ struct OctCtx {   // device pointers of one fp_build_chunk_octree call
     const uint32_t* counts;    // points per level-g cell: the hierarchy
     const uint32_t* rcounts;   // records per level-g cell: the points at hand (a chunk group's, or all)
     uint32_t leaf_base;        // position of the first record in the whole distributed array
-    const uint32_t* pyr;
     const uint32_t* cstart;
+    const uint32_t* cursor;    // ends of the cells as k_cell_scatter left them (cursor_slot)
     uint8_t* cell_leaf;
     uint4* rec;           // cell-grouped records (rec_key, rec_j)
-    Piece* pieces;
-    uint32_t* npieces;
-    uint32_t piece_cap;
-    uint32_t* dups;       // pieces of more than kPieceMax points (equal keys to the deepest level)
-    uint32_t* ndups;
+    Piece *tab, *small, *gen, *dups;   // the pieces by the way their lambda is found (emit_piece), any order
+    uint32_t *ntab, *nsmall, *ngen, *ndups;
+    uint32_t piece_cap;                // of each list
     NodeRec* nrec;
     uint32_t* nnode;
     uint32_t node_cap_ws;
@@ -104,16 +99,8 @@ struct OctCtx {   // device pointers of one fp_build_chunk_octree call
     uint32_t* err;
 };
 
-// code of record position jj (owner level, leaf level and the level-g cell of
-// its key21), checked against the record count (an inconsistent grouping must
-// not turn into a stray store)
-FP_DEV void put_code(const OctCtx& c, uint32_t jj, int K, int leafl, uint64_t key21)
-{
-    if (jj < c.n) c.codes[jj] = code_make(K, leafl, (uint32_t)(key21 >> (3 * (kKeyLevels - c.g))));
-    else raise(c.err, FP_ERR_CAPACITY, 17);
-}
-
-// record i of the cell-grouped array, checked likewise (a zero record beyond it)
+// record i of the cell-grouped array, checked against the record count (a zero
+// record beyond it: an inconsistent grouping must not turn into a stray access)
 FP_DEV uint4 get_rec(const OctCtx& c, uint64_t i)
 {
     if (i < c.n) return c.rec[i];
@@ -121,26 +108,9 @@ FP_DEV uint4 get_rec(const OctCtx& c, uint64_t i)
     return make_uint4(0u, 0u, 0u, 0u);
 }
 
-FP_DEV uint32_t pyr_at(const uint32_t* pyr, const uint32_t* counts, int g, int l, uint64_t key)
+FP_DEV void put_node(const OctCtx& c, uint32_t id, uint64_t key, int level, uint32_t count, uint32_t leaf_first,
+                     bool leaf)
 {
-    return l == g ? counts[key] : pyr[((1ull << (3 * l)) - 1) / 7 + key];
-}
-
-__global__ void k_pyr_level(const uint32_t* __restrict__ child, uint32_t* __restrict__ parent, uint64_t np)
-{
-    uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= np) return;
-    // level offsets (8^l - 1) / 7 are only 4-byte aligned: scalar loads
-    const uint32_t* c = child + 8 * k;
-    uint32_t s = 0;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) s += c[q];
-    parent[k] = s;
-}
-
-FP_DEV void emit_node(const OctCtx& c, uint64_t key, int level, uint32_t count, uint32_t leaf_first, bool leaf)
-{
-    uint32_t id = atomicAdd(c.nnode, 1u);
     if (id >= c.node_cap_ws) { raise(c.err, FP_ERR_CAPACITY, 1); return; }
     NodeRec r;
     r.key = key;
@@ -152,24 +122,42 @@ FP_DEV void emit_node(const OctCtx& c, uint64_t key, int level, uint32_t count, 
     c.nrec[id] = r;
 }
 
-FP_DEV void emit_piece(const OctCtx& c, uint32_t begin, uint32_t count, int q, uint8_t hier, uint8_t A, int srt)
+FP_DEV void emit_node(const OctCtx& c, uint64_t key, int level, uint32_t count, uint32_t leaf_first, bool leaf)
 {
-    uint32_t id = atomicAdd(c.npieces, 1u);
-    if (id >= c.piece_cap) { raise(c.err, FP_ERR_CAPACITY, 2); return; }
+    put_node(c, atomicAdd(c.nnode, 1u), key, level, count, leaf_first, leaf);
+}
+
+// levels below a piece of level q (leaf level hier, not inner) that can decide
+// lambda: an owner at level hier or deeper is the leaf itself
+FP_DEV int piece_depth(const OctCtx& c, int q, int hier) { return max(0, min(kKeyLevels, c.s + hier - 1) - q); }
+
+constexpr int kSmallMax = 32;   // largest piece done by pairs of points
+constexpr int kHashMaxD = 10;   // deepest piece on the tables: 3 * 10 cell bits beside a 30-bit index in 64 bits
+
+FP_DEV Piece make_piece(uint32_t begin, uint32_t count, int q, uint8_t hier, uint8_t A, int srt)
+{
     Piece p;
     p.begin = begin;
     p.count = count;
     p.q = (uint8_t)q;
     p.hier = hier;
     p.A = A;
-    p.dup = count > (uint32_t)kPieceMax ? 1 : 0;
     p.srt = (uint8_t)srt;
-    p.pad[0] = p.pad[1] = p.pad[2] = 0;
-    c.pieces[id] = p;
-    if (p.dup) {
-        const uint32_t k = atomicAdd(c.ndups, 1u);
-        if (k < c.piece_cap) c.dups[k] = id;
-    }
+    p.pad[0] = p.pad[1] = p.pad[2] = p.pad[3] = 0;
+    return p;
+}
+
+FP_DEV void emit_piece(const OctCtx& c, uint32_t begin, uint32_t count, int q, uint8_t hier, uint8_t A, int srt)
+{
+    Piece* list = c.tab;
+    uint32_t* n = c.ntab;
+    if (count > (uint32_t)kPieceMax) { list = c.dups; n = c.ndups; }
+    else if (hier == kInner) { list = c.gen; n = c.ngen; }
+    else if (count <= (uint32_t)kSmallMax) { list = c.small; n = c.nsmall; }
+    else if (piece_depth(c, q, hier) > kHashMaxD) { list = c.gen; n = c.ngen; }
+    const uint32_t id = atomicAdd(n, 1u);
+    if (id >= c.piece_cap) { raise(c.err, FP_ERR_CAPACITY, 2); return; }
+    list[id] = make_piece(begin, count, q, hier, A, srt);
 }
 
 // ---------------------------------------------------------------- cells
@@ -182,14 +170,8 @@ FP_DEV void emit_piece(const OctCtx& c, uint32_t begin, uint32_t count, int q, u
 // chunk by chunk, so the cells in use at any time are consecutive: cursors sit
 // at bit-reversed cell ids, which spreads those atomics over the whole array
 // (and every L2 slice).  A cursor that does not end at cstart[m + 1] means the
-// count grid was not the grid of these points (reported by k_cell_check).
+// count grid was not the grid of these points (reported by k_small_pieces).
 FP_DEV uint32_t cursor_slot(uint32_t m, int g) { return __brev(m) >> (32 - 3 * g); }
-
-__global__ void k_cell_cursor_init(const uint32_t* __restrict__ cstart, uint64_t cells, uint32_t* cursor, int g)
-{
-    for (uint64_t m = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; m < cells; m += (uint64_t)gridDim.x * blockDim.x)
-        cursor[cursor_slot((uint32_t)m, g)] = cstart[m];
-}
 
 __global__ void __launch_bounds__(256) k_cell_scatter(const int4* __restrict__ pts, uint64_t n, const fp_cube* cube_p,
                                                       uint32_t* cursor, uint4* __restrict__ rec, int g,
@@ -220,64 +202,141 @@ __global__ void __launch_bounds__(256) k_cell_scatter(const int4* __restrict__ p
     }
 }
 
-__global__ void k_cell_check(const uint32_t* __restrict__ cstart, uint64_t cells, const uint32_t* cursor, int g,
-                             uint32_t* err)
+// One block per tile of the grid (k_grid_tiles before it).  With `cells`: every
+// cell's start among the records and its cursor; its leaf level when the
+// hierarchy ends at or above g, kInner if the cell's node is inner, kEmpty
+// without a record.  Cells with at most kPieceMax records become pieces
+// (k_small_pieces finds the smallest by itself); larger ones open the split
+// tree.  With `upper`: the nodes at levels <= g, each by the thread of its first
+// cell.  Pieces for the tables, nearly all of them on large clouds, and nodes are
+// appended with one atomic per tile, the pieces in cell order: those in work at
+// one time then lie in one or two tiles, and their scattered codes stay in L2
+// (appended one by one as the atomics fell, k_tab_pieces took 15.5 instead of
+// 13.0 ms for 5 * 10^8 uniform points).
+__global__ void __launch_bounds__(kGtNT) k_cells_open(OctCtx c, const uint32_t* __restrict__ pyr,
+                                                      const uint32_t* __restrict__ rsum, int cells, int upper,
+                                                      uint32_t* __restrict__ cstart, uint32_t* __restrict__ cursor,
+                                                      OpenNode* open0, uint32_t* nopen0)
 {
-    for (uint64_t m = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; m < cells; m += (uint64_t)gridDim.x * blockDim.x)
-        if (cursor[cursor_slot((uint32_t)m, g)] != cstart[m + 1]) raise(err, FP_ERR_CAPACITY, 4);
-}
-
-// Per level-g cell: leaf level if the hierarchy ends at or above g, kInner if
-// the cell node is inner, kEmpty for an empty cell.  Nonempty cells with at
-// most kPieceMax points become pieces; larger ones open the split tree.
-__global__ void k_cell_setup(OctCtx c, OpenNode* open0, uint32_t* nopen0)
-{
-    uint64_t m = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const uint64_t cells = 1ull << (3 * c.g);
-    if (m >= cells) return;
-    uint32_t cnt = c.rcounts[m];
-    if (cnt == 0) { c.cell_leaf[m] = kEmpty; return; }
-    uint8_t hier = kInner;
-    for (int l = 0; l <= c.g; ++l) {
-        uint32_t v = pyr_at(c.pyr, c.counts, c.g, l, m >> (3 * (c.g - l)));
-        if (v <= c.C || l == c.lmax) { hier = (uint8_t)l; break; }
-    }
-    c.cell_leaf[m] = hier;
-    if (cnt <= (uint32_t)kPieceMax) {
-        emit_piece(c, c.cstart[m], cnt, c.g, hier, (uint8_t)c.g, c.g);
+    __shared__ GridTop top;
+    __shared__ uint32_t s_warp[kGtNT / 32], s_base[2];
+    const int g = c.g, tid = threadIdx.x;
+    const uint32_t ncell = 1u << (3 * g), tile = blockIdx.x, base = tile * kGtCells + tid * kGtPer;
+    uint32_t v[kGtPer], rv[kGtPer];
+    grid_load16(c.counts, base, ncell, v);
+    const GridSums s = grid_sums(v, s_warp);
+    const int up = grid_top(top, pyr, g, s.s4);
+    uint32_t before = 0;
+    for (uint32_t i = tid; i < tile; i += kGtNT) before += rsum[i];
+    before = block_sum(before, s_warp);
+    if (c.rcounts == c.counts) {
+#pragma unroll
+        for (int q = 0; q < kGtPer; ++q) rv[q] = v[q];
     } else {
-        uint32_t id = atomicAdd(nopen0, 1u);
-        if (id >= c.open_cap) { raise(c.err, FP_ERR_CAPACITY, 5); return; }
-        OpenNode o;
-        o.key = m;
-        o.begin = c.cstart[m];
-        o.count = cnt;
-        o.q = (uint8_t)c.g;
-        o.hier = hier;
-        o.A = (uint8_t)c.g;
-        o.pad = 0;
-        o.rb = o.pad2 = o.pad3 = 0;
-        open0[id] = o;
+        grid_load16(c.rcounts, base, ncell, rv);
     }
-}
+    uint32_t mine = 0;
+#pragma unroll
+    for (int q = 0; q < kGtPer; ++q) mine += rv[q];
+    uint32_t total;
+    const uint32_t at0 = before + block_exclusive_scan<kGtNT, uint32_t>(mine, s_warp, total);
 
-// nodes at levels <= g, from the count pyramid
-__global__ void k_nodes_upper(OctCtx c)
-{
-    uint64_t f = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int L = 0;
-    uint64_t base = 0;
-    while (L <= c.g && f >= base + (1ull << (3 * L))) { base += 1ull << (3 * L); ++L; }
-    if (L > c.g) return;
-    uint64_t k = f - base;
-    uint32_t cnt = pyr_at(c.pyr, c.counts, c.g, L, k);
-    if (cnt == 0) return;
-    for (int a = 0; a < L; ++a) {   // every ancestor must be inner
-        uint32_t v = pyr_at(c.pyr, c.counts, c.g, a, k >> (3 * (L - a)));
-        if (v <= c.C || a >= c.lmax) return;
+    // leaf level of the nodes around this thread's cells, down to the 64-cell one (255: all inner)
+    int hl = 255;
+    if (s.s2 <= c.C) hl = g - 2;
+    if (s.s3 <= c.C) hl = g - 3;
+    for (int a = 0; a <= up; ++a)
+        if (top.at(a, tile) <= c.C) hl = g - 4 - a;
+    if (hl < 0) hl = 0;   // (a grid of fewer than 4096 cells)
+    uint8_t hier[kGtPer];
+    uint32_t tab = 0;   // bit q: cell q is a piece for the tables
+    if (cells) {
+        uint32_t at = at0;
+#pragma unroll
+        for (int q = 0; q < kGtPer; ++q) {
+            const uint32_t m = base + q;
+            hier[q] = kEmpty;
+            if (m < ncell) {
+                cstart[m] = at;
+                cursor[cursor_slot(m, g)] = at;
+            }
+            if (rv[q]) {
+                hier[q] = hl != 255 ? (uint8_t)hl
+                                    : (s.s1[q >> 3] <= c.C ? (uint8_t)max(g - 1, 0)
+                                                           : (v[q] <= c.C || g == c.lmax ? (uint8_t)g : kInner));
+                if (rv[q] > (uint32_t)kPieceMax) {
+                    const uint32_t id = atomicAdd(nopen0, 1u);
+                    if (id >= c.open_cap) {
+                        raise(c.err, FP_ERR_CAPACITY, 5);
+                    } else {
+                        OpenNode o;
+                        o.key = m;
+                        o.begin = at;
+                        o.count = rv[q];
+                        o.q = (uint8_t)g;
+                        o.hier = hier[q];
+                        o.A = (uint8_t)g;
+                        o.pad = 0;
+                        o.rb = o.pad2 = o.pad3 = 0;
+                        open0[id] = o;
+                    }
+                } else if (hier[q] == kInner || (rv[q] > (uint32_t)kSmallMax && piece_depth(c, g, hier[q]) > kHashMaxD)) {
+                    emit_piece(c, at, rv[q], g, hier[q], (uint8_t)g, g);
+                } else if (rv[q] > (uint32_t)kSmallMax) {
+                    tab |= 1u << q;
+                }
+            }
+            at += rv[q];
+        }
+        if (tile == gridDim.x - 1 && tid == 0) cstart[ncell] = before + total;
+#pragma unroll
+        for (int q = 0; q < kGtPer; ++q)
+            if (base + q < ncell) c.cell_leaf[base + q] = hier[q];
     }
-    bool leaf = cnt <= c.C || L == c.lmax;
-    emit_node(c, k, L, cnt, c.cstart[k << (3 * (c.g - L))], leaf);
+
+    // nodes of this thread: bits 0..15 its cells, 16, 17 the runs of 8, 18 the 64 cells, 19 the warp's
+    // 512, 20 the tile, 20 + a the node a levels above it
+    auto exists = [&](int L, uint32_t cnt, uint32_t parent) { return L >= 0 && cnt && (L == 0 || parent > c.C); };
+    uint32_t nf = 0;
+    if (upper && base < ncell) {
+#pragma unroll
+        for (int q = 0; q < kGtPer; ++q)
+            if (base + q < ncell && exists(g, v[q], s.s1[q >> 3])) nf |= 1u << q;
+        if (exists(g - 1, s.s1[0], s.s2)) nf |= 1u << 16;
+        if (base + 8 < ncell && exists(g - 1, s.s1[1], s.s2)) nf |= 1u << 17;
+        if ((tid & 3) == 0 && exists(g - 2, s.s2, s.s3)) nf |= 1u << 18;
+        if ((tid & 31) == 0 && exists(g - 3, s.s3, s.s4)) nf |= 1u << 19;
+        if (tid == 0)
+            for (int a = 0; a <= up; ++a)
+                if ((tile & ((1u << (3 * a)) - 1)) == 0 &&
+                    exists(g - 4 - a, top.at(a, tile), a < up ? top.at(a + 1, tile) : 0u))
+                    nf |= 1u << (20 + a);
+    }
+    // both appends: one scan (tables in the low half, nodes in the high half: at most 5 * 4096 each)
+    const uint32_t ex = block_exclusive_scan<kGtNT, uint32_t>(__popc(tab) | (__popc(nf) << 16), s_warp, total);
+    if (tid == 0) {
+        s_base[0] = (total & 0xFFFFu) ? atomicAdd(c.ntab, total & 0xFFFFu) : 0u;
+        s_base[1] = (total >> 16) ? atomicAdd(c.nnode, total >> 16) : 0u;
+    }
+    __syncthreads();
+    uint32_t pi = s_base[0] + (ex & 0xFFFFu), ni = s_base[1] + (ex >> 16), at = at0;
+#pragma unroll
+    for (int q = 0; q < kGtPer; ++q) {
+        if ((tab >> q) & 1u) {
+            if (pi >= c.piece_cap) raise(c.err, FP_ERR_CAPACITY, 2);
+            else c.tab[pi] = make_piece(at, rv[q], g, hier[q], (uint8_t)g, g);
+            ++pi;
+        }
+        if ((nf >> q) & 1u) put_node(c, ni++, base + q, g, v[q], at, v[q] <= c.C || g == c.lmax);
+        if (q == 7 && ((nf >> 17) & 1u)) put_node(c, ni++, (base >> 3) + 1, g - 1, s.s1[1], at + rv[7], s.s1[1] <= c.C);
+        at += rv[q];
+    }
+    if ((nf >> 16) & 1u) put_node(c, ni++, base >> 3, g - 1, s.s1[0], at0, s.s1[0] <= c.C);
+    if ((nf >> 18) & 1u) put_node(c, ni++, base >> 6, g - 2, s.s2, at0, s.s2 <= c.C);
+    if ((nf >> 19) & 1u) put_node(c, ni++, base >> 9, g - 3, s.s3, at0, s.s3 <= c.C);
+    for (int a = 0; a <= up; ++a)
+        if ((nf >> (20 + a)) & 1u)
+            put_node(c, ni++, tile >> (3 * a), g - 4 - a, top.at(a, tile), at0, top.at(a, tile) <= c.C);
 }
 
 // ------------------------------------------------------- big cells: rounds
@@ -497,59 +556,308 @@ __global__ void k_split(OctCtx c, const OpenNode* cur, const uint32_t* ncur, Ope
     }
 }
 
-// ------------------------------------------------------------ units
-struct UnitSmem {
-    uint64_t key[kUnitCap];
-    uint64_t key2[kUnitCap];
-    uint32_t j[kUnitCap];       // by local index
-    uint32_t mt[kUnitCap];      // min-tree over hj: internal nodes 1..P-1 (the leaves are hj itself)
-    uint16_t v[kUnitCap];       // local index by sorted position
-    uint16_t v2[kUnitCap];
-    uint16_t piece[kUnitCap];   // piece of a local index
-    uint8_t cl[kUnitCap];       // by run: common level with the nearest smaller index on the left (255: none)
-    uint8_t cr[kUnitCap];       // ... on the right
-    uint32_t hj[kUnitCap];      // by run: smallest index of the run
-    uint16_t hid[kUnitCap];     // by sorted position: run number
-    uint8_t leaf[kUnitCap];     // leaf level by sorted position (pieces with a deep subtree)
-    uint32_t pbeg[kWindow + 1];
-    uint16_t pcnt[kWindow + 1]; // 0 for an oversized piece (handled elsewhere)
-    uint16_t psrt[kWindow + 1]; // start of each piece in the unit (load order = sorted order)
-    uint8_t pq[kWindow + 1], phier[kWindow + 1], pA[kWindow + 1], pkind[kWindow + 1];
-    uint16_t pn[kWindow + 1];   // points of the piece (0 for an oversized one)
-    uint16_t ptab[kWindow + 1]; // table pieces: first entry of the piece's level tables
-    uint16_t pfst[kWindow + 1]; // table pieces: start of the piece's records in the table phase
-    uint8_t pD[kWindow + 1];    // table pieces: levels below the piece that decide lambda
-    uint32_t pmin[kWindow + 1]; // table pieces: smallest index of the piece
-    uint16_t whist[kUnitWarps][256];
+// ------------------------------------------------------------ pieces
+// Lambda of every record, by the size and depth of its piece:
+//   * level-g cells of at most kSmallMax points: k_small_pieces, one lane per
+//     point, straight from the count grid (no piece is listed);
+//   * pieces whose node is not inner, at most kHashMaxD levels deep: k_tab_pieces,
+//     one block per piece, smallest index per occupied cell in tables;
+//   * inner pieces, and deeper ones: k_general_pieces, one block per piece, sort
+//     and nearest-smaller search, which also finds the nodes inside the piece;
+//   * more than kPieceMax equal keys: k_general_pieces too, by a minimum.
+// A piece is worked on by itself, so nothing about a record (its piece, the
+// levels that decide it) is looked up per record, the lists need no order, and
+// blocks wait on nothing but themselves.  (Windows of 1024 records with all of
+// their pieces in one 512-thread block, and the pieces sorted into record order
+// first, spent 950 instructions per point at 238 points per cell, where the
+// fourth and fifth table of a window did not fit its shared memory: 26.1 ms for
+// 5 * 10^8 uniform points.)
+constexpr int kTabNT = 128;
+constexpr int kTabCtas = 10;                  // blocks per SM (20 KB of tables each)
+constexpr int kTabDirect = 4;                 // levels in direct-mapped tables
+constexpr int kTabWords = 4680;               // 8 + 64 + 512 + 4096 entries
+constexpr uint64_t kHashEmpty = ~0ull;
+constexpr int kHashSlots = kPieceMax + kPieceMax / 2;
+constexpr int kTabBytes = sizeof(uint64_t) * (kPieceMax + kHashSlots);   // records and hash table
+static_assert(kTabWords * sizeof(uint32_t) <= kTabBytes, "the direct tables overlay the hash path's arrays");
+
+// owner level of a record with first-minimum level lambda, and its code
+FP_DEV void put_lambda(const OctCtx& c, uint32_t jj, int lambda, int leafl, uint32_t cell)
+{
+    int K = lambda - c.s;
+    K = K < 0 ? 0 : (K > leafl ? leafl : K);
+    if (jj < c.n) c.codes[jj] = code_make(K, leafl, cell);
+    else raise(c.err, FP_ERR_CAPACITY, 17);
+}
+
+// The points of up to 32 small pieces, one piece per lane (cnt 0: none), spread
+// over the lanes of the warp one record each: lambda is one more than the
+// deepest level shared with any point of smaller index in the piece (every pair
+// of the piece; its records are a few consecutive words, read through L1).
+FP_DEV void small_warp(const OctCtx& c, uint32_t begin, uint32_t cnt, uint32_t q, uint32_t leafl, uint32_t A)
+{
+    const int lane = threadIdx.x & 31;
+    if ((uint64_t)begin + cnt > c.n) { raise(c.err, FP_ERR_CAPACITY, 18); cnt = 0; }
+    uint32_t inc = cnt;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    const uint32_t total = __shfl_sync(0xFFFFFFFFu, inc, 31);
+    const uint32_t what = q | (leafl << 8) | (A << 16);
+    for (uint32_t r0 = 0; r0 < total; r0 += 32) {
+        const uint32_t r = r0 + lane;
+        int o = 0;   // lanes whose pieces end at or before r
+#pragma unroll
+        for (int b = 16; b > 0; b >>= 1)
+            if (__shfl_sync(0xFFFFFFFFu, inc, (o + b - 1) & 31) <= r) o += b;
+        o &= 31;
+        const uint32_t w = __shfl_sync(0xFFFFFFFFu, what, o);
+        const uint32_t cn = __shfl_sync(0xFFFFFFFFu, cnt, o);
+        const uint32_t b0 = __shfl_sync(0xFFFFFFFFu, begin, o);
+        const uint32_t at = b0 + r - (__shfl_sync(0xFFFFFFFFu, inc, o) - cn);
+        if (r >= total) continue;   // (no shuffle below)
+        const uint4 me = c.rec[at];
+        const uint64_t k = rec_key(me);
+        uint64_t near = ~0ull;   // smallest key difference to a smaller index: the deepest shared level
+        for (uint32_t t = 0; t < cn; ++t) {
+            const uint4 other = c.rec[b0 + t];
+            const uint64_t x = rec_key(other) ^ k;
+            if (other.z < me.z && x < near) near = x;
+        }
+        int lambda = (int)(w >> 16);   // the piece minimum: from the split tree
+        if (near != ~0ull) lambda = (near == 0 ? kKeyLevels : (__clzll((long long)near) - 1) / 3) + 1;
+        put_lambda(c, me.z, lambda, (int)((w >> 8) & 255u), (uint32_t)(k >> (3 * (kKeyLevels - c.g))));
+    }
+}
+
+// level-g cells of 1 .. kSmallMax points (not inner), one cell per lane, then the
+// small pieces of the split rounds
+__global__ void __launch_bounds__(256) k_small_pieces(OctCtx c)
+{
+    const int lane = threadIdx.x & 31;
+    const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
+    const uint32_t cells = 1u << (3 * c.g);
+    for (uint32_t m0 = warp * 32; m0 < cells; m0 += nwarps * 32) {
+        const uint32_t m = m0 + lane;
+        uint32_t cnt = m < cells ? c.rcounts[m] : 0u, leafl = 0, begin = 0;
+        // a cursor that does not end at the next cell's start: a count grid of other points
+        if (m < cells && c.cursor[cursor_slot(m, c.g)] != c.cstart[m + 1]) raise(c.err, FP_ERR_CAPACITY, 4);
+        if (cnt > (uint32_t)kSmallMax) cnt = 0;
+        if (cnt) {
+            leafl = c.cell_leaf[m];
+            if (leafl == kInner) cnt = 0;
+            else begin = c.cstart[m];
+        }
+        if (__any_sync(0xFFFFFFFFu, cnt != 0)) small_warp(c, begin, cnt, c.g, leafl, c.g);
+    }
+    const uint32_t ns = min(*c.nsmall, c.piece_cap);
+    for (uint32_t p0 = warp * 32; p0 < ns; p0 += nwarps * 32) {
+        Piece p{};
+        if (p0 + lane < ns) p = c.small[p0 + lane];
+        small_warp(c, p.begin, p.count, p.q, p.hier, p.A);
+    }
+}
+
+// A record that is not the smallest index of its cell at some level is not at
+// any coarser one either, so levels are taken deepest first and a record stops
+// at the first level it loses; lambda is the last level it held.
+
+// A piece of at most R * kTabNT records and kTabDirect levels: a direct-mapped
+// table of 8^d entries per level, the whole chain entered first and read back
+// after one barrier.
+template <int R>
+FP_DEV void direct_piece(const OctCtx& c, const Piece& p, int D, uint32_t* tab, uint32_t* s_min)
+{
+    const int tid = threadIdx.x;
+    const int n = (int)p.count, leafl = p.hier, q = p.q;
+    const int sh = 3 * (kKeyLevels - q - D);
+    const uint32_t cmask = (1u << (3 * D)) - 1u;
+    uint32_t kk[R], j[R], cell = 0;
+    {
+        uint4 rec[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            rec[r] = make_uint4(0u, 0u, 0u, 0u);
+            if (r * kTabNT + tid < n) rec[r] = get_rec(c, (uint64_t)p.begin + r * kTabNT + tid);
+        }
+        // clear the tables while the records arrive
+        const int words4 = (int)((((1u << (3 * (D + 1))) - 8u) / 7u + 3u) / 4u);
+        for (int x = tid; x < words4; x += kTabNT)
+            reinterpret_cast<uint4*>(tab)[x] = make_uint4(kNone, kNone, kNone, kNone);
+        if (tid == 0) *s_min = kNone;
+        cell = (uint32_t)(rec_key(rec[0]) >> (3 * (kKeyLevels - c.g)));   // the piece lies in one level-g cell
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            kk[r] = (uint32_t)(rec_key(rec[r]) >> sh) & cmask;
+            j[r] = rec[r].z;
+        }
+    }
+    __syncthreads();
+    int lost[R];   // level at which the record met a smaller index (0: none)
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        lost[r] = 0;
+        if (r * kTabNT + tid >= n) continue;
+        const uint32_t jv = j[r];
+        bool least = true;
+#pragma unroll
+        for (int d = kTabDirect; d >= 1; --d) {
+            if (d <= D && least) {
+                uint32_t* t = &tab[((1u << (3 * d)) - 8u) / 7u + (kk[r] >> (3 * (D - d)))];
+                if (*t < jv) { least = false; lost[r] = d; }
+                else atomicMin(t, jv);
+            }
+        }
+        if (least && *s_min > jv) atomicMin(s_min, jv);
+    }
+    __syncthreads();
+    const uint32_t jmin = *s_min;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        if (r * kTabNT + tid >= n) continue;
+        int top = kKeyLevels + 1 - q;   // never its cell's minimum down to the piece's depth
+        bool held = true;
+#pragma unroll
+        for (int d = kTabDirect; d >= 1; --d) {
+            if (d <= D && held) {
+                held = d > lost[r] && tab[((1u << (3 * d)) - 8u) / 7u + (kk[r] >> (3 * (D - d)))] == j[r];
+                if (held) top = d;
+            }
+        }
+        put_lambda(c, j[r], j[r] == jmin ? (int)p.A : q + top, leafl, cell);   // (the minimum: from the split tree)
+    }
+    __syncthreads();   // the tables are free for the next piece
+}
+
+// A deeper piece: level by level, one hash table of (cell << 30 | index) words,
+// entered by the records still holding; loops instead of registers, since few
+// records hold on at the coarser levels and unrolled code overran the
+// instruction cache (the top stall).
+FP_DEV void hash_piece(const OctCtx& c, const Piece& p, int D, uint64_t* mine /* kPieceMax */,
+                       unsigned long long* ht /* kHashSlots */, uint32_t* s_min)
+{
+    const int tid = threadIdx.x;
+    const int n = (int)p.count, leafl = p.hier, q = p.q;
+    const int sh = 3 * (kKeyLevels - q - D);
+    const uint32_t cmask = (uint32_t)((1ull << (3 * D)) - 1);
+    const uint32_t cell = (uint32_t)(rec_key_at(c.rec, p.begin) >> (3 * (kKeyLevels - c.g)));
+    const uint32_t slots = (uint32_t)(n + (n >> 1)) & ~1u;   // even; at most two thirds are taken
+    if (tid == 0) *s_min = kNone;
+#pragma unroll 4
+    for (int r = tid; r < n; r += kTabNT) {
+        const uint4 rec = get_rec(c, (uint64_t)p.begin + r);
+        mine[r] = ((uint64_t)((uint32_t)(rec_key(rec) >> sh) & cmask) << 30) | rec.z;
+    }
+    constexpr uint32_t kJMask = (1u << 30) - 1u;
+    for (int d = D; d >= 1; --d) {
+        for (uint32_t x = tid; x < slots / 2; x += kTabNT)
+            reinterpret_cast<uint4*>(ht)[x] = make_uint4(kNone, kNone, kNone, kNone);
+        __syncthreads();
+        const int lambda = d == D ? kKeyLevels + 1 : q + d + 1;   // of a record that loses level d
+        for (int r = tid; r < n; r += kTabNT) {
+            const uint64_t m0 = mine[r];
+            if (m0 == kHashEmpty) continue;   // lost before
+            const uint32_t key = (uint32_t)(m0 >> 30) >> (3 * (D - d));
+            const unsigned long long m = ((unsigned long long)key << 30) | (m0 & kJMask);
+            uint32_t h = __umulhi(key * 2654435761u, slots);
+            for (;;) {   // fewer cells than slots: an empty one is reached
+                unsigned long long e = ht[h];
+                if (e == kHashEmpty && (e = atomicCAS(&ht[h], kHashEmpty, m)) == kHashEmpty) break;
+                if ((uint32_t)(e >> 30) == key) {
+                    if (e > m) e = atomicMin(&ht[h], m);   // (words of one cell differ by the index)
+                    if (e < m) {
+                        mine[r] = kHashEmpty;
+                        put_lambda(c, (uint32_t)m & kJMask, lambda, leafl, cell);
+                    }
+                    break;
+                }
+                h = h + 1 == slots ? 0 : h + 1;
+            }
+        }
+        __syncthreads();
+        for (int r = tid; r < n; r += kTabNT) {
+            const uint64_t m0 = mine[r];
+            if (m0 == kHashEmpty) continue;
+            const uint32_t key = (uint32_t)(m0 >> 30) >> (3 * (D - d)), jv = (uint32_t)m0 & kJMask;
+            uint32_t h = __umulhi(key * 2654435761u, slots);
+            unsigned long long e = ht[h];
+            while ((uint32_t)(e >> 30) != key) {   // the record's cell is in the table
+                h = h + 1 == slots ? 0 : h + 1;
+                e = ht[h];
+            }
+            if (((uint32_t)e & kJMask) != jv) {
+                mine[r] = kHashEmpty;
+                put_lambda(c, jv, lambda, leafl, cell);
+            } else if (d == 1) {
+                atomicMin(s_min, jv);
+            }
+        }
+        __syncthreads();
+    }
+    const uint32_t jmin = *s_min;
+    for (int r = tid; r < n; r += kTabNT)
+        if (mine[r] != kHashEmpty) {
+            const uint32_t jv = (uint32_t)mine[r] & kJMask;
+            put_lambda(c, jv, jv == jmin ? (int)p.A : q + 1, leafl, cell);
+        }
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(kTabNT, kTabCtas) k_tab_pieces(OctCtx c)
+{
+    __shared__ __align__(16) unsigned char buf[kTabBytes];
+    __shared__ uint32_t s_min;
+    const uint32_t nt = min(*c.ntab, c.piece_cap);
+    Piece next{};
+    if (blockIdx.x < nt) next = c.tab[blockIdx.x];
+    for (uint32_t k = blockIdx.x; k < nt; k += gridDim.x) {
+        const Piece p = next;
+        if (k + gridDim.x < nt) {   // the next piece's records on their way to L2 during this one's work
+            next = c.tab[k + gridDim.x];
+            const uint32_t line = threadIdx.x * 8;   // 128 bytes a thread
+            if (line < next.count && (uint64_t)next.begin + line < c.n) prefetch_l2(c.rec + next.begin + line);
+        }
+        const int D = piece_depth(c, p.q, p.hier);
+        uint32_t* tab = reinterpret_cast<uint32_t*>(buf);
+        if (D > kTabDirect)
+            hash_piece(c, p, D, reinterpret_cast<uint64_t*>(buf),
+                       reinterpret_cast<unsigned long long*>(buf + sizeof(uint64_t) * kPieceMax), &s_min);
+        else if (p.count <= 2 * kTabNT) direct_piece<2>(c, p, D, tab, &s_min);
+        else if (p.count <= 4 * kTabNT) direct_piece<4>(c, p, D, tab, &s_min);
+        else direct_piece<kPieceMax / kTabNT>(c, p, D, tab, &s_min);
+    }
+}
+
+// ---- general pieces
+constexpr int kGenNT = 256;
+constexpr int kGenWarps = kGenNT / 32;
+struct GenSmem {
+    uint64_t key[kPieceMax];
+    uint64_t key2[kPieceMax];
+    uint32_t j[kPieceMax];       // by load order
+    uint32_t mt[kPieceMax];      // min-tree over hj: internal nodes 1..P-1 (the leaves are hj itself)
+    uint32_t hj[kPieceMax];      // by run: smallest index of the run
+    uint16_t v[kPieceMax];       // load position by sorted position
+    uint16_t v2[kPieceMax];
+    uint16_t hid[kPieceMax];     // by sorted position: run number
+    uint8_t cl[kPieceMax];       // by run: common level with the nearest smaller index on the left (255: none)
+    uint8_t cr[kPieceMax];       // ... on the right
+    uint8_t leaf[kPieceMax];     // leaf level by sorted position (inner pieces)
+    uint16_t whist[kGenWarps][256];
     uint32_t scan[64];
-    uint64_t wmin[kUnitWarps], wmax[kUnitWarps];
+    uint64_t wmin[kGenWarps], wmax[kGenWarps];
     unsigned long long kmin, kmax;
-    uint32_t np, cnt, p0, dl, nh, smin, fcnt, tabn;
+    uint32_t nh;
 };
 
-// two units per SM: 228 KB of shared memory, 1 KB of it reserved per CTA
-static_assert(sizeof(UnitSmem) <= 113 * 1024, "UnitSmem must leave room for two CTAs per SM");
-
-// Table pieces.  A piece whose node is not inner needs lambda only at the
-// levels q+1 .. dl of the piece (coarser: the piece minimum's rule; deeper: the
-// leaf).  When there are at most kTabLevels of them, one direct-mapped table
-// per level (8^d entries at q+d) takes the smallest index of every occupied
-// cell by shared-memory atomicMin, and lambda of a record is the shallowest of
-// those levels at which it is its cell's minimum -- no sort and no
-// nearest-smaller search.  The tables overlay the arrays of the general path
-// (key .. v2), which runs after them.
-constexpr int kTabLevels = 4;
-constexpr int kTabCap = (int)((offsetof(UnitSmem, piece) - offsetof(UnitSmem, key)) / sizeof(uint32_t));
-static_assert(kTabCap >= 3 * 4680, "tables of three pieces of four levels");
-FP_DEV uint32_t tab_size(int D) { return D <= 0 ? 0u : (uint32_t)(((1u << (3 * (D + 1))) - 8u) / 7u); }
-
-// stable LSD pass over the unit's records by 8 key bits at `shift`
-FP_DEV void unit_sort_pass(UnitSmem& S, const uint64_t* kin, const uint16_t* vin, uint64_t* kout, uint16_t* vout,
-                           int cnt, int shift)
+// stable LSD pass over the piece's records by 8 key bits at `shift`
+FP_DEV void gen_sort_pass(GenSmem& S, const uint64_t* kin, const uint16_t* vin, uint64_t* kout, uint16_t* vout,
+                          int cnt, int shift)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr int per_warp = kUnitCap / kUnitWarps;   // records per warp
-    for (int q = threadIdx.x; q < kUnitWarps * 256; q += kUnitNT) (&S.whist[0][0])[q] = 0;
+    constexpr int per_warp = kPieceMax / kGenWarps;   // records per warp
+    for (int q = threadIdx.x; q < kGenWarps * 256; q += kGenNT) (&S.whist[0][0])[q] = 0;
     __syncthreads();
     uint32_t pack[per_warp / 32];
 #pragma unroll
@@ -568,19 +876,16 @@ FP_DEV void unit_sort_pass(UnitSmem& S, const uint64_t* kin, const uint16_t* vin
         __syncwarp();
     }
     __syncthreads();
-    // exclusive prefix over (digit, warp): the first 256 threads own one digit each
+    // exclusive prefix over (digit, warp): each thread owns one digit
     uint32_t tot_d = 0;
-    if (threadIdx.x < 256) {
-        for (int w = 0; w < kUnitWarps; ++w) {
-            uint32_t v = S.whist[w][threadIdx.x];
-            S.whist[w][threadIdx.x] = (uint16_t)tot_d;
-            tot_d += v;
-        }
+    for (int w = 0; w < kGenWarps; ++w) {
+        uint32_t v = S.whist[w][threadIdx.x];
+        S.whist[w][threadIdx.x] = (uint16_t)tot_d;
+        tot_d += v;
     }
     uint32_t tot;
-    uint32_t ex = block_exclusive_scan<kUnitNT, uint32_t>(threadIdx.x < 256 ? tot_d : 0u, S.scan, tot);
-    if (threadIdx.x < 256)
-        for (int w = 0; w < kUnitWarps; ++w) S.whist[w][threadIdx.x] = (uint16_t)(S.whist[w][threadIdx.x] + ex);
+    uint32_t ex = block_exclusive_scan<kGenNT, uint32_t>(tot_d, S.scan, tot);
+    for (int w = 0; w < kGenWarps; ++w) S.whist[w][threadIdx.x] = (uint16_t)(S.whist[w][threadIdx.x] + ex);
     __syncthreads();
 #pragma unroll
     for (int r = 0; r < per_warp / 32; ++r) {
@@ -594,568 +899,241 @@ FP_DEV void unit_sort_pass(UnitSmem& S, const uint64_t* kin, const uint16_t* vin
     }
     __syncthreads();
 }
+static_assert(kGenNT == 256, "gen_sort_pass: one thread per digit");
 
-// last piece whose start is <= r (pieces of zero length share starts)
-FP_DEV int piece_of(const UnitSmem& S, int np, int r)
+// One piece per block: sort the records by key (stable, 8-bit LSD passes in
+// shared memory); nearest smaller index on each side along the key order
+// (min-tree walks over one representative per run of equal keys).  The deeper
+// of the levels shared with those two neighbours, plus one, is lambda unless
+// the record is the minimum of its piece, whose lambda comes from the split
+// tree; deep subtrees of inner pieces by binary search on the sorted keys.
+FP_DEV void general_piece(const OctCtx& c, GenSmem& S, const Piece& pc)
 {
-    int a = 0, b = np;
-    while (a < b) {
-        int m = (a + b) >> 1;
-        if ((int)S.psrt[m] <= r) a = m + 1;
-        else b = m;
-    }
-    return a - 1;
-}
-
-// last piece whose table-phase start is <= r
-FP_DEV int piece_of_tab(const UnitSmem& S, int np, int r)
-{
-    int a = 0, b = np;
-    while (a < b) {
-        int m = (a + b) >> 1;
-        if ((int)S.pfst[m] <= r) a = m + 1;
-        else b = m;
-    }
-    return a - 1;
-}
-
-// One CTA per window of kWindow record positions: the pieces starting in it.
-// Per unit:
-//   sort the records by key (stable, 8-bit LSD passes in shared memory);
-//   nearest smaller index on each side along the key order (min-tree walks
-//   over one representative per run of equal keys).  The deeper of the levels
-//   shared with those two neighbours, plus one, is lambda unless the record is
-//   the minimum of its piece, whose lambda comes from the split tree;
-//   deep subtrees of inner pieces by binary search on the sorted keys.
-// first piece of every unit: lower bound of the unit's window start over the sorted piece begins
-__global__ void k_unit_ranges(const uint64_t* piece_begin_sorted, const uint32_t* npieces, uint32_t cap,
-                              uint64_t nunits, uint32_t* unit_p0)
-{
-    uint64_t u = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (u > nunits) return;
-    const uint32_t np_all = *npieces < cap ? *npieces : cap;
-    const uint64_t w = u * kWindow;
-    uint32_t a = 0, b = np_all;
-    while (a < b) { uint32_t m = (a + b) >> 1; if (piece_begin_sorted[m] < w) a = m + 1; else b = m; }
-    unit_p0[u] = a;
-}
-
-// Per-window piece descriptors, one warp per window, ahead of k_units (which
-// then reads them with one load per piece instead of waiting, every warp of a
-// CTA, on the piece loads and two block scans).  Pieces in window order:
-//   kind 0: one point; 1: 2..32 points, not inner; 2: general path (larger, or
-//   inner); 3: more than kPieceMax equal keys (k_dup_pieces); 4: table path --
-//   a kind-2 piece, not inner, whose lambda is decided within kTabLevels levels,
-//   while the tables of the candidates up to it fit in kTabCap entries.
-// pdesc[p] = {begin, pn | psrt << 16, pcnt | pfst << 16, ptab | q << 16 | hier << 24},
-// pdesc2[p] = A | kind << 8 | D << 16 (p = window's first piece + index);
-// uhead[u] = {first piece, pieces, general records | table records << 16,
-//             table entries | deepest needed level << 16 | smallest sorted level << 24}.
-__global__ void __launch_bounds__(256) k_unit_desc(OctCtx c, const uint32_t* unit_p0, const uint32_t* piece_order,
-                                                   uint64_t nunits, uint4* pdesc, uint32_t* pdesc2, uint4* uhead)
-{
-    const int lane = threadIdx.x & 31;
-    const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    constexpr uint32_t kSat = (uint32_t)kTabCap + 1u;   // table prefixes saturate here (past it nothing fits)
-    for (uint64_t u = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < nunits; u += nw) {
-        const uint32_t p0 = unit_p0[u], np = unit_p0[u + 1] - p0;
-        uint32_t tcarry = 0, rcarry = 0, dmax = 0, smin = 255;
-        for (uint32_t b0 = 0; b0 < np; b0 += 32) {   // warp-uniform
-            const uint32_t pi = b0 + lane;
-            const bool valid = pi < np;
-            Piece p{};
-            if (valid) p = c.pieces[piece_order[p0 + pi]];
-            uint32_t kind = 0, tz = 0, D = 0;
-            bool cand = false;
-            if (valid) {
-                const bool large = !p.dup && (p.count > 32 || p.hier == kInner);
-                kind = p.dup ? 3u : (large ? 2u : (p.count == 1 ? 0u : 1u));
-                if (large && p.hier != kInner) {
-                    const int Dv = min(kKeyLevels, c.s + (int)p.hier - 1) - (int)p.q;
-                    if (Dv <= kTabLevels) { cand = true; tz = tab_size(Dv); D = (uint32_t)max(Dv, 0); }
-                }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int cnt = (int)pc.count;
+    const int dl = pc.hier == kInner ? c.dl : min(kKeyLevels, c.s + (int)pc.hier - 1);
+    {
+        uint64_t mn = ~0ull, mx = 0;
+        constexpr int kPer = kPieceMax / kGenNT;   // records per thread
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) {
+            const int r = threadIdx.x + q * kGenNT;
+            if (r < cnt) {
+                const uint4 rec = get_rec(c, (uint64_t)pc.begin + r);
+                const uint64_t k = rec_key(rec);
+                S.key[r] = k;
+                S.j[r] = rec.z;
+                S.v[r] = (uint16_t)r;
+                mn = min(mn, k);
+                mx = max(mx, k);
             }
-            uint32_t inc = tz;   // saturating inclusive scan of the candidates' table sizes
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
-                if (lane >= o) inc = min(inc + y, kSat);
-            }
-            uint32_t tex = __shfl_up_sync(0xFFFFFFFFu, inc, 1);
-            tex = min(tcarry + (lane ? tex : 0u), kSat);
-            uint32_t cn = 0, fn = 0, ptab = 0;
-            if (valid && kind == 2) {
-                if (cand && tex + tz <= (uint32_t)kTabCap) {
-                    kind = 4;
-                    ptab = tex;
-                    fn = p.count;
-                } else {
-                    cn = p.count;
-                    const uint32_t d = p.hier == kInner ? (uint32_t)c.dl
-                                                        : (uint32_t)min(kKeyLevels, c.s + (int)p.hier - 1);
-                    dmax = max(dmax, d);
-                    smin = min(smin, (uint32_t)p.srt);
-                }
-            }
-            uint32_t inc2 = cn | (fn << 16);   // records of both paths, in window order
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc2, o);
-                if (lane >= o) inc2 += y;
-            }
-            uint32_t ex = __shfl_up_sync(0xFFFFFFFFu, inc2, 1);
-            ex = rcarry + (lane ? ex : 0u);
-            if (valid) {
-                const uint32_t pn = p.dup ? 0u : p.count;
-                pdesc[p0 + pi] = make_uint4(p.begin, pn | (ex << 16), cn | ((ex >> 16) << 16),
-                                            ptab | ((uint32_t)p.q << 16) | ((uint32_t)p.hier << 24));
-                pdesc2[p0 + pi] = (uint32_t)p.A | (kind << 8) | (D << 16);
-            }
-            tcarry = min(tcarry + __shfl_sync(0xFFFFFFFFu, inc, 31), kSat);
-            rcarry += __shfl_sync(0xFFFFFFFFu, inc2, 31);
         }
-        dmax = __reduce_max_sync(0xFFFFFFFFu, dmax);
-        smin = __reduce_min_sync(0xFFFFFFFFu, smin);
-        if (lane == 0)
-            uhead[u] = make_uint4(p0, np, rcarry, min(tcarry, (uint32_t)kTabCap) | (dmax << 16) | (smin << 24));
+        for (int o = 16; o > 0; o >>= 1) {
+            mn = min(mn, (uint64_t)__shfl_xor_sync(0xFFFFFFFFu, (unsigned long long)mn, o));
+            mx = max(mx, (uint64_t)__shfl_xor_sync(0xFFFFFFFFu, (unsigned long long)mx, o));
+        }
+        if (lane == 0) { S.wmin[warp] = mn; S.wmax[warp] = mx; }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 0; w < kGenWarps; ++w) { mn = min(mn, S.wmin[w]); mx = max(mx, S.wmax[w]); }
+            S.kmin = mn;
+            S.kmax = mx;
+        }
     }
+    __syncthreads();
+    const int clev = common_level(S.kmin, S.kmax);
+    const int lo_bit = 3 * (kKeyLevels - max(dl, clev));
+    {
+        // records already in key order down to the needed depth need no sort
+        const int hi_bit = (int)pc.srt >= max(dl, clev) ? 0 : 3 * (kKeyLevels - clev);
+        bool in_key = true;
+        for (int sh = lo_bit; sh < hi_bit; sh += 8) {
+            if (in_key) gen_sort_pass(S, S.key, S.v, S.key2, S.v2, cnt, sh);
+            else gen_sort_pass(S, S.key2, S.v2, S.key, S.v, cnt, sh);
+            in_key = !in_key;
+        }
+        if (!in_key) {
+            for (int r = threadIdx.x; r < cnt; r += kGenNT) { S.key[r] = S.key2[r]; S.v[r] = S.v2[r]; }
+        }
+    }
+    __syncthreads();
+    // ---- runs: records equal down to the sorted depth share every cell down
+    // to that depth, so only the smallest index of a run can be the minimum of
+    // any of those cells and the others inherit "never" (lambda beyond the
+    // depth).  The search below runs over one representative per run: the
+    // run's smallest index, with the run's key.
+    {
+        constexpr int per_h = kPieceMax / kGenNT;   // records per thread, contiguous
+        const int h0 = threadIdx.x * per_h;
+        uint32_t flags = 0, cntf = 0;
+        for (int q = 0; q < per_h; ++q) {
+            const int r = h0 + q;
+            bool head = false;
+            if (r < cnt) head = r == 0 || ((S.key[r] ^ S.key[r - 1]) >> lo_bit) != 0;
+            flags |= (uint32_t)head << q;
+            cntf += head;
+        }
+        uint32_t tot;
+        const uint32_t ex0 = block_exclusive_scan<kGenNT, uint32_t>(cntf, S.scan, tot);
+        for (uint32_t x = threadIdx.x; x < tot; x += kGenNT) S.hj[x] = 0xFFFFFFFFu;
+        __syncthreads();
+        int run = (int)ex0 - 1;   // run of the record before this thread's block
+        uint32_t mn = 0xFFFFFFFFu;
+        for (int q = 0; q < per_h; ++q) {
+            const int r = h0 + q;
+            if (r >= cnt) break;
+            if ((flags >> q) & 1u) {
+                if (run >= 0 && mn != 0xFFFFFFFFu) atomicMin(&S.hj[run], mn);
+                ++run;
+                mn = 0xFFFFFFFFu;
+                S.key2[run] = S.key[r];
+            }
+            S.hid[r] = (uint16_t)run;
+            mn = min(mn, S.j[S.v[r]]);
+        }
+        if (run >= 0 && mn != 0xFFFFFFFFu) atomicMin(&S.hj[run], mn);
+        if (threadIdx.x == 0) S.nh = tot;
+    }
+    __syncthreads();
+    const int nh = (int)S.nh;
+    // ---- nearest smaller index on each side of every representative, by a
+    // min-tree over hj (the leaves are hj itself, padded to a power of two
+    // P >= 32): climb to the first sibling subtree that holds a smaller
+    // index, then descend into it towards the near side.  The five levels
+    // above the leaves are built per warp with shuffles, the rest by one
+    // warp.  The level shared with that neighbour is the deepest level at
+    // which the representative is not its cell's minimum on that side (keys
+    // are sorted, so nearer records share at least as many levels).
+    int P = 32;
+    while (P < nh) P <<= 1;
+    for (int b = warp; b < (P >> 5); b += kGenWarps) {
+        const int i = (b << 5) + lane;
+        uint32_t v = i < nh ? S.hj[i] : 0xFFFFFFFFu;
+#pragma unroll
+        for (int t = 1; t <= 5; ++t) {
+            v = min(v, __shfl_xor_sync(0xFFFFFFFFu, v, 1 << (t - 1)));
+            if ((lane & ((1 << t) - 1)) == 0) S.mt[(P + i) >> t] = v;
+        }
+    }
+    __syncthreads();
+    if (warp == 0) {
+        for (int m = P >> 6; m >= 1; m >>= 1) {
+            for (int k = m + lane; k < 2 * m; k += 32) S.mt[k] = min(S.mt[2 * k], S.mt[2 * k + 1]);
+            __syncwarp();
+        }
+    }
+    __syncthreads();
+    auto tv = [&](int k) -> uint32_t {
+        return k >= P ? (k - P < nh ? S.hj[k - P] : 0xFFFFFFFFu) : S.mt[k];
+    };
+    for (int r = threadIdx.x; r < nh; r += kGenNT) {
+        const uint32_t jr = S.hj[r];
+        const uint64_t kr = S.key2[r];
+        int left = -1, right = -1;
+        for (int k = P + r; k > 1; k >>= 1) {
+            if ((k & 1) && tv(k - 1) < jr) {
+                k = k - 1;
+                while (k < P) k = tv(2 * k + 1) < jr ? 2 * k + 1 : 2 * k;
+                left = k - P;
+                break;
+            }
+        }
+        for (int k = P + r; k > 1; k >>= 1) {
+            if (!(k & 1) && tv(k + 1) < jr) {
+                k = k + 1;
+                while (k < P) k = tv(2 * k) < jr ? 2 * k : 2 * k + 1;
+                right = k - P;
+                break;
+            }
+        }
+        S.cl[r] = left >= 0 ? (uint8_t)common_level(kr, S.key2[left]) : (uint8_t)255;
+        S.cr[r] = right >= 0 ? (uint8_t)common_level(kr, S.key2[right]) : (uint8_t)255;
+    }
+    // ---- deep subtree of a piece whose node is still inner (one warp)
+    if (warp == 0 && pc.hier == kInner) {
+        int st_b[8 * 22], st_e[8 * 22], st_l[8 * 22];   // used by lane 0 only
+        int sp = 0;
+        if (lane == 0) { st_b[0] = 0; st_e[0] = cnt; st_l[0] = pc.q; sp = 1; }
+        for (;;) {
+            int nb_ = 0, ne_ = 0, L = 0, more = 0;
+            if (lane == 0 && sp > 0) { --sp; nb_ = st_b[sp]; ne_ = st_e[sp]; L = st_l[sp]; more = 1; }
+            more = __shfl_sync(0xFFFFFFFFu, more, 0);
+            if (!more) break;
+            nb_ = __shfl_sync(0xFFFFFFFFu, nb_, 0);
+            ne_ = __shfl_sync(0xFFFFFFFFu, ne_, 0);
+            L = __shfl_sync(0xFFFFFFFFu, L, 0);
+            const int L1 = L + 1;
+            const int sh = 3 * (kKeyLevels - L1);
+            int lo = ne_;
+            if (lane <= 8) {   // lane d: first position whose child digit is >= d
+                int a2 = nb_, b2 = ne_;
+                while (a2 < b2) {
+                    int mid = (a2 + b2) >> 1;
+                    if ((int)((S.key[mid] >> sh) & 7) < lane) a2 = mid + 1;
+                    else b2 = mid;
+                }
+                lo = a2;
+            }
+            for (int d = 0; d < 8; ++d) {
+                const int cb = __shfl_sync(0xFFFFFFFFu, lo, d);
+                const int ce = __shfl_sync(0xFFFFFFFFu, lo, d + 1);
+                const int cn = ce - cb;
+                if (cn <= 0) continue;
+                const bool leaf = (uint64_t)cn <= c.C || L1 == c.lmax;
+                if (lane == 0) {
+                    emit_node(c, S.key[cb] >> sh, L1, (uint32_t)cn, pc.begin + (uint32_t)cb, leaf);
+                    if (!leaf && sp < 8 * 22) { st_b[sp] = cb; st_e[sp] = ce; st_l[sp] = L1; ++sp; }
+                }
+                if (leaf)
+                    for (int r = cb + lane; r < ce; r += 32) S.leaf[r] = (uint8_t)L1;
+            }
+        }
+    }
+    __syncthreads();
+    // ---- owner level and leaf level of every record
+    for (int r = threadIdx.x; r < cnt; r += kGenNT) {
+        const int vv = S.v[r];
+        const int h = S.hid[r];
+        int lm = kKeyLevels;   // not its run's minimum: shares the sorted depth with a smaller index
+        if (S.j[vv] == S.hj[h]) {
+            const int ql = S.cl[h] == 255 ? -1 : (int)S.cl[h];
+            const int qr = S.cr[h] == 255 ? -1 : (int)S.cr[h];
+            lm = max(ql, qr);
+        }
+        const int lambda = lm < (int)pc.q ? (int)pc.A : lm + 1;   // the piece minimum: from the split tree
+        const int leafl = pc.hier == kInner ? (int)S.leaf[r] : (int)pc.hier;
+        put_lambda(c, S.j[vv], lambda, leafl, (uint32_t)(S.key[r] >> (3 * (kKeyLevels - c.g))));
+    }
+    __syncthreads();
 }
 
-__global__ void __launch_bounds__(kUnitNT, 2) k_units(OctCtx c, const uint4* uhead, const uint4* pdesc,
-                                                      const uint32_t* pdesc2, uint64_t n)
+// the general pieces, then the oversized ones (more than kPieceMax identical keys
+// down to the deepest needed level): only their smallest index can be a minimum
+__global__ void __launch_bounds__(kGenNT) k_general_pieces(OctCtx c)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    UnitSmem& S = *reinterpret_cast<UnitSmem*>(smem_raw);
-    const uint64_t nunits = (n + kWindow - 1) / kWindow;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint4 hn = blockIdx.x < nunits ? uhead[blockIdx.x] : make_uint4(0, 0, 0, 0);
-    for (uint64_t u = blockIdx.x; u < nunits; u += gridDim.x) {
-        // piece descriptors of the window (k_unit_desc); the next window's
-        // header is in flight while this one is worked on
-        {
-            const uint4 h = hn;
-            if (u + gridDim.x < nunits) hn = uhead[u + gridDim.x];
-            if (threadIdx.x == 0) {
-                S.p0 = h.x;
-                S.np = h.y;
-                S.cnt = h.z & 0xFFFFu;
-                S.fcnt = h.z >> 16;
-                S.tabn = h.w & 0xFFFFu;
-                S.dl = (h.w >> 16) & 0xFFu;
-                S.smin = h.w >> 24;
-            }
-            for (int pi = threadIdx.x; pi < (int)h.y; pi += kUnitNT) {
-                const uint4 d = pdesc[h.x + pi];
-                const uint32_t d2 = pdesc2[h.x + pi];
-                S.pbeg[pi] = d.x;
-                S.pn[pi] = (uint16_t)(d.y & 0xFFFFu);
-                S.psrt[pi] = (uint16_t)(d.y >> 16);
-                S.pcnt[pi] = (uint16_t)(d.z & 0xFFFFu);
-                S.pfst[pi] = (uint16_t)(d.z >> 16);
-                S.ptab[pi] = (uint16_t)(d.w & 0xFFFFu);
-                S.pq[pi] = (uint8_t)(d.w >> 16);
-                S.phier[pi] = (uint8_t)(d.w >> 24);
-                S.pA[pi] = (uint8_t)d2;
-                S.pkind[pi] = (uint8_t)(d2 >> 8);
-                S.pD[pi] = (uint8_t)(d2 >> 16);
-            }
-        }
-        __syncthreads();
-        const int np = (int)S.np;
-        // ---- pieces of one point: the point is its piece's minimum
-        for (int pi = threadIdx.x; pi < np; pi += kUnitNT) {
-            if (S.pkind[pi] != 0) continue;
-            const uint4 rr = get_rec(c, S.pbeg[pi]);
-            const int leafl = S.phier[pi];
-            int K = (int)S.pA[pi] - c.s;
-            K = K < 0 ? 0 : (K > leafl ? leafl : K);
-            put_code(c, rr.z, K, leafl, rec_key(rr));
-        }
-        // ---- pieces of 2..32 points: lambda from the deepest level shared with any
-        // point of smaller index in the piece (all pairs, by shuffles); a warp
-        // loads the records of kSmallB of its pieces before working on them
-        constexpr int kSmallB = 4;
-        for (int pb = warp; pb < np; pb += kUnitWarps * kSmallB) {
-            uint64_t kb[kSmallB];
-            uint32_t jb[kSmallB];
-            int nb[kSmallB];
-#pragma unroll
-            for (int t = 0; t < kSmallB; ++t) {
-                const int pi = pb + t * kUnitWarps;
-                nb[t] = pi < np && S.pkind[pi] == 1 ? (int)S.pn[pi] : 0;
-                kb[t] = 0;
-                jb[t] = 0xFFFFFFFFu;
-                if (lane < nb[t]) {
-                    const uint4 r = get_rec(c, S.pbeg[pi] + lane);
-                    kb[t] = rec_key(r);
-                    jb[t] = r.z;
-                }
-            }
-#pragma unroll
-            for (int t = 0; t < kSmallB; ++t) {
-                const int cnum = nb[t];   // warp-uniform
-                if (cnum == 0) continue;
-                const int pi = pb + t * kUnitWarps;
-                const uint64_t k = kb[t];
-                const uint32_t jj = jb[t];
-                int lm = -1;
-                for (int q = 0; q < cnum; ++q) {
-                    const uint64_t kt = __shfl_sync(0xFFFFFFFFu, k, q);
-                    const uint32_t jt = __shfl_sync(0xFFFFFFFFu, jj, q);
-                    if (jt < jj) lm = max(lm, common_level(k, kt));
-                }
-                if (lane < cnum) {
-                    const int q0 = S.pq[pi];
-                    const int lambda = lm < q0 ? (int)S.pA[pi] : lm + 1;
-                    const int leafl = S.phier[pi];
-                    int K = lambda - c.s;
-                    K = K < 0 ? 0 : (K > leafl ? leafl : K);
-                    put_code(c, jj, K, leafl, k);
-                }
-            }
-        }
-        // ---- table pieces: per-level smallest index of every occupied cell
-        if (S.fcnt) {
-            const int fcnt = (int)S.fcnt;
-            uint32_t* tab = reinterpret_cast<uint32_t*>(S.key);
-            const int tabn4 = (int)((S.tabn + 3u) >> 2);
-            for (int x = threadIdx.x; x < tabn4; x += kUnitNT)
-                reinterpret_cast<uint4*>(tab)[x] = make_uint4(kNone, kNone, kNone, kNone);
-            for (int pi = threadIdx.x; pi < np; pi += kUnitNT)
-                if (S.pkind[pi] == 4) S.pmin[pi] = kNone;
-            constexpr int kPer = kUnitCap / kUnitNT;
-            uint32_t gi[kPer], jq[kPer];
-            uint64_t kq[kPer];
-            int pp[kPer];
-#pragma unroll
-            for (int q = 0; q < kPer; ++q) {
-                const int r = threadIdx.x + q * kUnitNT;
-                pp[q] = -1;
-                gi[q] = 0;
-                if (r < fcnt) {
-                    pp[q] = piece_of_tab(S, np, r);
-                    gi[q] = S.pbeg[pp[q]] + (uint32_t)(r - S.pfst[pp[q]]);
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < kPer; ++q)   // all loads in flight together
-                if (pp[q] >= 0) {
-                    const uint4 r = get_rec(c, gi[q]);
-                    kq[q] = rec_key(r);
-                    jq[q] = r.z;
-                }
-            __syncthreads();   // tables cleared
-            // deepest level first: a record that finds a smaller index in its cell
-            // stops (that index lies in every coarser cell too); a cell's minimum
-            // never does, so every cell ends with its minimum
-#pragma unroll
-            for (int q = 0; q < kPer; ++q) {
-                if (pp[q] < 0) continue;
-                const int pi = pp[q], D = S.pD[pi], q0 = S.pq[pi];
-                const uint32_t jv = jq[q];
-                bool least = true;
-                for (int d = D; d >= 1 && least; --d) {
-                    const uint32_t idx = (uint32_t)(kq[q] >> (3 * (kKeyLevels - q0 - d))) & ((1u << (3 * d)) - 1u);
-                    uint32_t* t = &tab[S.ptab[pi] + tab_size(d - 1) + idx];
-                    if (*t < jv) least = false;
-                    else atomicMin(t, jv);
-                }
-                if (least && S.pmin[pi] > jv) atomicMin(&S.pmin[pi], jv);
-            }
-            __syncthreads();
-#pragma unroll
-            for (int q = 0; q < kPer; ++q) {
-                if (pp[q] < 0) continue;
-                const int pi = pp[q], D = S.pD[pi], q0 = S.pq[pi];
-                int lambda = kKeyLevels + 1;   // never its cell's minimum down to the piece's depth
-                if (jq[q] == S.pmin[pi]) {
-                    lambda = S.pA[pi];           // the piece minimum: from the split tree
-                } else {
-                    uint32_t off = S.ptab[pi];
-                    for (int d = 1; d <= D; ++d) {
-                        const uint32_t idx =
-                            (uint32_t)(kq[q] >> (3 * (kKeyLevels - q0 - d))) & ((1u << (3 * d)) - 1u);
-                        if (tab[off + idx] == jq[q]) { lambda = q0 + d; break; }
-                        off += 1u << (3 * d);
-                    }
-                }
-                const int leafl = S.phier[pi];
-                int K = lambda - c.s;
-                K = K < 0 ? 0 : (K > leafl ? leafl : K);
-                put_code(c, jq[q], K, leafl, kq[q]);
-            }
-            __syncthreads();   // the tables overlay the general path's arrays
-        }
-        const int cnt = (int)S.cnt;
-        if (cnt == 0) { __syncthreads(); continue; }
-        // records; local index = position in load order
-        {
-            uint64_t mn = ~0ull, mx = 0;
-            constexpr int kPer = kUnitCap / kUnitNT;   // records per thread
-            uint32_t gi[kPer];
-#pragma unroll
-            for (int q = 0; q < kPer; ++q) {
-                const int r = threadIdx.x + q * kUnitNT;
-                gi[q] = 0;
-                if (r < cnt) {
-                    const int pi = piece_of(S, np, r);
-                    gi[q] = S.pbeg[pi] + (uint32_t)(r - S.psrt[pi]);
-                    S.v[r] = (uint16_t)r;
-                    S.piece[r] = (uint16_t)pi;
-                }
-            }
-            uint64_t kq[kPer];
-            uint32_t jq[kPer];
-#pragma unroll
-            for (int q = 0; q < kPer; ++q)   // all loads in flight together
-                if ((int)threadIdx.x + q * kUnitNT < cnt) {
-                    const uint4 r = get_rec(c, gi[q]);
-                    kq[q] = rec_key(r);
-                    jq[q] = r.z;
-                }
-#pragma unroll
-            for (int q = 0; q < kPer; ++q) {
-                const int r = threadIdx.x + q * kUnitNT;
-                if (r < cnt) {
-                    S.key[r] = kq[q];
-                    S.j[r] = jq[q];
-                    mn = min(mn, kq[q]);
-                    mx = max(mx, kq[q]);
-                }
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                mn = min(mn, (uint64_t)__shfl_xor_sync(0xFFFFFFFFu, (unsigned long long)mn, o));
-                mx = max(mx, (uint64_t)__shfl_xor_sync(0xFFFFFFFFu, (unsigned long long)mx, o));
-            }
-            if (lane == 0) { S.wmin[warp] = mn; S.wmax[warp] = mx; }
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                for (int w = 1; w < kUnitWarps; ++w) { mn = min(mn, S.wmin[w]); mx = max(mx, S.wmax[w]); }
-                mn = min(mn, S.wmin[0]); mx = max(mx, S.wmax[0]);
-                S.kmin = mn;
-                S.kmax = mx;
-            }
-        }
-        __syncthreads();
-        {
-            const int dl_unit = (int)S.dl;
-            const int clev = common_level(S.kmin, S.kmax);
-            // records already in key order down to the needed depth (every large
-            // piece sorted that deep; pieces lie in key order) need no sort
-            const int hi_bit = (int)S.smin >= max(dl_unit, clev) ? 0 : 3 * (kKeyLevels - clev);
-            const int lo_bit = 3 * (kKeyLevels - max(dl_unit, clev));
-            bool in_key = true;
-            for (int sh = lo_bit; sh < hi_bit; sh += 8) {
-                if (in_key) unit_sort_pass(S, S.key, S.v, S.key2, S.v2, cnt, sh);
-                else unit_sort_pass(S, S.key2, S.v2, S.key, S.v, cnt, sh);
-                in_key = !in_key;
-            }
-            if (!in_key) {
-                for (int r = threadIdx.x; r < cnt; r += kUnitNT) { S.key[r] = S.key2[r]; S.v[r] = S.v2[r]; }
-            }
-        }
-        __syncthreads();
-        // ---- runs: records equal down to the sorted depth share every cell down
-        // to that depth, so only the smallest index of a run can be the minimum of
-        // any of those cells and the others inherit "never" (lambda beyond the
-        // depth).  The search below runs over one representative per run: the
-        // run's smallest index, with the run's key.
-        int lo_bit_u = 0;
-        {
-            const int dl_unit = (int)S.dl;
-            const int clev = common_level(S.kmin, S.kmax);
-            lo_bit_u = 3 * (kKeyLevels - max(dl_unit, clev));
-        }
-        {
-            constexpr int per_h = kUnitCap / kUnitNT;   // records per thread, contiguous
-            const int h0 = threadIdx.x * per_h;
-            uint32_t flags = 0, cntf = 0;
-            for (int q = 0; q < per_h; ++q) {
-                const int r = h0 + q;
-                bool head = false;
-                if (r < cnt) head = r == 0 || ((S.key[r] ^ S.key[r - 1]) >> lo_bit_u) != 0;
-                flags |= (uint32_t)head << q;
-                cntf += head;
-            }
-            uint32_t tot;
-            const uint32_t ex0 = block_exclusive_scan<kUnitNT, uint32_t>(cntf, S.scan, tot);
-            for (uint32_t x = threadIdx.x; x < tot; x += kUnitNT) S.hj[x] = 0xFFFFFFFFu;
-            __syncthreads();
-            int run = (int)ex0 - 1;   // run of the record before this thread's block
-            uint32_t mn = 0xFFFFFFFFu;
-            for (int q = 0; q < per_h; ++q) {
-                const int r = h0 + q;
-                if (r >= cnt) break;
-                if ((flags >> q) & 1u) {
-                    if (run >= 0 && mn != 0xFFFFFFFFu) atomicMin(&S.hj[run], mn);
-                    ++run;
-                    mn = 0xFFFFFFFFu;
-                    S.key2[run] = S.key[r];
-                }
-                S.hid[r] = (uint16_t)run;
-                mn = min(mn, S.j[S.v[r]]);
-            }
-            if (run >= 0 && mn != 0xFFFFFFFFu) atomicMin(&S.hj[run], mn);
-            if (threadIdx.x == 0) S.nh = tot;
-        }
-        __syncthreads();
-        const int nh = (int)S.nh;
-        // ---- nearest smaller index on each side of every representative, by a
-        // min-tree over hj (the leaves are hj itself, padded to a power of two
-        // P >= 32): climb to the first sibling subtree that holds a smaller
-        // index, then descend into it towards the near side.  The five levels
-        // above the leaves are built per warp with shuffles, the rest by one
-        // warp.  The level shared with that neighbour is the deepest level at
-        // which the representative is not its cell's minimum on that side (keys
-        // are sorted, so nearer records share at least as many levels).
-        int P = 32;
-        while (P < nh) P <<= 1;
-        for (int b = warp; b < (P >> 5); b += kUnitWarps) {
-            const int i = (b << 5) + lane;
-            uint32_t v = i < nh ? S.hj[i] : 0xFFFFFFFFu;
-#pragma unroll
-            for (int t = 1; t <= 5; ++t) {
-                v = min(v, __shfl_xor_sync(0xFFFFFFFFu, v, 1 << (t - 1)));
-                if ((lane & ((1 << t) - 1)) == 0) S.mt[(P + i) >> t] = v;
-            }
-        }
-        __syncthreads();
-        if (warp == 0) {
-            for (int m = P >> 6; m >= 1; m >>= 1) {
-                for (int k = m + lane; k < 2 * m; k += 32) S.mt[k] = min(S.mt[2 * k], S.mt[2 * k + 1]);
-                __syncwarp();
-            }
-        }
-        __syncthreads();
-        auto tv = [&](int k) -> uint32_t {
-            return k >= P ? (k - P < nh ? S.hj[k - P] : 0xFFFFFFFFu) : S.mt[k];
-        };
-        for (int r = threadIdx.x; r < nh; r += kUnitNT) {
-            const uint32_t jr = S.hj[r];
-            const uint64_t kr = S.key2[r];
-            int left = -1, right = -1;
-            for (int k = P + r; k > 1; k >>= 1) {
-                if ((k & 1) && tv(k - 1) < jr) {
-                    k = k - 1;
-                    while (k < P) k = tv(2 * k + 1) < jr ? 2 * k + 1 : 2 * k;
-                    left = k - P;
-                    break;
-                }
-            }
-            for (int k = P + r; k > 1; k >>= 1) {
-                if (!(k & 1) && tv(k + 1) < jr) {
-                    k = k + 1;
-                    while (k < P) k = tv(2 * k) < jr ? 2 * k : 2 * k + 1;
-                    right = k - P;
-                    break;
-                }
-            }
-            S.cl[r] = left >= 0 ? (uint8_t)common_level(kr, S.key2[left]) : (uint8_t)255;
-            S.cr[r] = right >= 0 ? (uint8_t)common_level(kr, S.key2[right]) : (uint8_t)255;
-        }
-        __syncthreads();
-        // ---- deep subtrees inside pieces whose node is still inner: one warp per piece
-        for (int pi = warp; pi < np; pi += kUnitWarps) {
-            if (S.phier[pi] != kInner || S.pcnt[pi] == 0) continue;
-            const int ps0 = S.psrt[pi], pn = S.pcnt[pi];
-            int st_b[8 * 22], st_e[8 * 22], st_l[8 * 22];   // used by lane 0 only
-            int sp = 0;
-            if (lane == 0) { st_b[0] = ps0; st_e[0] = ps0 + pn; st_l[0] = S.pq[pi]; sp = 1; }
-            for (;;) {
-                int nb_ = 0, ne_ = 0, L = 0, more = 0;
-                if (lane == 0 && sp > 0) { --sp; nb_ = st_b[sp]; ne_ = st_e[sp]; L = st_l[sp]; more = 1; }
-                more = __shfl_sync(0xFFFFFFFFu, more, 0);
-                if (!more) break;
-                nb_ = __shfl_sync(0xFFFFFFFFu, nb_, 0);
-                ne_ = __shfl_sync(0xFFFFFFFFu, ne_, 0);
-                L = __shfl_sync(0xFFFFFFFFu, L, 0);
-                const int L1 = L + 1;
-                const int sh = 3 * (kKeyLevels - L1);
-                int lo = ne_;
-                if (lane <= 8) {   // lane d: first position whose child digit is >= d
-                    int a2 = nb_, b2 = ne_;
-                    while (a2 < b2) {
-                        int mid = (a2 + b2) >> 1;
-                        if ((int)((S.key[mid] >> sh) & 7) < lane) a2 = mid + 1;
-                        else b2 = mid;
-                    }
-                    lo = a2;
-                }
-                for (int d = 0; d < 8; ++d) {
-                    const int cb = __shfl_sync(0xFFFFFFFFu, lo, d);
-                    const int ce = __shfl_sync(0xFFFFFFFFu, lo, d + 1);
-                    const int cn = ce - cb;
-                    if (cn <= 0) continue;
-                    const bool leaf = (uint64_t)cn <= c.C || L1 == c.lmax;
-                    if (lane == 0) {
-                        emit_node(c, S.key[cb] >> sh, L1, (uint32_t)cn, S.pbeg[pi] + (uint32_t)(cb - ps0), leaf);
-                        if (!leaf && sp < 8 * 22) { st_b[sp] = cb; st_e[sp] = ce; st_l[sp] = L1; ++sp; }
-                    }
-                    if (leaf)
-                        for (int r = cb + lane; r < ce; r += 32) S.leaf[r] = (uint8_t)L1;
-                }
-            }
-        }
-        __syncthreads();
-        // ---- owner level and leaf level of every record
-        for (int r = threadIdx.x; r < cnt; r += kUnitNT) {
-            const int vv = S.v[r];
-            const int pi = S.piece[vv];
-            const int h = S.hid[r];
-            int lm = kKeyLevels;   // not its run's minimum: shares the sorted depth with a smaller index
-            if (S.j[vv] == S.hj[h]) {
-                const int ql = S.cl[h] == 255 ? -1 : (int)S.cl[h];
-                const int qr = S.cr[h] == 255 ? -1 : (int)S.cr[h];
-                lm = max(ql, qr);
-            }
-            const int q = S.pq[pi];
-            const int lambda = lm < q ? (int)S.pA[pi] : lm + 1;   // the piece minimum: from the split tree
-            const int leafl = S.phier[pi] == kInner ? (int)S.leaf[r] : (int)S.phier[pi];
-            int K = lambda - c.s;
-            if (K < 0) K = 0;
-            if (K > leafl) K = leafl;
-            const uint32_t jj = S.j[vv];
-            put_code(c, jj, K, leafl, S.key[r]);
-        }
-        __syncthreads();
-    }
-}
-
-// oversized pieces (more than kPieceMax identical keys down to the deepest
-// needed level): only their first record, the smallest index, can be a minimum
-__global__ void __launch_bounds__(256) k_dup_pieces(OctCtx c)
-{
-    __shared__ uint32_t s_min[8];
-    const uint32_t nd = *c.ndups < c.piece_cap ? *c.ndups : c.piece_cap;
+    GenSmem& S = *reinterpret_cast<GenSmem*>(smem_raw);
+    const uint32_t ng = min(*c.ngen, c.piece_cap);
+    for (uint32_t k = blockIdx.x; k < ng; k += gridDim.x) general_piece(c, S, c.gen[k]);
+    const uint32_t nd = min(*c.ndups, c.piece_cap);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (uint32_t k = blockIdx.x; k < nd; k += gridDim.x) {
-        const Piece p = c.pieces[c.dups[k]];
+        const Piece p = c.dups[k];
         const int leafl = p.hier == kInner ? c.lmax : (int)p.hier;
         uint32_t mn = kNone;
-        for (uint32_t r = threadIdx.x; r < p.count; r += blockDim.x) mn = min(mn, get_rec(c, (uint64_t)p.begin + r).z);
+        for (uint32_t r = threadIdx.x; r < p.count; r += kGenNT) mn = min(mn, get_rec(c, (uint64_t)p.begin + r).z);
         mn = __reduce_min_sync(0xFFFFFFFFu, mn);
-        if (lane == 0) s_min[warp] = mn;
+        if (lane == 0) S.scan[warp] = mn;
         __syncthreads();
-        mn = s_min[0];
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) mn = min(mn, s_min[w]);
-        for (uint32_t r = threadIdx.x; r < p.count; r += blockDim.x) {
+        mn = S.scan[0];
+        for (int w = 1; w < kGenWarps; ++w) mn = min(mn, S.scan[w]);
+        for (uint32_t r = threadIdx.x; r < p.count; r += kGenNT) {
             const uint4 rr = get_rec(c, (uint64_t)p.begin + r);
-            const uint32_t jj = rr.z;
-            int K = leafl;
-            if (jj == mn) {
-                K = (int)p.A - c.s;
-                if (K < 0) K = 0;
-                if (K > leafl) K = leafl;
-            }
-            put_code(c, jj, K, leafl, rec_key(rr));
+            put_lambda(c, rr.z, rr.z == mn ? (int)p.A : kKeyLevels + 1, leafl,
+                       (uint32_t)(rec_key(rr) >> (3 * (kKeyLevels - c.g))));
         }
         __syncthreads();
     }
-}
-
-__global__ void k_piece_keys(const Piece* pieces, const uint32_t* npieces, uint32_t cap, uint64_t* keys)
-{
-    uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    uint32_t np = *npieces < cap ? *npieces : cap;
-    if (i < np) keys[i] = pieces[i].begin;
 }
 
 __global__ void k_clamp(uint32_t* v, uint32_t cap)
@@ -1428,14 +1406,11 @@ struct OctBufs {
     uint4* trec;   // split rounds: the copied records with their slots
     int4* lt_pt;
     uint32_t *lt_val, *lt_k32;
-    uint32_t *pyr, *cstart, *cursor;
+    uint32_t *pyr, *rsum, *cstart, *cursor;
     uint8_t* cell_leaf;
     uint4* rec;           // cell-grouped records (rec_key, rec_j)
-    Piece* pieces;
-    uint32_t* counters;   // [0] pieces, [1] pieces of equal keys, [3] node records
-    uint32_t* dups;
-    uint64_t *pk, *pk2, *pk3;
-    uint32_t *pv, *pv2;
+    Piece* pieces[4];     // table, small, general, oversized
+    uint32_t* counters;   // [0], [1], [2], [4] their numbers, [3] node records
     OpenNode* open[2];
     uint32_t *ocount, *bigstart;
     NodeRec* nrec;
@@ -1445,9 +1420,6 @@ struct OctBufs {
     uint32_t *idxtab, *leafw, *nown;
     uint32_t* codes;
     uint32_t* leafid;
-    uint32_t* unit_p0;
-    uint4 *pdesc, *uhead;   // window descriptors (k_unit_desc)
-    uint32_t* pdesc2;
     uint32_t* ndesc;
     SegScratch seg;
 };
@@ -1457,7 +1429,7 @@ static OctBufs oct_carve(const Workspace& ws, uint64_t n, const OctLayout& Ly)
 {
     OctBufs B;
     const uint64_t N = n ? n : 1;
-    B.sc = take_sort_scratch(ws, std::max<uint64_t>(N, std::max(Ly.node_cap, Ly.piece_cap)));
+    B.sc = take_sort_scratch(ws, std::max<uint64_t>(N, Ly.node_cap));
     B.rcnt = ws.take<uint32_t>(Ly.open_cap << (3 * kRoundLevels));
     B.rmin = ws.take<uint32_t>(Ly.open_cap << (3 * kRoundLevels));
     // aliased phase region: grouping temporaries, later the leaf scatter temporaries
@@ -1468,18 +1440,15 @@ static OctBufs oct_carve(const Workspace& ws, uint64_t n, const OctLayout& Ly)
     B.lt_pt = ws.take<int4>(N); B.lt_val = ws.take<uint32_t>(N); B.lt_k32 = ws.take<uint32_t>(N);
     ws.used = std::max(phase_end, ws.used);
     B.pyr = ws.take<uint32_t>(Ly.npyr ? Ly.npyr : 1);
+    B.rsum = ws.take<uint32_t>(kGtMaxTiles);
     B.cstart = ws.take<uint32_t>(Ly.cells + 1);
     B.cursor = ws.take<uint32_t>(Ly.cells);
     B.cell_leaf = ws.take<uint8_t>(Ly.cells);
     B.rec = ws.take<uint4>(N);
-    B.pieces = ws.take<Piece>(Ly.piece_cap);
-    B.counters = ws.take<uint32_t>(4);
-    B.dups = ws.take<uint32_t>(Ly.piece_cap);
-    B.pk = ws.take<uint64_t>(Ly.piece_cap); B.pk2 = ws.take<uint64_t>(Ly.piece_cap);
-    B.pk3 = ws.take<uint64_t>(Ly.piece_cap);
-    B.pv = ws.take<uint32_t>(Ly.piece_cap); B.pv2 = ws.take<uint32_t>(Ly.piece_cap);
+    for (Piece*& p : B.pieces) p = ws.take<Piece>(Ly.piece_cap);
+    B.counters = ws.take<uint32_t>(8 + 4);
+    B.ocount = B.counters + 8;
     B.open[0] = ws.take<OpenNode>(Ly.open_cap); B.open[1] = ws.take<OpenNode>(Ly.open_cap);
-    B.ocount = ws.take<uint32_t>(4);
     B.bigstart = ws.take<uint32_t>(Ly.open_cap + 1);
     B.nrec = ws.take<NodeRec>(Ly.node_cap);
     B.nk = ws.take<uint64_t>(Ly.node_cap); B.nk2 = ws.take<uint64_t>(Ly.node_cap);
@@ -1492,10 +1461,6 @@ static OctBufs oct_carve(const Workspace& ws, uint64_t n, const OctLayout& Ly)
     B.nown = ws.take<uint32_t>(Ly.node_cap);
     B.codes = ws.take<uint32_t>(N);
     B.leafid = ws.take<uint32_t>(N);
-    B.unit_p0 = ws.take<uint32_t>((N + kWindow - 1) / kWindow + 2);
-    B.pdesc = ws.take<uint4>(Ly.piece_cap);
-    B.pdesc2 = ws.take<uint32_t>(Ly.piece_cap);
-    B.uhead = ws.take<uint4>((N + kWindow - 1) / kWindow + 1);
     B.ndesc = ws.take<uint32_t>(Ly.node_cap);
     B.seg = take_seg_scratch(ws, N, Ly.cells, 1);
     return B;
@@ -1598,43 +1563,31 @@ cudaError_t launch_octree_impl(const fp_point* sorted, const uint32_t* perm, uin
     const uint64_t N = n;
     const OctBufs B = oct_carve(ws, n, Ly);
     const SortScratch& sc = B.sc;
-    uint32_t* npieces = B.counters;
     uint32_t* nnode = B.counters + 3;
-    if ((e = cudaMemsetAsync(B.counters, 0, 4 * sizeof(uint32_t), st))) return e;
-    if ((e = cudaMemsetAsync(B.ocount, 0, 4 * sizeof(uint32_t), st))) return e;
-
-    // 1. pyramid and per-cell starts
-    for (int l = g - 1; l >= 0; --l) {
-        uint64_t np_ = 1ull << (3 * l);
-        const uint32_t* child = l + 1 == g ? counts : B.pyr + ((1ull << (3 * (l + 1))) - 1) / 7;
-        k_pyr_level<<<(unsigned)((np_ + 255) / 256), 256, 0, st>>>(child, B.pyr + (np_ - 1) / 7, np_);
-    }
-    if ((e = scan_exclusive<uint32_t, uint32_t>(rcounts, B.cstart, Ly.cells, nullptr, B.leafw, B.cstart + Ly.cells,
-                                                (uint32_t*)nullptr, st)))
-        return e;
     OctCtx c;
     c.counts = counts; c.rcounts = rcounts; c.leaf_base = grp ? grp->leaf_base : 0u;
-    c.pyr = B.pyr; c.cstart = B.cstart; c.cell_leaf = B.cell_leaf;
-    c.rec = B.rec; c.pieces = B.pieces; c.npieces = npieces; c.piece_cap = (uint32_t)Ly.piece_cap;
-    c.dups = B.dups; c.ndups = B.counters + 1;
+    c.cstart = B.cstart; c.cursor = B.cursor; c.cell_leaf = B.cell_leaf;
+    c.rec = B.rec; c.piece_cap = (uint32_t)Ly.piece_cap;
+    c.tab = B.pieces[0]; c.small = B.pieces[1]; c.gen = B.pieces[2]; c.dups = B.pieces[3];
+    c.ntab = B.counters; c.nsmall = B.counters + 1; c.ngen = B.counters + 2; c.ndups = B.counters + 4;
     c.nrec = B.nrec; c.nnode = nnode; c.node_cap_ws = (uint32_t)Ly.node_cap;
     c.codes = grp ? grp->codes : B.codes;
     c.open_cap = (uint32_t)Ly.open_cap;
     c.g = g; c.s = s; c.lmax = lmax; c.dl = dl; c.C = prm.node_capacity; c.n = N; c.err = ws.err;
 
+    // 1. the grid's levels, every cell's start, leaf level and piece, the nodes at
+    // levels <= g (a chunk group leaves those to the whole-cloud node table)
+    const int ntile = grid_tiles(g);
+    k_grid_tiles<<<ntile, kGtNT, 0, st>>>(counts, g, B.pyr, rcounts, B.rsum, nullptr, 0, B.counters, 12);
+    k_cells_open<<<ntile, kGtNT, 0, st>>>(c, B.pyr, B.rsum, 1, grp ? 0 : 1, B.cstart, B.cursor, B.open[0], B.ocount);
     // 2. group by level-g cell: (key21, j) scattered by cell id
     {
-        const int gcell = (int)std::max<uint64_t>(1, std::min<uint64_t>((Ly.cells + 255) / 256, ws.num_sms * 8ull));
-        k_cell_cursor_init<<<gcell, 256, 0, st>>>(B.cstart, Ly.cells, B.cursor, g);
         const int gs = (int)std::max<uint64_t>(1, std::min<uint64_t>((N + 255) / 256, (uint64_t)ws.num_sms * 8));
         KTimerScope kt(FP_KERNEL_CELL_GROUP, st);
         k_cell_scatter<<<gs, 256, 0, st>>>(reinterpret_cast<const int4*>(sorted), N, cube, B.cursor, B.rec, g,
                                            ws.err);
-        k_cell_check<<<gcell, 256, 0, st>>>(B.cstart, Ly.cells, B.cursor, g, ws.err);
     }
-    // 3. cells: pieces, leaf levels, open big cells
-    k_cell_setup<<<(unsigned)((Ly.cells + 255) / 256), 256, 0, st>>>(c, B.open[0], B.ocount);
-    // 4. big cells: split tree.  Rounds of up to three levels: the records of
+    // 3. big cells: split tree.  Rounds of up to three levels: the records of
     // the open nodes are grouped by their cell three levels down (one counting
     // scatter: copy out with per-(node, cell) counts, starts, scatter back),
     // which puts them in key order down to that depth; then the splits of
@@ -1666,37 +1619,17 @@ cudaError_t launch_octree_impl(const fp_point* sorted, const uint32_t* perm, uin
             q += k;
         }
     }
-    // 5. nodes at levels <= g (a chunk group leaves them to the whole-cloud node table)
-    if (!grp) {
-        uint64_t total = (Ly.cells * 8 - 1) / 7;
-        k_nodes_upper<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(c);
-    }
-    // 6. pieces in record order, then the units
+    // 4. lambda of every record: owner level and leaf level
     {
-        const uint32_t pcap = (uint32_t)Ly.piece_cap;
-        k_clamp<<<1, 1, 0, st>>>(npieces, pcap);
-        k_piece_keys<<<(pcap + 255) / 256, 256, 0, st>>>(B.pieces, npieces, pcap, B.pk);
-        int bits = 1;
-        while ((1ull << bits) <= N) ++bits;
-        if ((e = sort_plan_keys(sc, B.pk, pcap, npieces, 0, (uint32_t)bits, st))) return e;
-        SortArgs a{};
-        a.b.k64_src = B.pk; a.b.k64_tmp = B.pk2; a.b.k64_dst = B.pk3;
-        a.b.val_src = nullptr; a.b.val_tmp = B.pv2; a.b.val_dst = B.pv;
-        a.n = pcap; a.d_n = npieces; a.err = ws.err;
-        if ((e = run_sort<DIG_K64, false, true, false>(sc, a, sort_passes(bits), ws, st))) return e;
-        const size_t smem = sizeof(UnitSmem);
-        if ((e = cudaFuncSetAttribute(k_units, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
-        const uint64_t nunits = (N + kWindow - 1) / kWindow;
-        k_unit_ranges<<<(unsigned)((nunits + 1 + 255) / 256), 256, 0, st>>>(B.pk3, npieces, pcap, nunits, B.unit_p0);
-        const int gd =
-            (int)std::max<uint64_t>(1, std::min<uint64_t>((nunits * 32 + 255) / 256, (uint64_t)ws.num_sms * 8));
-        k_unit_desc<<<gd, 256, 0, st>>>(c, B.unit_p0, B.pv, nunits, B.pdesc, B.pdesc2, B.uhead);
-        int grid = (int)std::min<uint64_t>(nunits, (uint64_t)ws.num_sms * 2);
-        {
-            KTimerScope kt(FP_KERNEL_UNITS, st);
-            k_units<<<grid, kUnitNT, smem, st>>>(c, B.uhead, B.pdesc, B.pdesc2, N);
-        }
-        k_dup_pieces<<<ws.num_sms, 256, 0, st>>>(c);
+        KTimerScope kt(FP_KERNEL_UNITS, st);
+        const uint64_t blk = N / (kSmallMax + 1) + 1;   // at most that many table pieces
+        k_tab_pieces<<<(int)std::min<uint64_t>(blk, (uint64_t)ws.num_sms * kTabCtas), kTabNT, 0, st>>>(c);
+        k_small_pieces<<<(int)std::max<uint64_t>(1, std::min<uint64_t>(Ly.cells / 256, ws.num_sms * 8ull)), 256, 0,
+                         st>>>(c);
+        const size_t smem = sizeof(GenSmem);
+        if ((e = cudaFuncSetAttribute(k_general_pieces, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
+            return e;
+        k_general_pieces<<<(int)std::min<uint64_t>(blk, ws.num_sms * 4ull), kGenNT, smem, st>>>(c);
     }
     if (grp) {   // a chunk group: its nodes below level g are appended to the caller's list
         const unsigned ga = (unsigned)std::max(1, std::min(ws.num_sms * 8, (int)((Ly.node_cap + 255) / 256)));
@@ -1705,7 +1638,7 @@ cudaError_t launch_octree_impl(const fp_point* sorted, const uint32_t* perm, uin
         k_add_u32<<<1, 1, 0, st>>>(grp->num_deep, nnode, (uint32_t)Ly.node_cap);
         return cudaGetLastError();
     }
-    // 7. node table in preorder: stable sort by level, then by start at max_level resolution
+    // 5. node table in preorder: stable sort by level, then by start at max_level resolution
     {
         NodeSortBufs nb{B.nk, B.nk2, B.nk3, B.nk4, B.nl, B.nv2, B.nv3, B.slevel, B.idxtab, B.leafw, B.ndesc};
         KTimerScope kt(FP_KERNEL_NODE_TABLE, st);
@@ -1713,7 +1646,7 @@ cudaError_t launch_octree_impl(const fp_point* sorted, const uint32_t* perm, uin
             return e;
         if ((e = cudaMemsetAsync(B.nown, 0, (size_t)Ly.node_cap * sizeof(uint32_t), st))) return e;
     }
-    // 8. owner and leaf ids per distributed point, owned counts
+    // 6. owner and leaf ids per distributed point, owned counts
     {
         const int grid = (int)std::max<uint64_t>(
             1, std::min<uint64_t>((N + kResolveTile - 1) / kResolveTile, (uint64_t)ws.num_sms * 8));
@@ -1724,7 +1657,7 @@ cudaError_t launch_octree_impl(const fp_point* sorted, const uint32_t* perm, uin
                                    B.nown, g, lmax, ws.err);
         k_write_nown<<<(unsigned)((Ly.node_cap + 255) / 256), 256, 0, st>>>(nodes, nnode, node_cap, B.nown);
     }
-    // 9. leaf-grouped points: stable scatter by leaf id, chunk by chunk (every
+    // 7. leaf-grouped points: stable scatter by leaf id, chunk by chunk (every
     // leaf lies in the subtree of its points' chunk); the whole-array sort by
     // leaf id runs instead, gated on the device, when a chunk does not fit
     if (leaf_pts || leaf_perm) {
@@ -1762,7 +1695,7 @@ __global__ void k_copy_u32(uint32_t* dst, const uint32_t* src) { *dst = *src; }
 
 struct NodesBufs {
     SortScratch sc;
-    uint32_t *pyr, *cstart;
+    uint32_t *pyr, *rsum;
     NodeSortBufs nb;
 };
 
@@ -1773,7 +1706,7 @@ static NodesBufs nodes_carve(const Workspace& ws, const fp_params& p, uint64_t r
     const uint64_t R = rec_cap ? rec_cap : 1;
     B.sc = take_sort_scratch(ws, R);
     B.pyr = ws.take<uint32_t>((cells - 1) / 7 ? (cells - 1) / 7 : 1);
-    B.cstart = ws.take<uint32_t>(cells + 1);
+    B.rsum = ws.take<uint32_t>(kGtMaxTiles);
     B.nb.nk2 = ws.take<uint64_t>(R); B.nb.nk3 = ws.take<uint64_t>(R); B.nb.nk4 = ws.take<uint64_t>(R);
     B.nb.nl = ws.take<uint32_t>(R); B.nb.nv2 = ws.take<uint32_t>(R); B.nb.nv3 = ws.take<uint32_t>(R);
     B.nb.leafw = ws.take<uint32_t>(std::max<uint64_t>(R, kScanMaxTiles));
@@ -1787,30 +1720,20 @@ size_t nodes_ws_bytes(const fp_params& p, uint64_t rec_cap)
     return dry.used;
 }
 
-uint64_t upper_node_bound(const fp_params& p) { return ((1ull << (3 * p.grid_log2)) * 8 - 1) / 7; }
-
 cudaError_t launch_octree_nodes(const uint32_t* counts, const fp_params& prm, NodeRec* recs, uint64_t rec_cap,
                                 const uint32_t* num_deep, fp_node* nodes, uint32_t node_cap, uint32_t* num_nodes,
                                 const NodeTables& T, const Workspace& ws, cudaStream_t st)
 {
     cudaError_t e;
     const int g = (int)prm.grid_log2, lmax = (int)prm.max_level;
-    const uint64_t cells = 1ull << (3 * g);
     const NodesBufs B = nodes_carve(ws, prm, rec_cap);
-    for (int l = g - 1; l >= 0; --l) {
-        uint64_t np_ = 1ull << (3 * l);
-        const uint32_t* child = l + 1 == g ? counts : B.pyr + ((1ull << (3 * (l + 1))) - 1) / 7;
-        k_pyr_level<<<(unsigned)((np_ + 255) / 256), 256, 0, st>>>(child, B.pyr + (np_ - 1) / 7, np_);
-    }
-    if ((e = scan_exclusive<uint32_t, uint32_t>(counts, B.cstart, cells, nullptr, B.nb.leafw, B.cstart + cells,
-                                                (uint32_t*)nullptr, st)))
-        return e;
     k_copy_u32<<<1, 1, 0, st>>>(T.nnode, num_deep);
     OctCtx c{};
     c.counts = counts; c.rcounts = counts; c.leaf_base = 0;
-    c.pyr = B.pyr; c.cstart = B.cstart; c.nrec = recs; c.nnode = T.nnode; c.node_cap_ws = (uint32_t)rec_cap;
+    c.nrec = recs; c.nnode = T.nnode; c.node_cap_ws = (uint32_t)rec_cap;
     c.g = g; c.s = (int)prm.sub_log2; c.lmax = lmax; c.C = prm.node_capacity; c.err = ws.err;
-    k_nodes_upper<<<(unsigned)((upper_node_bound(prm) + 255) / 256), 256, 0, st>>>(c);
+    k_grid_tiles<<<grid_tiles(g), kGtNT, 0, st>>>(counts, g, B.pyr, counts, B.rsum, nullptr, 0, nullptr, 0);
+    k_cells_open<<<grid_tiles(g), kGtNT, 0, st>>>(c, B.pyr, B.rsum, 0, 1, nullptr, nullptr, nullptr, nullptr);
     NodeSortBufs nb = B.nb;
     nb.nk = T.starts; nb.slevel = T.slevel; nb.idxtab = T.idxtab; nb.ndesc = T.ndesc;
     if ((e = node_table(B.sc, recs, T.nnode, (uint32_t)rec_cap, nb, nodes, node_cap, num_nodes, g, lmax, ws, st)))
