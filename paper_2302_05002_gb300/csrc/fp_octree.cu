@@ -86,7 +86,7 @@ struct OctCtx {   // device pointers of one fp_build_chunk_octree call
     uint8_t* cell_leaf;
     uint4* rec;           // cell-grouped records (rec_key, rec_j)
     Piece *tab, *small, *gen, *dups;   // the pieces by the way their lambda is found (emit_piece), any order
-    uint32_t *ntab, *nsmall, *ngen, *ndups;
+    uint32_t *ntab, *nsmall, *ngen, *ndups, *tab_claim;
     uint32_t piece_cap;                // of each list
     NodeRec* nrec;
     uint32_t* nnode;
@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(256) k_cell_scatter(const int4* __restrict__ p
 // appended with one atomic per tile, the pieces in cell order: those in work at
 // one time then lie in one or two tiles, and their scattered codes stay in L2
 // (appended one by one as the atomics fell, k_tab_pieces took 15.5 instead of
-// 13.0 ms for 5 * 10^8 uniform points).
+// 13.0 ms for 5 * 10^8 uniform points, before it took its pieces in order).
 __global__ void __launch_bounds__(kGtNT) k_cells_open(OctCtx c, const uint32_t* __restrict__ pyr,
                                                       const uint32_t* __restrict__ rsum, int cells, int upper,
                                                       uint32_t* __restrict__ cstart, uint32_t* __restrict__ cursor,
@@ -571,8 +571,9 @@ __global__ void k_split(OctCtx c, const OpenNode* cur, const uint32_t* ncur, Ope
 // their pieces in one 512-thread block, and the pieces sorted into record order
 // first, spent 950 instructions per point at 238 points per cell, where the
 // fourth and fifth table of a window did not fit its shared memory: 26.1 ms for
-// 5 * 10^8 uniform points.)
+// 5 * 10^8 uniform points, 6.1 ms now at about 300 instructions per point.)
 constexpr int kTabNT = 128;
+constexpr int kTabRun = 8;                    // pieces taken at a time
 constexpr int kTabCtas = 10;                  // blocks per SM (20 KB of tables each)
 constexpr int kTabDirect = 4;                 // levels in direct-mapped tables
 constexpr int kTabWords = 4680;               // 8 + 64 + 512 + 4096 entries
@@ -808,13 +809,25 @@ __global__ void __launch_bounds__(kTabNT, kTabCtas) k_tab_pieces(OctCtx c)
 {
     __shared__ __align__(16) unsigned char buf[kTabBytes];
     __shared__ uint32_t s_min;
+    __shared__ uint32_t s_next;
     const uint32_t nt = min(*c.ntab, c.piece_cap);
+    // runs of up to kTabRun pieces (fewer when that would leave blocks without
+    // work: 10^7 points, 0.23 against 0.29 ms) are taken in order from a counter: with a fixed share
+    // per block the blocks drifted apart over a large cloud until their scattered
+    // codes no longer met in L2 (5 * 10^8 points: 19.4 GB read and 12.5 GB
+    // written instead of 8 and 2, 13.0 instead of 6.1 ms)
+    const uint32_t run = max(1u, min((uint32_t)kTabRun, nt / (gridDim.x * 16)));
+    if (threadIdx.x == 0) s_next = atomicAdd(c.tab_claim, run);
+    __syncthreads();
+    uint32_t k = s_next, k1 = k + run;
     Piece next{};
-    if (blockIdx.x < nt) next = c.tab[blockIdx.x];
-    for (uint32_t k = blockIdx.x; k < nt; k += gridDim.x) {
+    if (k < nt) next = c.tab[k];
+    while (k < nt) {
         const Piece p = next;
-        if (k + gridDim.x < nt) {   // the next piece's records on their way to L2 during this one's work
-            next = c.tab[k + gridDim.x];
+        if (k + 1 == k1) {   // (every block barrier of a piece lies between this write and the read below)
+            if (threadIdx.x == 0) s_next = atomicAdd(c.tab_claim, run);
+        } else if (k + 1 < nt) {   // the next piece's records on their way to L2 during this one's work
+            next = c.tab[k + 1];
             const uint32_t line = threadIdx.x * 8;   // 128 bytes a thread
             if (line < next.count && (uint64_t)next.begin + line < c.n) prefetch_l2(c.rec + next.begin + line);
         }
@@ -826,6 +839,12 @@ __global__ void __launch_bounds__(kTabNT, kTabCtas) k_tab_pieces(OctCtx c)
         else if (p.count <= 2 * kTabNT) direct_piece<2>(c, p, D, tab, &s_min);
         else if (p.count <= 4 * kTabNT) direct_piece<4>(c, p, D, tab, &s_min);
         else direct_piece<kPieceMax / kTabNT>(c, p, D, tab, &s_min);
+        if (++k == k1) {
+            k = s_next;
+            k1 = k + run;
+            if (k < nt) next = c.tab[k];
+            __syncthreads();   // s_next is read before it is written again
+        }
     }
 }
 
@@ -1410,7 +1429,7 @@ struct OctBufs {
     uint8_t* cell_leaf;
     uint4* rec;           // cell-grouped records (rec_key, rec_j)
     Piece* pieces[4];     // table, small, general, oversized
-    uint32_t* counters;   // [0], [1], [2], [4] their numbers, [3] node records
+    uint32_t* counters;   // [0], [1], [2], [4] their numbers, [3] node records, [5] table pieces taken
     OpenNode* open[2];
     uint32_t *ocount, *bigstart;
     NodeRec* nrec;
@@ -1569,7 +1588,7 @@ cudaError_t launch_octree_impl(const fp_point* sorted, const uint32_t* perm, uin
     c.cstart = B.cstart; c.cursor = B.cursor; c.cell_leaf = B.cell_leaf;
     c.rec = B.rec; c.piece_cap = (uint32_t)Ly.piece_cap;
     c.tab = B.pieces[0]; c.small = B.pieces[1]; c.gen = B.pieces[2]; c.dups = B.pieces[3];
-    c.ntab = B.counters; c.nsmall = B.counters + 1; c.ngen = B.counters + 2; c.ndups = B.counters + 4;
+    c.ntab = B.counters; c.nsmall = B.counters + 1; c.ngen = B.counters + 2; c.ndups = B.counters + 4; c.tab_claim = B.counters + 5;
     c.nrec = B.nrec; c.nnode = nnode; c.node_cap_ws = (uint32_t)Ly.node_cap;
     c.codes = grp ? grp->codes : B.codes;
     c.open_cap = (uint32_t)Ly.open_cap;
