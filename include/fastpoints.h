@@ -140,7 +140,7 @@ fp_status fp_get_device_error(cudaStream_t stream, uint32_t* h_bits, int clear);
 fp_status fp_get_device_error_sites(cudaStream_t stream, uint32_t* h_sites);
 
 /* Test hook of the bounded waits.  The radix passes (fp_distribute with more
- * than 2048 chunks, the sorts of the octree and subsample stages) find each
+ * than 4096 chunks, the sorts of the octree and subsample stages) find each
  * tile's output offsets by a decoupled look-back over the earlier tiles'
  * published counts; every such wait gives up after a bounded number of
  * rounds, raises FP_ERR_TIMEOUT in the device error word and lets the kernel
@@ -285,10 +285,9 @@ fp_status fp_distribute(const fp_point* d_pts, uint64_t n, const fp_cube* d_cube
 
 /* fp_distribute with the points' level-g cells given (d_cells from
  * fp_count_cells, same cube and grid_log2): the chunk of point i is
- * d_lut[d_cells[i]] instead of being computed from the point.  With d_cells
- * 16-byte aligned, up to 4096 chunks take a counting pass and a double-buffered
- * sweep (no wait between blocks); otherwise up to 2048 chunks the one-sweep
- * scatter; more chunks take the radix passes, which compute the cell.  Every
+ * d_lut[d_cells[i]] instead of being computed from the point.  Both calls: up to
+ * 4096 chunks take a counting pass and a double-buffered sweep (no wait between
+ * blocks); more chunks the radix passes, which compute the cell.  Every
  * d_cells[i] must be below 8^grid_log2 (else FP_ERR_CAPACITY, outputs invalid).
  * Outputs identical to fp_distribute's. */
 fp_status fp_distribute_cells(const fp_point* d_pts, const uint32_t* d_cells, uint64_t n, const fp_cube* d_cube,

@@ -1492,16 +1492,6 @@ size_t octree_ws_bytes(uint64_t n, const fp_params& p)
     return dry.used;
 }
 
-template <int DIG, bool CPT, bool CK64, bool CK32>
-static cudaError_t run_sort(const SortScratch& sc, SortArgs a, int npass, const Workspace& ws, cudaStream_t st)
-{
-    for (int slot = 0; slot < npass; ++slot) {
-        cudaError_t e = sort_run_pass<DIG, CPT, CK64, CK32>(sc, a, slot, ws.num_sms, st);
-        if (e) return e;
-    }
-    return cudaSuccess;
-}
-
 // node records -> fp_node table in preorder, the level-g id table, sorted starts,
 // levels and subtree sizes (the lookups of the id resolution)
 struct NodeSortBufs {
@@ -1520,19 +1510,19 @@ static cudaError_t node_table(const SortScratch& sc, const NodeRec* nrec, uint32
     k_clamp<<<1, 1, 0, st>>>(nnode, ncap);
     k_node_keys<<<gn, 256, 0, st>>>(nrec, nnode, B.nk, B.nl, lmax);
     k_level_keys<<<gn, 256, 0, st>>>(B.nl, nnode, B.nk3);
-    if ((e = sort_plan_keys(sc, B.nk3, ncap, nnode, 0, 5, st))) return e;
     SortArgs a{};
     a.b.k64_src = B.nk3; a.b.k64_tmp = B.nk2; a.b.k64_dst = B.nk4;
     a.b.val_src = nullptr; a.b.val_tmp = B.nv2; a.b.val_dst = B.nv3;
     a.n = ncap; a.d_n = nnode; a.err = ws.err;
-    if ((e = run_sort<DIG_K64, false, true, false>(sc, a, sort_passes(5), ws, st))) return e;
+    if ((e = sort_plan_keys(sc, a, 0, 5, nullptr, false, ws.num_sms, st))) return e;
+    if ((e = sort_run<DIG_K64, false, true, false>(a, sort_passes(5), ws.num_sms, st))) return e;
     k_gather_u64<<<gn, 256, 0, st>>>(B.nk, B.nv3, nnode, B.nk3);
-    if ((e = sort_plan_keys(sc, B.nk3, ncap, nnode, 0, (uint32_t)std::max(1, 3 * lmax), st))) return e;
     SortArgs b2{};
     b2.b.k64_src = B.nk3; b2.b.k64_tmp = B.nk2; b2.b.k64_dst = B.nk;   // nk <- sorted starts
     b2.b.val_src = B.nv3; b2.b.val_tmp = B.nv2; b2.b.val_dst = B.nl;   // nl <- record of preorder position
     b2.n = ncap; b2.d_n = nnode; b2.err = ws.err;
-    if ((e = run_sort<DIG_K64, false, true, false>(sc, b2, sort_passes(3 * lmax), ws, st))) return e;
+    if ((e = sort_plan_keys(sc, b2, 0, (uint32_t)std::max(1, 3 * lmax), nullptr, false, ws.num_sms, st))) return e;
+    if ((e = sort_run<DIG_K64, false, true, false>(b2, sort_passes(3 * lmax), ws.num_sms, st))) return e;
     k_node_write<<<gn, 256, 0, st>>>(nrec, nnode, B.nl, B.nk, B.slevel, nodes, node_cap, num_nodes, B.idxtab, B.leafw,
                                      g, lmax, ws.err);
     k_node_fill<<<gn, 256, 0, st>>>(nrec, nnode, B.nl, B.nk, B.slevel, nodes, node_cap, B.ndesc, lmax);
@@ -1693,7 +1683,6 @@ cudaError_t launch_octree_impl(const fp_point* sorted, const uint32_t* perm, uin
         sg.first = reinterpret_cast<const uint64_t*>(nodes) + offsetof(fp_node, leaf_first) / sizeof(uint64_t);
         sg.first_stride = sizeof(fp_node) / sizeof(uint64_t);
         if ((e = seg_scatter(B.seg, sg, ws, st))) return e;
-        if ((e = sort_plan_weights(sc, B.leafw, nullptr, nnode, Ly.node_cap, 0, st))) return e;
         SortArgs a{};
         a.b.pt_src = reinterpret_cast<const int4*>(sorted);
         a.b.pt_tmp = B.lt_pt;
@@ -1701,9 +1690,10 @@ cudaError_t launch_octree_impl(const fp_point* sorted, const uint32_t* perm, uin
         a.b.val_src = perm; a.b.val_tmp = B.lt_val; a.b.val_dst = leaf_perm;
         a.b.k32_src = B.leafid; a.b.k32_tmp = B.lt_k32; a.b.k32_dst = nullptr;
         a.n = N; a.d_n = B.seg.cnt + 5; a.err = ws.err;
+        if ((e = sort_plan_weights(sc, a, B.leafw, nullptr, nnode, Ly.node_cap, false, ws.num_sms, st))) return e;
         const int np = sort_passes(count_bits(Ly.node_cap));   // leaf ids below node_cap
-        if (leaf_pts) e = run_sort<DIG_K32, true, false, true>(sc, a, np, ws, st);
-        else e = run_sort<DIG_K32, false, false, true>(sc, a, np, ws, st);
+        if (leaf_pts) e = sort_run<DIG_K32, true, false, true>(a, np, ws.num_sms, st);
+        else e = sort_run<DIG_K32, false, false, true>(a, np, ws.num_sms, st);
         if (e) return e;
     }
     return cudaGetLastError();
@@ -2015,15 +2005,14 @@ cudaError_t launch_subsample(fp_node* nodes, const uint32_t* num_nodes, uint32_t
     if ((e = scan_exclusive<uint32_t, uint32_t>(B.scnt, soff, M, nm, B.tiles32, (uint32_t*)nullptr,
                                                 (uint32_t*)nullptr, st)))
         return e;
-    if ((e = sort_plan_keys(sc, B.s_key, N, nstaged, 0, (uint32_t)pbits, st, nrank))) return e;
     {
         SortArgs b{};
         b.b.k64_src = B.s_key; b.b.k64_tmp = B.s_key2; b.b.k64_dst = B.s_key3;
         b.b.val_src = B.s_val; b.b.val_tmp = B.s_val2; b.b.val_dst = B.s_val3;
         b.n = N; b.d_n = nstaged; b.err = ws.err;
+        if ((e = sort_plan_keys(sc, b, 0, (uint32_t)pbits, nrank, false, ws.num_sms, st))) return e;
         const int np = sort_passes(pbits + count_bits(M));   // node ids below M above the index bits
-        for (int slot = 0; slot < np; ++slot)
-            if ((e = sort_run_pass<DIG_K64, false, true, false>(sc, b, slot, ws.num_sms, st))) return e;
+        if ((e = sort_run<DIG_K64, false, true, false>(b, np, ws.num_sms, st))) return e;
     }
     k_stitch_place<<<gN, 256, 0, st>>>(nstaged, B.s_key3, B.s_val3, pbits, B.slist, nrank, nm, soff, first,
                                        reinterpret_cast<const int4*>(sorted), perm, N,
@@ -2034,15 +2023,14 @@ cudaError_t launch_subsample(fp_node* nodes, const uint32_t* num_nodes, uint32_t
     // whole-array path (runs with seg cnt[5] = n records when a chunk did not fit, else on none):
     // stable scatter by owner id, then the owner segments spanning several chunks re-sorted
     const uint32_t* gate = B.seg.cnt + 5;
-    if ((e = sort_plan_weights(sc, nown, nullptr, nm, M, 0, st))) return e;
     SortArgs a{};
     a.b.pt_src = reinterpret_cast<const int4*>(sorted); a.b.pt_tmp = B.t_pt;
     a.b.pt_dst = reinterpret_cast<int4*>(final_pts);
     a.b.val_src = perm; a.b.val_tmp = B.t_val; a.b.val_dst = final_perm;
     a.b.k32_src = owner; a.b.k32_tmp = B.t_k32; a.b.k32_dst = B.fown;
     a.n = N; a.d_n = gate; a.err = ws.err;
-    for (int slot = 0; slot < sort_passes(count_bits(M)); ++slot)
-        if ((e = sort_run_pass<DIG_K32, true, false, true>(sc, a, slot, ws.num_sms, st))) return e;
+    if ((e = sort_plan_weights(sc, a, nown, nullptr, nm, M, false, ws.num_sms, st))) return e;
+    if ((e = sort_run<DIG_K32, true, false, true>(a, sort_passes(count_bits(M)), ws.num_sms, st))) return e;
     if ((e = cudaMemsetAsync(mark, 0, (size_t)M * 4, st))) return e;
     if ((e = cudaMemsetAsync(cnt, 0, 2 * sizeof(uint32_t), st))) return e;
     k_mark_unsorted<<<gN, 256, 0, st>>>(B.fown, final_perm, N, gate, mark, nm);
@@ -2054,13 +2042,12 @@ cudaError_t launch_subsample(fp_node* nodes, const uint32_t* num_nodes, uint32_t
     k_stitch_keys<<<ws.num_sms * 8, 256, 0, st>>>(mlist, cnt, soff, cnt + 1, first, final_perm, B.s_key, B.s_val);
     int rank_bits = 1;
     while ((1ull << rank_bits) < M) ++rank_bits;
-    if ((e = sort_plan_keys(sc, B.s_key, N, cnt + 1, 0, (uint32_t)(32 + rank_bits), st))) return e;
     SortArgs b{};
     b.b.k64_src = B.s_key; b.b.k64_tmp = B.s_key2; b.b.k64_dst = B.s_key3;
     b.b.val_src = B.s_val; b.b.val_tmp = B.s_val2; b.b.val_dst = B.s_val3;
     b.n = N; b.d_n = cnt + 1; b.err = ws.err;
-    for (int slot = 0; slot < sort_passes(32 + rank_bits); ++slot)
-        if ((e = sort_run_pass<DIG_K64, false, true, false>(sc, b, slot, ws.num_sms, st))) return e;
+    if ((e = sort_plan_keys(sc, b, 0, (uint32_t)(32 + rank_bits), nullptr, false, ws.num_sms, st))) return e;
+    if ((e = sort_run<DIG_K64, false, true, false>(b, sort_passes(32 + rank_bits), ws.num_sms, st))) return e;
     k_stitch_gather<<<gN, 256, 0, st>>>(cnt + 1, B.s_val3,
                                                                   reinterpret_cast<const int4*>(final_pts),
                                                                   final_perm, B.s_pt, B.s_perm);

@@ -682,13 +682,12 @@ fp_status build(const fp_point* h_pts, uint64_t n, const fp_params& prm, uint64_
         if ((e = cudaMemcpyAsync(B.owner, H.owner + b0, ng * 4, cudaMemcpyHostToDevice, st))) return cu(e);
         k_owner_keys<<<grid_for(ng, base.num_sms), 256, 0, st>>>(B.owner, ng, B.key);
         ws.used = ws_after_sc;
-        if ((e = sort_plan_keys(sc, B.key, ng, nullptr, 0, (uint32_t)mbits, st))) return cu(e);
         SortArgs a{};
         a.b.k64_src = B.key; a.b.k64_tmp = B.key2; a.b.k64_dst = B.key3;
         a.b.val_src = nullptr; a.b.val_tmp = B.val2; a.b.val_dst = B.val3;
         a.n = ng; a.err = base.err;
-        for (int slot = 0; slot < sort_passes(mbits); ++slot)
-            if ((e = sort_run_pass<DIG_K64, false, true, false>(sc, a, slot, base.num_sms, st))) return cu(e);
+        if ((e = sort_plan_keys(sc, a, 0, (uint32_t)mbits, nullptr, false, base.num_sms, st))) return cu(e);
+        if ((e = sort_run<DIG_K64, false, true, false>(a, sort_passes(mbits), base.num_sms, st))) return cu(e);
         k_run_starts<<<grid_for(ng, base.num_sms), 256, 0, st>>>(B.key3, ng, 0, F.soff, M);
         k_group_place<<<grid_for(ng, base.num_sms), 256, 0, st>>>(
             B.key3, B.val3, ng, F.soff, F.nodes, M, prm.chunk_threshold, g, F.first, B.pts, B.perm, b0,
@@ -715,13 +714,12 @@ fp_status build(const fp_point* h_pts, uint64_t n, const fp_params& prm, uint64_
         const SortScratch sf = take_sort_scratch(wf, S);
         if (wf.used > wf.bytes) return FP_ERR_WORKSPACE;
         if ((e = cudaMemcpyAsync(k1, H.st_key, S * 8, cudaMemcpyHostToDevice, st))) return cu(e);
-        if ((e = sort_plan_keys(sf, k1, S, nullptr, 0, (uint32_t)(pbits + mbits), st))) return cu(e);
         SortArgs a{};
         a.b.k64_src = k1; a.b.k64_tmp = k2; a.b.k64_dst = k3;
         a.b.val_src = nullptr; a.b.val_tmp = v2; a.b.val_dst = v3;
         a.n = S; a.err = base.err;
-        for (int slot = 0; slot < sort_passes(pbits + mbits); ++slot)
-            if ((e = sort_run_pass<DIG_K64, false, true, false>(sf, a, slot, base.num_sms, st))) return cu(e);
+        if ((e = sort_plan_keys(sf, a, 0, (uint32_t)(pbits + mbits), nullptr, false, base.num_sms, st))) return cu(e);
+        if ((e = sort_run<DIG_K64, false, true, false>(a, sort_passes(pbits + mbits), base.num_sms, st))) return cu(e);
         k_run_starts<<<grid_for(S, base.num_sms), 256, 0, st>>>(k3, S, pbits, F.soff, M);
         k_stitch_final<<<grid_for(S, base.num_sms), 256, 0, st>>>(k3, v3, S, pbits, F.soff, F.first, H.st_src, H.pts,
                                                                   H.perm, resident ? 1 : 0,

@@ -133,15 +133,15 @@ static cudaError_t seg_launch(SegArgs a, const SegScratch& sc, int v, int num_sm
     return cudaGetLastError();
 }
 
-// ---- the distribution with each point's cell given, up to 4096 chunks, in four
-// launches and without any wait between blocks (the sweep below for up to 512
-// chunks, k_dist_sweep_wide further down for 513 .. 4096):
+// ---- the distribution into up to 4096 chunks, in four launches and without any
+// wait between blocks (the sweep with per-warp histograms for up to 512 chunks,
+// the one that sorts each tile for 513 .. 4096; chosen on the device):
 //   k_dist_table: per node of level L = min(g, 5), its chunk when every
 //     occupied cell of the node lies in that one chunk (else none) -- a 64 KB
 //     table that spares most points the gather of the cell -> chunk table;
-//   k_dist_count: one block per group of kDistGroup consecutive tiles writes
-//     every point's chunk, and per tile the points of each chunk in the group's
-//     earlier tiles, and per group its totals;
+//   k_dist_count: one block per group of consecutive tiles writes every point's
+//     chunk (from its cell, given or computed), and per tile the points of each
+//     chunk in the group's earlier tiles, and per group its totals;
 //   k_dist_colscan: per chunk, the exclusive prefix of the group totals plus the
 //     chunk's offset -- each group's output start in every chunk;
 //   k_dist_sweep: one CTA of 1024 threads per SM; tiles taken in order from a
@@ -157,7 +157,8 @@ constexpr int kDistBits = 9;
 constexpr int kDistDig = 1 << kDistBits;
 constexpr int kDistWideBits = 12;               // the wide sweep: 513 .. 4096 chunks
 constexpr int kDistWideDig = 1 << kDistWideBits;
-constexpr int kDistGroup = 64;                  // tiles per block of k_dist_count
+constexpr int kDistGroup = 64;                  // most tiles per block of k_dist_count
+constexpr int kDistSpread = 608;                // small clouds: about this many blocks (4 per SM) instead
 constexpr int kDistCountNT = 512;               // thread d of k_dist_count owns chunks d, d + 512, ...
 constexpr int kDistCountIPT = kSortTile / kDistCountNT;
 constexpr int kDistTabLevel = 5;                // level of the node -> chunk table
@@ -165,32 +166,48 @@ constexpr uint16_t kDistSplit = 0xFFFFu;        // the node's points lie in seve
 
 struct DistSweepArgs {
     const int4* pts;
-    const uint32_t* cells;      // level-g cell of every point
+    const uint32_t* cells;      // nullable: level-g cell of every point (else computed from the point)
+    const fp_cube* cube;
     const uint32_t* lut;        // cell -> chunk (kNone: empty cell)
     const uint64_t* offsets;    // chunk c = output positions [offsets[c], offsets[c + 1])
     int4* out;
     uint32_t* perm;             // nullable
     uint16_t* tab;              // [8^tl]: chunk of a level-tl node, or kDistSplit
     uint16_t* chunk;            // chunk of every point, 16-byte aligned
+    uint32_t group;             // consecutive tiles of one k_dist_count block
     uint32_t* before;           // [tile][DIG]: points of the chunk in the group's earlier tiles
     uint32_t* gstart;           // [group][DIG]: group totals, then the group's start in the chunk
-    uint32_t* counter;
-    const uint32_t* d_ntiles;   // tiles of this sweep (0: another path runs)
-    uint64_t ntiles_max;
-    const uint32_t* nb;         // chunks (1 .. DIG, the sweep's width)
+    uint32_t* counter;          // the sweep's tile counter
+    uint64_t ntiles;
+    const uint32_t* num_chunks; // more than kDistWideDig: the radix passes run instead
+    uint32_t* run_sort;         // set to 1 then, else 0
+    uint32_t* hist;             // the radix passes' histogram, cleared here
     uint64_t n;
     uint32_t ncell;             // cells of the grid (bound of a cell id)
     int g, tl;                  // grid level, table level (tl <= g)
     uint32_t* err;
 };
 
-// one warp per level-tl node: the chunks of its occupied cells (built for both
-// sweeps, whichever of them runs)
-__global__ void k_dist_table(DistSweepArgs a)
+FP_DEV uint32_t dist_chunks(const DistSweepArgs& a)   // 0: not this path
 {
+    const uint32_t K = *a.num_chunks;
+    return K <= (uint32_t)kDistWideDig ? K : 0u;
+}
+
+// one warp per level-tl node: the chunks of its occupied cells
+__global__ void __launch_bounds__(256) k_dist_table(DistSweepArgs a)
+{
+    const uint32_t nb = dist_chunks(a);
+    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t == 0) {
+        *a.counter = 0;
+        *a.run_sort = nb ? 0u : 1u;
+    }
+    if (!nb)
+        for (uint32_t q = t; q < (uint32_t)kSortHistWords; q += gridDim.x * blockDim.x) a.hist[q] = 0;
     const int lane = threadIdx.x & 31;
-    const uint32_t k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (k >= (1u << (3 * a.tl))) return;
+    const uint32_t k = t >> 5;
+    if (!nb || k >= (1u << (3 * a.tl))) return;
     const uint32_t span = 1u << (3 * (a.g - a.tl)), lo = k * span;
     uint32_t cmin = kNone, cmax = 0;
     for (uint32_t q = lane; q < span; q += 32) {
@@ -202,40 +219,45 @@ __global__ void k_dist_table(DistSweepArgs a)
     if (lane == 0) a.tab[k] = (cmin == cmax && cmin < (uint32_t)kDistWideDig) ? (uint16_t)cmin : kDistSplit;
 }
 
-template <int DIG>
-__global__ void __launch_bounds__(kDistCountNT) k_dist_count(DistSweepArgs a)
+template <int DIG, bool CELLS>
+FP_DEV void dist_count(const DistSweepArgs& a, uint32_t nb, const uint16_t* dist_tab, uint32_t* h)
 {
     constexpr int kOwn = DIG / kDistCountNT;   // chunks per thread
-    extern __shared__ __align__(16) uint16_t dist_tab[];   // 8^tl entries
-    __shared__ uint32_t h[DIG];
-    const uint64_t ntiles = min((uint64_t)*a.d_ntiles, a.ntiles_max);
-    if (ntiles == 0) return;
-    const uint64_t ngroups = (ntiles + kDistGroup - 1) / kDistGroup;
-    const uint32_t nb = min(*a.nb, (uint32_t)DIG);
+    const uint64_t ngroups = (a.ntiles + a.group - 1) / a.group;
     const uint32_t d = threadIdx.x;
     const int tsh = 3 * (a.g - a.tl);
-    {
-        const uint32_t nt4 = (1u << (3 * a.tl)) / 8;   // uint4 words of the table (8^tl >= 8 when tl >= 1)
-        if (a.tl >= 1) {
-            for (uint32_t q = d; q < nt4; q += kDistCountNT)
-                reinterpret_cast<uint4*>(dist_tab)[q] = __ldg(reinterpret_cast<const uint4*>(a.tab) + q);
-        } else if (d == 0) {
-            dist_tab[0] = a.tab[0];
-        }
+    CubeDev cube;
+    float sg = 0.f;
+    if (!CELLS) {
+        cube = load_cube(a.cube);
+        sg = scale_at(cube, a.g);
     }
     for (uint64_t gi = blockIdx.x; gi < ngroups; gi += gridDim.x) {
-        const uint64_t t0 = gi * kDistGroup, t1 = min(ntiles, t0 + kDistGroup);
+        const uint64_t t0 = gi * a.group, t1 = min(a.ntiles, t0 + a.group);
         uint32_t run[kOwn];
 #pragma unroll
         for (int o = 0; o < kOwn; ++o) { run[o] = 0; h[d + o * kDistCountNT] = 0; }
-        // the cells of the next tile are loaded while the current one is counted
+        // given cells: those of the next tile are loaded while the current one is counted
         uint32_t c[kDistCountIPT];
         auto load = [&](uint64_t t) {
             const uint64_t base = t * kSortTile;
+            if (CELLS) {
 #pragma unroll
-            for (int r = 0; r < kDistCountIPT; ++r) {
-                const uint64_t i = base + (uint64_t)r * kDistCountNT + d;
-                c[r] = i < a.n ? __ldg(a.cells + i) : kNone;
+                for (int r = 0; r < kDistCountIPT; ++r) {
+                    const uint64_t i = base + (uint64_t)r * kDistCountNT + d;
+                    c[r] = i < a.n ? __ldg(a.cells + i) : kNone;
+                }
+            } else {
+                int4 p[kDistCountIPT];
+#pragma unroll
+                for (int r = 0; r < kDistCountIPT; ++r) {   // all loads in flight together
+                    const uint64_t i = base + (uint64_t)r * kDistCountNT + d;
+                    p[r] = i < a.n ? __ldg(a.pts + i) : make_int4(cube.o[0], cube.o[1], cube.o[2], 0);
+                }
+#pragma unroll
+                for (int r = 0; r < kDistCountIPT; ++r)
+                    c[r] = base + (uint64_t)r * kDistCountNT + d < a.n ? key_small(p[r].x, p[r].y, p[r].z, cube, sg, a.g)
+                                                                      : kNone;
             }
         };
         load(t0);
@@ -256,12 +278,14 @@ __global__ void __launch_bounds__(kDistCountNT) k_dist_count(DistSweepArgs a)
                 }
             const uint64_t base = t * kSortTile;
 #pragma unroll
-            for (int r = 0; r < kDistCountIPT; ++r)
-                if (k[r] != kNone) {
+            for (int r = 0; r < kDistCountIPT; ++r) {
+                const uint64_t i = base + (uint64_t)r * kDistCountNT + d;
+                if (i < a.n) {
                     if (k[r] >= nb) { raise(a.err, FP_ERR_CAPACITY, 13); k[r] = nb - 1; }   // not a chunk
-                    a.chunk[base + (uint64_t)r * kDistCountNT + d] = (uint16_t)k[r];
+                    a.chunk[i] = (uint16_t)k[r];
                     atomicAdd(&h[k[r]], 1u);
                 }
+            }
             __syncthreads();
 #pragma unroll
             for (int o = 0; o < kOwn; ++o) {
@@ -280,27 +304,40 @@ __global__ void __launch_bounds__(kDistCountNT) k_dist_count(DistSweepArgs a)
     }
 }
 
-// one warp per chunk: exclusive prefix of the group totals, plus the chunk's offset
-template <int DIG>
-__global__ void k_dist_colscan(DistSweepArgs a)
+template <bool CELLS>
+__global__ void __launch_bounds__(kDistCountNT) k_dist_count(DistSweepArgs a)
 {
-    const uint64_t ntiles = min((uint64_t)*a.d_ntiles, a.ntiles_max);
-    const uint64_t ngroups = (ntiles + kDistGroup - 1) / kDistGroup;
-    const uint32_t nb = min(*a.nb, (uint32_t)DIG);
+    extern __shared__ __align__(16) uint16_t dist_tab[];   // 8^tl entries
+    __shared__ uint32_t h[kDistWideDig];
+    const uint32_t nb = dist_chunks(a);
+    if (!nb) return;
+    const uint32_t nt4 = (1u << (3 * a.tl)) / 8;   // uint4 words of the table (8^tl >= 8: tl >= 1)
+    for (uint32_t q = threadIdx.x; q < nt4; q += kDistCountNT)
+        reinterpret_cast<uint4*>(dist_tab)[q] = __ldg(reinterpret_cast<const uint4*>(a.tab) + q);
+    if (nb <= (uint32_t)kDistDig) dist_count<kDistDig, CELLS>(a, nb, dist_tab, h);
+    else dist_count<kDistWideDig, CELLS>(a, nb, dist_tab, h);
+}
+
+// one warp per chunk: exclusive prefix of the group totals, plus the chunk's offset
+__global__ void __launch_bounds__(256) k_dist_colscan(DistSweepArgs a)
+{
+    const uint64_t ngroups = (a.ntiles + a.group - 1) / a.group;
+    const uint32_t nb = dist_chunks(a);
+    const uint32_t dig = nb <= (uint32_t)kDistDig ? kDistDig : kDistWideDig;
     const int lane = threadIdx.x & 31;
     const uint32_t d = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (d >= nb || ngroups == 0) return;
+    if (d >= nb) return;
     uint32_t run = (uint32_t)a.offsets[d];
     for (uint64_t g0 = 0; g0 < ngroups; g0 += 32) {
         const uint64_t gi = g0 + lane;
-        const uint32_t v = gi < ngroups ? a.gstart[gi * DIG + d] : 0u;
+        const uint32_t v = gi < ngroups ? a.gstart[gi * dig + d] : 0u;
         uint32_t x = v;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
             if (lane >= o) x += y;
         }
-        if (gi < ngroups) a.gstart[gi * DIG + d] = run + x - v;
+        if (gi < ngroups) a.gstart[gi * dig + d] = run + x - v;
         run += __shfl_sync(0xFFFFFFFFu, x, 31);
     }
 }
@@ -317,15 +354,11 @@ struct DistSmem {
     uint64_t bar[2];
 };
 
-__global__ void __launch_bounds__(kDistNT, 1) k_dist_sweep(DistSweepArgs a)
+FP_DEV void dist_sweep(const DistSweepArgs& a, DistSmem& S, int nb)
 {
-    extern __shared__ __align__(128) unsigned char dist_smem[];
-    DistSmem& S = *reinterpret_cast<DistSmem*>(dist_smem);
-    const uint64_t ntiles = min((uint64_t)*a.d_ntiles, a.ntiles_max);
-    if (ntiles == 0) return;
+    const uint64_t ntiles = a.ntiles;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint64_t n = a.n;
-    const int nb = (int)min(*a.nb, (uint32_t)kDistDig);
     // a full tile by bulk copy into buffer b (thread 0); a partial one is loaded by the threads
     auto issue = [&](uint64_t t, int b) {
         const uint64_t base = t * kSortTile;
@@ -355,7 +388,7 @@ __global__ void __launch_bounds__(kDistNT, 1) k_dist_sweep(DistSweepArgs a)
         // this tile's start in every chunk, in flight during the ranking
         uint32_t start = 0;
         if (threadIdx.x < (unsigned)nb)
-            start = __ldg(a.gstart + (tile / kDistGroup) * kDistDig + threadIdx.x) +
+            start = __ldg(a.gstart + (tile / a.group) * kDistDig + threadIdx.x) +
                     __ldg(a.before + tile * kDistDig + threadIdx.x);
         const uint64_t base = tile * kSortTile;
         const int tn = (int)(n - base < (uint64_t)kSortTile ? n - base : (uint64_t)kSortTile);
@@ -515,14 +548,10 @@ FP_DEV void wide_pass(WideSmem& S, int b, const uint32_t* src, uint32_t* dst, in
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(kDistNT, 1) k_dist_sweep_wide(DistSweepArgs a)
+FP_DEV void dist_sweep_wide(const DistSweepArgs& a, WideSmem& S, uint32_t nb)
 {
-    extern __shared__ __align__(128) unsigned char wide_smem[];
-    WideSmem& S = *reinterpret_cast<WideSmem*>(wide_smem);
-    const uint64_t ntiles = min((uint64_t)*a.d_ntiles, a.ntiles_max);
-    if (ntiles == 0) return;
+    const uint64_t ntiles = a.ntiles;
     const uint64_t n = a.n;
-    const uint32_t nb = min(*a.nb, (uint32_t)kDistWideDig);
     auto issue = [&](uint64_t t, int b) {
         const uint64_t base = t * kSortTile;
         if (base + kSortTile > n) return;
@@ -568,7 +597,7 @@ __global__ void __launch_bounds__(kDistNT, 1) k_dist_sweep_wide(DistSweepArgs a)
         }
         wide_pass(S, b, S.s0, S.s1, tn, kWideRadix, false);
         // ---- every chunk present: its first slot and its output start
-        const uint64_t g = tile / kDistGroup;
+        const uint64_t g = tile / a.group;
         for (int q = threadIdx.x; q < tn; q += kDistNT) {
             const uint32_t c = S.s1[q] >> 12;
             if (q == 0 || (S.s1[q - 1] >> 12) != c) {
@@ -592,42 +621,19 @@ __global__ void __launch_bounds__(kDistNT, 1) k_dist_sweep_wide(DistSweepArgs a)
     }
 }
 
-// ------------------------------------------------ distribution in one sweep
-// one segment [0, n) with K digits when k_lo < K <= 2048 (k_lo: 256, or 0 when
-// the cells are given and the double-buffered sweep takes the small counts
-// too): its tiles, the segment bounds, and the flag that gates the radix passes
-constexpr int kDistMidBits = 9;   // up to 512 chunks: two CTAs per SM
-static_assert(kDistMidBits == kDistBits, "the sweep with the cells given is the 9-bit variant");
-
-__global__ void k_dist_setup(const uint32_t* num_chunks, uint64_t n, uint32_t k_lo, uint32_t k_hi, uint64_t* seg_off,
-                             uint32_t* seg_lo, uint32_t* seg_nb, SegTile* tiles, uint32_t* cnt, uint32_t* run_sort)
+__global__ void __launch_bounds__(kDistNT, 1) k_dist_sweep(DistSweepArgs a)
 {
-    const uint32_t K = *num_chunks;
-    const bool wide = K > k_lo && K <= k_hi;
-    const uint64_t ntl = wide ? (n + kSortTile - 1) / kSortTile : 0;
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < ntl; t += stride)
-        tiles[t] = SegTile{0u, (uint32_t)t};
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        const bool mid = K <= (1u << kDistMidBits);
-        seg_off[0] = 0;
-        seg_off[1] = n;
-        seg_lo[0] = 0;
-        seg_nb[0] = wide ? K : 1u;
-        cnt[0] = mid ? (uint32_t)ntl : 0u;   // tiles of the 9-bit pass
-        cnt[3] = mid ? 0u : (uint32_t)ntl;   // tiles of the 11-bit pass (the wide sweep with the cells)
-        cnt[1] = cnt[4] = 0;                 // tile counters
-        cnt[2] = 0;                          // fail word (never set here)
-        *run_sort = wide ? 0u : 1u;
-    }
+    extern __shared__ __align__(128) unsigned char dist_smem[];
+    const uint32_t nb = dist_chunks(a);
+    if (!nb) return;
+    if (nb <= (uint32_t)kDistDig) dist_sweep(a, *reinterpret_cast<DistSmem*>(dist_smem), (int)nb);
+    else dist_sweep_wide(a, *reinterpret_cast<WideSmem*>(dist_smem), nb);
 }
 
 struct DistScratch {
-    uint64_t* seg_off;
-    uint32_t *lo, *nb, *cnt, *status, *gstart;
+    uint32_t *counter, *before, *gstart;
     uint16_t* tab;
-    SegTile* tiles;
-    uint64_t ntiles;
+    uint64_t ntiles, group;
 };
 
 static DistScratch dist_carve(const Workspace& ws, uint64_t n)
@@ -635,30 +641,12 @@ static DistScratch dist_carve(const Workspace& ws, uint64_t n)
     DistScratch d;
     d.ntiles = (n + kSortTile - 1) / kSortTile;
     const uint64_t T = d.ntiles ? d.ntiles : 1;
-    d.seg_off = ws.take<uint64_t>(2);
-    d.lo = ws.take<uint32_t>(1);
-    d.nb = ws.take<uint32_t>(1);
-    d.cnt = ws.take<uint32_t>(8);
-    d.tiles = ws.take<SegTile>(T);
-    d.status = ws.take<uint32_t>(T << kDistWideBits);   // (also the wide sweep's per-tile starts)
-    d.gstart = ws.take<uint32_t>(((T + kDistGroup - 1) / kDistGroup) << kDistWideBits);
+    d.group = std::max<uint64_t>(1, std::min<uint64_t>(kDistGroup, T / kDistSpread));
+    d.counter = ws.take<uint32_t>(1);
+    d.before = ws.take<uint32_t>(T << kDistWideBits);
+    d.gstart = ws.take<uint32_t>(((T + d.group - 1) / d.group) << kDistWideBits);
     d.tab = ws.take<uint16_t>(1u << (3 * kDistTabLevel));
     return d;
-}
-
-template <int MAXB>
-static cudaError_t dist_launch(const SegArgs& a, uint64_t ntiles, int num_sms, cudaStream_t st)
-{
-    using SM = SegSmem<true, MAXB, true>;
-    auto kern = k_seg_pass<true, MAXB, true>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::total);
-    if (e) return e;
-    int per_sm = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kSortNT, SM::total))) return e;
-    if (per_sm < 1) per_sm = 1;
-    const int grid = (int)std::max<uint64_t>(1, std::min<uint64_t>(ntiles, (uint64_t)num_sms * per_sm));
-    kern<<<grid, kSortNT, SM::total, st>>>(a);
-    return cudaGetLastError();
 }
 
 size_t dist_wide_bytes(uint64_t n)
@@ -670,70 +658,32 @@ size_t dist_wide_bytes(uint64_t n)
 
 cudaError_t dist_wide(const int4* pts, uint64_t n, const fp_cube* cube, int g, const uint32_t* lut,
                       const uint64_t* offsets, const uint32_t* num_chunks, int4* out, uint32_t* perm,
-                      uint32_t* run_sort, const Workspace& ws, cudaStream_t st, const uint32_t* cells,
+                      uint32_t* run_sort, uint32_t* hist, const Workspace& ws, cudaStream_t st, const uint32_t* cells,
                       uint16_t* chunk_tmp)
 {
     const DistScratch d = dist_carve(ws, n);
-    // the cells given and a scratch array for every point's chunk: up to 4096
-    // chunks take the counting pass and a double-buffered sweep
-    const bool sweep = cells && chunk_tmp && ((uintptr_t)chunk_tmp & 15) == 0 && ((uintptr_t)pts & 15) == 0;
-    const int gs = (int)std::max<uint64_t>(1, std::min<uint64_t>((d.ntiles + 255) / 256, (uint64_t)ws.num_sms * 4));
-    k_dist_setup<<<gs, 256, 0, st>>>(num_chunks, n, sweep ? 0u : (1u << kSegSmallBits),
-                                     sweep ? (uint32_t)kDistWideDig : (1u << kSegMaxBits), d.seg_off, d.lo, d.nb,
-                                     d.tiles, d.cnt, run_sort);
+    DistSweepArgs b{};
+    b.pts = pts; b.cells = cells; b.cube = cube; b.lut = lut; b.offsets = offsets;
+    b.out = out; b.perm = perm; b.tab = d.tab; b.chunk = chunk_tmp;
+    b.group = (uint32_t)d.group; b.before = d.before; b.gstart = d.gstart;
+    b.counter = d.counter; b.ntiles = d.ntiles;
+    b.num_chunks = num_chunks; b.run_sort = run_sort; b.hist = hist;
+    b.n = n; b.ncell = 1u << (3 * g); b.g = g; b.tl = std::min(g, kDistTabLevel); b.err = ws.err;
+    const uint32_t nodes = 1u << (3 * b.tl);
+    k_dist_table<<<(nodes * 32 + 255) / 256, 256, 0, st>>>(b);
+    const uint64_t ngroups = (d.ntiles + d.group - 1) / d.group;
+    const int tsm = (int)(nodes * sizeof(uint16_t));
+    const int gc = (int)std::max<uint64_t>(1, std::min<uint64_t>(ngroups, (uint64_t)ws.num_sms * 2));
+    const int grid = (int)std::max<uint64_t>(1, std::min<uint64_t>(d.ntiles, (uint64_t)ws.num_sms));
     cudaError_t e;
-    if (sweep) {
-        DistSweepArgs b{};
-        b.pts = pts; b.cells = cells; b.lut = lut; b.offsets = offsets;
-        b.out = out; b.perm = perm; b.tab = d.tab; b.chunk = chunk_tmp;
-        b.before = d.status; b.gstart = d.gstart;
-        b.ntiles_max = d.ntiles; b.nb = d.nb;
-        b.n = n; b.ncell = 1u << (3 * g); b.g = g; b.tl = std::min(g, kDistTabLevel); b.err = ws.err;
-        const uint32_t nodes = 1u << (3 * b.tl);
-        k_dist_table<<<(nodes * 32 + 255) / 256, 256, 0, st>>>(b);
-        const uint64_t ngroups = (d.ntiles + kDistGroup - 1) / kDistGroup;
-        const int tsm = (int)(nodes * sizeof(uint16_t) < 16 ? 16 : nodes * sizeof(uint16_t));
-        const int gc = (int)std::max<uint64_t>(1, std::min<uint64_t>(ngroups, (uint64_t)ws.num_sms * 3));
-        const int grid = (int)std::max<uint64_t>(1, std::min<uint64_t>(d.ntiles, (uint64_t)ws.num_sms));
-        // up to 512 chunks: per-warp histograms in the sweep (tiles cnt[0], counter cnt[1])
-        b.d_ntiles = d.cnt; b.counter = d.cnt + 1;
-        if ((e = cudaFuncSetAttribute(k_dist_count<kDistDig>, cudaFuncAttributeMaxDynamicSharedMemorySize, tsm)))
-            return e;
-        k_dist_count<kDistDig><<<gc, kDistCountNT, tsm, st>>>(b);
-        k_dist_colscan<kDistDig><<<kDistDig * 32 / 256, 256, 0, st>>>(b);
-        const int smem = (int)sizeof(DistSmem);
-        if ((e = cudaFuncSetAttribute(k_dist_sweep, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
-        k_dist_sweep<<<grid, kDistNT, smem, st>>>(b);
-        // 513 .. 4096 chunks: the tile's ranks by a two-pass sort (tiles cnt[3], counter cnt[4])
-        b.d_ntiles = d.cnt + 3; b.counter = d.cnt + 4;
-        if ((e = cudaFuncSetAttribute(k_dist_count<kDistWideDig>, cudaFuncAttributeMaxDynamicSharedMemorySize, tsm)))
-            return e;
-        k_dist_count<kDistWideDig><<<gc, kDistCountNT, tsm, st>>>(b);
-        k_dist_colscan<kDistWideDig><<<kDistWideDig * 32 / 256, 256, 0, st>>>(b);
-        const int wsm = (int)sizeof(WideSmem);
-        if ((e = cudaFuncSetAttribute(k_dist_sweep_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, wsm))) return e;
-        k_dist_sweep_wide<<<grid, kDistNT, wsm, st>>>(b);
-        return cudaGetLastError();
-    }
-    const int gz = std::max(1, ws.num_sms * 8);
-    k_seg_zero<kDistMidBits><<<gz, 256, 0, st>>>(d.tiles, d.cnt, d.ntiles, d.seg_off, d.nb, d.status, d.cnt + 2);
-    k_seg_zero<kSegMaxBits><<<gz, 256, 0, st>>>(d.tiles, d.cnt + 3, d.ntiles, d.seg_off, d.nb, d.status, d.cnt + 2);
-    SegArgs a{};
-    a.pt_in = pts; a.pt_out = out;
-    a.val_in = nullptr; a.val_out = perm;
-    a.offsets = d.seg_off;
-    a.seg_lo = d.lo; a.seg_nb = d.nb;
-    a.tiles = d.tiles; a.d_ntiles = d.cnt; a.ntiles_max = d.ntiles;
-    a.first = offsets; a.first_stride = 1;
-    a.status = d.status; a.counter = d.cnt + 1;
-    a.stitch = 0;
-    a.n = n;
-    a.d_fail = d.cnt + 2;
-    a.err = ws.err;
-    a.cube = cube; a.lut = lut; a.cells = cells; a.g = g;
-    if ((e = dist_launch<kDistMidBits>(a, d.ntiles, ws.num_sms, st))) return e;
-    a.d_ntiles = d.cnt + 3; a.counter = d.cnt + 4;
-    return dist_launch<kSegMaxBits>(a, d.ntiles, ws.num_sms, st);
+    auto kcount = cells ? k_dist_count<true> : k_dist_count<false>;
+    if ((e = cudaFuncSetAttribute(kcount, cudaFuncAttributeMaxDynamicSharedMemorySize, tsm))) return e;
+    kcount<<<gc, kDistCountNT, tsm, st>>>(b);
+    k_dist_colscan<<<kDistWideDig * 32 / 256, 256, 0, st>>>(b);
+    const int smem = (int)std::max(sizeof(DistSmem), sizeof(WideSmem));
+    if ((e = cudaFuncSetAttribute(k_dist_sweep, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
+    k_dist_sweep<<<grid, kDistNT, smem, st>>>(b);
+    return cudaGetLastError();
 }
 
 cudaError_t seg_scatter(const SegScratch& sc, const SegCall& c, const Workspace& ws, cudaStream_t st)

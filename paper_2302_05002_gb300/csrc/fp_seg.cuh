@@ -24,8 +24,7 @@ namespace fp {
 static_assert(sizeof(fp_node) == 40 && offsetof(fp_node, leaf_first) % 8 == 0, "fp_node layout");
 
 constexpr int kSegSmallBits = 8;
-// earlier tiles' words one look-back round trip reads per digit (16 measured
-// no faster than 8 on the 10^9-point distribution)
+// earlier tiles' words one look-back round trip reads per digit
 constexpr int kSegLookBatch = 8;
 constexpr int kSegMaxBits = 11;
 
@@ -60,15 +59,9 @@ struct SegArgs {
 
     const uint32_t* d_fail;
     uint32_t* err;
-
-    // distribution (DIST): the digit is the chunk of the point's level-g cell
-    const fp_cube* cube;
-    const uint32_t* lut;
-    const uint32_t* cells;                // nullable: the level-g cell of every point (else computed)
-    int g;
 };
 
-template <bool CPT, int MAXB, bool DIST = false>
+template <bool CPT, int MAXB>
 struct SegSmem {
     using dig_t = typename std::conditional<(MAXB <= 8), uint8_t, uint16_t>::type;
     static constexpr size_t pt = CPT ? sizeof(int4) * kSortTile : 0;
@@ -76,7 +69,7 @@ struct SegSmem {
     static constexpr size_t val = sizeof(uint32_t) * kSortTile;
     static constexpr size_t cnt = sizeof(uint32_t) * (1 << MAXB);
     static constexpr size_t off = sizeof(uint32_t) * (1 << MAXB);
-    static constexpr size_t pos = DIST ? 0 : sizeof(uint16_t) * kSortTile;   // tile position of a staged record
+    static constexpr size_t pos = sizeof(uint16_t) * kSortTile;   // tile position of a staged record
     static constexpr size_t dig = sizeof(dig_t) * kSortTile;
     static constexpr size_t whist = sizeof(uint16_t) * kSortWarps * (1 << MAXB);
     static constexpr size_t misc = 4 * (1 + kSortWarps + 15);
@@ -84,22 +77,15 @@ struct SegSmem {
     static constexpr size_t total = pt + gbase + val + cnt + off + pos + dig + whist + misc + tiles;
 };
 
-// two CTAs per SM while the shared memory allows it (8-bit digits; 9-bit
-// digits without the staging positions, i.e. in the distribution)
-template <bool CPT, int MAXB, bool DIST>
-constexpr int seg_ctas() { return SegSmem<CPT, MAXB, DIST>::total <= 113 * 1024 ? 2 : 1; }
+// two CTAs per SM while the shared memory allows it (8-bit digits)
+template <bool CPT, int MAXB>
+constexpr int seg_ctas() { return SegSmem<CPT, MAXB>::total <= 113 * 1024 ? 2 : 1; }
 
-template <bool CPT, int MAXB, bool DIST = false>
-__global__ void __launch_bounds__(kSortNT, (seg_ctas<CPT, MAXB, DIST>())) k_seg_pass(SegArgs a)
+template <bool CPT, int MAXB>
+__global__ void __launch_bounds__(kSortNT, (seg_ctas<CPT, MAXB>())) k_seg_pass(SegArgs a)
 {
     if (*a.d_fail) return;
-    CubeDev cube;
-    float scale_g = 0.f;
-    if (DIST && !a.cells) {
-        cube = load_cube(a.cube);
-        scale_g = scale_at(cube, a.g);
-    }
-    using SM = SegSmem<CPT, MAXB, DIST>;
+    using SM = SegSmem<CPT, MAXB>;
     using dig_t = typename SM::dig_t;
     extern __shared__ __align__(16) unsigned char smem[];
     unsigned char* sp = smem;
@@ -144,28 +130,7 @@ __global__ void __launch_bounds__(kSortNT, (seg_ctas<CPT, MAXB, DIST>())) k_seg_
 #pragma unroll
         for (int r = 0; r < kSortIPT; ++r) {
             const int p = warp * (kSortIPT * 32) + r * 32 + lane;
-            if (DIST) {
-                uint32_t cell = 0;
-                if (p < tn) {
-                    if (a.cells) {
-                        cell = __ldg(a.cells + base + p);
-                        if (cell >> (3 * a.g)) { raise(a.err, FP_ERR_CAPACITY, 19); cell = 0; }   // not a cell of the grid
-                    } else {
-                        const int4 q = __ldg(a.pt_in + base + p);
-                        cell = key_small(q.x, q.y, q.z, cube, scale_g, a.g);
-                    }
-                }
-                dg[r] = cell;
-            } else {
-                dg[r] = p < tn ? a.id_in[base + p] - lo : 0xFFFFFFFFu;
-            }
-        }
-        if (DIST) {   // cell -> chunk, all gathers in flight together
-#pragma unroll
-            for (int r = 0; r < kSortIPT; ++r) {
-                const int p = warp * (kSortIPT * 32) + r * 32 + lane;
-                dg[r] = p < tn ? a.lut[dg[r]] - lo : 0xFFFFFFFFu;
-            }
+            dg[r] = p < tn ? a.id_in[base + p] - lo : 0xFFFFFFFFu;
         }
         uint32_t pack[kSortIPT];
 #pragma unroll
@@ -225,8 +190,8 @@ __global__ void __launch_bounds__(kSortNT, (seg_ctas<CPT, MAXB, DIST>())) k_seg_
                 const uint32_t lp = s_off[d] + s_whist[warp * nb + d] + (pack[r] >> 16);
                 const uint64_t i = base + p;
                 if (CPT) s_pt[lp] = __ldg(a.pt_in + i);
-                s_val[lp] = DIST ? (uint32_t)i : a.val_in[i];
-                if (!DIST) s_pos[lp] = (uint16_t)p;
+                s_val[lp] = a.val_in[i];
+                s_pos[lp] = (uint16_t)p;
                 s_dig[lp] = (dig_t)d;
             }
         }
@@ -301,18 +266,16 @@ struct SegCall {
     uint32_t *st_rank, *st_list, *st_nrank, *st_tiles;
 };
 
-// Distribution of n points into chunks without the radix passes: with the
-// cells and a 16-byte aligned scratch of n chunk ids given, 1..512 chunks take
-// the counting pass and the double-buffered sweep (fp_seg.cu); else 257..512
-// chunks the 9-bit segmented sweep; 513..2048 chunks the 11-bit one (digit =
-// chunk of the point's cell, bucket bases = the chunk offsets).  *run_sort is
-// set to 1 when the count is outside these ranges (the radix passes run
-// instead), 0 when one of them ran.
+// Distribution of n points into up to 4096 chunks by the counting pass and a
+// double-buffered sweep (fp_seg.cu); the points' cells given or computed.
+// chunk_tmp: n chunk ids, 16-byte aligned.  *run_sort is set to 1, and hist
+// (kSortHistWords) cleared, when there are more chunks (the radix passes run
+// instead), else 0.
 size_t dist_wide_bytes(uint64_t n);
 cudaError_t dist_wide(const int4* pts, uint64_t n, const fp_cube* cube, int g, const uint32_t* lut,
                       const uint64_t* offsets, const uint32_t* num_chunks, int4* out, uint32_t* perm,
-                      uint32_t* run_sort, const Workspace& ws, cudaStream_t st, const uint32_t* cells = nullptr,
-                      uint16_t* chunk_tmp = nullptr);
+                      uint32_t* run_sort, uint32_t* hist, const Workspace& ws, cudaStream_t st, const uint32_t* cells,
+                      uint16_t* chunk_tmp);
 
 // Setup (chunk node ids, digits, tiles), status reset, both pass variants.
 // Afterwards cnt[2] != 0 means a chunk did not fit (the caller's whole-array

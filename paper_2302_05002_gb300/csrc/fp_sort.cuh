@@ -11,10 +11,15 @@
 //   3. stages the records in shared memory in digit order and writes each digit
 //      run contiguously (coalesced).
 // Several passes (least significant digit first) sort by a wider key.  The
-// number of passes and the digit width are read from a device-side plan, so a
+// number of passes and the digit width follow from counts on the device (every
+// block derives them, and its digits' bases from the histogram, by itself), so a
 // whole multi-pass sort can be enqueued without knowing the key range on the
 // host: surplus pass slots return at once, and slot k reads from the source,
 // or the temporaries, and writes to the destination when it is the last pass.
+// A sort is one histogram launch and one launch per pass: the histogram clears
+// the first pass's look-back words, every pass the next one's (two sets, in
+// turn).  (A launch to clear them before each pass and one to turn the histogram
+// into bases took 29 more launches in a build, about 2 us of host time each.)
 #pragma once
 #include "fp_internal.cuh"
 
@@ -67,12 +72,30 @@ FP_DEV uint32_t look_back(Word word, int64_t t, int64_t t_first, uint32_t* err, 
     return excl;
 }
 
-struct SortPlan {
-    uint32_t npass;    // passes to run (1..kSortMaxPass)
-    uint32_t bits;     // digit width of every pass
-    uint32_t shift0;   // key bit of digit 0
-    uint32_t pad;
+// What decides the passes of a sort and the bases of their buckets.
+struct SortSpec {
+    const uint32_t* d_nw;      // ids below *d_nw (nw_max when null); their bits unless fixed_bits is given
+    uint64_t nw_max;
+    uint32_t fixed_bits;       // 0, or the key's bits above shift0 ...
+    const uint32_t* d_rank_n;  // ... plus, when given, the bits of values below *d_rank_n
+    uint32_t shift0;           // key bit of digit 0
+    uint32_t* hist;            // [kSortMaxPass][1 << kSortMaxBits] digit counts, then the pass slots' tile counters
 };
+constexpr int kSortHistWords = (kSortMaxPass << kSortMaxBits) + 8;   // all zero before the histogram
+
+// bits of the largest value below n (at least 1)
+FP_DEV uint32_t bits_below(uint64_t n) { return n <= 2 ? 1u : 64u - (uint32_t)__clzll((long long)(n - 1)); }
+
+// Passes and digit width for a key of `need` bits (at most 64): the fewest
+// passes of at most 8 bits, the bits spread evenly over them.
+FP_DEV void sort_shape(const SortSpec& p, uint32_t& npass, uint32_t& bits)
+{
+    uint32_t need = p.fixed_bits ? p.fixed_bits + (p.d_rank_n ? bits_below(*p.d_rank_n) : 0u)
+                                 : bits_below(p.d_nw ? (uint64_t)*p.d_nw : p.nw_max);
+    need = min(need, 64u);
+    npass = (need + kSortMaxBits - 1) / kSortMaxBits;
+    bits = (need + npass - 1) / npass;
+}
 
 // Buffers of one multi-pass sort.  Null pointers mean "field not present".
 // Passes ping-pong between dst and one temporary so that the last pass lands
@@ -88,10 +111,8 @@ struct SortArgs {
     SortBufs b;
     uint64_t n;               // records (upper bound when d_n is set)
     const uint32_t* d_n;      // device-side record count (nullable)
-    const SortPlan* plan;
-    const uint64_t* bases;    // [kSortMaxPass][1 << kSortMaxBits]
-    uint32_t* status;         // [tiles][1 << bits]
-    uint32_t* counter;        // tile counter of the pass
+    SortSpec spec;
+    uint32_t* status[2];      // [tiles][1 << bits] look-back words of the even and the odd passes
     // digit from points
     const fp_cube* cube;
     const uint32_t* lut;      // DIG_CHUNK: cell -> chunk
@@ -147,8 +168,9 @@ struct SortSmem {
 template <int DIG, bool CPT, bool CK64, bool CK32>
 __global__ void __launch_bounds__(kSortNT, 2) k_sort_pass(SortArgs a, int slot)
 {
-    const SortPlan plan = *a.plan;
-    if (slot >= (int)plan.npass || (a.run_if && !*a.run_if)) return;
+    uint32_t npass_u, bits_u;
+    sort_shape(a.spec, npass_u, bits_u);
+    if (slot >= (int)npass_u || (a.run_if && !*a.run_if)) return;
     using SM = SortSmem<DIG, CPT, CK64, CK32>;
     using dig_t = typename SM::dig_t;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -169,13 +191,14 @@ __global__ void __launch_bounds__(kSortNT, 2) k_sort_pass(SortArgs a, int slot)
     uint32_t* s_tile = reinterpret_cast<uint32_t*>(sp);
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int bits = (int)plan.bits;
+    const int bits = (int)bits_u;
     const int nb = 1 << bits;
     const uint32_t dmask = (uint32_t)nb - 1;
-    const int shift = (int)(plan.shift0 + slot * plan.bits);
+    const int shift = (int)a.spec.shift0 + slot * bits;
     const uint64_t n = a.d_n ? min((uint64_t)*a.d_n, a.n) : a.n;
     const uint64_t ntiles = (n + kSortTile - 1) / kSortTile;
-    const int npass = (int)plan.npass;
+    const int npass = (int)npass_u;
+    if (ntiles == 0) return;
 
     const int4* in_pt = pick_src(slot, npass, a.b.pt_src, a.b.pt_dst, a.b.pt_tmp);
     const uint32_t* in_val = pick_src(slot, npass, a.b.val_src, a.b.val_dst, a.b.val_tmp);
@@ -185,7 +208,16 @@ __global__ void __launch_bounds__(kSortNT, 2) k_sort_pass(SortArgs a, int slot)
     uint32_t* out_val = pick_dst(slot, npass, a.b.val_dst, a.b.val_tmp);
     uint64_t* out_k64 = pick_dst(slot, npass, a.b.k64_dst, a.b.k64_tmp);
     uint32_t* out_k32 = pick_dst(slot, npass, a.b.k32_dst, a.b.k32_tmp);
-    const uint64_t* bases = a.bases + (size_t)slot * (1 << kSortMaxBits);
+    uint32_t* const status = a.status[slot & 1];
+    uint32_t* const status_next = slot + 1 < npass ? a.status[(slot + 1) & 1] : nullptr;
+    uint32_t* const counter = a.spec.hist + (kSortMaxPass << kSortMaxBits) + slot;
+    // first output position of bucket threadIdx.x
+    uint32_t base_d;
+    {
+        const uint32_t h = (int)threadIdx.x < nb ? a.spec.hist[(slot << kSortMaxBits) + threadIdx.x] : 0u;
+        uint32_t tot;
+        base_d = block_exclusive_scan<kSortNT, uint32_t>(h, s_misc + 1, tot);
+    }
 
     CubeDev cube;
     if (DIG == DIG_CHUNK) cube = load_cube(a.cube);
@@ -208,7 +240,7 @@ __global__ void __launch_bounds__(kSortNT, 2) k_sort_pass(SortArgs a, int slot)
     // smaller ones, so holding one in reserve cannot deadlock the look-back).
     if (threadIdx.x == 0) {
         if (use_bulk) mbar_init(s_bar, 1);
-        s_tile[0] = atomicAdd(a.counter, 1u);
+        s_tile[0] = atomicAdd(counter, 1u);
         if (use_bulk) issue(s_tile[0]);
     }
     for (int it = 0;; ++it) {
@@ -218,7 +250,7 @@ __global__ void __launch_bounds__(kSortNT, 2) k_sort_pass(SortArgs a, int slot)
         __syncthreads();
         const uint64_t tile = s_tile[it & 1];
         if (tile >= ntiles) break;
-        if (threadIdx.x == 0) s_tile[(it + 1) & 1] = atomicAdd(a.counter, 1u);
+        if (threadIdx.x == 0) s_tile[(it + 1) & 1] = atomicAdd(counter, 1u);
         const uint64_t base = tile * kSortTile;
         const int tn = (int)(n - base < (uint64_t)kSortTile ? n - base : (uint64_t)kSortTile);
         uint16_t* wh = s_whist + warp * nb;
@@ -289,7 +321,8 @@ __global__ void __launch_bounds__(kSortNT, 2) k_sort_pass(SortArgs a, int slot)
                 s += v;
             }
             s_cnt[d] = s;
-            if (tile != a.withhold) a.status[tile * nb + d] = (tile == 0 ? kStFlagInc : kStFlagAgg) | s;
+            if (tile != a.withhold) status[tile * nb + d] = (tile == 0 ? kStFlagInc : kStFlagAgg) | s;
+            if (status_next) status_next[tile * nb + d] = 0;
         }
         __syncthreads();
         // exclusive scan of s_cnt over digits -> s_off (each thread a run of digits)
@@ -327,14 +360,15 @@ __global__ void __launch_bounds__(kSortNT, 2) k_sort_pass(SortArgs a, int slot)
         }
 
         // ---- look-back: exclusive prefix of every digit over earlier tiles
-        for (int d = threadIdx.x; d < nb; d += kSortNT) {
+        if ((int)threadIdx.x < nb) {
+            const int d = threadIdx.x;
             uint32_t excl = 0;
             if (tile > 0) {
-                auto word = [&](int64_t t) { return &a.status[(uint64_t)t * nb + d]; };
+                auto word = [&](int64_t t) { return &status[(uint64_t)t * nb + d]; };
                 excl = look_back<decltype(word), kLookBatch>(word, (int64_t)tile - 1, 0, a.err, a.spin_limit);
-                if (tile != a.withhold) atomicExch(&a.status[tile * nb + d], kStFlagInc | (excl + s_cnt[d]));
+                if (tile != a.withhold) atomicExch(&status[tile * nb + d], kStFlagInc | (excl + s_cnt[d]));
             }
-            s_gbase[d] = bases[d] + excl - s_off[d];
+            s_gbase[d] = (uint64_t)base_d + excl - s_off[d];
         }
         __syncthreads();
 
@@ -350,21 +384,6 @@ __global__ void __launch_bounds__(kSortNT, 2) k_sort_pass(SortArgs a, int slot)
         __syncthreads();
     }
 }
-
-// zero the status words and the tile counter of one pass slot
-__global__ void k_sort_zero(uint32_t* status, uint32_t* counter, uint64_t n, const uint32_t* d_n, const SortPlan* plan,
-                            int slot);
-
-// Plan from per-id weights (ids 0..*d_nw-1, or nw_max when d_nw is null; the id
-// is the key above bit shift0):
-// digit histograms of every pass -> bucket bases.  hist: kSortMaxPass << kSortMaxBits u32, zeroed by the caller.
-__global__ void k_plan_hist_weights(const uint32_t* weights, const uint64_t* offsets, const uint32_t* d_nw,
-                                    uint64_t nw_max, uint32_t* hist);
-__global__ void k_plan_finalize(const uint32_t* d_nw, uint64_t nw_max, uint32_t fixed_bits, uint32_t shift0,
-                                const uint32_t* hist, SortPlan* plan, uint64_t* bases, const uint32_t* d_rank_n);
-// Plan of a fixed-width key sort: digits of bits [shift0, shift0 + total_bits) of k64 keys.
-__global__ void k_plan_hist_keys(const uint64_t* keys, uint64_t n, const uint32_t* d_n, uint32_t shift0,
-                                 uint32_t total_bits, uint32_t* hist, const uint32_t* d_rank_n);
 
 // host helpers
 // Launch bound of a sort: the device plan of keys with `bits` significant bits
@@ -382,22 +401,21 @@ inline uint32_t count_bits(uint64_t v)   // bits of v - 1, at least 1, as the de
     return b;
 }
 struct SortScratch {
-    SortPlan* plan;
-    uint64_t* bases;
-    uint32_t* hist;
-    uint32_t* status;
-    uint32_t* counter;
+    uint32_t* hist;        // kSortHistWords
+    uint32_t* status[2];
 };
 size_t sort_scratch_bytes(uint64_t n);
 SortScratch take_sort_scratch(const Workspace& ws, uint64_t n);
 
-// plan from weights of ids; then run the passes of the given kind
-cudaError_t sort_plan_weights(const SortScratch& sc, const uint32_t* weights, const uint64_t* offsets,
-                              const uint32_t* d_nw, uint64_t nw_max, uint32_t shift0, cudaStream_t st);
-// total_bits of key above shift0, plus the bit width of *d_rank_n when given
-cudaError_t sort_plan_keys(const SortScratch& sc, const uint64_t* keys, uint64_t n, const uint32_t* d_n,
-                           uint32_t shift0, uint32_t total_bits, cudaStream_t st,
-                           const uint32_t* d_rank_n = nullptr);
+// Histogram of a sort; returns its spec in a.spec and the look-back words in
+// a.status.  From weights of ids: record counts per id (weights, or differences
+// of offsets).  From 64-bit keys: a.b.k64_src, total_bits above shift0, plus the
+// bits of values below *d_rank_n when given.  a.n, a.d_n and a.run_if are set
+// already.  zeroed: a kernel before on the stream has cleared sc.hist.
+cudaError_t sort_plan_weights(const SortScratch& sc, SortArgs& a, const uint32_t* weights, const uint64_t* offsets,
+                              const uint32_t* d_nw, uint64_t nw_max, bool zeroed, int num_sms, cudaStream_t st);
+cudaError_t sort_plan_keys(const SortScratch& sc, SortArgs& a, uint32_t shift0, uint32_t total_bits,
+                           const uint32_t* d_rank_n, bool zeroed, int num_sms, cudaStream_t st);
 
 template <int DIG, bool CPT, bool CK64, bool CK32>
 cudaError_t sort_launch(const SortArgs& a, int slot, int num_sms, cudaStream_t st)
@@ -416,26 +434,21 @@ cudaError_t sort_launch(const SortArgs& a, int slot, int num_sms, cudaStream_t s
     return cudaGetLastError();
 }
 
+// passes [0, npass) of a planned sort
 template <int DIG, bool CPT, bool CK64, bool CK32>
-cudaError_t sort_run_pass(const SortScratch& sc, const SortArgs& a0, int slot, int num_sms, cudaStream_t st)
+cudaError_t sort_run(SortArgs a, int npass, int num_sms, cudaStream_t st)
 {
-    cudaError_t e;
-    SortArgs a = a0;
     debug_wait_config(&a.withhold, &a.spin_limit);
-    a.plan = sc.plan;
-    a.bases = sc.bases;
-    a.status = sc.status;
-    a.counter = sc.counter + slot;
-    uint64_t ntiles = (a.n + kSortTile - 1) / kSortTile;
-    k_sort_zero<<<std::max(1, std::min(num_sms * 4, (int)((ntiles * (1 << kSortMaxBits) + 1023) / 1024))), 256, 0,
-                  st>>>(sc.status, sc.counter + slot, a.n, a.d_n, sc.plan, slot);
-    if ((e = cudaGetLastError())) return e;
     if (sort_bulk_layout<DIG, CPT, CK64, CK32>()) {
         auto al = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
         a.bulk = al(a.b.k64_src) && al(a.b.k64_tmp) && al(a.b.k64_dst) && al(a.b.val_src) && al(a.b.val_tmp) &&
                  al(a.b.val_dst);
     }
-    return sort_launch<DIG, CPT, CK64, CK32>(a, slot, num_sms, st);
+    for (int slot = 0; slot < npass; ++slot) {
+        cudaError_t e = sort_launch<DIG, CPT, CK64, CK32>(a, slot, num_sms, st);
+        if (e) return e;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace fp
