@@ -1,0 +1,75 @@
+// fp_cluster.cuh -- steps over a few thousand nodes or chunks in one launch: a
+// cluster of 8 CTAs of 1024 threads whose phases are separated by the hardware
+// cluster barrier.  Such a step used to be a chain of grid launches (scans of
+// three, sorts of two per pass); at these sizes a launch costs more, on the host
+// (about 2 us) and on the device (2 - 5 us), than the work between two barriers.
+#pragma once
+#include "fp_internal.cuh"
+
+namespace fp {
+
+constexpr int kClCtas = 8;        // portable cluster size
+constexpr int kClNT = 1024;
+constexpr int kClThreads = kClCtas * kClNT;
+
+FP_DEV uint32_t cl_rank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// barrier of the cluster; orders global memory between its CTAs (release, acquire)
+FP_DEV void cl_sync()
+{
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// Exclusive prefix sums over i in [0, n) of value(i) (a pair packed into 64
+// bits, each half below 2^32 in all), handed to store(i, prefix); returns the
+// total.  part: kClCtas words of global memory.  All threads of the cluster.
+template <typename Value, typename Store>
+FP_DEV uint64_t cl_scan(uint32_t n, uint64_t* part, uint64_t* smem_warp /* 32 words */, Value value, Store store)
+{
+    const uint32_t per = (n + kClCtas - 1) / kClCtas, lo = min(n, cl_rank() * per), hi = min(n, lo + per);
+    uint64_t s = 0;
+    for (uint32_t i = lo + threadIdx.x; i < hi; i += kClNT) s += value(i);
+    uint64_t tot;
+    block_exclusive_scan<kClNT, uint64_t>(s, smem_warp, tot);
+    if (threadIdx.x == 0) part[cl_rank()] = tot;
+    cl_sync();
+    uint64_t run = 0, all = 0;
+    for (int r = 0; r < kClCtas; ++r) {
+        const uint64_t v = *(volatile const uint64_t*)(part + r);
+        if (r < (int)cl_rank()) run += v;
+        all += v;
+    }
+    for (uint32_t i0 = lo; i0 < hi; i0 += kClNT) {
+        const uint32_t i = i0 + threadIdx.x;
+        const uint64_t v = i < hi ? value(i) : 0;
+        const uint64_t ex = run + block_exclusive_scan<kClNT, uint64_t>(v, smem_warp, tot);
+        if (i < hi) store(i, ex);
+        run += tot;
+    }
+    cl_sync();   // (part may be written again)
+    return all;
+}
+
+// launch of kernel(args) as one cluster
+template <typename Args>
+inline cudaError_t cl_launch(void (*kernel)(Args), const Args& args, cudaStream_t st)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(kClCtas);
+    cfg.blockDim = dim3(kClNT);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kClCtas;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args);
+}
+
+}  // namespace fp

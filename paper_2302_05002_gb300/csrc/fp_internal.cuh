@@ -115,7 +115,7 @@ struct NodeTables {                  // lookups of the id resolution, kept betwe
     uint32_t* nnode;                 // node count
 };
 size_t nodes_ws_bytes(const fp_params& p, uint64_t rec_cap);
-cudaError_t launch_octree_nodes(const uint32_t* counts, const fp_params& prm, NodeRec* recs, uint64_t rec_cap,
+cudaError_t launch_octree_nodes(const uint32_t* counts, uint64_t n, const fp_params& prm, NodeRec* recs, uint64_t rec_cap,
                                 const uint32_t* num_deep, fp_node* nodes, uint32_t node_cap, uint32_t* num_nodes,
                                 const NodeTables& T, const Workspace& ws, cudaStream_t st);
 cudaError_t launch_octree_resolve(const fp_point* pts, uint64_t n, const fp_cube* cube, const uint32_t* codes,

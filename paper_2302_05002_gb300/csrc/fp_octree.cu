@@ -31,6 +31,7 @@
 //   5. the points are scattered stably by leaf id (leaf-grouped output) and,
 //      in fp_subsample, by owner id (final output); owner segments of nodes
 //      above the chunks (the stitch) are re-sorted by original index.
+#include "fp_cluster.cuh"
 #include "fp_grid.cuh"
 #include "fp_seg.cuh"
 
@@ -1251,6 +1252,175 @@ __global__ void k_node_children(const uint32_t* nnode, const uint64_t* sorted_st
     }
 }
 
+// The node table in one launch of one cluster, for at most kNodeClusterMax nodes
+// by the host's bound (28 launches otherwise; 1M points: 110 -> NODEUS us).  Stable
+// least-significant-digit-first passes over (level, start): every CTA counts the
+// digits of its slice, all CTAs' counts give every digit's base, and each tile of
+// 1024 records is ranked by ballots.  A pass in which all records share the digit
+// is left out (without nodes below the count grid: all bits below level g).
+constexpr uint64_t kNodeClusterMax = 1ull << 18;
+
+struct NodeClusterArgs {
+    const NodeRec* rec;
+    uint32_t* nnode;
+    uint32_t ncap;
+    uint64_t *key[2];
+    uint32_t *val[2];
+    uint32_t* hist;        // [kClCtas][256]
+    uint64_t* part;        // [kClCtas]
+    uint64_t* starts;      // (not one of key[])
+    uint8_t* slevel;
+    uint32_t *ndesc, *idxtab, *leafw;
+    fp_node* nodes;
+    uint32_t node_cap;
+    uint32_t* num_nodes;
+    int g, lmax;
+    uint32_t* err;
+};
+
+__global__ void __launch_bounds__(kClNT, 1) k_node_cluster(NodeClusterArgs a)
+{
+    __shared__ uint32_t s_whist[kClNT / 32][256];
+    __shared__ uint32_t s_cnt[256], s_base[256], s_warp[32];
+    __shared__ unsigned long long s_mask;
+    const uint32_t rank = cl_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t M = min(*a.nnode, a.ncap);
+    const int lmax = a.lmax;
+    if (rank == 0 && tid == 0) {
+        *a.num_nodes = M;
+        if (M > a.node_cap) raise(a.err, FP_ERR_CAPACITY, 8);
+    }
+    // starts, and the bits in which any two of them differ
+    if (tid == 0) s_mask = 0;
+    __syncthreads();
+    uint64_t diff = 0;
+    const uint64_t s0 = M ? a.rec[0].key << (3 * (lmax - a.rec[0].level)) : 0;
+    for (uint32_t i = rank * kClNT + tid; i < M; i += kClThreads) {
+        const uint64_t s = a.rec[i].key << (3 * (lmax - a.rec[i].level));
+        a.key[0][i] = s;
+        a.val[0][i] = i;
+        diff |= s ^ s0;
+    }
+    diff |= __shfl_xor_sync(0xFFFFFFFFu, diff, 16);
+    diff |= __shfl_xor_sync(0xFFFFFFFFu, diff, 8);
+    diff |= __shfl_xor_sync(0xFFFFFFFFu, diff, 4);
+    diff |= __shfl_xor_sync(0xFFFFFFFFu, diff, 2);
+    diff |= __shfl_xor_sync(0xFFFFFFFFu, diff, 1);
+    if (lane == 0) atomicOr(&s_mask, (unsigned long long)diff);
+    __syncthreads();
+    if (tid == 0) a.part[rank] = s_mask;
+    cl_sync();
+    uint64_t mask = 0;
+    for (int r = 0; r < kClCtas; ++r) mask |= *(volatile const uint64_t*)(a.part + r);
+
+    const uint32_t per = (M + kClCtas - 1) / kClCtas, lo = min(M, rank * per), hi = min(M, lo + per);
+    int cur = 0;
+    for (int pass = -1; pass < 8; ++pass) {   // -1: the level
+        if (pass >= 0 && !((mask >> (8 * pass)) & 255u)) continue;
+        const uint64_t* kin = a.key[cur];
+        const uint32_t* vin = a.val[cur];
+        auto digit = [&](uint32_t i) -> uint32_t {
+            return pass < 0 ? a.rec[vin[i]].level : (uint32_t)(kin[i] >> (8 * pass)) & 255u;
+        };
+        if (tid < 256) s_cnt[tid] = 0;
+        __syncthreads();
+        for (uint32_t i0 = lo; i0 < hi; i0 += kClNT) {
+            const uint32_t i = i0 + tid;
+            const uint32_t d = i < hi ? digit(i) : 0u;
+            const uint32_t peers = match_bits<8>(d, i < hi);
+            if (i < hi && lane == (uint32_t)__ffs(peers) - 1) atomicAdd(&s_cnt[d], (uint32_t)__popc(peers));
+        }
+        __syncthreads();
+        if (tid < 256) a.hist[rank * 256 + tid] = s_cnt[tid];
+        cl_sync();
+        {
+            uint32_t before = 0, total = 0;
+            if (tid < 256)
+                for (int r = 0; r < kClCtas; ++r) {
+                    const uint32_t v = ld_volatile(a.hist + r * 256 + tid);
+                    if (r < (int)rank) before += v;
+                    total += v;
+                }
+            uint32_t all;
+            const uint32_t ex = block_exclusive_scan<kClNT, uint32_t>(total, s_warp, all);
+            if (tid < 256) s_base[tid] = ex + before;
+        }
+        uint64_t* kout = a.key[cur ^ 1];
+        uint32_t* vout = a.val[cur ^ 1];
+        for (uint32_t i0 = lo; i0 < hi; i0 += kClNT) {
+            for (uint32_t q = tid; q < (kClNT / 32) * 256 / 4; q += kClNT)
+                reinterpret_cast<uint4*>(&s_whist[0][0])[q] = make_uint4(0, 0, 0, 0);
+            __syncthreads();
+            const uint32_t i = i0 + tid;
+            const bool valid = i < hi;
+            const uint32_t d = valid ? digit(i) : 0u;
+            const uint32_t peers = match_bits<8>(d, valid);
+            if (valid && lane == (uint32_t)__ffs(peers) - 1) s_whist[warp][d] = __popc(peers);
+            __syncthreads();
+            if (tid < 256) {
+                uint32_t run = s_base[tid];
+                for (int w = 0; w < kClNT / 32; ++w) {
+                    const uint32_t c = s_whist[w][tid];
+                    s_whist[w][tid] = run;
+                    run += c;
+                }
+                s_base[tid] = run;
+            }
+            __syncthreads();
+            if (valid) {
+                const uint32_t at = s_whist[warp][d] + __popc(peers & lanemask_lt());
+                kout[at] = kin[i];
+                vout[at] = vin[i];
+            }
+            __syncthreads();
+        }
+        cl_sync();
+        cur ^= 1;
+    }
+    // records in preorder and the lookups
+    const uint64_t* ks = a.key[cur];
+    const uint32_t* vs = a.val[cur];
+    for (uint32_t i = rank * kClNT + tid; i < M; i += kClThreads) {
+        const NodeRec r = a.rec[vs[i]];
+        const uint64_t end = (r.key + 1) << (3 * (lmax - r.level));
+        uint32_t b0 = i + 1, b1 = M;
+        while (b0 < b1) {
+            const uint32_t m = (b0 + b1) >> 1;
+            if (ks[m] < end) b0 = m + 1;
+            else b1 = m;
+        }
+        fp_node o;
+        o.key = r.key;
+        o.first = 0;
+        o.leaf_first = r.leaf_first;
+        o.count = r.count;
+        o.n_own = 0;
+        o.n_desc = b0 - i - 1;
+        o.level = r.level;
+        o.child_mask = 0;
+        o.is_leaf = r.is_leaf;
+        o.pad = 0;
+        if (i < a.node_cap) a.nodes[i] = o;
+        a.starts[i] = ks[i];
+        a.slevel[i] = r.level;
+        a.ndesc[i] = o.n_desc;
+        a.leafw[i] = r.is_leaf ? r.count : 0;
+        if (r.level <= a.g) a.idxtab[((1ull << (3 * r.level)) - 1) / 7 + r.key] = i;
+    }
+    cl_sync();
+    for (uint32_t i = rank * kClNT + tid; i < M; i += kClThreads) {
+        const NodeRec r = a.rec[vs[i]];
+        if (r.level == 0) continue;
+        uint32_t p;
+        if (r.level - 1 <= a.g) p = a.idxtab[((1ull << (3 * (r.level - 1))) - 1) / 7 + (r.key >> 3)];
+        else p = node_lookup(ks, a.slevel, M, (r.key >> 3) << (3 * (lmax - r.level + 1)), r.level - 1);
+        if (p < M && p < a.node_cap)   // child_mask is byte 37 of the 40-byte record
+            atomicOr(reinterpret_cast<uint32_t*>(reinterpret_cast<unsigned char*>(a.nodes + p) + 36),
+                     (1u << (r.key & 7)) << 8);
+    }
+    if (rank == 0 && tid == 0 && *a.nnode > M) *a.nnode = M;   // (every CTA has read it: barriers above)
+}
+
 // owner and leaf ids of every distributed point; owned counts per node.
 // A node at a level <= g is found from the level-g cell in the point's code
 // (the id table of levels <= g); a node deeper than g lies in the subtree of its
@@ -1271,7 +1441,16 @@ constexpr int kOwnProbes = 32;
 constexpr int kResolveTabLevel = 4;   // node ids of the levels 0..4 in shared memory
 constexpr int kResolveTab = ((1 << (3 * (kResolveTabLevel + 1))) - 1) / 7;
 
-FP_DEV void own_add(uint32_t* keys, uint32_t* cnt, uint32_t* n_own, uint32_t id, uint32_t v)
+struct OwnCounts {   // the owned count of node id < cap: word id * stride
+    uint32_t* n_own;
+    uint32_t stride, cap;
+    FP_DEV void add(uint32_t id, uint32_t v) const
+    {
+        if (id < cap) atomicAdd(&n_own[(uint64_t)id * stride], v);
+    }
+};
+
+FP_DEV void own_add(uint32_t* keys, uint32_t* cnt, const OwnCounts& own, uint32_t id, uint32_t v)
 {
     uint32_t h = (id * 2654435761u) & (kOwnSlots - 1);
     for (int q = 0; q < kOwnProbes; ++q) {
@@ -1283,7 +1462,7 @@ FP_DEV void own_add(uint32_t* keys, uint32_t* cnt, uint32_t* n_own, uint32_t id,
         if (k == id) { atomicAdd(&cnt[h], v); return; }
         h = (h + 1) & (kOwnSlots - 1);
     }
-    atomicAdd(&n_own[id], v);   // the table is crowded: straight to the global count
+    own.add(id, v);   // the table is crowded: straight to the global count
 }
 
 // id of the node at level L > g holding distributed point j (kNone when absent):
@@ -1311,7 +1490,7 @@ __global__ void __launch_bounds__(kResolveNT) k_resolve(const fp_point* __restri
                                                         const uint32_t* idxtab, const uint64_t* sorted_start,
                                                         const uint8_t* sorted_level, const uint32_t* ndesc,
                                                         const uint32_t* nnode, uint32_t* owner, uint32_t* leafid,
-                                                        uint32_t* n_own, int g, int lmax, uint32_t* err)
+                                                        OwnCounts own, int g, int lmax, uint32_t* err)
 {
     __shared__ uint32_t s_key[kOwnSlots], s_cnt[kOwnSlots];
     __shared__ uint32_t s_idx[kResolveTab];   // the node ids of the coarse levels' cells
@@ -1359,13 +1538,13 @@ __global__ void __launch_bounds__(kResolveNT) k_resolve(const fp_point* __restri
                 if (leafid) leafid[j] = ids[1];
                 oid = ids[0];
             }
-            if (oid != kNone) own_add(s_key, s_cnt, n_own, oid, 1u);
+            if (oid != kNone) own_add(s_key, s_cnt, own, oid, 1u);
         }
         __syncthreads();
         for (int q = threadIdx.x; q < kOwnSlots; q += kResolveNT) {   // flush, and clear for the next tile
             const uint32_t k = s_key[q];
             if (k != kNone) {
-                atomicAdd(&n_own[k], s_cnt[q]);
+                own.add(k, s_cnt[q]);
                 s_key[q] = kNone;
                 s_cnt[q] = 0;
             }
@@ -1418,6 +1597,16 @@ static OctLayout oct_layout(uint64_t n, const fp_params& p)
 
 uint64_t node_capacity_bound(uint64_t n, const fp_params& p) { return oct_layout(n, p).node_cap; }
 
+// nodes of a cloud of n points: every node but the root is the child of an inner
+// node, and the inner nodes of a level hold more than C points each
+static uint64_t node_bound(uint64_t n, const fp_params& p)
+{
+    uint64_t b = 1;
+    for (uint32_t l = 0; l < p.max_level; ++l)
+        b += 8 * std::min(l < 20 ? 1ull << (3 * l) : ~0ull, (unsigned long long)(n / (p.node_capacity + 1)));
+    return b;
+}
+
 struct OctBufs {
     SortScratch sc;
     uint32_t* rcnt;        // counting slots of a split round: 8^3 per open node
@@ -1436,7 +1625,7 @@ struct OctBufs {
     uint64_t *nk, *nk2, *nk3, *nk4;
     uint32_t *nl, *nv2, *nv3;
     uint8_t* slevel;
-    uint32_t *idxtab, *leafw, *nown;
+    uint32_t *idxtab, *leafw;
     uint32_t* codes;
     uint32_t* leafid;
     uint32_t* ndesc;
@@ -1477,7 +1666,6 @@ static OctBufs oct_carve(const Workspace& ws, uint64_t n, const OctLayout& Ly)
     B.slevel = ws.take<uint8_t>(Ly.node_cap);
     B.idxtab = ws.take<uint32_t>(Ly.cells * 8 / 7 + 8);
     B.leafw = ws.take<uint32_t>(std::max<uint64_t>(Ly.node_cap, kScanMaxTiles));
-    B.nown = ws.take<uint32_t>(Ly.node_cap);
     B.codes = ws.take<uint32_t>(N);
     B.leafid = ws.take<uint32_t>(N);
     B.ndesc = ws.take<uint32_t>(Ly.node_cap);
@@ -1502,10 +1690,20 @@ struct NodeSortBufs {
 };
 
 static cudaError_t node_table(const SortScratch& sc, const NodeRec* nrec, uint32_t* nnode, uint32_t ncap,
-                              const NodeSortBufs& B, fp_node* nodes, uint32_t node_cap, uint32_t* num_nodes, int g,
-                              int lmax, const Workspace& ws, cudaStream_t st)
+                              uint64_t bound, const NodeSortBufs& B, fp_node* nodes, uint32_t node_cap,
+                              uint32_t* num_nodes, int g, int lmax, const Workspace& ws, cudaStream_t st)
 {
     cudaError_t e;
+    if (bound <= kNodeClusterMax) {
+        NodeClusterArgs a{};
+        a.rec = nrec; a.nnode = nnode; a.ncap = ncap;
+        a.key[0] = B.nk2; a.key[1] = B.nk3; a.val[0] = B.nl; a.val[1] = B.nv2;
+        a.hist = sc.hist; a.part = B.nk4;
+        a.starts = B.nk; a.slevel = B.slevel; a.ndesc = B.ndesc; a.idxtab = B.idxtab; a.leafw = B.leafw;
+        a.nodes = nodes; a.node_cap = node_cap; a.num_nodes = num_nodes;
+        a.g = g; a.lmax = lmax; a.err = ws.err;
+        return cl_launch(k_node_cluster, a, st);
+    }
     const unsigned gn = (ncap + 255) / 256;
     k_clamp<<<1, 1, 0, st>>>(nnode, ncap);
     k_node_keys<<<gn, 256, 0, st>>>(nrec, nnode, B.nk, B.nl, lmax);
@@ -1651,20 +1849,22 @@ cudaError_t launch_octree_impl(const fp_point* sorted, const uint32_t* perm, uin
     {
         NodeSortBufs nb{B.nk, B.nk2, B.nk3, B.nk4, B.nl, B.nv2, B.nv3, B.slevel, B.idxtab, B.leafw, B.ndesc};
         KTimerScope kt(FP_KERNEL_NODE_TABLE, st);
-        if ((e = node_table(sc, B.nrec, nnode, (uint32_t)Ly.node_cap, nb, nodes, node_cap, num_nodes, g, lmax, ws, st)))
+        if ((e = node_table(sc, B.nrec, nnode, (uint32_t)Ly.node_cap, node_bound(N, prm), nb, nodes, node_cap,
+                            num_nodes, g, lmax, ws, st)))
             return e;
-        if ((e = cudaMemsetAsync(B.nown, 0, (size_t)Ly.node_cap * sizeof(uint32_t), st))) return e;
     }
     // 6. owner and leaf ids per distributed point, owned counts
     {
         const int grid = (int)std::max<uint64_t>(
             1, std::min<uint64_t>((N + kResolveTile - 1) / kResolveTile, (uint64_t)ws.num_sms * 8));
         auto kres = lmax <= 10 ? k_resolve<true> : k_resolve<false>;
+        // counted in the node records (zeroed with the table)
+        const OwnCounts own{reinterpret_cast<uint32_t*>(nodes) + offsetof(fp_node, n_own) / sizeof(uint32_t),
+                            sizeof(fp_node) / sizeof(uint32_t), node_cap};
         KTimerScope kt(FP_KERNEL_RESOLVE, st);
         kres<<<grid, kResolveNT, 0, st>>>(sorted, N, cube, B.codes, B.idxtab, B.nk, B.slevel, B.ndesc, nnode, owner,
                                    (leaf_pts || leaf_perm) ? B.leafid : nullptr,
-                                   B.nown, g, lmax, ws.err);
-        k_write_nown<<<(unsigned)((Ly.node_cap + 255) / 256), 256, 0, st>>>(nodes, nnode, node_cap, B.nown);
+                                   own, g, lmax, ws.err);
     }
     // 7. leaf-grouped points: stable scatter by leaf id, chunk by chunk (every
     // leaf lies in the subtree of its points' chunk); the whole-array sort by
@@ -1682,6 +1882,7 @@ cudaError_t launch_octree_impl(const fp_point* sorted, const uint32_t* perm, uin
         sg.n = N;
         sg.first = reinterpret_cast<const uint64_t*>(nodes) + offsetof(fp_node, leaf_first) / sizeof(uint64_t);
         sg.first_stride = sizeof(fp_node) / sizeof(uint64_t);
+        sg.hist = sc.hist;
         if ((e = seg_scatter(B.seg, sg, ws, st))) return e;
         SortArgs a{};
         a.b.pt_src = reinterpret_cast<const int4*>(sorted);
@@ -1689,8 +1890,8 @@ cudaError_t launch_octree_impl(const fp_point* sorted, const uint32_t* perm, uin
         a.b.pt_dst = reinterpret_cast<int4*>(leaf_pts);
         a.b.val_src = perm; a.b.val_tmp = B.lt_val; a.b.val_dst = leaf_perm;
         a.b.k32_src = B.leafid; a.b.k32_tmp = B.lt_k32; a.b.k32_dst = nullptr;
-        a.n = N; a.d_n = B.seg.cnt + 5; a.err = ws.err;
-        if ((e = sort_plan_weights(sc, a, B.leafw, nullptr, nnode, Ly.node_cap, false, ws.num_sms, st))) return e;
+        a.n = N; a.run_if = B.seg.cnt + 2; a.err = ws.err;
+        if ((e = sort_plan_weights(sc, a, B.leafw, nullptr, nnode, Ly.node_cap, true, ws.num_sms, st))) return e;
         const int np = sort_passes(count_bits(Ly.node_cap));   // leaf ids below node_cap
         if (leaf_pts) e = sort_run<DIG_K32, true, false, true>(a, np, ws.num_sms, st);
         else e = sort_run<DIG_K32, false, false, true>(a, np, ws.num_sms, st);
@@ -1729,7 +1930,7 @@ size_t nodes_ws_bytes(const fp_params& p, uint64_t rec_cap)
     return dry.used;
 }
 
-cudaError_t launch_octree_nodes(const uint32_t* counts, const fp_params& prm, NodeRec* recs, uint64_t rec_cap,
+cudaError_t launch_octree_nodes(const uint32_t* counts, uint64_t n, const fp_params& prm, NodeRec* recs, uint64_t rec_cap,
                                 const uint32_t* num_deep, fp_node* nodes, uint32_t node_cap, uint32_t* num_nodes,
                                 const NodeTables& T, const Workspace& ws, cudaStream_t st)
 {
@@ -1745,7 +1946,8 @@ cudaError_t launch_octree_nodes(const uint32_t* counts, const fp_params& prm, No
     k_cells_open<<<grid_tiles(g), kGtNT, 0, st>>>(c, B.pyr, B.rsum, 0, 1, nullptr, nullptr, nullptr, nullptr);
     NodeSortBufs nb = B.nb;
     nb.nk = T.starts; nb.slevel = T.slevel; nb.idxtab = T.idxtab; nb.ndesc = T.ndesc;
-    if ((e = node_table(B.sc, recs, T.nnode, (uint32_t)rec_cap, nb, nodes, node_cap, num_nodes, g, lmax, ws, st)))
+    if ((e = node_table(B.sc, recs, T.nnode, (uint32_t)rec_cap, n ? node_bound(n, prm) : rec_cap, nb, nodes, node_cap,
+                        num_nodes, g, lmax, ws, st)))
         return e;
     return cudaMemsetAsync(T.nown, 0, rec_cap * sizeof(uint32_t), st);
 }
@@ -1759,7 +1961,7 @@ cudaError_t launch_octree_resolve(const fp_point* pts, uint64_t n, const fp_cube
         1, std::min<uint64_t>((n + kResolveTile - 1) / kResolveTile, (uint64_t)ws.num_sms * 8));
     auto kres = prm.max_level <= 10 ? k_resolve<true> : k_resolve<false>;
     kres<<<grid, kResolveNT, 0, st>>>(pts, n, cube, codes, T.idxtab, T.starts, T.slevel, T.ndesc, T.nnode, owner, nullptr,
-                               T.nown, (int)prm.grid_log2, (int)prm.max_level, ws.err);
+                               OwnCounts{T.nown, 1u, 0xFFFFFFFFu}, (int)prm.grid_log2, (int)prm.max_level, ws.err);
     return cudaGetLastError();
 }
 
@@ -1768,13 +1970,6 @@ cudaError_t launch_node_first(fp_node* nodes, const uint32_t* num_nodes, uint32_
                               uint64_t* first, uint32_t* nm, uint64_t* tiles64, cudaStream_t st);
 
 // ------------------------------------------------------------ subsample
-__global__ void k_nown_in(const fp_node* nodes, const uint32_t* num_nodes, uint32_t node_cap, uint32_t* nown)
-{
-    uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    uint32_t M = *num_nodes < node_cap ? *num_nodes : node_cap;
-    if (i < M) nown[i] = nodes[i].n_own;
-}
-
 __global__ void k_first_out(fp_node* nodes, const uint32_t* num_nodes, uint32_t node_cap, const uint64_t* first)
 {
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1782,78 +1977,7 @@ __global__ void k_first_out(fp_node* nodes, const uint32_t* num_nodes, uint32_t 
     if (i < M) nodes[i].first = first[i];
 }
 
-// owner segments whose original indices are not ascending (owners above the chunks)
-__global__ void k_mark_unsorted(const uint32_t* fown, const uint32_t* fperm, uint64_t n, const uint32_t* d_n,
-                                uint32_t* mark, const uint32_t* nm)
-{
-    const uint32_t M = *nm;
-    if (*d_n < n) n = *d_n;
-    uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t f = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; f + 1 < n; f += stride)
-        if (fown[f] == fown[f + 1] && fperm[f] > fperm[f + 1] && fown[f] < M) mark[fown[f]] = 1;
-}
-
 __global__ void k_clamp_copy(const uint32_t* v, uint32_t cap, uint32_t* out) { *out = *v < cap ? *v : cap; }
-
-__global__ void k_stitch_list(const uint32_t* mark, const uint32_t* mrank, const uint32_t* num_nodes,
-                              uint32_t node_cap, uint32_t* mlist, const uint32_t* nown, uint32_t* mown)
-{
-    uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    uint32_t M = *num_nodes < node_cap ? *num_nodes : node_cap;
-    if (i < M && mark[i]) {
-        mlist[mrank[i]] = i;
-        mown[mrank[i]] = nown[i];
-    }
-}
-
-// keys (rank << 32 | original index) of the points of marked nodes, value = final position;
-// one thread per stitch record, its node found by binary search over the segment offsets
-__global__ void k_stitch_keys(const uint32_t* mlist, const uint32_t* nmarked, const uint32_t* soff,
-                              const uint32_t* nstitch, const uint64_t* first, const uint32_t* fperm, uint64_t* key,
-                              uint32_t* val)
-{
-    const uint32_t nm = *nmarked, S = *nstitch;
-    for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < S; t += gridDim.x * blockDim.x) {
-        uint32_t a = 0, b = nm;
-        while (a < b) { uint32_t m = (a + b) >> 1; if (soff[m] <= t) a = m + 1; else b = m; }
-        const uint32_t r = a - 1;
-        const uint64_t f = first[mlist[r]] + (t - soff[r]);
-        key[t] = ((uint64_t)r << 32) | fperm[f];
-        val[t] = (uint32_t)f;
-    }
-}
-
-__global__ void k_stitch_gather(const uint32_t* nstitch, const uint32_t* val, const int4* fin, const uint32_t* fperm,
-                                int4* tpt, uint32_t* tperm)
-{
-    const uint32_t S = *nstitch;
-    for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < S; t += gridDim.x * blockDim.x) {
-        tpt[t] = fin[val[t]];
-        tperm[t] = fperm[val[t]];
-    }
-}
-
-__global__ void k_stitch_put(const uint32_t* nstitch, const uint64_t* key, const uint32_t* mlist, const uint32_t* soff,
-                             const uint64_t* first, const int4* tpt, const uint32_t* tperm, int4* fin, uint32_t* fperm)
-{
-    const uint32_t S = *nstitch;
-    for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < S; t += gridDim.x * blockDim.x) {
-        uint32_t r = (uint32_t)(key[t] >> 32);
-        uint64_t f = first[mlist[r]] + (t - soff[r]);
-        fin[f] = tpt[t];
-        fperm[f] = tperm[t];
-    }
-}
-
-// stitch records staged by the segmented scatter: a node above the chunks keeps
-// all of its points through the staging area, the others none of theirs
-__global__ void k_stitch_counts(const uint8_t* inside, const uint32_t* nown, const uint32_t* nm, uint32_t* scnt,
-                                uint32_t cap)
-{
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= cap) return;
-    scnt[i] = i < *nm && !inside[i] ? nown[i] : 0u;
-}
 
 // sorted staging record t = (rank of node X, original index): final position
 // first[X] + rank inside X
@@ -1887,22 +2011,34 @@ cudaError_t launch_node_first(fp_node* nodes, const uint32_t* num_nodes, uint32_
     return cudaGetLastError();
 }
 
-static const uint64_t kMaxScanNodes = (uint64_t)kScanTile * kScanMaxTiles;
+// Whole-array path, where a chunk holds more nodes than the segmented scatter
+// takes: the points and owners in original order, from which one stable sort by
+// owner gives the final layout.
+__global__ void __launch_bounds__(256) k_original_order(const uint32_t* gate, const int4* pts, const uint32_t* perm,
+                                                        const uint32_t* owner, uint64_t n, int4* opts,
+                                                        uint32_t* oowner, uint32_t* err)
+{
+    if (!*gate) return;
+    for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (uint64_t)gridDim.x * blockDim.x) {
+        const uint32_t i = perm[j];
+        if (i >= n) { raise(err, FP_ERR_CAPACITY, 11); continue; }
+        opts[i] = __ldg(pts + j);
+        oowner[i] = owner[j];
+    }
+}
+
+constexpr uint64_t kMaxNodes = 1ull << 23;   // node_cap of a subsample call
 
 struct SubBufs {
     SortScratch sc;
-    uint32_t *nown, *mark, *mrank, *mlist, *mown, *soff, *cnt;
-    uint32_t *srank, *slist;   // staging: rank of a node outside every chunk subtree, and back
+    uint32_t* hist2;           // histogram of the whole-array sort
+    uint32_t *nown, *soff, *cnt;
+    uint32_t *srank, *slist;   // rank of a node outside every chunk subtree, and back
     uint64_t* first;
-    int4* t_pt;
-    uint32_t *t_val, *t_k32, *fown;
+    int4 *o_pt, *t_pt;
+    uint32_t *o_own, *t_val, *t_k32;
     uint64_t *s_key, *s_key2, *s_key3;
     uint32_t *s_val, *s_val2, *s_val3;
-    int4* s_pt;
-    uint32_t* s_perm;
-    uint64_t* tiles64;
-    uint32_t* tiles32;
-    uint32_t* scnt;
     SegScratch seg;
 };
 
@@ -1914,34 +2050,21 @@ static SubBufs sub_carve(const Workspace& ws, uint64_t n, uint64_t M)
     SubBufs B;
     const uint64_t N = n ? n : 1;
     B.sc = take_sort_scratch(ws, N);
+    B.hist2 = ws.take<uint32_t>(kSortHistWords);
     B.nown = ws.take<uint32_t>(M); B.first = ws.take<uint64_t>(M + 1);
-    B.mark = ws.take<uint32_t>(M); B.mrank = ws.take<uint32_t>(M); B.mlist = ws.take<uint32_t>(M);
-    B.mown = ws.take<uint32_t>(M); B.soff = ws.take<uint32_t>(M + 1); B.cnt = ws.take<uint32_t>(8);
+    B.soff = ws.take<uint32_t>(M + 1); B.cnt = ws.take<uint32_t>(8);
     B.srank = ws.take<uint32_t>(M); B.slist = ws.take<uint32_t>(M);
-    // One region serves three sets of per-point buffers that are never live
-    // together: the whole-array path's sort temporaries and owner copy (dead
-    // once its unsorted segments are marked), the stitch records and their
-    // sort buffers, and the stitch's gathered points (written over the sort's
-    // source and temporary, both dead after the sort).
+    // One region serves two sets of per-point buffers that are never live
+    // together: the whole-array path's, and the staged records and their sort's.
     const size_t region = ws.used;
+    B.o_pt = ws.take<int4>(N); B.o_own = ws.take<uint32_t>(N);
     B.t_pt = ws.take<int4>(N); B.t_val = ws.take<uint32_t>(N); B.t_k32 = ws.take<uint32_t>(N);
-    B.fown = ws.take<uint32_t>(N);
     const size_t end_t = ws.used;
     ws.used = region;
     B.s_key = ws.take<uint64_t>(N); B.s_val = ws.take<uint32_t>(N);
     B.s_key2 = ws.take<uint64_t>(N); B.s_val2 = ws.take<uint32_t>(N);
-    const size_t end_src = ws.used;
     B.s_key3 = ws.take<uint64_t>(N); B.s_val3 = ws.take<uint32_t>(N);
-    const size_t end_s = ws.used;
-    ws.used = region;
-    B.s_pt = ws.take<int4>(N); B.s_perm = ws.take<uint32_t>(N);
-    if (ws.used > end_src) {   // (20 bytes per point fit in 24 unless rounding says otherwise: then after)
-        ws.used = end_s;
-        B.s_pt = ws.take<int4>(N); B.s_perm = ws.take<uint32_t>(N);
-    }
-    ws.used = std::max(std::max(end_t, end_s), ws.used);
-    B.tiles64 = ws.take<uint64_t>(kScanMaxTiles); B.tiles32 = ws.take<uint32_t>(kScanMaxTiles);
-    B.scnt = ws.take<uint32_t>(M + 1);
+    ws.used = std::max(end_t, ws.used);
     B.seg = take_seg_scratch(ws, N, chunk_bound(n), M);
     return B;
 }
@@ -1959,26 +2082,16 @@ cudaError_t launch_subsample(fp_node* nodes, const uint32_t* num_nodes, uint32_t
                              uint32_t* final_perm, const Workspace& ws, cudaStream_t st)
 {
     if (n == 0) return cudaSuccess;
-    if (node_cap > kMaxScanNodes) return cudaErrorInvalidValue;
+    if (node_cap > kMaxNodes) return cudaErrorInvalidValue;
     cudaError_t e;
     const uint64_t N = n;
     const uint32_t M = node_cap;
     const SubBufs B = sub_carve(ws, n, M);
     const SortScratch& sc = B.sc;
-    uint32_t *nown = B.nown, *mark = B.mark, *mrank = B.mrank, *mlist = B.mlist, *mown = B.mown, *soff = B.soff;
-    uint32_t* cnt = B.cnt;
-    uint64_t* first = B.first;
-    const unsigned gM = (M + 255) / 256;
+    uint32_t* nm = B.cnt + 2;   // node count clamped to the capacity
+    uint32_t* nstaged = B.cnt + 3;
+    uint32_t* nrank = B.cnt + 4;   // nodes outside every chunk subtree
     const unsigned gN = (unsigned)std::min<uint64_t>((N + 255) / 256, (uint64_t)ws.num_sms * 16);
-
-    uint32_t* nm = cnt + 2;   // node count clamped to the capacity
-    uint32_t* nstaged = cnt + 3;
-    k_clamp_copy<<<1, 1, 0, st>>>(num_nodes, node_cap, nm);
-    k_nown_in<<<gM, 256, 0, st>>>(nodes, num_nodes, node_cap, nown);
-    if ((e = scan_exclusive<uint32_t, uint64_t>(nown, first, M, nm, B.tiles64, (uint64_t*)nullptr,
-                                                (uint64_t*)nullptr, st)))
-        return e;
-    k_first_out<<<gM, 256, 0, st>>>(nodes, num_nodes, node_cap, first);
 
     // 1. stable scatter by owner id, chunk by chunk; owners above the chunk are staged
     int pbits = 1;
@@ -1991,70 +2104,43 @@ cudaError_t launch_subsample(fp_node* nodes, const uint32_t* num_nodes, uint32_t
     sg.val_in = perm; sg.val_out = final_perm;
     sg.id_in = owner;
     sg.n = N;
-    sg.first = first; sg.first_stride = 1;
+    sg.first = B.first; sg.first_stride = 1;
+    sg.hist = sc.hist; sg.hist2 = B.hist2;
+    sg.nown = B.nown; sg.first_out = B.first; sg.nm = nm;
     sg.st_key = B.s_key; sg.st_src = B.s_val; sg.st_count = nstaged; sg.st_shift = pbits;
-    uint32_t* nrank = cnt + 4;   // nodes outside every chunk subtree
-    sg.st_rank = B.srank; sg.st_list = B.slist; sg.st_nrank = nrank; sg.st_tiles = B.tiles32;
+    sg.st_rank = B.srank; sg.st_list = B.slist; sg.st_nrank = nrank; sg.st_soff = B.soff;
     {
         KTimerScope kt(FP_KERNEL_OWNER_SCATTER, st);
         if ((e = seg_scatter(B.seg, sg, ws, st))) return e;
     }
     // 2. the stitch: staged records sorted by (node, original index), then placed
-    KTimerScope kt_stitch(FP_KERNEL_STITCH, st);
-    k_stitch_counts<<<gM, 256, 0, st>>>(B.seg.inside, nown, nm, B.scnt, M);
-    if ((e = scan_exclusive<uint32_t, uint32_t>(B.scnt, soff, M, nm, B.tiles32, (uint32_t*)nullptr,
-                                                (uint32_t*)nullptr, st)))
-        return e;
     {
+        KTimerScope kt(FP_KERNEL_STITCH, st);
         SortArgs b{};
         b.b.k64_src = B.s_key; b.b.k64_tmp = B.s_key2; b.b.k64_dst = B.s_key3;
         b.b.val_src = B.s_val; b.b.val_tmp = B.s_val2; b.b.val_dst = B.s_val3;
         b.n = N; b.d_n = nstaged; b.err = ws.err;
-        if ((e = sort_plan_keys(sc, b, 0, (uint32_t)pbits, nrank, false, ws.num_sms, st))) return e;
-        const int np = sort_passes(pbits + count_bits(M));   // node ids below M above the index bits
-        if ((e = sort_run<DIG_K64, false, true, false>(b, np, ws.num_sms, st))) return e;
+        if ((e = sort_plan_keys(sc, b, 0, (uint32_t)pbits, nrank, true, ws.num_sms, st))) return e;
+        // a node outside every chunk subtree lies above the count grid's cells: at most 8^0 + .. + 8^6 of them
+        const uint64_t above = std::min<uint64_t>(M, 299593);
+        if ((e = sort_run<DIG_K64, false, true, false>(b, sort_passes(pbits + count_bits(above)), ws.num_sms, st)))
+            return e;
+        k_stitch_place<<<gN, 256, 0, st>>>(nstaged, B.s_key3, B.s_val3, pbits, B.slist, nrank, nm, B.soff, B.first,
+                                           reinterpret_cast<const int4*>(sorted), perm, N,
+                                           reinterpret_cast<int4*>(final_pts), final_perm, ws.err);
     }
-    k_stitch_place<<<gN, 256, 0, st>>>(nstaged, B.s_key3, B.s_val3, pbits, B.slist, nrank, nm, soff, first,
-                                       reinterpret_cast<const int4*>(sorted), perm, N,
-                                       reinterpret_cast<int4*>(final_pts), final_perm, ws.err);
-    ktimer_mark(FP_KERNEL_STITCH, false, st);   // the gated whole-array path below is not timed with it
-    kt_stitch.id = FP_KERNEL_NONE;
-
-    // whole-array path (runs with seg cnt[5] = n records when a chunk did not fit, else on none):
-    // stable scatter by owner id, then the owner segments spanning several chunks re-sorted
-    const uint32_t* gate = B.seg.cnt + 5;
+    // whole-array path, when a chunk did not fit
+    const uint32_t* gate = B.seg.cnt + 2;
+    k_original_order<<<gN, 256, 0, st>>>(gate, reinterpret_cast<const int4*>(sorted), perm, owner, N, B.o_pt, B.o_own,
+                                         ws.err);
     SortArgs a{};
-    a.b.pt_src = reinterpret_cast<const int4*>(sorted); a.b.pt_tmp = B.t_pt;
-    a.b.pt_dst = reinterpret_cast<int4*>(final_pts);
-    a.b.val_src = perm; a.b.val_tmp = B.t_val; a.b.val_dst = final_perm;
-    a.b.k32_src = owner; a.b.k32_tmp = B.t_k32; a.b.k32_dst = B.fown;
-    a.n = N; a.d_n = gate; a.err = ws.err;
-    if ((e = sort_plan_weights(sc, a, nown, nullptr, nm, M, false, ws.num_sms, st))) return e;
-    if ((e = sort_run<DIG_K32, true, false, true>(a, sort_passes(count_bits(M)), ws.num_sms, st))) return e;
-    if ((e = cudaMemsetAsync(mark, 0, (size_t)M * 4, st))) return e;
-    if ((e = cudaMemsetAsync(cnt, 0, 2 * sizeof(uint32_t), st))) return e;
-    k_mark_unsorted<<<gN, 256, 0, st>>>(B.fown, final_perm, N, gate, mark, nm);
-    if ((e = scan_exclusive<uint32_t, uint32_t>(mark, mrank, M, nm, B.tiles32, cnt, (uint32_t*)nullptr, st)))
-        return e;
-    k_stitch_list<<<gM, 256, 0, st>>>(mark, mrank, num_nodes, node_cap, mlist, nown, mown);
-    if ((e = scan_exclusive<uint32_t, uint32_t>(mown, soff, M, cnt, B.tiles32, cnt + 1, (uint32_t*)nullptr, st)))
-        return e;
-    k_stitch_keys<<<ws.num_sms * 8, 256, 0, st>>>(mlist, cnt, soff, cnt + 1, first, final_perm, B.s_key, B.s_val);
-    int rank_bits = 1;
-    while ((1ull << rank_bits) < M) ++rank_bits;
-    SortArgs b{};
-    b.b.k64_src = B.s_key; b.b.k64_tmp = B.s_key2; b.b.k64_dst = B.s_key3;
-    b.b.val_src = B.s_val; b.b.val_tmp = B.s_val2; b.b.val_dst = B.s_val3;
-    b.n = N; b.d_n = cnt + 1; b.err = ws.err;
-    if ((e = sort_plan_keys(sc, b, 0, (uint32_t)(32 + rank_bits), nullptr, false, ws.num_sms, st))) return e;
-    if ((e = sort_run<DIG_K64, false, true, false>(b, sort_passes(32 + rank_bits), ws.num_sms, st))) return e;
-    k_stitch_gather<<<gN, 256, 0, st>>>(cnt + 1, B.s_val3,
-                                                                  reinterpret_cast<const int4*>(final_pts),
-                                                                  final_perm, B.s_pt, B.s_perm);
-    k_stitch_put<<<gN, 256, 0, st>>>(cnt + 1, B.s_key3, mlist, soff, first, B.s_pt,
-                                                               B.s_perm, reinterpret_cast<int4*>(final_pts),
-                                                               final_perm);
-    return cudaGetLastError();
+    a.b.pt_src = B.o_pt; a.b.pt_tmp = B.t_pt; a.b.pt_dst = reinterpret_cast<int4*>(final_pts);
+    a.b.val_src = nullptr; a.b.val_tmp = B.t_val; a.b.val_dst = final_perm;   // the original index
+    a.b.k32_src = B.o_own; a.b.k32_tmp = B.t_k32; a.b.k32_dst = nullptr;
+    a.n = N; a.run_if = gate; a.err = ws.err;
+    const SortScratch sc2{B.hist2, {sc.status[0], sc.status[1]}};
+    if ((e = sort_plan_weights(sc2, a, B.nown, nullptr, nm, M, true, ws.num_sms, st))) return e;
+    return sort_run<DIG_K32, true, false, true>(a, sort_passes(count_bits(M)), ws.num_sms, st);
 }
 
 }  // namespace fp

@@ -640,7 +640,7 @@ fp_status build(const fp_point* h_pts, uint64_t n, const fp_params& prm, uint64_
 
     // ---- node table of the whole cloud
     ws.used = 0;
-    if ((e = launch_octree_nodes(F.counts, prm, F.recs, node_cap, F.num_deep, F.nodes, node_cap, F.num_nodes, F.T, ws,
+    if ((e = launch_octree_nodes(F.counts, n, prm, F.recs, node_cap, F.num_deep, F.nodes, node_cap, F.num_nodes, F.T, ws,
                                  st)))
         return cu(e);
 

@@ -1,4 +1,5 @@
 // fp_seg.cu -- setup and launch of the chunk-segmented scatter (fp_seg.cuh).
+#include "fp_cluster.cuh"
 #include "fp_seg.cuh"
 
 namespace fp {
@@ -21,79 +22,165 @@ FP_DEV uint32_t find_node(const fp_node* nodes, uint32_t M, uint64_t key, uint32
     return kNone;
 }
 
-// Per chunk: its node, digits, and its tiles appended to the variant's list.
-__global__ void k_seg_setup(int mode, const fp_node* nodes, const uint32_t* num_nodes, uint32_t node_cap,
-                            const fp_chunk* chunks, const uint32_t* num_chunks, const uint64_t* offsets,
-                            uint64_t kmax, uint64_t n, uint32_t* seg_lo, uint32_t* seg_nb, SegTile* t0,
-                            SegTile* t1, uint64_t tiles_max, uint32_t* cnt, uint8_t* inside, uint32_t* err)
+// What the segmented scatter needs before its passes, in three steps:
+//   A (owner layout): first point of every node (prefix of the owned counts),
+//     the scratch words cleared;
+//   B: per chunk its node, digits and tiles, and the flags of the nodes inside
+//     chunk subtrees; the look-back words of tiles that others will read cleared;
+//   C (owner layout): the nodes outside every chunk subtree ranked in order, and
+//     where each one's staged points start.
+// One cluster does all of them for up to kSegClusterMax points (a chain of 20
+// launches before: PLANUS); step B, whose work grows with chunks and tiles, takes
+// the whole GPU for larger clouds.
+struct SegPlan {
+    int owner;               // 1: owner layout, 0: leaf grouping
+    int steps;               // 1: A, 2: B, 4: C
+    fp_node* nodes;
+    const uint32_t* num_nodes;
+    uint32_t node_cap;
+    const fp_chunk* chunks;
+    const uint32_t* num_chunks;
+    const uint64_t* offsets;
+    uint64_t kmax, n, tiles_max;
+    uint32_t *seg_lo, *seg_nb;
+    SegTile* tiles[2];
+    uint32_t* status[2];
+    uint32_t* cnt;           // SegScratch::cnt
+    uint8_t* inside;
+    uint64_t* part;
+    // owner layout
+    uint32_t* nown;
+    uint64_t* first;
+    uint32_t *rank, *list, *nrank, *soff, *nm, *nstaged;
+    uint32_t *hist, *hist2;  // the sorts' histograms, cleared in A
+    uint32_t* err;
+};
+constexpr uint64_t kSegClusterMax = 1ull << 18;
+
+// step B for the chunk of this lane (c < K); all 32 lanes of the warp take part.
+// Callers spread the chunks over the warps first (a few large chunks: one each).
+FP_DEV void seg_chunk(const SegPlan& a, uint64_t c, uint64_t K, uint32_t M)
 {
-    const uint64_t K = min((uint64_t)*num_chunks, kmax);
-    const uint32_t M = min(*num_nodes, node_cap);
-    if (blockIdx.x == 0 && threadIdx.x == 0 && (*num_chunks > kmax || offsets[K] != n)) atomicOr(&cnt[2], 1u);
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t c = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; c < K; c += stride) {
-        const uint64_t beg = offsets[c], end = offsets[c + 1], cn = end - beg;
-        seg_lo[c] = 0;
-        seg_nb[c] = 1;
-        if (end > n || end < beg) { atomicOr(&cnt[2], 1u); continue; }   // offsets not a partition of [0, n)
-        if (cn == 0) continue;
-        const fp_chunk ch = chunks[c];
-        const uint32_t id = find_node(nodes, M, ch.key, ch.level);
-        if (id == kNone) { atomicOr(&cnt[2], 1u); continue; }   // not in the table: the whole-array path runs
-        const uint32_t nd = nodes[id].n_desc;
-        if ((uint64_t)id + nd >= M) { atomicOr(&cnt[2], 1u); continue; }
-        const uint64_t nb = (uint64_t)nd + (mode == SEG_OWNER ? 2 : 1);
-        if (nb > (1u << kSegMaxBits)) { atomicOr(&cnt[2], 1u); continue; }
-        const int v = nb <= (1u << kSegSmallBits) ? 0 : 1;
-        const uint32_t ntl = (uint32_t)((cn + kSortTile - 1) / kSortTile);
-        const uint32_t at = atomicAdd(&cnt[v], ntl);
-        if ((uint64_t)at + ntl > tiles_max) {
-            raise(err, FP_ERR_CAPACITY, 12);
-            atomicOr(&cnt[2], 1u);
-            continue;
+    const int lane = threadIdx.x & 31;
+    uint32_t id = 0, nd = 0, ntl = 0, at = 0, nb = 1;
+    uint64_t beg = 0;
+    int v = 0;
+    if (c < K) {
+        beg = a.offsets[c];
+        const uint64_t end = a.offsets[c + 1], cn = end - beg;
+        bool ok = true;
+        if (end > a.n || end < beg) ok = false;   // offsets not a partition of [0, n)
+        if (ok && cn) {
+            const fp_chunk ch = a.chunks[c];
+            id = find_node(a.nodes, M, ch.key, ch.level);
+            if (id == kNone) ok = false;          // not in the table: the whole-array path runs
+            if (ok) {
+                nd = a.nodes[id].n_desc;
+                const uint64_t b = (uint64_t)nd + (a.owner ? 2 : 1);
+                if ((uint64_t)id + nd >= M || b > (1u << kSegMaxBits)) ok = false;
+                else nb = (uint32_t)b;
+            }
+            if (ok) {
+                v = nb <= (1u << kSegSmallBits) ? 0 : 1;
+                ntl = (uint32_t)((cn + kSortTile - 1) / kSortTile);
+                at = atomicAdd(&a.cnt[v], ntl);
+                if ((uint64_t)at + ntl > a.tiles_max) {
+                    raise(a.err, FP_ERR_CAPACITY, 12);
+                    ok = false;
+                }
+            }
         }
-        SegTile* tl = v ? t1 : t0;
-        for (uint32_t i = 0; i < ntl; ++i) tl[at + i] = SegTile{(uint32_t)c, i};
-        seg_lo[c] = id;
-        seg_nb[c] = (uint32_t)nb;
-        if (inside)
-            for (uint32_t x = 0; x <= nd && id + x < M; ++x) inside[id + x] = 1;
+        if (!ok) {
+            atomicOr(&a.cnt[2], 1u);
+            id = 0; nb = 1; ntl = 0;
+        }
+        a.seg_lo[c] = id;
+        a.seg_nb[c] = nb;
+    }
+    // the lists of every lane's chunk, by the whole warp
+    for (uint32_t todo = __ballot_sync(0xFFFFFFFFu, ntl != 0); todo; todo &= todo - 1) {
+        const int l = __ffs(todo) - 1;
+        const uint32_t nt = __shfl_sync(0xFFFFFFFFu, ntl, l), t0 = __shfl_sync(0xFFFFFFFFu, at, l);
+        const uint32_t b = __shfl_sync(0xFFFFFFFFu, nb, l), x0 = __shfl_sync(0xFFFFFFFFu, id, l);
+        const uint32_t vv = __shfl_sync(0xFFFFFFFFu, (uint32_t)v, l);
+        const uint32_t cc = __shfl_sync(0xFFFFFFFFu, (uint32_t)c, l);
+        const uint64_t base = __shfl_sync(0xFFFFFFFFu, (unsigned long long)beg, l);
+        SegTile* tl = a.tiles[vv];
+        uint32_t* st = a.status[vv];
+        const int sb = vv ? kSegMaxBits : kSegSmallBits;
+        for (uint32_t i = lane; i < nt; i += 32) tl[t0 + i] = SegTile{cc, i};
+        for (uint32_t i = 0; i + 1 < nt; ++i) {   // (the last tile publishes nothing)
+            uint32_t* row = st + ((base / kSortTile + i) << sb);
+            for (uint32_t d = lane; d < b; d += 32) row[d] = 0;
+        }
+        if (a.owner)
+            for (uint32_t x = lane; x < b - 1; x += 32) a.inside[x0 + x] = 1;   // the chunk's node and n_desc below it
     }
 }
 
-// owner layout: 1 for a node outside every chunk subtree (then its rank, by the scan)
-__global__ void k_outside_flags(const uint8_t* inside, const uint32_t* num_nodes, uint32_t cap, uint32_t* flag)
-{
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < cap) flag[i] = i < min(*num_nodes, cap) && !inside[i] ? 1u : 0u;
+FP_DEV void seg_chunks(const SegPlan& a, uint32_t warp, uint32_t nwarps, uint64_t K, uint32_t M)
+{   // lane l of warp w: chunks w + l * nwarps, + 32 * nwarps, ...
+    for (uint64_t c0 = warp; c0 < K; c0 += 32ull * nwarps) seg_chunk(a, c0 + (uint64_t)(threadIdx.x & 31) * nwarps, K, M);
 }
 
-__global__ void k_outside_list(const uint8_t* inside, const uint32_t* num_nodes, uint32_t cap, const uint32_t* rank,
-                               uint32_t* list)
+FP_DEV void seg_chunk_head(const SegPlan& a, uint64_t K)
 {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < min(*num_nodes, cap) && !inside[i]) list[rank[i]] = i;
+    if (*a.num_chunks > a.kmax || a.offsets[K] != a.n) atomicOr(&a.cnt[2], 1u);
 }
 
-// clear the status words that later tiles of the same chunk will read
-template <int MAXB>
-__global__ void k_seg_zero(const SegTile* tiles, const uint32_t* d_ntiles, uint64_t tiles_max,
-                           const uint64_t* offsets, const uint32_t* seg_nb, uint32_t* status, const uint32_t* fail)
+__global__ void __launch_bounds__(256) k_seg_chunks(SegPlan a)
 {
-    if (*fail) return;
-    const uint64_t T = min((uint64_t)*d_ntiles, tiles_max);
-    for (uint64_t t = blockIdx.x; t < T; t += gridDim.x) {
-        const SegTile td = tiles[t];
-        const uint64_t base = offsets[td.chunk] + (uint64_t)td.index * kSortTile;
-        if (base + kSortTile >= offsets[td.chunk + 1]) continue;   // the chunk's last tile publishes nothing
-        const uint64_t row = base / kSortTile;
-        const int nb = (int)seg_nb[td.chunk];
-        for (int d = threadIdx.x; d < nb; d += blockDim.x) status[(row << MAXB) + d] = 0;
+    const uint64_t K = min((uint64_t)*a.num_chunks, a.kmax);
+    const uint32_t M = min(*a.num_nodes, a.node_cap);
+    if (blockIdx.x == 0 && threadIdx.x == 0) seg_chunk_head(a, K);
+    seg_chunks(a, (blockIdx.x * blockDim.x + threadIdx.x) >> 5, (gridDim.x * blockDim.x) >> 5, K, M);
+}
+
+__global__ void __launch_bounds__(kClNT, 1) k_seg_plan(SegPlan a)
+{
+    __shared__ uint64_t s_warp[32];
+    const uint32_t t = cl_rank() * kClNT + threadIdx.x;
+    const uint32_t M = min(*a.num_nodes, a.node_cap);
+    if (a.steps & 1) {
+        for (uint32_t q = t; q < 8; q += kClThreads) a.cnt[q] = 0;
+        for (uint32_t q = t; q < (uint32_t)kSortHistWords; q += kClThreads) {
+            a.hist[q] = 0;
+            if (a.hist2) a.hist2[q] = 0;
+        }
+        if (a.owner) {
+            if (t == 0) { *a.nm = M; *a.nstaged = 0; }
+            for (uint32_t i = t; i < M; i += kClThreads) {
+                a.nown[i] = a.nodes[i].n_own;
+                a.inside[i] = 0;
+            }
+            cl_sync();
+            cl_scan(M, a.part, s_warp, [&](uint32_t i) -> uint64_t { return a.nown[i]; },
+                    [&](uint32_t i, uint64_t ex) {
+                        a.first[i] = ex;
+                        a.nodes[i].first = ex;
+                    });
+        } else {
+            cl_sync();
+        }
+    }
+    if (a.steps & 2) {
+        const uint64_t K = min((uint64_t)*a.num_chunks, a.kmax);
+        if (t == 0) seg_chunk_head(a, K);
+        seg_chunks(a, t >> 5, kClThreads / 32, K, M);
+        cl_sync();
+    }
+    if (a.steps & 4) {
+        const uint64_t all = cl_scan(
+            M, a.part, s_warp,
+            [&](uint32_t i) -> uint64_t { return a.inside[i] ? 0ull : (1ull << 32) | a.nown[i]; },
+            [&](uint32_t i, uint64_t ex) {
+                a.soff[i] = (uint32_t)ex;
+                a.rank[i] = (uint32_t)(ex >> 32);
+                if (!a.inside[i]) a.list[ex >> 32] = i;
+            });
+        if (t == 0) *a.nrank = (uint32_t)(all >> 32);
     }
 }
-
-// record count of the whole-array path: n when a chunk did not fit, else 0
-__global__ void k_seg_gate(uint32_t* cnt, uint32_t n) { cnt[5] = cnt[2] ? n : 0u; }
 
 SegScratch take_seg_scratch(const Workspace& ws, uint64_t n, uint64_t kmax, uint64_t node_cap)
 {
@@ -110,6 +197,7 @@ SegScratch take_seg_scratch(const Workspace& ws, uint64_t n, uint64_t kmax, uint
     s.status[1] = ws.take<uint32_t>(s.rows << kSegMaxBits);
     s.cnt = ws.take<uint32_t>(8);
     s.inside = ws.take<uint8_t>(s.node_cap);
+    s.part = ws.take<uint64_t>(kClCtas);
     return s;
 }
 
@@ -689,29 +777,30 @@ cudaError_t dist_wide(const int4* pts, uint64_t n, const fp_cube* cube, int g, c
 cudaError_t seg_scatter(const SegScratch& sc, const SegCall& c, const Workspace& ws, cudaStream_t st)
 {
     cudaError_t e;
-    if ((e = cudaMemsetAsync(sc.cnt, 0, 8 * sizeof(uint32_t), st))) return e;
     const bool owner = c.mode == SEG_OWNER;
-    if (owner) {
-        if ((e = cudaMemsetAsync(sc.inside, 0, sc.node_cap, st))) return e;
-        if ((e = cudaMemsetAsync(c.st_count, 0, sizeof(uint32_t), st))) return e;
+    SegPlan p{};
+    p.owner = owner;
+    p.nodes = c.nodes; p.num_nodes = c.num_nodes; p.node_cap = c.node_cap;
+    p.chunks = c.chunks; p.num_chunks = c.num_chunks; p.offsets = c.offsets;
+    p.kmax = sc.kmax; p.n = c.n; p.tiles_max = sc.tiles_max;
+    p.seg_lo = sc.lo; p.seg_nb = sc.nb;
+    for (int v = 0; v < 2; ++v) { p.tiles[v] = sc.tiles[v]; p.status[v] = sc.status[v]; }
+    p.cnt = sc.cnt; p.inside = sc.inside; p.part = sc.part;
+    p.nown = c.nown; p.first = c.first_out;
+    p.rank = c.st_rank; p.list = c.st_list; p.nrank = c.st_nrank; p.soff = c.st_soff; p.nm = c.nm; p.nstaged = c.st_count;
+    p.hist = c.hist; p.hist2 = c.hist2;
+    p.err = ws.err;
+    if (c.n <= kSegClusterMax) {
+        p.steps = owner ? 7 : 3;
+        if ((e = cl_launch(k_seg_plan, p, st))) return e;
+    } else {
+        p.steps = 1;
+        if ((e = cl_launch(k_seg_plan, p, st))) return e;
+        const int gk = (int)std::max<uint64_t>(1, std::min<uint64_t>((sc.kmax + 255) / 256, (uint64_t)ws.num_sms * 8));
+        k_seg_chunks<<<gk, 256, 0, st>>>(p);
+        p.steps = 4;
+        if (owner && (e = cl_launch(k_seg_plan, p, st))) return e;
     }
-    const int gk = (int)std::max<uint64_t>(1, std::min<uint64_t>((sc.kmax + 255) / 256, (uint64_t)ws.num_sms * 8));
-    k_seg_setup<<<gk, 256, 0, st>>>((int)c.mode, c.nodes, c.num_nodes, c.node_cap, c.chunks, c.num_chunks,
-                                    c.offsets, sc.kmax, c.n, sc.lo, sc.nb, sc.tiles[0], sc.tiles[1], sc.tiles_max, sc.cnt,
-                                    owner ? sc.inside : nullptr, ws.err);
-    if (owner && c.st_rank) {
-        const unsigned gn = (c.node_cap + 255) / 256;
-        k_outside_flags<<<gn, 256, 0, st>>>(sc.inside, c.num_nodes, c.node_cap, c.st_rank);
-        if ((e = scan_exclusive<uint32_t, uint32_t>(c.st_rank, c.st_rank, c.node_cap, nullptr, c.st_tiles, c.st_nrank,
-                                                    (uint32_t*)nullptr, st)))
-            return e;
-        k_outside_list<<<gn, 256, 0, st>>>(sc.inside, c.num_nodes, c.node_cap, c.st_rank, c.st_list);
-    }
-    const int gz = std::max(1, ws.num_sms * 8);
-    k_seg_zero<kSegSmallBits><<<gz, 256, 0, st>>>(sc.tiles[0], sc.cnt + 0, sc.tiles_max, c.offsets, sc.nb,
-                                                   sc.status[0], sc.cnt + 2);
-    k_seg_zero<kSegMaxBits><<<gz, 256, 0, st>>>(sc.tiles[1], sc.cnt + 1, sc.tiles_max, c.offsets, sc.nb,
-                                                 sc.status[1], sc.cnt + 2);
     SegArgs a{};
     a.pt_in = c.pt_in; a.pt_out = c.pt_out;
     a.val_in = c.val_in; a.val_out = c.val_out;
@@ -721,20 +810,17 @@ cudaError_t seg_scatter(const SegScratch& sc, const SegCall& c, const Workspace&
     a.first = c.first; a.first_stride = c.first_stride;
     a.stitch = owner ? 1 : 0;
     a.st_key = c.st_key; a.st_src = c.st_src; a.st_count = c.st_count; a.st_cap = c.n; a.st_shift = c.st_shift;
-    a.st_rank = owner ? c.st_rank : nullptr;
-    a.n = c.out_n ? c.out_n : c.n;
+    a.st_rank = c.st_rank;
+    a.n = c.n;
     a.d_fail = sc.cnt + 2;
     a.err = ws.err;
     const bool cpt = c.pt_in && c.pt_out;
     if (cpt) {
         if ((e = seg_launch<true, kSegSmallBits>(a, sc, 0, ws.num_sms, st))) return e;
-        if ((e = seg_launch<true, kSegMaxBits>(a, sc, 1, ws.num_sms, st))) return e;
-    } else {
-        if ((e = seg_launch<false, kSegSmallBits>(a, sc, 0, ws.num_sms, st))) return e;
-        if ((e = seg_launch<false, kSegMaxBits>(a, sc, 1, ws.num_sms, st))) return e;
+        return seg_launch<true, kSegMaxBits>(a, sc, 1, ws.num_sms, st);
     }
-    k_seg_gate<<<1, 1, 0, st>>>(sc.cnt, (uint32_t)c.n);
-    return cudaGetLastError();
+    if ((e = seg_launch<false, kSegSmallBits>(a, sc, 0, ws.num_sms, st))) return e;
+    return seg_launch<false, kSegMaxBits>(a, sc, 1, ws.num_sms, st);
 }
 
 }  // namespace fp

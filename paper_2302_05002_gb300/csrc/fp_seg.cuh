@@ -49,8 +49,8 @@ struct SegArgs {
     uint32_t* status;                     // [row][1 << MAXB], row = tile start / kSortTile
     uint32_t* counter;
     int stitch;                           // nonzero: the chunk's last digit is the staging digit
-    uint64_t* st_key;                     // (node << st_shift) | original index, node = st_rank[id] or id
-    const uint32_t* st_rank;              // nullable: rank of a node among those outside every chunk subtree
+    uint64_t* st_key;                     // (st_rank[node] << st_shift) | original index
+    const uint32_t* st_rank;              // rank of a node among those outside every chunk subtree (stitch)
     uint32_t* st_src;                     // position in the chunk array
     uint32_t* st_count;
     uint64_t st_cap;
@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(kSortNT, (seg_ctas<CPT, MAXB>())) k_seg_pass(S
                 if (o >= a.st_cap) { raise(a.err, FP_ERR_CAPACITY, 14); continue; }
                 const uint64_t src = base + s_pos[q];
                 const uint32_t id = a.id_in[src];
-                a.st_key[o] = ((uint64_t)(a.st_rank ? a.st_rank[id] : id) << a.st_shift) | s_val[q];
+                a.st_key[o] = ((uint64_t)a.st_rank[id] << a.st_shift) | s_val[q];
                 a.st_src[o] = (uint32_t)src;
             } else {
                 if (o >= a.n) { raise(a.err, FP_ERR_CAPACITY, 15); continue; }   // inconsistent node table
@@ -239,8 +239,9 @@ struct SegScratch {
     uint32_t* nb;          // [kmax]
     SegTile* tiles[2];     // [tiles_max] per variant
     uint32_t* status[2];   // [rows][256] and [rows][2048]
-    uint32_t* cnt;         // [0..1] tiles per variant, [2] fail, [3..4] tile counters, [5] gated record count
+    uint32_t* cnt;         // [0..1] tiles per variant, [2] fail, [3..4] tile counters
     uint8_t* inside;       // [node_cap] owner layout: node lies in a chunk's subtree
+    uint64_t* part;        // cluster scan scratch
     uint64_t kmax, tiles_max, rows, node_cap;
 };
 SegScratch take_seg_scratch(const Workspace& ws, uint64_t n, uint64_t kmax, uint64_t node_cap);
@@ -249,21 +250,22 @@ enum SegMode { SEG_LEAF = 0, SEG_OWNER = 1 };
 
 struct SegCall {
     SegMode mode;
-    const fp_node* nodes; const uint32_t* num_nodes; uint32_t node_cap;
+    fp_node* nodes; const uint32_t* num_nodes; uint32_t node_cap;
     const fp_chunk* chunks; const uint32_t* num_chunks; const uint64_t* offsets;
     const int4* pt_in; int4* pt_out;
     const uint32_t* val_in; uint32_t* val_out;
     const uint32_t* id_in;
     uint64_t n;
-    uint64_t out_n;       // bound of the output positions (0: n)
     const uint64_t* first; uint32_t first_stride;
-    // owner layout: staging
+    uint32_t *hist, *hist2;   // sort histograms to clear (kSortHistWords each; hist2 nullable)
+    // owner layout: owned counts and starts of the nodes (written, also into the node records)
+    uint32_t* nown; uint64_t* first_out; uint32_t* nm;
+    // owner layout: staging, keyed by rank among the nodes outside every chunk
+    // subtree (in node order, so the sorted order is that of node ids):
+    // st_rank[node] (node_cap), st_list[rank] = node, *st_nrank = their number,
+    // st_soff[node] = staged points of the nodes before it
     uint64_t* st_key; uint32_t* st_src; uint32_t* st_count; int st_shift;
-    // owner layout, nullable: staging keys by rank among the nodes outside every
-    // chunk subtree (in node order, so the sorted order is that of node ids):
-    // st_rank[node] (node_cap), st_list[rank] = node, *st_nrank = their number;
-    // st_tiles: scan scratch (kScanMaxTiles)
-    uint32_t *st_rank, *st_list, *st_nrank, *st_tiles;
+    uint32_t *st_rank, *st_list, *st_nrank, *st_soff;
 };
 
 // Distribution of n points into up to 4096 chunks by the counting pass and a
@@ -277,9 +279,9 @@ cudaError_t dist_wide(const int4* pts, uint64_t n, const fp_cube* cube, int g, c
                       uint32_t* run_sort, uint32_t* hist, const Workspace& ws, cudaStream_t st, const uint32_t* cells,
                       uint16_t* chunk_tmp);
 
-// Setup (chunk node ids, digits, tiles), status reset, both pass variants.
-// Afterwards cnt[2] != 0 means a chunk did not fit (the caller's whole-array
-// path must run; it is gated on cnt[5] = n in that case, 0 otherwise).
+// The plan (k_seg_plan) and both pass variants.
+// Afterwards cnt[2] != 0 means a chunk did not fit: the caller's whole-array
+// path, gated on it, must run.
 cudaError_t seg_scatter(const SegScratch& sc, const SegCall& call, const Workspace& ws, cudaStream_t st);
 
 }  // namespace fp
