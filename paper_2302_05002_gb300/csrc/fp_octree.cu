@@ -53,15 +53,16 @@ struct Piece {
     uint32_t begin, count;   // record range in the cell-grouped arrays
     uint8_t q, hier, A;      // level, leaf level or kInner, first-min level of its minimum
     uint8_t srt;             // its records are in key order down to this level
-    uint8_t pad[4];
+    uint8_t buf;             // record buffer that holds them (OctCtx::recs)
+    uint8_t pad[3];
 };
 static_assert(sizeof(Piece) == 16, "Piece layout");
 
 struct OpenNode {
     uint64_t key;
     uint32_t begin, count;
-    uint8_t q, hier, A, pad;
-    uint32_t rb;          // its ancestor-or-self in the open list the current round started from
+    uint8_t q, hier, A, buf;
+    uint32_t tile0;       // large nodes of a round: first tile
     uint32_t pad2, pad3;
 };
 static_assert(sizeof(OpenNode) == 32, "OpenNode layout");
@@ -75,8 +76,6 @@ FP_DEV uint4 rec_make(uint64_t key, uint32_t j, uint32_t w)
     return make_uint4((uint32_t)key, (uint32_t)(key >> 32), j, w);
 }
 FP_DEV uint64_t rec_key(const uint4& r) { return (uint64_t)r.x | ((uint64_t)r.y << 32); }
-FP_DEV uint64_t rec_key_at(const uint4* rec, uint64_t i) { return *reinterpret_cast<const uint64_t*>(rec + i); }
-FP_DEV uint32_t rec_j_at(const uint4* rec, uint64_t i) { return reinterpret_cast<const uint32_t*>(rec + i)[2]; }
 
 struct OctCtx {   // device pointers of one fp_build_chunk_octree call
     const uint32_t* counts;    // points per level-g cell: the hierarchy
@@ -85,26 +84,26 @@ struct OctCtx {   // device pointers of one fp_build_chunk_octree call
     const uint32_t* cstart;
     const uint32_t* cursor;    // ends of the cells as k_cell_scatter left them (cursor_slot)
     uint8_t* cell_leaf;
-    uint4* rec;           // cell-grouped records (rec_key, rec_j)
-    Piece *tab, *small, *gen, *dups;   // the pieces by the way their lambda is found (emit_piece), any order
-    uint32_t *ntab, *nsmall, *ngen, *ndups, *tab_claim;
-    uint32_t piece_cap;                // of each list
+    uint4* recs[2];       // cell-grouped records (rec_key, rec_j), and the split rounds' second buffer
+    uint64_t nrec_max;    // records
+    Piece* list[4];       // the pieces by the way their lambda is found (PieceList), any order
+    uint32_t* n[4];       // their numbers
+    uint32_t* tab_claim;  // table pieces taken
+    uint32_t piece_cap;   // of each list
     NodeRec* nrec;
     uint32_t* nnode;
     uint32_t node_cap_ws;
     uint32_t* codes;      // per record position j: code_make(LOD owner level, leaf level, level-g cell)
-    uint32_t open_cap;
     int g, s, lmax, dl;
     uint64_t C;
-    uint64_t n;           // records (bound of record positions j and of record indices)
     uint32_t* err;
 };
 
 // record i of the cell-grouped array, checked against the record count (a zero
 // record beyond it: an inconsistent grouping must not turn into a stray access)
-FP_DEV uint4 get_rec(const OctCtx& c, uint64_t i)
+FP_DEV uint4 get_rec(const OctCtx& c, int buf, uint64_t i)
 {
-    if (i < c.n) return c.rec[i];
+    if (i < c.nrec_max) return c.recs[buf][i];
     raise(c.err, FP_ERR_CAPACITY, 18);
     return make_uint4(0u, 0u, 0u, 0u);
 }
@@ -135,7 +134,17 @@ FP_DEV int piece_depth(const OctCtx& c, int q, int hier) { return max(0, min(kKe
 constexpr int kSmallMax = 32;   // largest piece done by pairs of points
 constexpr int kHashMaxD = 10;   // deepest piece on the tables: 3 * 10 cell bits beside a 30-bit index in 64 bits
 
-FP_DEV Piece make_piece(uint32_t begin, uint32_t count, int q, uint8_t hier, uint8_t A, int srt)
+enum PieceList : uint8_t { LIST_TAB = 0, LIST_SMALL = 1, LIST_GEN = 2, LIST_DUP = 3 };
+
+FP_DEV PieceList piece_list(const OctCtx& c, uint32_t count, int q, uint8_t hier)
+{
+    if (count > (uint32_t)kPieceMax) return LIST_DUP;
+    if (hier == kInner) return LIST_GEN;
+    if (count <= (uint32_t)kSmallMax) return LIST_SMALL;
+    return piece_depth(c, q, hier) > kHashMaxD ? LIST_GEN : LIST_TAB;
+}
+
+FP_DEV Piece make_piece(uint32_t begin, uint32_t count, int q, uint8_t hier, uint8_t A, int srt, int buf)
 {
     Piece p;
     p.begin = begin;
@@ -144,21 +153,15 @@ FP_DEV Piece make_piece(uint32_t begin, uint32_t count, int q, uint8_t hier, uin
     p.hier = hier;
     p.A = A;
     p.srt = (uint8_t)srt;
-    p.pad[0] = p.pad[1] = p.pad[2] = p.pad[3] = 0;
+    p.buf = (uint8_t)buf;
+    p.pad[0] = p.pad[1] = p.pad[2] = 0;
     return p;
 }
 
-FP_DEV void emit_piece(const OctCtx& c, uint32_t begin, uint32_t count, int q, uint8_t hier, uint8_t A, int srt)
+FP_DEV void put_piece(const OctCtx& c, PieceList l, uint32_t id, const Piece& p)
 {
-    Piece* list = c.tab;
-    uint32_t* n = c.ntab;
-    if (count > (uint32_t)kPieceMax) { list = c.dups; n = c.ndups; }
-    else if (hier == kInner) { list = c.gen; n = c.ngen; }
-    else if (count <= (uint32_t)kSmallMax) { list = c.small; n = c.nsmall; }
-    else if (piece_depth(c, q, hier) > kHashMaxD) { list = c.gen; n = c.ngen; }
-    const uint32_t id = atomicAdd(n, 1u);
     if (id >= c.piece_cap) { raise(c.err, FP_ERR_CAPACITY, 2); return; }
-    list[id] = make_piece(begin, count, q, hier, A, srt);
+    c.list[l][id] = p;
 }
 
 // ---------------------------------------------------------------- cells
@@ -203,6 +206,341 @@ __global__ void __launch_bounds__(256) k_cell_scatter(const int4* __restrict__ p
     }
 }
 
+// ------------------------------------------------- big cells: split rounds
+// Cells of more than kPieceMax records are split into node-aligned pieces, three
+// levels a round, all rounds in one cooperative launch (70 launches before: most
+// clouds have few open nodes or none, and then the launches were all there was).
+// The records of an open node are grouped by their cell three levels down, which
+// puts them in key order down to that depth, and the nodes of those levels follow
+// from the 512 counts and smallest indices:
+//   * nodes of at most kRoundTile records by one block each, records in
+//     registers, counted, ranked (any order inside a cell) and put back in place
+//     with shared-memory atomics: 16 bytes read and written per record, no
+//     global atomic;
+//   * larger nodes in tiles of kRoundTile records by all blocks: counts and
+//     minima per tile into the node's column (phase 1), columns into starts (2),
+//     every tile's records to the other record buffer at slots taken once per
+//     tile and cell (3), one block per node for the split (4), with a barrier of
+//     the grid between the phases.
+// (Copying every open node's records out, counting per record with global
+// atomics, and scattering them back moved 64 bytes per record and round: 4.1 ms
+// of 10^8 LiDAR points, 1.5 ms now.)
+constexpr int kRoundNT = 512;
+constexpr int kRoundIPT = 8;
+constexpr int kRoundTile = kRoundNT * kRoundIPT;   // 4096
+static_assert(kRoundNT == 1 << (3 * kRoundLevels), "one thread per cell of a round");
+
+struct RoundCnt {          // open nodes of one round
+    unsigned long long big;    // nodes of more than kRoundTile records << 32 | their tiles
+    uint32_t small, pad;
+};
+constexpr int kMaxRounds = (kKeyLevels + kRoundLevels - 1) / kRoundLevels;
+
+struct RoundArgs {
+    OctCtx c;
+    OpenNode *small[2], *big[2];   // open nodes of even and odd rounds
+    RoundCnt* cnt;                 // [kMaxRounds + 1], zeroed
+    uint32_t small_cap, big_cap;
+    uint32_t *slots, *smin;        // [512][big_cap]: counts, then starts, then ends; smallest index
+    uint32_t* bar;                 // barrier word, zeroed
+};
+
+FP_DEV void open_node(const RoundArgs& a, int round, const OpenNode& node)
+{
+    OpenNode o = node;
+    if (o.count <= (uint32_t)kRoundTile) {
+        const uint32_t id = atomicAdd(&a.cnt[round].small, 1u);
+        if (id >= a.small_cap) { raise(a.c.err, FP_ERR_CAPACITY, 7); return; }
+        a.small[round & 1][id] = o;
+    } else {
+        const uint32_t nt = (o.count + kRoundTile - 1) / kRoundTile;
+        const unsigned long long at = atomicAdd(&a.cnt[round].big, (1ull << 32) | nt);
+        const uint32_t id = (uint32_t)(at >> 32);
+        if (id >= a.big_cap) { raise(a.c.err, FP_ERR_CAPACITY, 7); return; }
+        o.tile0 = (uint32_t)at;   // (ids and first tiles grow together)
+        a.big[round & 1][id] = o;
+    }
+}
+
+// barrier number `k` (from 1) of the grid, every block of which is resident
+// (cooperative launch); false when the bounded wait ran out
+FP_DEV bool grid_barrier(uint32_t* word, uint32_t k, uint32_t* err)
+{
+    __shared__ int s_ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(word, 1u);
+        const uint32_t target = k * gridDim.x;
+        uint32_t spins = 0;
+        s_ok = 1;
+        while (ld_volatile(word) < target) {
+            if (++spins > (1u << 22)) { raise(err, FP_ERR_TIMEOUT); s_ok = 0; break; }
+            __nanosleep(64);
+        }
+        __threadfence();
+    }
+    __syncthreads();
+    return s_ok != 0;
+}
+
+struct RoundSmem {
+    uint32_t h[kRoundNT], st[kRoundNT], mn[kRoundNT];   // per cell three levels down: count, start, smallest index
+    uint32_t c2[64], m2[64], m1[8];
+    uint64_t warp[kRoundNT / 32];
+    uint32_t warp32[kRoundNT / 32];
+    uint32_t base[3], tile[2];
+};
+
+// The nodes of the three levels below open node o (level q), thread d the cell d
+// three levels down: children of more than kPieceMax records stay open down to
+// the round's end, the others become pieces; inner nodes' children are nodes.
+FP_DEV void split_node(const RoundArgs& a, RoundSmem& S, const OpenNode& o, int round, int buf)
+{
+    const OctCtx& c = a.c;
+    const int d = threadIdx.x, q = o.q;
+    const uint32_t begin = S.st[d];
+    uint32_t cn[4], mn[4];   // by levels below o
+    cn[3] = S.h[d];
+    mn[3] = S.mn[d];
+    cn[2] = cn[3]; mn[2] = mn[3];
+#pragma unroll
+    for (int x = 1; x < 8; x <<= 1) {
+        cn[2] += __shfl_xor_sync(0xFFFFFFFFu, cn[2], x);
+        mn[2] = min(mn[2], __shfl_xor_sync(0xFFFFFFFFu, mn[2], x));
+    }
+    if ((d & 7) == 0) { S.c2[d >> 3] = cn[2]; S.m2[d >> 3] = mn[2]; }
+    __syncthreads();
+    cn[1] = 0; mn[1] = kNone;
+#pragma unroll
+    for (int x = 0; x < 8; ++x) {
+        cn[1] += S.c2[(d >> 6) * 8 + x];
+        mn[1] = min(mn[1], S.m2[(d >> 6) * 8 + x]);
+    }
+    if ((d & 63) == 0) S.m1[d >> 6] = mn[1];
+    __syncthreads();
+    mn[0] = kNone;
+#pragma unroll
+    for (int x = 0; x < 8; ++x) mn[0] = min(mn[0], S.m1[x]);
+
+    // per level: is this thread the child's first cell, the child's hierarchy and first-min level
+    bool node[4] = {false, false, false, false}, piece[4] = {false, false, false, false};
+    uint8_t hier[4], A[4];
+    hier[0] = o.hier;
+    A[0] = o.A;
+    bool open = true;
+#pragma unroll
+    for (int t = 1; t <= 3; ++t) {
+        const int lev = q + t;
+        hier[t] = hier[t - 1] != kInner ? hier[t - 1] : ((cn[t] <= c.C || lev == c.lmax) ? (uint8_t)lev : kInner);
+        // the child's minimum is the parent's minimum: it keeps the parent's first-min level
+        A[t] = mn[t] == mn[t - 1] ? A[t - 1] : (uint8_t)lev;
+        const bool here = open && cn[t] && (d & ((1 << (3 * (3 - t))) - 1)) == 0;
+        open = open && cn[t] > (uint32_t)kPieceMax && lev < c.dl;
+        if (here) {
+            node[t] = hier[t - 1] == kInner;
+            if (!open) {
+                piece[t] = true;
+            } else if (t == 3) {
+                OpenNode ch;
+                ch.key = (o.key << 9) | (uint64_t)d;
+                ch.begin = begin;
+                ch.count = cn[3];
+                ch.q = (uint8_t)lev;
+                ch.hier = hier[3];
+                ch.A = A[3];
+                ch.buf = (uint8_t)buf;
+                ch.tile0 = ch.pad2 = ch.pad3 = 0;
+                open_node(a, round + 1, ch);
+            }
+        }
+    }
+    // appends of table pieces, small pieces and nodes: one scan, one atomic each
+    const int srt = min(q + kRoundLevels, kKeyLevels);
+    uint64_t want = 0;
+    PieceList list[4];
+#pragma unroll
+    for (int t = 1; t <= 3; ++t) {
+        list[t] = piece_list(c, cn[t], q + t, hier[t]);
+        if (piece[t] && list[t] == LIST_TAB) want += 1;
+        if (piece[t] && list[t] == LIST_SMALL) want += 1ull << 21;
+        if (node[t]) want += 1ull << 42;
+    }
+    uint64_t total;
+    const uint64_t ex = block_exclusive_scan<kRoundNT, uint64_t>(want, S.warp, total);
+    constexpr uint32_t kF = (1u << 21) - 1;
+    if (d < 3) {
+        const uint32_t n = (uint32_t)(total >> (21 * d)) & kF;
+        uint32_t* ctr = d == 0 ? c.n[LIST_TAB] : (d == 1 ? c.n[LIST_SMALL] : c.nnode);
+        S.base[d] = n ? atomicAdd(ctr, n) : 0u;
+    }
+    __syncthreads();
+    uint32_t ti = S.base[0] + ((uint32_t)ex & kF), si = S.base[1] + ((uint32_t)(ex >> 21) & kF),
+             ni = S.base[2] + (uint32_t)(ex >> 42);
+#pragma unroll
+    for (int t = 1; t <= 3; ++t) {
+        if (node[t])
+            put_node(c, ni++, (o.key << (3 * t)) | (uint64_t)(d >> (3 * (3 - t))), q + t, cn[t], begin, hier[t] != kInner);
+        if (piece[t]) {
+            const Piece p = make_piece(begin, cn[t], q + t, hier[t], A[t], srt, buf);
+            if (list[t] == LIST_TAB) put_piece(c, LIST_TAB, ti++, p);
+            else if (list[t] == LIST_SMALL) put_piece(c, LIST_SMALL, si++, p);
+            else put_piece(c, list[t], atomicAdd(c.n[list[t]], 1u), p);
+        }
+    }
+    __syncthreads();   // the arrays are free for the next node
+}
+
+__global__ void __launch_bounds__(kRoundNT, 2) k_rounds(RoundArgs a)
+{
+    __shared__ RoundSmem S;
+    const OctCtx& c = a.c;
+    const int tid = threadIdx.x, lane = tid & 31;
+    uint32_t nbar = 0;
+    for (int round = 0, q = c.g; q < c.dl; ++round, q += kRoundLevels) {
+        const uint32_t ns = min(ld_volatile(&a.cnt[round].small), a.small_cap);
+        const uint64_t bp = ld_volatile64(reinterpret_cast<const uint64_t*>(&a.cnt[round].big));
+        const uint32_t nb = min((uint32_t)(bp >> 32), a.big_cap), ntile = nb ? (uint32_t)bp : 0u;
+        if (ns == 0 && nb == 0) return;   // (the same in every block)
+        const OpenNode* small = a.small[round & 1];
+        const OpenNode* big = a.big[round & 1];
+        // the record's cell three levels below q (beyond the key's last level: zeros)
+        const int sh = 3 * (kKeyLevels - q - kRoundLevels);
+        auto digit = [&](const uint4& r) {
+            const uint64_t k = rec_key(r);
+            return (uint32_t)(sh >= 0 ? k >> sh : k << -sh) & (kRoundNT - 1);
+        };
+        if (nb) {
+            for (uint64_t x = (uint64_t)blockIdx.x * kRoundNT + tid; x < (uint64_t)nb * kRoundNT;
+                 x += (uint64_t)gridDim.x * kRoundNT) {
+                const uint64_t slot = (x / nb) * a.big_cap + x % nb;
+                a.slots[slot] = 0;
+                a.smin[slot] = kNone;
+            }
+            if (!grid_barrier(a.bar, ++nbar, c.err)) return;
+        }
+        // loads a run of at most kRoundTile records, counts them per cell; returns each one's cell | rank << 16
+        uint4 rec[kRoundIPT];
+        uint32_t pk[kRoundIPT];
+        auto count_run = [&](const uint4* src, uint32_t n, bool minima) {
+            S.h[tid] = 0;
+            S.mn[tid] = kNone;
+            __syncthreads();
+#pragma unroll
+            for (int r = 0; r < kRoundIPT; ++r)
+                if (r * kRoundNT + tid < n) rec[r] = src[r * kRoundNT + tid];
+#pragma unroll
+            for (int r = 0; r < kRoundIPT; ++r)
+                if (r * kRoundNT + tid < n) {
+                    const uint32_t d = digit(rec[r]);
+                    pk[r] = d | (atomicAdd(&S.h[d], 1u) << 16);
+                    if (minima && S.mn[d] > rec[r].z) atomicMin(&S.mn[d], rec[r].z);
+                }
+            __syncthreads();
+        };
+        for (uint32_t i = blockIdx.x; i < ns; i += gridDim.x) {
+            const OpenNode o = small[i];
+            if ((uint64_t)o.begin + o.count > c.nrec_max) { raise(c.err, FP_ERR_CAPACITY, 6); continue; }
+            uint4* buf = c.recs[o.buf];
+            count_run(buf + o.begin, o.count, true);
+            uint32_t tot;
+            const uint32_t ex = block_exclusive_scan<kRoundNT, uint32_t>(S.h[tid], S.warp32, tot);
+            S.st[tid] = o.begin + ex;
+            __syncthreads();
+#pragma unroll
+            for (int r = 0; r < kRoundIPT; ++r)
+                if (r * kRoundNT + tid < o.count) buf[S.st[pk[r] & 0xFFFFu] + (pk[r] >> 16)] = rec[r];
+            split_node(a, S, o, round, o.buf);
+        }
+        // tile t of the large nodes: its node and its first record
+        auto tile_of = [&](uint32_t t) {
+            if (tid == 0) {
+                uint32_t x = 0, y = nb;
+                while (y - x > 1) {
+                    const uint32_t m = (x + y) >> 1;
+                    if (big[m].tile0 <= t) x = m;
+                    else y = m;
+                }
+                S.tile[0] = x;
+                S.tile[1] = (t - big[x].tile0) * kRoundTile;
+            }
+            __syncthreads();
+        };
+        for (uint32_t t = blockIdx.x; t < ntile; t += gridDim.x) {
+            tile_of(t);
+            const uint32_t b = S.tile[0], off = S.tile[1];
+            const OpenNode o = big[b];
+            const bool ok = off < o.count && (uint64_t)o.begin + o.count <= c.nrec_max;
+            if (!ok && tid == 0) raise(c.err, FP_ERR_CAPACITY, 6);
+            count_run(c.recs[o.buf] + o.begin + off, ok ? min((uint32_t)kRoundTile, o.count - off) : 0u, true);
+            if (S.h[tid]) {
+                atomicAdd(&a.slots[(uint64_t)tid * a.big_cap + b], S.h[tid]);
+                atomicMin(&a.smin[(uint64_t)tid * a.big_cap + b], S.mn[tid]);
+            }
+            __syncthreads();
+        }
+        if (nb) {
+            if (!grid_barrier(a.bar, ++nbar, c.err)) return;
+            // counts -> starts, one warp per node
+            const uint32_t warp = (blockIdx.x * kRoundNT + tid) >> 5, nwarps = (gridDim.x * kRoundNT) >> 5;
+            for (uint32_t b = warp; b < nb; b += nwarps) {
+                uint32_t v[kRoundNT / 32], sum = 0;
+#pragma unroll
+                for (int x = 0; x < kRoundNT / 32; ++x) {
+                    v[x] = a.slots[(uint64_t)(lane * (kRoundNT / 32) + x) * a.big_cap + b];
+                    sum += v[x];
+                }
+                uint32_t inc = sum;
+                for (int s = 1; s < 32; s <<= 1) {
+                    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, s);
+                    if (lane >= s) inc += y;
+                }
+                uint32_t run = big[b].begin + inc - sum;
+#pragma unroll
+                for (int x = 0; x < kRoundNT / 32; ++x) {
+                    a.slots[(uint64_t)(lane * (kRoundNT / 32) + x) * a.big_cap + b] = run;
+                    run += v[x];
+                }
+            }
+            if (!grid_barrier(a.bar, ++nbar, c.err)) return;
+            for (uint32_t t = blockIdx.x; t < ntile; t += gridDim.x) {
+                tile_of(t);
+                const uint32_t b = S.tile[0], off = S.tile[1];
+                const OpenNode o = big[b];
+                const uint32_t n = off < o.count && (uint64_t)o.begin + o.count <= c.nrec_max
+                                       ? min((uint32_t)kRoundTile, o.count - off) : 0u;
+                count_run(c.recs[o.buf] + o.begin + off, n, false);
+                S.st[tid] = S.h[tid] ? atomicAdd(&a.slots[(uint64_t)tid * a.big_cap + b], S.h[tid]) : 0u;
+                __syncthreads();
+                uint4* dst = c.recs[o.buf ^ 1];
+#pragma unroll
+                for (int r = 0; r < kRoundIPT; ++r)
+                    if (r * kRoundNT + tid < n) {
+                        const uint64_t at = (uint64_t)S.st[pk[r] & 0xFFFFu] + (pk[r] >> 16);
+                        if (at < c.nrec_max) dst[at] = rec[r];
+                        else raise(c.err, FP_ERR_CAPACITY, 6);
+                    }
+                __syncthreads();
+            }
+            if (!grid_barrier(a.bar, ++nbar, c.err)) return;
+            for (uint32_t b = blockIdx.x; b < nb; b += gridDim.x) {   // slots hold the cells' ends now
+                const OpenNode o = big[b];
+                const uint32_t end = a.slots[(uint64_t)tid * a.big_cap + b];
+                S.mn[tid] = a.smin[(uint64_t)tid * a.big_cap + b];
+                S.h[tid] = end;
+                __syncthreads();
+                const uint32_t from = tid ? S.h[tid - 1] : o.begin;
+                __syncthreads();
+                S.st[tid] = from;
+                S.h[tid] = end - from;
+                __syncthreads();
+                split_node(a, S, o, round, o.buf ^ 1);
+            }
+        }
+        if (!grid_barrier(a.bar, ++nbar, c.err)) return;
+    }
+}
+
 // One block per tile of the grid (k_grid_tiles before it).  With `cells`: every
 // cell's start among the records and its cursor; its leaf level when the
 // hierarchy ends at or above g, kInner if the cell's node is inner, kEmpty
@@ -214,11 +552,11 @@ __global__ void __launch_bounds__(256) k_cell_scatter(const int4* __restrict__ p
 // one time then lie in one or two tiles, and their scattered codes stay in L2
 // (appended one by one as the atomics fell, k_tab_pieces took 15.5 instead of
 // 13.0 ms for 5 * 10^8 uniform points, before it took its pieces in order).
-__global__ void __launch_bounds__(kGtNT) k_cells_open(OctCtx c, const uint32_t* __restrict__ pyr,
+__global__ void __launch_bounds__(kGtNT) k_cells_open(RoundArgs ra, const uint32_t* __restrict__ pyr,
                                                       const uint32_t* __restrict__ rsum, int cells, int upper,
-                                                      uint32_t* __restrict__ cstart, uint32_t* __restrict__ cursor,
-                                                      OpenNode* open0, uint32_t* nopen0)
+                                                      uint32_t* __restrict__ cstart, uint32_t* __restrict__ cursor)
 {
+    const OctCtx& c = ra.c;
     __shared__ GridTop top;
     __shared__ uint32_t s_warp[kGtNT / 32], s_base[2];
     const int g = c.g, tid = threadIdx.x;
@@ -266,25 +604,21 @@ __global__ void __launch_bounds__(kGtNT) k_cells_open(OctCtx c, const uint32_t* 
                                     : (s.s1[q >> 3] <= c.C ? (uint8_t)max(g - 1, 0)
                                                            : (v[q] <= c.C || g == c.lmax ? (uint8_t)g : kInner));
                 if (rv[q] > (uint32_t)kPieceMax) {
-                    const uint32_t id = atomicAdd(nopen0, 1u);
-                    if (id >= c.open_cap) {
-                        raise(c.err, FP_ERR_CAPACITY, 5);
-                    } else {
-                        OpenNode o;
-                        o.key = m;
-                        o.begin = at;
-                        o.count = rv[q];
-                        o.q = (uint8_t)g;
-                        o.hier = hier[q];
-                        o.A = (uint8_t)g;
-                        o.pad = 0;
-                        o.rb = o.pad2 = o.pad3 = 0;
-                        open0[id] = o;
-                    }
-                } else if (hier[q] == kInner || (rv[q] > (uint32_t)kSmallMax && piece_depth(c, g, hier[q]) > kHashMaxD)) {
-                    emit_piece(c, at, rv[q], g, hier[q], (uint8_t)g, g);
-                } else if (rv[q] > (uint32_t)kSmallMax) {
-                    tab |= 1u << q;
+                    OpenNode o;
+                    o.key = m;
+                    o.begin = at;
+                    o.count = rv[q];
+                    o.q = (uint8_t)g;
+                    o.hier = hier[q];
+                    o.A = (uint8_t)g;
+                    o.buf = 0;
+                    o.tile0 = o.pad2 = o.pad3 = 0;
+                    open_node(ra, 0, o);
+                } else {
+                    const PieceList l = piece_list(c, rv[q], g, hier[q]);
+                    if (l == LIST_TAB) tab |= 1u << q;
+                    else if (l == LIST_GEN)
+                        put_piece(c, l, atomicAdd(c.n[l], 1u), make_piece(at, rv[q], g, hier[q], (uint8_t)g, g, 0));
                 }
             }
             at += rv[q];
@@ -316,7 +650,7 @@ __global__ void __launch_bounds__(kGtNT) k_cells_open(OctCtx c, const uint32_t* 
     // both appends: one scan (tables in the low half, nodes in the high half: at most 5 * 4096 each)
     const uint32_t ex = block_exclusive_scan<kGtNT, uint32_t>(__popc(tab) | (__popc(nf) << 16), s_warp, total);
     if (tid == 0) {
-        s_base[0] = (total & 0xFFFFu) ? atomicAdd(c.ntab, total & 0xFFFFu) : 0u;
+        s_base[0] = (total & 0xFFFFu) ? atomicAdd(c.n[LIST_TAB], total & 0xFFFFu) : 0u;
         s_base[1] = (total >> 16) ? atomicAdd(c.nnode, total >> 16) : 0u;
     }
     __syncthreads();
@@ -324,9 +658,7 @@ __global__ void __launch_bounds__(kGtNT) k_cells_open(OctCtx c, const uint32_t* 
 #pragma unroll
     for (int q = 0; q < kGtPer; ++q) {
         if ((tab >> q) & 1u) {
-            if (pi >= c.piece_cap) raise(c.err, FP_ERR_CAPACITY, 2);
-            else c.tab[pi] = make_piece(at, rv[q], g, hier[q], (uint8_t)g, g);
-            ++pi;
+            put_piece(c, LIST_TAB, pi++, make_piece(at, rv[q], g, hier[q], (uint8_t)g, g, 0));
         }
         if ((nf >> q) & 1u) put_node(c, ni++, base + q, g, v[q], at, v[q] <= c.C || g == c.lmax);
         if (q == 7 && ((nf >> 17) & 1u)) put_node(c, ni++, (base >> 3) + 1, g - 1, s.s1[1], at + rv[7], s.s1[1] <= c.C);
@@ -338,223 +670,6 @@ __global__ void __launch_bounds__(kGtNT) k_cells_open(OctCtx c, const uint32_t* 
     for (int a = 0; a <= up; ++a)
         if ((nf >> (20 + a)) & 1u)
             put_node(c, ni++, tile >> (3 * a), g - 4 - a, top.at(a, tile), at0, top.at(a, tile) <= c.C);
-}
-
-// ------------------------------------------------------- big cells: rounds
-// position p of the records of the open nodes, copied out one node after another
-FP_DEV uint32_t big_of(const uint32_t* bigstart, uint32_t nb, uint32_t p)
-{
-    uint32_t a = 0, b = nb;
-    while (a < b) { uint32_t m = (a + b) >> 1; if (bigstart[m] <= p) a = m + 1; else b = m; }
-    return a - 1;
-}
-
-// records of each open node; a round's records are copied out compactly (bigstart)
-__global__ void k_open_counts(const OpenNode* open0, const uint32_t* nopen0, uint32_t* cnt_out, uint32_t cap,
-                              const uint64_t* d_skip, uint64_t skip_min)
-{
-    uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= cap) return;
-    const bool skip = d_skip && *d_skip > skip_min;
-    cnt_out[i] = i < *nopen0 && !skip ? open0[i].count : 0;
-}
-
-// Counting slots of a round are digit-major (slot = d * cap + node): the cells
-// of one node, used together, lie far apart in the array (and in L2 slices).
-__global__ void k_round_zero(const uint32_t* nopen, uint32_t cap, int nd, uint32_t* cnt, uint32_t* smin)
-{
-    const uint32_t nb = min(*nopen, cap);
-    const uint64_t tot = (uint64_t)nb * nd;
-    for (uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; x < tot; x += (uint64_t)gridDim.x * blockDim.x) {
-        const uint64_t slot = (x / nb) * cap + x % nb;
-        cnt[slot] = 0;
-        smin[slot] = kNone;
-    }
-}
-
-// copy of the open nodes' records (key, j) and their slot (node, cell of the
-// round's depth), counted per slot with one atomic per slot and warp, and the
-// smallest index of every slot (the splits of the round take their children's
-// minima from these)
-__global__ void k_round_copy(const OpenNode* open, const uint32_t* nopen, uint32_t cap, const uint32_t* bigstart,
-                             const uint32_t* total, const uint4* __restrict__ rec, uint4* __restrict__ trec, int sh,
-                             uint32_t dmask, uint32_t* cnt, uint32_t* smin)
-{
-    const uint32_t nb = min(*nopen, cap), T = *total;
-    const int lane = threadIdx.x & 31;
-    const uint32_t stride = gridDim.x * blockDim.x;
-    for (uint32_t p0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); p0 < T; p0 += stride) {   // warp-uniform
-        const uint32_t p = p0 + lane;
-        uint32_t slot = kNone, jv = kNone;
-        if (p < T) {
-            const uint32_t b = big_of(bigstart, nb, p);
-            const uint32_t src = open[b].begin + (p - bigstart[b]);
-            const uint4 r = rec[src];
-            slot = (uint32_t)((rec_key(r) >> sh) & dmask) * cap + b;
-            jv = r.z;
-            trec[p] = make_uint4(r.x, r.y, r.z, slot);
-        }
-        // a warp whose neighbouring lanes hold distinct slots adds per lane (no match,
-        // no reduction over each slot's lanes); otherwise equal slots are merged first
-        const uint32_t snext = __shfl_down_sync(0xFFFFFFFFu, slot, 1);   // (lane 31: its own)
-        if (__any_sync(0xFFFFFFFFu, lane < 31 && slot != kNone && slot == snext)) {
-            const uint32_t peers = __match_any_sync(0xFFFFFFFFu, slot);
-            if (slot != kNone) {   // every lane of a slot's group takes part in its reduction
-                const uint32_t m = __reduce_min_sync(peers, jv);
-                if (lane == __ffs(peers) - 1) {
-                    atomicAdd(&cnt[slot], (uint32_t)__popc(peers));
-                    atomicMin(&smin[slot], m);
-                }
-            }
-        } else if (slot != kNone) {
-            atomicAdd(&cnt[slot], 1u);
-            atomicMin(&smin[slot], jv);
-        }
-    }
-}
-
-// counts -> absolute starts: node b's cells in digit order from open[b].begin (one warp per node)
-__global__ void k_round_bases(const OpenNode* open, const uint32_t* nopen, uint32_t cap, int nd, uint32_t* cnt)
-{
-    const uint32_t nb = min(*nopen, cap);
-    const int lane = threadIdx.x & 31;
-    const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
-    const int per = (nd + 31) / 32;   // <= 16
-    for (uint32_t b = warp; b < nb; b += nwarps) {
-        uint32_t v[16];
-        uint32_t sum = 0;
-#pragma unroll
-        for (int q = 0; q < 16; ++q) {
-            const int d = lane * per + q;
-            v[q] = q < per && d < nd ? cnt[(uint64_t)d * cap + b] : 0u;
-            sum += v[q];
-        }
-        uint32_t x = sum;
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-            if (lane >= o) x += y;
-        }
-        uint32_t run = open[b].begin + (x - sum);
-#pragma unroll
-        for (int q = 0; q < 16; ++q) {
-            const int d = lane * per + q;
-            if (q < per && d < nd) {
-                cnt[(uint64_t)d * cap + b] = run;
-                run += v[q];
-            }
-        }
-    }
-}
-
-// the copied records back into their nodes' ranges, grouped by slot (any order inside a slot)
-__global__ void k_round_scatter(const uint32_t* total, const uint4* __restrict__ trec, uint32_t* cnt,
-                                uint4* __restrict__ rec, uint64_t n, uint32_t* err)
-{
-    const uint32_t T = *total;
-    const int lane = threadIdx.x & 31;
-    const uint32_t stride = gridDim.x * blockDim.x;
-    for (uint32_t p0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); p0 < T; p0 += stride) {   // warp-uniform
-        const uint32_t p = p0 + lane;
-        const uint4 r = p < T ? trec[p] : make_uint4(0u, 0u, 0u, kNone);
-        const uint32_t slot = r.w;
-        // as in k_round_copy: one slot per lane when neighbouring lanes differ
-        const uint32_t snext = __shfl_down_sync(0xFFFFFFFFu, slot, 1);   // (lane 31: its own)
-        uint32_t at = 0;
-        if (__any_sync(0xFFFFFFFFu, lane < 31 && slot != kNone && slot == snext)) {
-            const uint32_t peers = __match_any_sync(0xFFFFFFFFu, slot);
-            const int leader = __ffs(peers) - 1;
-            if (slot != kNone && lane == leader) at = atomicAdd(&cnt[slot], (uint32_t)__popc(peers));
-            at = __shfl_sync(0xFFFFFFFFu, at, leader) + (uint32_t)__popc(peers & lanemask_lt());
-        } else if (slot != kNone) {
-            at = atomicAdd(&cnt[slot], 1u);
-        }
-        if (slot == kNone) continue;
-        if (at >= n) { raise(err, FP_ERR_CAPACITY, 6); continue; }
-        rec[at] = make_uint4(r.x, r.y, r.z, 0u);
-    }
-}
-
-// --------------------------------------------------- big cells: split tree
-// One warp per open node at level q: child ranges by binary search on the
-// key-sorted records, smallest index of every child, hierarchy status, first-min
-// level; children that are still too large stay open, the others become pieces.
-__global__ void k_split(OctCtx c, const OpenNode* cur, const uint32_t* ncur, OpenNode* nxt, uint32_t* nnxt,
-                        uint32_t open_cap, int srt, const uint32_t* smin, int q0)
-{
-    const uint32_t nc = *ncur;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    for (uint32_t w = warp; w < nc; w += nwarps) {
-        const OpenNode o = cur[w];
-        const uint32_t rb = o.q == q0 ? w : o.rb;   // slot column of the round (q0: the round's first level)
-        const int q1 = o.q + 1;
-        const int sh = 3 * (kKeyLevels - q1);
-        // lane d (0..8): first record whose child digit is >= d
-        uint32_t lo = o.begin + o.count;
-        if (lane <= 8) {
-            uint32_t a = o.begin, b = o.begin + o.count;
-            while (a < b) {
-                uint32_t mid = (a + b) >> 1;
-                if ((int)((rec_key_at(c.rec, mid) >> sh) & 7) < lane) a = mid + 1;
-                else b = mid;
-            }
-            lo = a;
-        }
-        // smallest index of every child, and of the node (the smallest of those):
-        // from the round's per-slot minima -- child d covers the slots whose
-        // digits below q0 start with the node's digits below q0, then d
-        // (8^(srt - q1) of them)
-        uint32_t mjd[8];
-        uint32_t pmin = 0xFFFFFFFFu;
-        const int span = 3 * (srt - q1);
-        const uint32_t pre = (uint32_t)(o.key & ((1ull << (3 * (o.q - q0))) - 1));
-#pragma unroll
-        for (int d = 0; d < 8; ++d) {
-            const uint32_t d0 = ((pre << 3) | (uint32_t)d) << span;
-            uint32_t mj = 0xFFFFFFFFu;
-            for (uint32_t t = lane; t < (1u << span); t += 32) mj = min(mj, smin[(uint64_t)(d0 + t) * open_cap + rb]);
-            for (int off = 16; off > 0; off >>= 1) mj = min(mj, __shfl_xor_sync(0xFFFFFFFFu, mj, off));
-            mjd[d] = mj;
-            pmin = min(pmin, mj);
-        }
-#pragma unroll
-        for (int d = 0; d < 8; ++d) {
-            uint32_t cb = __shfl_sync(0xFFFFFFFFu, lo, d);
-            uint32_t ce = __shfl_sync(0xFFFFFFFFu, lo, d + 1);
-            uint32_t cn = ce - cb;
-            if (cn == 0) continue;
-            const uint32_t mj = mjd[d];
-            if (lane == 0) {
-                uint64_t key = (o.key << 3) | (uint64_t)d;
-                uint8_t hier;
-                if (o.hier != kInner) hier = o.hier;
-                else hier = (cn <= c.C || q1 == c.lmax) ? (uint8_t)q1 : kInner;
-                // the child's minimum is the parent's minimum: it keeps the parent's first-min level
-                uint8_t A = mj == pmin ? o.A : (uint8_t)q1;
-                if (o.hier == kInner) emit_node(c, key, q1, cn, cb, hier != kInner);
-                uint32_t id = 0;
-                const bool open_child = cn > (uint32_t)kPieceMax && q1 < c.dl;
-                if (open_child) id = atomicAdd(nnxt, 1u);
-                if (open_child && id >= open_cap) {
-                    raise(c.err, FP_ERR_CAPACITY, 7);
-                } else if (open_child) {
-                    OpenNode ch;
-                    ch.key = key;
-                    ch.begin = cb;
-                    ch.count = cn;
-                    ch.q = (uint8_t)q1;
-                    ch.hier = hier;
-                    ch.A = A;
-                    ch.pad = 0;
-                    ch.rb = rb;
-                    ch.pad2 = ch.pad3 = 0;
-                    nxt[id] = ch;
-                } else {
-                    emit_piece(c, cb, cn, q1, hier, A, srt);
-                }
-            }
-        }
-    }
 }
 
 // ------------------------------------------------------------ pieces
@@ -588,7 +703,7 @@ FP_DEV void put_lambda(const OctCtx& c, uint32_t jj, int lambda, int leafl, uint
 {
     int K = lambda - c.s;
     K = K < 0 ? 0 : (K > leafl ? leafl : K);
-    if (jj < c.n) c.codes[jj] = code_make(K, leafl, cell);
+    if (jj < c.nrec_max) c.codes[jj] = code_make(K, leafl, cell);
     else raise(c.err, FP_ERR_CAPACITY, 17);
 }
 
@@ -596,17 +711,17 @@ FP_DEV void put_lambda(const OctCtx& c, uint32_t jj, int lambda, int leafl, uint
 // over the lanes of the warp one record each: lambda is one more than the
 // deepest level shared with any point of smaller index in the piece (every pair
 // of the piece; its records are a few consecutive words, read through L1).
-FP_DEV void small_warp(const OctCtx& c, uint32_t begin, uint32_t cnt, uint32_t q, uint32_t leafl, uint32_t A)
+FP_DEV void small_warp(const OctCtx& c, uint32_t begin, uint32_t cnt, uint32_t buf, uint32_t leafl, uint32_t A)
 {
     const int lane = threadIdx.x & 31;
-    if ((uint64_t)begin + cnt > c.n) { raise(c.err, FP_ERR_CAPACITY, 18); cnt = 0; }
+    if ((uint64_t)begin + cnt > c.nrec_max) { raise(c.err, FP_ERR_CAPACITY, 18); cnt = 0; }
     uint32_t inc = cnt;
     for (int o = 1; o < 32; o <<= 1) {
         const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
         if (lane >= o) inc += y;
     }
     const uint32_t total = __shfl_sync(0xFFFFFFFFu, inc, 31);
-    const uint32_t what = q | (leafl << 8) | (A << 16);
+    const uint32_t what = buf | (leafl << 8) | (A << 16);
     for (uint32_t r0 = 0; r0 < total; r0 += 32) {
         const uint32_t r = r0 + lane;
         int o = 0;   // lanes whose pieces end at or before r
@@ -619,11 +734,12 @@ FP_DEV void small_warp(const OctCtx& c, uint32_t begin, uint32_t cnt, uint32_t q
         const uint32_t b0 = __shfl_sync(0xFFFFFFFFu, begin, o);
         const uint32_t at = b0 + r - (__shfl_sync(0xFFFFFFFFu, inc, o) - cn);
         if (r >= total) continue;   // (no shuffle below)
-        const uint4 me = c.rec[at];
+        const uint4* rec = c.recs[w & 1u];
+        const uint4 me = rec[at];
         const uint64_t k = rec_key(me);
         uint64_t near = ~0ull;   // smallest key difference to a smaller index: the deepest shared level
         for (uint32_t t = 0; t < cn; ++t) {
-            const uint4 other = c.rec[b0 + t];
+            const uint4 other = rec[b0 + t];
             const uint64_t x = rec_key(other) ^ k;
             if (other.z < me.z && x < near) near = x;
         }
@@ -651,13 +767,13 @@ __global__ void __launch_bounds__(256) k_small_pieces(OctCtx c)
             if (leafl == kInner) cnt = 0;
             else begin = c.cstart[m];
         }
-        if (__any_sync(0xFFFFFFFFu, cnt != 0)) small_warp(c, begin, cnt, c.g, leafl, c.g);
+        if (__any_sync(0xFFFFFFFFu, cnt != 0)) small_warp(c, begin, cnt, 0, leafl, c.g);
     }
-    const uint32_t ns = min(*c.nsmall, c.piece_cap);
+    const uint32_t ns = min(*c.n[LIST_SMALL], c.piece_cap);
     for (uint32_t p0 = warp * 32; p0 < ns; p0 += nwarps * 32) {
         Piece p{};
-        if (p0 + lane < ns) p = c.small[p0 + lane];
-        small_warp(c, p.begin, p.count, p.q, p.hier, p.A);
+        if (p0 + lane < ns) p = c.list[LIST_SMALL][p0 + lane];
+        small_warp(c, p.begin, p.count, p.buf, p.hier, p.A);
     }
 }
 
@@ -681,7 +797,7 @@ FP_DEV void direct_piece(const OctCtx& c, const Piece& p, int D, uint32_t* tab, 
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             rec[r] = make_uint4(0u, 0u, 0u, 0u);
-            if (r * kTabNT + tid < n) rec[r] = get_rec(c, (uint64_t)p.begin + r * kTabNT + tid);
+            if (r * kTabNT + tid < n) rec[r] = get_rec(c, p.buf, (uint64_t)p.begin + r * kTabNT + tid);
         }
         // clear the tables while the records arrive
         const int words4 = (int)((((1u << (3 * (D + 1))) - 8u) / 7u + 3u) / 4u);
@@ -743,12 +859,12 @@ FP_DEV void hash_piece(const OctCtx& c, const Piece& p, int D, uint64_t* mine /*
     const int n = (int)p.count, leafl = p.hier, q = p.q;
     const int sh = 3 * (kKeyLevels - q - D);
     const uint32_t cmask = (uint32_t)((1ull << (3 * D)) - 1);
-    const uint32_t cell = (uint32_t)(rec_key_at(c.rec, p.begin) >> (3 * (kKeyLevels - c.g)));
+    const uint32_t cell = (uint32_t)(rec_key(get_rec(c, p.buf, p.begin)) >> (3 * (kKeyLevels - c.g)));
     const uint32_t slots = (uint32_t)(n + (n >> 1)) & ~1u;   // even; at most two thirds are taken
     if (tid == 0) *s_min = kNone;
 #pragma unroll 4
     for (int r = tid; r < n; r += kTabNT) {
-        const uint4 rec = get_rec(c, (uint64_t)p.begin + r);
+        const uint4 rec = get_rec(c, p.buf, (uint64_t)p.begin + r);
         mine[r] = ((uint64_t)((uint32_t)(rec_key(rec) >> sh) & cmask) << 30) | rec.z;
     }
     constexpr uint32_t kJMask = (1u << 30) - 1u;
@@ -811,7 +927,7 @@ __global__ void __launch_bounds__(kTabNT, kTabCtas) k_tab_pieces(OctCtx c)
     __shared__ __align__(16) unsigned char buf[kTabBytes];
     __shared__ uint32_t s_min;
     __shared__ uint32_t s_next;
-    const uint32_t nt = min(*c.ntab, c.piece_cap);
+    const uint32_t nt = min(*c.n[LIST_TAB], c.piece_cap);
     // runs of up to kTabRun pieces (fewer when that would leave blocks without
     // work: 10^7 points, 0.23 against 0.29 ms) are taken in order from a counter: with a fixed share
     // per block the blocks drifted apart over a large cloud until their scattered
@@ -822,15 +938,16 @@ __global__ void __launch_bounds__(kTabNT, kTabCtas) k_tab_pieces(OctCtx c)
     __syncthreads();
     uint32_t k = s_next, k1 = k + run;
     Piece next{};
-    if (k < nt) next = c.tab[k];
+    if (k < nt) next = c.list[LIST_TAB][k];
     while (k < nt) {
         const Piece p = next;
         if (k + 1 == k1) {   // (every block barrier of a piece lies between this write and the read below)
             if (threadIdx.x == 0) s_next = atomicAdd(c.tab_claim, run);
         } else if (k + 1 < nt) {   // the next piece's records on their way to L2 during this one's work
-            next = c.tab[k + 1];
+            next = c.list[LIST_TAB][k + 1];
             const uint32_t line = threadIdx.x * 8;   // 128 bytes a thread
-            if (line < next.count && (uint64_t)next.begin + line < c.n) prefetch_l2(c.rec + next.begin + line);
+            if (line < next.count && (uint64_t)next.begin + line < c.nrec_max)
+                prefetch_l2(c.recs[next.buf] + next.begin + line);
         }
         const int D = piece_depth(c, p.q, p.hier);
         uint32_t* tab = reinterpret_cast<uint32_t*>(buf);
@@ -843,7 +960,7 @@ __global__ void __launch_bounds__(kTabNT, kTabCtas) k_tab_pieces(OctCtx c)
         if (++k == k1) {
             k = s_next;
             k1 = k + run;
-            if (k < nt) next = c.tab[k];
+            if (k < nt) next = c.list[LIST_TAB][k];
             __syncthreads();   // s_next is read before it is written again
         }
     }
@@ -939,7 +1056,7 @@ FP_DEV void general_piece(const OctCtx& c, GenSmem& S, const Piece& pc)
         for (int q = 0; q < kPer; ++q) {
             const int r = threadIdx.x + q * kGenNT;
             if (r < cnt) {
-                const uint4 rec = get_rec(c, (uint64_t)pc.begin + r);
+                const uint4 rec = get_rec(c, pc.buf, (uint64_t)pc.begin + r);
                 const uint64_t k = rec_key(rec);
                 S.key[r] = k;
                 S.j[r] = rec.z;
@@ -1133,22 +1250,22 @@ __global__ void __launch_bounds__(kGenNT) k_general_pieces(OctCtx c)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     GenSmem& S = *reinterpret_cast<GenSmem*>(smem_raw);
-    const uint32_t ng = min(*c.ngen, c.piece_cap);
-    for (uint32_t k = blockIdx.x; k < ng; k += gridDim.x) general_piece(c, S, c.gen[k]);
-    const uint32_t nd = min(*c.ndups, c.piece_cap);
+    const uint32_t ng = min(*c.n[LIST_GEN], c.piece_cap);
+    for (uint32_t k = blockIdx.x; k < ng; k += gridDim.x) general_piece(c, S, c.list[LIST_GEN][k]);
+    const uint32_t nd = min(*c.n[LIST_DUP], c.piece_cap);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (uint32_t k = blockIdx.x; k < nd; k += gridDim.x) {
-        const Piece p = c.dups[k];
+        const Piece p = c.list[LIST_DUP][k];
         const int leafl = p.hier == kInner ? c.lmax : (int)p.hier;
         uint32_t mn = kNone;
-        for (uint32_t r = threadIdx.x; r < p.count; r += kGenNT) mn = min(mn, get_rec(c, (uint64_t)p.begin + r).z);
+        for (uint32_t r = threadIdx.x; r < p.count; r += kGenNT) mn = min(mn, get_rec(c, p.buf, (uint64_t)p.begin + r).z);
         mn = __reduce_min_sync(0xFFFFFFFFu, mn);
         if (lane == 0) S.scan[warp] = mn;
         __syncthreads();
         mn = S.scan[0];
         for (int w = 1; w < kGenWarps; ++w) mn = min(mn, S.scan[w]);
         for (uint32_t r = threadIdx.x; r < p.count; r += kGenNT) {
-            const uint4 rr = get_rec(c, (uint64_t)p.begin + r);
+            const uint4 rr = get_rec(c, p.buf, (uint64_t)p.begin + r);
             put_lambda(c, rr.z, rr.z == mn ? (int)p.A : kKeyLevels + 1, leafl,
                        (uint32_t)(rec_key(rr) >> (3 * (kKeyLevels - c.g))));
         }
@@ -1253,7 +1370,7 @@ __global__ void k_node_children(const uint32_t* nnode, const uint64_t* sorted_st
 }
 
 // The node table in one launch of one cluster, for at most kNodeClusterMax nodes
-// by the host's bound (28 launches otherwise; 1M points: 110 -> NODEUS us).  Stable
+// by the host's bound (28 launches otherwise; 1M points: about 110 -> 19 us).  Stable
 // least-significant-digit-first passes over (level, start): every CTA counts the
 // digits of its slice, all CTAs' counts give every digit's base, and each tile of
 // 1024 records is ranked by ballots.  A pass in which all records share the digit
@@ -1574,7 +1691,7 @@ __global__ void k_gather_u64(const uint64_t* src, const uint32_t* idx, const uin
 
 // ------------------------------------------------------------ host: octree
 struct OctLayout {
-    uint64_t cells, npyr, piece_cap, open_cap, node_cap;
+    uint64_t cells, npyr, piece_cap, open_cap, big_cap, node_cap;
 };
 
 static OctLayout oct_layout(uint64_t n, const fp_params& p)
@@ -1583,7 +1700,8 @@ static OctLayout oct_layout(uint64_t n, const fp_params& p)
     L.cells = 1ull << (3 * p.grid_log2);
     L.npyr = (L.cells - 1) / 7;
     L.piece_cap = L.cells + 16 * (n / kPieceMax) + 4096;
-    L.open_cap = n / kPieceMax + 1024;
+    L.open_cap = n / kPieceMax + 1;   // open nodes are disjoint, of more than kPieceMax records each
+    L.big_cap = n / kRoundTile + 1;
     const uint64_t upper = (L.cells * 8 - 1) / 7;
     const uint64_t C = p.node_capacity ? p.node_capacity : 1;
     // every deep node is a child of an inner node, and an inner node holds more than C points:
@@ -1609,18 +1727,18 @@ static uint64_t node_bound(uint64_t n, const fp_params& p)
 
 struct OctBufs {
     SortScratch sc;
-    uint32_t* rcnt;        // counting slots of a split round: 8^3 per open node
+    uint32_t* rcnt;        // counting slots of a split round: 8^3 per large open node
     uint32_t* rmin;        // the smallest index of every slot
-    uint4* trec;   // split rounds: the copied records with their slots
+    uint4* trec;           // split rounds: the second record buffer
     int4* lt_pt;
     uint32_t *lt_val, *lt_k32;
     uint32_t *pyr, *rsum, *cstart, *cursor;
     uint8_t* cell_leaf;
     uint4* rec;           // cell-grouped records (rec_key, rec_j)
     Piece* pieces[4];     // table, small, general, oversized
-    uint32_t* counters;   // [0], [1], [2], [4] their numbers, [3] node records, [5] table pieces taken
-    OpenNode* open[2];
-    uint32_t *ocount, *bigstart;
+    uint32_t* counters;   // [0..3] their numbers, [4] node records, [5] table pieces taken, [6] barrier of the rounds
+    RoundCnt* rounds;
+    OpenNode *open[2], *big[2];
     NodeRec* nrec;
     uint64_t *nk, *nk2, *nk3, *nk4;
     uint32_t *nl, *nv2, *nv3;
@@ -1632,14 +1750,16 @@ struct OctBufs {
     SegScratch seg;
 };
 
+constexpr int kOctCounters = 8 + (kMaxRounds + 1) * (int)(sizeof(RoundCnt) / sizeof(uint32_t));   // words, zeroed
+
 // one carve-up serves both the size query (base == nullptr) and the launch
 static OctBufs oct_carve(const Workspace& ws, uint64_t n, const OctLayout& Ly)
 {
     OctBufs B;
     const uint64_t N = n ? n : 1;
     B.sc = take_sort_scratch(ws, std::max<uint64_t>(N, Ly.node_cap));
-    B.rcnt = ws.take<uint32_t>(Ly.open_cap << (3 * kRoundLevels));
-    B.rmin = ws.take<uint32_t>(Ly.open_cap << (3 * kRoundLevels));
+    B.rcnt = ws.take<uint32_t>(Ly.big_cap << (3 * kRoundLevels));
+    B.rmin = ws.take<uint32_t>(Ly.big_cap << (3 * kRoundLevels));
     // aliased phase region: grouping temporaries, later the leaf scatter temporaries
     const size_t phase_base = ws.used;
     B.trec = ws.take<uint4>(N);
@@ -1654,10 +1774,10 @@ static OctBufs oct_carve(const Workspace& ws, uint64_t n, const OctLayout& Ly)
     B.cell_leaf = ws.take<uint8_t>(Ly.cells);
     B.rec = ws.take<uint4>(N);
     for (Piece*& p : B.pieces) p = ws.take<Piece>(Ly.piece_cap);
-    B.counters = ws.take<uint32_t>(8 + 4);
-    B.ocount = B.counters + 8;
+    B.counters = ws.take<uint32_t>(kOctCounters);
+    B.rounds = reinterpret_cast<RoundCnt*>(B.counters + 8);
     B.open[0] = ws.take<OpenNode>(Ly.open_cap); B.open[1] = ws.take<OpenNode>(Ly.open_cap);
-    B.bigstart = ws.take<uint32_t>(Ly.open_cap + 1);
+    B.big[0] = ws.take<OpenNode>(Ly.big_cap); B.big[1] = ws.take<OpenNode>(Ly.big_cap);
     B.nrec = ws.take<NodeRec>(Ly.node_cap);
     B.nk = ws.take<uint64_t>(Ly.node_cap); B.nk2 = ws.take<uint64_t>(Ly.node_cap);
     B.nk3 = ws.take<uint64_t>(Ly.node_cap); B.nk4 = ws.take<uint64_t>(Ly.node_cap);
@@ -1770,23 +1890,27 @@ cudaError_t launch_octree_impl(const fp_point* sorted, const uint32_t* perm, uin
     const uint64_t N = n;
     const OctBufs B = oct_carve(ws, n, Ly);
     const SortScratch& sc = B.sc;
-    uint32_t* nnode = B.counters + 3;
+    uint32_t* nnode = B.counters + 4;
     OctCtx c;
     c.counts = counts; c.rcounts = rcounts; c.leaf_base = grp ? grp->leaf_base : 0u;
     c.cstart = B.cstart; c.cursor = B.cursor; c.cell_leaf = B.cell_leaf;
-    c.rec = B.rec; c.piece_cap = (uint32_t)Ly.piece_cap;
-    c.tab = B.pieces[0]; c.small = B.pieces[1]; c.gen = B.pieces[2]; c.dups = B.pieces[3];
-    c.ntab = B.counters; c.nsmall = B.counters + 1; c.ngen = B.counters + 2; c.ndups = B.counters + 4; c.tab_claim = B.counters + 5;
+    c.recs[0] = B.rec; c.recs[1] = B.trec; c.nrec_max = N; c.piece_cap = (uint32_t)Ly.piece_cap;
+    for (int l = 0; l < 4; ++l) { c.list[l] = B.pieces[l]; c.n[l] = B.counters + l; }
+    c.tab_claim = B.counters + 5;
     c.nrec = B.nrec; c.nnode = nnode; c.node_cap_ws = (uint32_t)Ly.node_cap;
     c.codes = grp ? grp->codes : B.codes;
-    c.open_cap = (uint32_t)Ly.open_cap;
-    c.g = g; c.s = s; c.lmax = lmax; c.dl = dl; c.C = prm.node_capacity; c.n = N; c.err = ws.err;
+    c.g = g; c.s = s; c.lmax = lmax; c.dl = dl; c.C = prm.node_capacity; c.err = ws.err;
+    RoundArgs ra{};
+    ra.c = c;
+    for (int l = 0; l < 2; ++l) { ra.small[l] = B.open[l]; ra.big[l] = B.big[l]; }
+    ra.cnt = B.rounds; ra.small_cap = (uint32_t)Ly.open_cap; ra.big_cap = (uint32_t)Ly.big_cap;
+    ra.slots = B.rcnt; ra.smin = B.rmin; ra.bar = B.counters + 6;
 
     // 1. the grid's levels, every cell's start, leaf level and piece, the nodes at
     // levels <= g (a chunk group leaves those to the whole-cloud node table)
     const int ntile = grid_tiles(g);
-    k_grid_tiles<<<ntile, kGtNT, 0, st>>>(counts, g, B.pyr, rcounts, B.rsum, nullptr, 0, B.counters, 12);
-    k_cells_open<<<ntile, kGtNT, 0, st>>>(c, B.pyr, B.rsum, 1, grp ? 0 : 1, B.cstart, B.cursor, B.open[0], B.ocount);
+    k_grid_tiles<<<ntile, kGtNT, 0, st>>>(counts, g, B.pyr, rcounts, B.rsum, nullptr, 0, B.counters, kOctCounters);
+    k_cells_open<<<ntile, kGtNT, 0, st>>>(ra, B.pyr, B.rsum, 1, grp ? 0 : 1, B.cstart, B.cursor);
     // 2. group by level-g cell: (key21, j) scattered by cell id
     {
         const int gs = (int)std::max<uint64_t>(1, std::min<uint64_t>((N + 255) / 256, (uint64_t)ws.num_sms * 8));
@@ -1794,37 +1918,22 @@ cudaError_t launch_octree_impl(const fp_point* sorted, const uint32_t* perm, uin
         k_cell_scatter<<<gs, 256, 0, st>>>(reinterpret_cast<const int4*>(sorted), N, cube, B.cursor, B.rec, g,
                                            ws.err);
     }
-    // 3. big cells: split tree.  Rounds of up to three levels: the records of
-    // the open nodes are grouped by their cell three levels down (one counting
-    // scatter: copy out with per-(node, cell) counts, starts, scatter back),
-    // which puts them in key order down to that depth; then the splits of
-    // those levels, whose children still too large stay open for the next round.
-    {
+    // 3. big cells split into pieces
+    if (N > (uint64_t)kPieceMax) {
         KTimerScope kt(FP_KERNEL_SPLIT_ROUNDS, st);
-        const uint32_t cap = (uint32_t)Ly.open_cap;
-        int gw = std::max(1, std::min(ws.num_sms * 16, (int)(((uint64_t)cap * 32 + 255) / 256)));
-        const int gr = std::max(1, std::min(ws.num_sms * 8, (int)((N + 255) / 256)));
-        int cur = 0;
-        for (int q = g; q < dl;) {
-            const int k = std::min(kRoundLevels, dl - q);
-            const int nd = 1 << (3 * k);
-            k_open_counts<<<(cap + 255) / 256, 256, 0, st>>>(B.open[cur], B.ocount + cur, B.bigstart, cap, nullptr, 0);
-            if ((e = scan_exclusive<uint32_t, uint32_t>(B.bigstart, B.bigstart, cap, nullptr, B.leafw, B.ocount + 3,
-                                                        (uint32_t*)nullptr, st)))
-                return e;
-            k_round_zero<<<gr, 256, 0, st>>>(B.ocount + cur, cap, nd, B.rcnt, B.rmin);
-            k_round_copy<<<gr, 256, 0, st>>>(B.open[cur], B.ocount + cur, cap, B.bigstart, B.ocount + 3, B.rec,
-                                             B.trec, 3 * (kKeyLevels - q - k), (uint32_t)(nd - 1), B.rcnt, B.rmin);
-            k_round_bases<<<gw, 256, 0, st>>>(B.open[cur], B.ocount + cur, cap, nd, B.rcnt);
-            k_round_scatter<<<gr, 256, 0, st>>>(B.ocount + 3, B.trec, B.rcnt, B.rec, N, ws.err);
-            for (int l = q; l < q + k; ++l) {
-                k_set_u32<<<1, 1, 0, st>>>(B.ocount + (1 - cur), 0);
-                k_split<<<gw, 256, 0, st>>>(c, B.open[cur], B.ocount + cur, B.open[1 - cur], B.ocount + (1 - cur),
-                                            cap, q + k, B.rmin, q);
-                cur = 1 - cur;
-            }
-            q += k;
-        }
+        int per_sm = 0;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rounds, kRoundNT, 0))) return e;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)std::min<uint64_t>((N + kRoundTile - 1) / kRoundTile,
+                                                        (uint64_t)ws.num_sms * std::max(per_sm, 1)));
+        cfg.blockDim = dim3(kRoundNT);
+        cfg.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeCooperative;   // its blocks wait for one another
+        at[0].val.cooperative = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        if ((e = cudaLaunchKernelEx(&cfg, k_rounds, ra))) return e;
     }
     // 4. lambda of every record: owner level and leaf level
     {
@@ -1889,7 +1998,8 @@ cudaError_t launch_octree_impl(const fp_point* sorted, const uint32_t* perm, uin
         a.b.pt_tmp = B.lt_pt;
         a.b.pt_dst = reinterpret_cast<int4*>(leaf_pts);
         a.b.val_src = perm; a.b.val_tmp = B.lt_val; a.b.val_dst = leaf_perm;
-        a.b.k32_src = B.leafid; a.b.k32_tmp = B.lt_k32; a.b.k32_dst = nullptr;
+        // (three passes read the ids back from dst; the codes are not needed any more)
+        a.b.k32_src = B.leafid; a.b.k32_tmp = B.lt_k32; a.b.k32_dst = B.codes;
         a.n = N; a.run_if = B.seg.cnt + 2; a.err = ws.err;
         if ((e = sort_plan_weights(sc, a, B.leafw, nullptr, nnode, Ly.node_cap, true, ws.num_sms, st))) return e;
         const int np = sort_passes(count_bits(Ly.node_cap));   // leaf ids below node_cap
@@ -1943,7 +2053,9 @@ cudaError_t launch_octree_nodes(const uint32_t* counts, uint64_t n, const fp_par
     c.nrec = recs; c.nnode = T.nnode; c.node_cap_ws = (uint32_t)rec_cap;
     c.g = g; c.s = (int)prm.sub_log2; c.lmax = lmax; c.C = prm.node_capacity; c.err = ws.err;
     k_grid_tiles<<<grid_tiles(g), kGtNT, 0, st>>>(counts, g, B.pyr, counts, B.rsum, nullptr, 0, nullptr, 0);
-    k_cells_open<<<grid_tiles(g), kGtNT, 0, st>>>(c, B.pyr, B.rsum, 0, 1, nullptr, nullptr, nullptr, nullptr);
+    RoundArgs ra{};
+    ra.c = c;
+    k_cells_open<<<grid_tiles(g), kGtNT, 0, st>>>(ra, B.pyr, B.rsum, 0, 1, nullptr, nullptr);
     NodeSortBufs nb = B.nb;
     nb.nk = T.starts; nb.slevel = T.slevel; nb.idxtab = T.idxtab; nb.ndesc = T.ndesc;
     if ((e = node_table(B.sc, recs, T.nnode, (uint32_t)rec_cap, n ? node_bound(n, prm) : rec_cap, nb, nodes, node_cap,
@@ -2036,7 +2148,7 @@ struct SubBufs {
     uint32_t *srank, *slist;   // rank of a node outside every chunk subtree, and back
     uint64_t* first;
     int4 *o_pt, *t_pt;
-    uint32_t *o_own, *t_val, *t_k32;
+    uint32_t *o_own, *o_own2, *t_val, *t_k32;
     uint64_t *s_key, *s_key2, *s_key3;
     uint32_t *s_val, *s_val2, *s_val3;
     SegScratch seg;
@@ -2057,7 +2169,7 @@ static SubBufs sub_carve(const Workspace& ws, uint64_t n, uint64_t M)
     // One region serves two sets of per-point buffers that are never live
     // together: the whole-array path's, and the staged records and their sort's.
     const size_t region = ws.used;
-    B.o_pt = ws.take<int4>(N); B.o_own = ws.take<uint32_t>(N);
+    B.o_pt = ws.take<int4>(N); B.o_own = ws.take<uint32_t>(N); B.o_own2 = ws.take<uint32_t>(N);
     B.t_pt = ws.take<int4>(N); B.t_val = ws.take<uint32_t>(N); B.t_k32 = ws.take<uint32_t>(N);
     const size_t end_t = ws.used;
     ws.used = region;
@@ -2136,7 +2248,7 @@ cudaError_t launch_subsample(fp_node* nodes, const uint32_t* num_nodes, uint32_t
     SortArgs a{};
     a.b.pt_src = B.o_pt; a.b.pt_tmp = B.t_pt; a.b.pt_dst = reinterpret_cast<int4*>(final_pts);
     a.b.val_src = nullptr; a.b.val_tmp = B.t_val; a.b.val_dst = final_perm;   // the original index
-    a.b.k32_src = B.o_own; a.b.k32_tmp = B.t_k32; a.b.k32_dst = nullptr;
+    a.b.k32_src = B.o_own; a.b.k32_tmp = B.t_k32; a.b.k32_dst = B.o_own2;
     a.n = N; a.run_if = gate; a.err = ws.err;
     const SortScratch sc2{B.hist2, {sc.status[0], sc.status[1]}};
     if ((e = sort_plan_weights(sc2, a, B.nown, nullptr, nm, M, true, ws.num_sms, st))) return e;

@@ -20,12 +20,12 @@ SIZES = [1, 2, 31, 32, 33, 127, 128, 129, 255, 256, 257, 511, 512, 513, 1023, 10
 SIDE = 1 << 21
 
 
-def cells_cloud(spread, seed):
+def cells_cloud(spread, seed, sizes=SIZES):
     """One level-3 cell of every size, points in random order; two far corners fix the cube."""
     rng = np.random.default_rng(seed)
     w = SIDE >> 3
     rows = [np.array([[0, 0, 0], [SIDE - 1] * 3])]
-    for k, n in enumerate(SIZES):
+    for k, n in enumerate(sizes):
         m = 9 + 17 * k   # cells apart from each other and from the corners'
         base = np.array([(m >> 6) & 7, (m >> 3) & 7, m & 7]) * w
         p = rng.integers(0, w, (n, 3))
@@ -71,6 +71,21 @@ def test_piece_sizes_and_depths(gpu_lib, spread, s):
 @pytest.mark.parametrize("s,lmax,C", [(3, 12, 20), (7, 15, 300), (5, 9, 1000), (11, 11, 40)])
 def test_pieces_below_leaves(gpu_lib, spread, s, lmax, C):
     check(gpu_lib, cells_cloud(spread, 7 * s + C), 3, s, lmax, 2000, C)
+
+
+# split rounds: nodes of one tile (4096 records) and of several, split again and again where
+# the points lie close together, down to runs of equal keys; leaves above and below the cells
+@pytest.mark.parametrize("spread", ["volume", "plane", "line", "spot"])
+@pytest.mark.parametrize("s,lmax,C", [(7, 15, 1 << 20), (7, 15, 3000), (10, 12, 700), (3, 18, 50), (5, 8, 5000)])
+def test_split_rounds(gpu_lib, spread, s, lmax, C):
+    sizes = [1025, 4095, 4096, 4097, 8193, 30_000, 70_000]
+    check(gpu_lib, cells_cloud(spread, 3 * s + lmax, sizes), 3, s, lmax, max(C, 20_000), C)
+
+
+# more nodes than the one-launch node table takes, and as few as one
+@pytest.mark.parametrize("n,g,s,lmax,C", [(60_000, 4, 5, 15, 1), (1, 4, 5, 15, 1), (60_000, 7, 7, 15, 1 << 20)])
+def test_node_counts(gpu_lib, n, g, s, lmax, C):
+    check(gpu_lib, synth.lidar(n, 77), g, s, lmax, max(C, 2000), C)
 
 
 @pytest.mark.parametrize("g", [1, 2, 3, 4, 5, 6, 7])
