@@ -65,7 +65,8 @@ struct FusedCloud {
     uint64_t prev_cap;
     uint64_t* prev_cnt;
     uint32_t* counts;
-    uint32_t modulus, g;
+    KeepMultiple mult;
+    uint32_t g;
 };
 
 struct FusedArgs {
@@ -143,8 +144,7 @@ __global__ void __launch_bounds__(kFbNT, 2) k_fused_bounds_decimate(const __grid
             const uint64_t i = base + (uint64_t)r * kFbNT + threadIdx.x;
             bool k = false;
             if (i < d.n) {
-                const uint64_t h = splitmix64(i);
-                k = (d.modulus & (d.modulus - 1)) == 0 ? (h & ((uint64_t)d.modulus - 1)) == 0 : (h % d.modulus) == 0;
+                k = d.mult(i);
             }
             const uint32_t bal = __ballot_sync(0xFFFFFFFFu, k);
             if (lane == 0) s_cnt[r][warp] = __popc(bal);
@@ -436,7 +436,7 @@ fp_status fused_first(const fp_cloud_desc* c, uint32_t g0, uint32_t g1, const fp
         f.prev_cap = d.d_preview ? d.preview_cap : 0;
         f.prev_cnt = d.d_preview_count;
         f.counts = d.d_counts;
-        f.modulus = d.prm.decim_modulus;
+        f.mult = KeepMultiple::of(d.prm.decim_modulus);
         f.g = d.prm.grid_log2;
         a.tile0[i - g0] = tiles;
         a.item0[i - g0] = items;

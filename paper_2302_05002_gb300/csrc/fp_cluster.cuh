@@ -1,4 +1,7 @@
-// fp_cluster.cuh -- steps over a few thousand nodes or chunks in one launch: a
+// fp_cluster.cuh -- several phases in one launch, by a barrier of the whole grid
+// (cooperative launch) or of one cluster.
+//
+// Steps over a few thousand nodes or chunks: a
 // cluster of 8 CTAs of 1024 threads whose phases are separated by the hardware
 // cluster barrier.  Such a step used to be a chain of grid launches (scans of
 // three, sorts of two per pass); at these sizes a launch costs more, on the host
@@ -52,6 +55,46 @@ FP_DEV uint64_t cl_scan(uint32_t n, uint64_t* part, uint64_t* smem_warp /* 32 wo
     }
     cl_sync();   // (part may be written again)
     return all;
+}
+
+// barrier number `k` (from 1) of the grid, every block of which is resident
+// (cooperative launch); false when the bounded wait ran out
+FP_DEV bool grid_barrier(uint32_t* word, uint32_t k, uint32_t* err)
+{
+    __shared__ int s_ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(word, 1u);
+        const uint32_t target = k * gridDim.x;
+        uint32_t spins = 0;
+        s_ok = 1;
+        while (ld_volatile(word) < target) {
+            if (++spins > (1u << 22)) { raise(err, FP_ERR_TIMEOUT); s_ok = 0; break; }
+            __nanosleep(64);
+        }
+        __threadfence();
+    }
+    __syncthreads();
+    return s_ok != 0;
+}
+
+// cooperative launch (all blocks resident, so that they may wait for one another)
+template <typename... Params, typename... Args>
+inline cudaError_t coop_launch(void (*kernel)(Params...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+                               Args... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 // launch of kernel(args) as one cluster

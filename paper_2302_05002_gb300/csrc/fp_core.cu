@@ -1,18 +1,20 @@
 // fp_core.cu -- bounds, preview decimation, count grid and chunk merge.
 //
-//   k_bounds_decimate  one pass over the cloud: per-axis min/max (Sec. 4.4) and,
+//   k_bounds_bulk      one pass over the cloud: per-axis min/max (Sec. 4.4) and,
 //                      optionally, the preview compaction (Sec. 3 / Sec. 4.2):
 //                      index i is kept iff splitmix64(first + i) % m == 0.  Kept
 //                      points keep ascending index order through a single-pass
-//                      scan with decoupled look-back across tiles.  With the
-//                      bounds (the main path, k_bounds_bulk) each tile arrives
-//                      in shared memory by one bulk copy issued when the tile is
-//                      claimed, in flight during the ranking and look-back.
+//                      scan with decoupled look-back across tiles.  Each tile
+//                      arrives in shared memory by one bulk copy issued when the
+//                      tile is claimed, in flight during the ranking and look-back.
+//   k_keep, k_keep_write   the previews without extents: the uniform one, and
+//                      the spatial one (with k_cell_min_hash before them).
 //   k_count            count grid: one level-g Morton key per point, warp-
 //                      aggregated atomics into an L2-resident 8^g histogram.
 //   k_merge_write      with k_grid_tiles' sums of the grid: the chunk rule of
 //                      Fig. "octree" (maximal nodes with 0 < count <= T, plus
 //                      overflowing finest cells), listed in Morton preorder.
+#include "fp_cluster.cuh"
 #include "fp_grid.cuh"
 
 namespace fp {
@@ -26,171 +28,193 @@ constexpr uint64_t kFlagAgg = 1ull << 62;
 constexpr uint64_t kFlagInc = 2ull << 62;
 constexpr uint64_t kValMask = (1ull << 62) - 1;
 
-// keep rule of the compaction: none, index hash modulo m (the uniform
-// preview), or the smallest index hash of the point's cell (the spatial one)
-enum KeepRule { KEEP_NONE = 0, KEEP_MODULUS = 1, KEEP_CELL_MIN = 2 };
-
-FP_DEV bool keep_modulus(uint64_t first, uint64_t i, uint32_t modulus)
+// The tile's output offset by decoupled look-back, by one warp: 32 earlier
+// tiles' words per round trip; the sum runs back to the nearest inclusive
+// prefix, and stops (and reads again) at the nearest word not yet published.
+// Publishes the tile's own words; the last tile writes the total.  (By the whole
+// block, 256 words a trip, the polling slowed the publishing: 0.21 -> 0.27 ms at
+// 51M points.)
+FP_DEV uint64_t preview_base(uint64_t* tile_status, uint64_t tile, uint64_t ntiles, uint32_t total, uint64_t out_cap,
+                             uint64_t* out_count, uint32_t* err)
 {
-    const uint64_t h = splitmix64(first + i);
-    return (modulus & (modulus - 1)) == 0 ? (h & ((uint64_t)modulus - 1)) == 0 : (h % modulus) == 0;
+    const int lane = threadIdx.x & 31;
+    uint64_t excl = 0;
+    if (tile == 0) {
+        if (lane == 0) atomicExch((unsigned long long*)&tile_status[0], (unsigned long long)(kFlagInc | total));
+    } else {
+        if (lane == 0) atomicExch((unsigned long long*)&tile_status[tile], (unsigned long long)(kFlagAgg | total));
+        int64_t t = (int64_t)tile - 1;
+        uint32_t spins = 0;
+        while (t >= 0) {
+            const int64_t q = t - lane;
+            const uint64_t w = q >= 0 ? ld_volatile64(&tile_status[q]) : kFlagInc;
+            const uint32_t inc = __ballot_sync(0xFFFFFFFFu, (w >> 62) == 2);
+            const uint32_t none = __ballot_sync(0xFFFFFFFFu, (w >> 62) == 0);
+            const int fi = inc ? __ffs(inc) - 1 : 32, fn = none ? __ffs(none) - 1 : 32;
+            // lanes [0, take) are summed: up to the first unpublished word, or
+            // through the first inclusive prefix, or all 32 aggregates
+            const int take = fn < fi ? fn : (fi < 32 ? fi + 1 : 32);
+            uint64_t v = lane < take ? (w & kValMask) : 0;
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+            excl += v;
+            if (fi < fn) break;   // reached an inclusive prefix
+            if (take == 0 && ++spins > kSpinLimit) {
+                if (lane == 0) raise(err, FP_ERR_TIMEOUT);
+                break;
+            }
+            t -= take;
+        }
+        if (lane == 0)
+            atomicExch((unsigned long long*)&tile_status[tile], (unsigned long long)(kFlagInc | (excl + total)));
+    }
+    if (lane == 0 && tile == ntiles - 1) {
+        *out_count = excl + total;
+        if (excl + total > out_cap) raise(err, FP_ERR_CAPACITY, 0);
+    }
+    return excl;
 }
 
-template <bool BOUNDS, int KEEP>
-__global__ void __launch_bounds__(kBdNT) k_bounds_decimate(const fp_point* __restrict__ pts, uint64_t n,
-                                                           uint64_t first, uint32_t modulus, fp_point* __restrict__ out,
-                                                           uint64_t out_cap, uint64_t* __restrict__ out_count,
-                                                           int32_t* __restrict__ partial, uint64_t* tile_status,
-                                                           uint32_t* tile_counter, uint64_t ntiles, uint32_t* err,
-                                                           const uint64_t* __restrict__ cell_min,
-                                                           const fp_cube* cube_p, int level)
+// The previews that need no extents, without a look-back.  Keep rule: the index
+// hash is a multiple of the modulus (the uniform preview: only the kept points
+// are read), or it is the smallest of the point's cell (the spatial one).  A
+// block takes a segment of consecutive tiles; a warp takes ROWS rows of 32
+// points, lane r holds row r's keep bits.  When every block has counted its
+// segment, a tile's output starts at the totals of the earlier segments plus its
+// place in its own.
+//   k_keep_all: both halves in one cooperative launch, the keep bits in shared
+//     memory across the barrier (the uniform rule, up to kKeepTiles tiles a block);
+//   k_keep, k_keep_write: in two launches (the spatial rule, its bits stored, and
+//     larger pieces, whose bits are computed again).
+// Both halves are bound by the hash's integer instructions (10 us for 8M points).
+// (In one launch with a look-back, all tiles of a wave publish at about the same
+// time and the last walks back over all of them: 38 us for 8M points, 25 us now,
+// and 880 us for the spatial pass over 10^8, 820 us now.)
+constexpr int kKeepSegs = 2048;
+constexpr int kKeepRows = 32, kKeepRowsCell = 8;   // rows per warp and tile
+
+struct KeepScratch {
+    uint32_t* words;      // spatial rule: keep bits, tile by tile, warp by warp, row by row
+    uint32_t* before;     // per tile: kept points of its segment before it
+    uint32_t* seg;        // per segment: kept points
+    uint64_t ntiles, per; // tiles, tiles per segment
+};
+
+// uniform rule: keep bits of ROWS rows of 32 indices from i (this lane's in the first), row r's in lane r
+template <int ROWS>
+FP_DEV uint32_t keep_word(uint64_t i, uint64_t n, uint64_t first, const KeepMultiple& mult)
 {
-    constexpr bool DECIM = KEEP != KEEP_NONE;
-    __shared__ uint32_t s_tile;
-    __shared__ uint32_t s_cnt[kBdIPT][kBdNT / 32];
-    __shared__ uint64_t s_base;
-    __shared__ int32_t s_red[6][kBdNT / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool pow2 = (modulus & (modulus - 1)) == 0;
-    const uint64_t mmask = (uint64_t)modulus - 1;
-
-    int32_t lo[3] = {INT32_MAX, INT32_MAX, INT32_MAX};
-    int32_t hi[3] = {INT32_MIN, INT32_MIN, INT32_MIN};
-    CubeDev cube;
-    if (KEEP == KEEP_CELL_MIN) cube = load_cube(cube_p);
-    const int csh = 3 * (kKeyLevels - level);
-
-    for (;;) {
-        if (threadIdx.x == 0) s_tile = atomicAdd(tile_counter, 1u);
-        __syncthreads();
-        const uint64_t tile = s_tile;
-        __syncthreads();
-        if (tile >= ntiles) break;
-        const uint64_t base = tile * kBdTile;
-
-        uint32_t keepmask = 0;   // bit r: item r of this thread kept
-        if (DECIM) {
-            // the keep decisions first (the uniform rule needs the index only), then publish
-#pragma unroll
-            for (int r = 0; r < kBdIPT; ++r) {
-                uint64_t i = base + (uint64_t)r * kBdNT + threadIdx.x;
-                bool k = false;
-                if (i < n) {
-                    uint64_t h = splitmix64(first + i);
-                    if (KEEP == KEEP_MODULUS) {
-                        k = pow2 ? (h & mmask) == 0 : (h % modulus) == 0;
-                    } else {
-                        const int4 q = ld_point(pts, i);
-                        k = cell_min[key21(q.x, q.y, q.z, cube) >> csh] == h;
-                    }
-                }
-                uint32_t bal = __ballot_sync(0xFFFFFFFFu, k);
-                if (lane == 0) s_cnt[r][warp] = __popc(bal);
-                keepmask |= (uint32_t)k << r;
-            }
-            __syncthreads();
-            // exclusive scan over (r, warp) order = index order
-            if (threadIdx.x < 32) {
-                uint32_t v[kBdIPT * (kBdNT / 32) / 32];   // 2 entries per lane
-                uint32_t s = 0;
-                constexpr int per = kBdIPT * (kBdNT / 32) / 32;
-#pragma unroll
-                for (int q = 0; q < per; ++q) {
-                    int e = lane * per + q;
-                    v[q] = s_cnt[e / (kBdNT / 32)][e % (kBdNT / 32)];
-                    s += v[q];
-                }
-                uint32_t x = s;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-                    if (lane >= o) x += y;
-                }
-                uint32_t total = __shfl_sync(0xFFFFFFFFu, x, 31);
-                uint32_t ex = x - s;
-#pragma unroll
-                for (int q = 0; q < per; ++q) {
-                    int e = lane * per + q;
-                    s_cnt[e / (kBdNT / 32)][e % (kBdNT / 32)] = ex;
-                    ex += v[q];
-                }
-                // decoupled look-back for the tile's global offset
-                if (lane == 0) {
-                    uint64_t excl = 0;
-                    if (tile == 0) {
-                        atomicExch((unsigned long long*)&tile_status[0], (unsigned long long)(kFlagInc | total));
-                    } else {
-                        atomicExch((unsigned long long*)&tile_status[tile], (unsigned long long)(kFlagAgg | total));
-                        int64_t t = (int64_t)tile - 1;
-                        uint32_t spins = 0;
-                        while (t >= 0) {
-                            uint64_t s2 = ld_volatile64(&tile_status[t]);
-                            if ((s2 >> 62) == 0) {
-                                if (++spins > kSpinLimit) { raise(err, FP_ERR_TIMEOUT); break; }
-                                continue;
-                            }
-                            excl += s2 & kValMask;
-                            if ((s2 >> 62) == 2) break;
-                            --t;
-                        }
-                        atomicExch((unsigned long long*)&tile_status[tile],
-                                   (unsigned long long)(kFlagInc | (excl + total)));
-                    }
-                    s_base = excl;
-                    if (tile == ntiles - 1) {
-                        *out_count = excl + total;
-                        if (excl + total > out_cap) raise(err, FP_ERR_CAPACITY, 0);
-                    }
-                }
-            }
-            __syncthreads();
-        }
-
-        if (BOUNDS) {
-#pragma unroll 4
-            for (int r = 0; r < kBdIPT; ++r) {
-                uint64_t i = base + (uint64_t)r * kBdNT + threadIdx.x;
-                if (i < n) {
-                    int4 p = ld_point_cs(pts, i);
-                    lo[0] = min(lo[0], p.x); hi[0] = max(hi[0], p.x);
-                    lo[1] = min(lo[1], p.y); hi[1] = max(hi[1], p.y);
-                    lo[2] = min(lo[2], p.z); hi[2] = max(hi[2], p.z);
-                }
-            }
-        }
-        if (DECIM) {
-            // second sweep for the writes (ballots need converged warps)
-#pragma unroll 4
-            for (int r = 0; r < kBdIPT; ++r) {
-                bool kept = (keepmask >> r) & 1u;
-                uint32_t bal = __ballot_sync(0xFFFFFFFFu, kept);
-                if (kept) {
-                    uint64_t i = base + (uint64_t)r * kBdNT + threadIdx.x;
-                    uint64_t pos = s_base + s_cnt[r][warp] + __popc(bal & lanemask_lt());
-                    if (pos < out_cap) st_point(out, pos, ld_point(pts, i));
-                }
-            }
-        }
-        __syncthreads();
+    uint32_t word = 0;
+    const uint32_t left = (uint32_t)min(n - min(n, i), (uint64_t)(32 * ROWS));   // rows reach n at 32 r >= left
+    const uint64_t v = first + i;
+#pragma unroll 8
+    for (int r = 0; r < ROWS; ++r) {
+        const uint32_t bal = __ballot_sync(0xFFFFFFFFu, mult(v + 32 * r) && 32u * r < left);
+        if ((int)(threadIdx.x & 31) == r) word = bal;
     }
+    return word;
+}
 
-    if (BOUNDS) {
+template <bool CELL_MIN, int ROWS>
+__global__ void __launch_bounds__(kBdNT) k_keep(const fp_point* __restrict__ pts, uint64_t n, uint64_t first,
+                                                KeepMultiple mult, KeepScratch s, const uint64_t* __restrict__ cell_min,
+                                                const fp_cube* cube_p, int level)
+{
+    constexpr int kWarps = kBdNT / 32;
+    __shared__ uint32_t s_tot[2][kWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    CubeDev cube;
+    float scale = 0.f;
+    if (CELL_MIN) {
+        cube = load_cube(cube_p);
+        scale = scale_at(cube, level);
+    }
+    const uint64_t t0 = blockIdx.x * s.per, t1 = min(s.ntiles, t0 + s.per);
+    uint32_t run = 0;
+    for (uint64_t tile = t0; tile < t1; ++tile) {
+        const uint64_t base = (tile * kWarps + warp) * (32 * ROWS) + lane;
+        uint32_t word = 0;
+        if (CELL_MIN) {
+            int4 q[ROWS];
+            uint64_t least[ROWS];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            for (int o = 16; o > 0; o >>= 1) {
-                lo[a] = min(lo[a], __shfl_xor_sync(0xFFFFFFFFu, lo[a], o));
-                hi[a] = max(hi[a], __shfl_xor_sync(0xFFFFFFFFu, hi[a], o));
+            for (int r = 0; r < ROWS; ++r)   // points, then minima, all in flight together
+                if (base + 32 * r < n) q[r] = ld_point_cs(pts, base + 32 * r);
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r)
+                if (base + 32 * r < n) least[r] = __ldcg(cell_min + key_small(q[r].x, q[r].y, q[r].z, cube, scale, level));
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r) {
+                const uint64_t i = base + 32 * r;
+                const uint32_t bal = __ballot_sync(0xFFFFFFFFu, i < n && least[r] == splitmix64(first + i));
+                if (lane == r) word = bal;
             }
+            if (lane < ROWS) s.words[(tile * kWarps + warp) * ROWS + lane] = word;
+        } else {
+            word = keep_word<ROWS>(base, n, first, mult);
         }
-        if (lane == 0) {
-            for (int a = 0; a < 3; ++a) { s_red[a][warp] = lo[a]; s_red[3 + a][warp] = hi[a]; }
-        }
+        const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, __popc(word));
+        uint32_t* tot = s_tot[(tile - t0) & 1];   // (two sets: one barrier a tile)
+        if (lane == 0) tot[warp] = total;
         __syncthreads();
-        if (threadIdx.x < 6) {
-            int a = threadIdx.x;
-            int32_t v = s_red[a][0];
-            for (int w = 1; w < kBdNT / 32; ++w) v = a < 3 ? min(v, s_red[a][w]) : max(v, s_red[a][w]);
-            partial[blockIdx.x * 6 + a] = v;
+        if (threadIdx.x == 0) s.before[tile] = run;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) run += tot[w];
+    }
+    if (threadIdx.x == 0) s.seg[blockIdx.x] = run;
+}
+
+template <bool CELL_MIN, int ROWS>
+__global__ void __launch_bounds__(kBdNT) k_keep_write(const fp_point* __restrict__ pts, uint64_t n, uint64_t first,
+                                                      KeepMultiple mult, KeepScratch s, uint32_t nseg,
+                                                      fp_point* __restrict__ out, uint64_t out_cap,
+                                                      uint64_t* __restrict__ out_count, uint32_t* err)
+{
+    constexpr int kWarps = kBdNT / 32;
+    __shared__ uint64_t s_sum[kWarps], s_all[kWarps];
+    __shared__ uint32_t s_tot[kWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint64_t tile = blockIdx.x;
+    const uint32_t g = (uint32_t)(tile / s.per);
+    const uint64_t w0 = (tile * kWarps + warp) * ROWS;
+    const uint32_t word = CELL_MIN ? (lane < ROWS ? s.words[w0 + lane] : 0u)
+                                   : keep_word<ROWS>(w0 * 32 + lane, n, first, mult);
+    uint64_t sum = 0, rest = 0;
+    for (uint32_t q = threadIdx.x; q < nseg; q += kBdNT) {
+        const uint32_t v = s.seg[q];
+        if (q < g) sum += v;
+        else rest += v;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+        rest += __shfl_xor_sync(0xFFFFFFFFu, rest, o);
+    }
+    uint32_t inc = __popc(word);
+#pragma unroll
+    for (int o = 1; o < ROWS; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    if (lane == 0) { s_sum[warp] = sum; s_all[warp] = sum + rest; }
+    if (lane == ROWS - 1) s_tot[warp] = inc;
+    __syncthreads();
+    uint64_t at = s.before[tile], all = 0;
+    for (int w = 0; w < kWarps; ++w) {
+        at += s_sum[w];
+        all += s_all[w];
+        if (w < warp) at += s_tot[w];
+    }
+    if (tile == 0 && threadIdx.x == 0) {
+        *out_count = all;
+        if (all > out_cap) raise(err, FP_ERR_CAPACITY, 0);
+    }
+    const uint32_t ex = inc - __popc(word);   // of row `lane`
+#pragma unroll 8
+    for (int r = 0; r < ROWS; ++r) {
+        const uint32_t bal = __shfl_sync(0xFFFFFFFFu, word, r);
+        const uint32_t rx = __shfl_sync(0xFFFFFFFFu, ex, r);
+        if ((bal >> lane) & 1u) {
+            const uint64_t pos = at + rx + __popc(bal & lanemask_lt());
+            if (pos < out_cap) st_point(out, pos, ld_point(pts, (w0 + r) * 32 + lane));
         }
     }
 }
@@ -398,7 +422,7 @@ constexpr size_t kBdBulkSmem = sizeof(int4) * kBdTile;
 
 template <bool DECIM>
 __global__ void __launch_bounds__(kBdNT) k_bounds_bulk(const fp_point* __restrict__ pts, uint64_t n, uint64_t first,
-                                                       uint32_t modulus, fp_point* __restrict__ out, uint64_t out_cap,
+                                                       KeepMultiple mult, fp_point* __restrict__ out, uint64_t out_cap,
                                                        uint64_t* __restrict__ out_count, int32_t* __restrict__ partial,
                                                        uint64_t* tile_status, uint32_t* tile_counter, uint64_t ntiles,
                                                        uint32_t* err)
@@ -437,7 +461,7 @@ __global__ void __launch_bounds__(kBdNT) k_bounds_bulk(const fp_point* __restric
 #pragma unroll
             for (int r = 0; r < kBdIPT; ++r) {
                 const uint64_t i = base + (uint64_t)r * kBdNT + threadIdx.x;
-                const bool k = i < n && keep_modulus(first, i, modulus);
+                const bool k = i < n && mult(first + i);
                 const uint32_t bal = __ballot_sync(0xFFFFFFFFu, k);
                 if (lane == 0) s_cnt[r][warp] = __popc(bal);
                 keepmask |= (uint32_t)k << r;
@@ -467,48 +491,8 @@ __global__ void __launch_bounds__(kBdNT) k_bounds_bulk(const fp_point* __restric
                     s_cnt[e / (kBdNT / 32)][e % (kBdNT / 32)] = ex;
                     ex += v[q];
                 }
-                // decoupled look-back by the whole warp: 32 earlier tiles' words per
-                // round trip; the sum runs back to the nearest inclusive prefix, and
-                // stops (and reads again) at the nearest word not yet published
-                uint64_t excl = 0;
-                if (tile == 0) {
-                    if (lane == 0)
-                        atomicExch((unsigned long long*)&tile_status[0], (unsigned long long)(kFlagInc | total));
-                } else {
-                    if (lane == 0)
-                        atomicExch((unsigned long long*)&tile_status[tile], (unsigned long long)(kFlagAgg | total));
-                    int64_t t = (int64_t)tile - 1;
-                    uint32_t spins = 0;
-                    while (t >= 0) {
-                        const int64_t q = t - lane;
-                        const uint64_t w = q >= 0 ? ld_volatile64(&tile_status[q]) : kFlagInc;
-                        const uint32_t inc = __ballot_sync(0xFFFFFFFFu, (w >> 62) == 2);
-                        const uint32_t none = __ballot_sync(0xFFFFFFFFu, (w >> 62) == 0);
-                        const int fi = inc ? __ffs(inc) - 1 : 32, fn = none ? __ffs(none) - 1 : 32;
-                        // lanes [0, take) are summed: up to the first unpublished word, or
-                        // through the first inclusive prefix, or all 32 aggregates
-                        const int take = fn < fi ? fn : (fi < 32 ? fi + 1 : 32);
-                        uint64_t v = lane < take ? (w & kValMask) : 0;
-                        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-                        excl += v;
-                        if (fi < fn) break;   // reached an inclusive prefix
-                        if (take == 0 && ++spins > kSpinLimit) {
-                            if (lane == 0) raise(err, FP_ERR_TIMEOUT);
-                            break;
-                        }
-                        t -= take;
-                    }
-                    if (lane == 0)
-                        atomicExch((unsigned long long*)&tile_status[tile],
-                                   (unsigned long long)(kFlagInc | (excl + total)));
-                }
-                if (lane == 0) {
-                    s_base = excl;
-                    if (tile == ntiles - 1) {
-                        *out_count = excl + total;
-                        if (excl + total > out_cap) raise(err, FP_ERR_CAPACITY, 0);
-                    }
-                }
+                const uint64_t excl = preview_base(tile_status, tile, ntiles, total, out_cap, out_count, err);
+                if (lane == 0) s_base = excl;
             }
         }
         // the tile's points have landed (bounded wait; on a time-out the copy is
@@ -559,44 +543,181 @@ __global__ void __launch_bounds__(kBdNT) k_bounds_bulk(const fp_point* __restric
 }
 
 // ----------------------------------------------------------------- host side
-// the carve of launch_bounds_decimate: block partials (grid <= 8 per SM), one
-// look-back word per tile, the tile counter
-size_t bounds_ws_bytes(uint64_t n, int num_sms)
+// the carve of the preview passes: block partials (grid <= 8 per SM), one
+// look-back word per tile and the tile counter behind them (cleared together)
+struct BoundsScratch {
+    int32_t* partial;
+    uint64_t* status;      // [ntiles], then the counter
+    uint32_t* counter;
+    uint64_t ntiles;       // of kBdTile points (the previews' larger tiles use fewer words)
+};
+
+static BoundsScratch bounds_carve(const Workspace& ws, uint64_t n, int num_sms)
 {
-    const size_t nt = (size_t)((n + kBdTile - 1) / kBdTile);
-    return Workspace::bytes_for({6 * 4 * (size_t)num_sms * 8, 8 * (nt ? nt : 1), 4 * sizeof(uint32_t)});
+    BoundsScratch b;
+    b.ntiles = (n + kBdTile - 1) / kBdTile;
+    b.partial = ws.take<int32_t>(6 * (size_t)num_sms * 8);
+    b.status = ws.take<uint64_t>(b.ntiles + 1);
+    b.counter = reinterpret_cast<uint32_t*>(b.status + b.ntiles);
+    return b;
+}
+
+size_t bounds_ws_bytes(uint64_t n, int num_sms)   // (the uniform preview's tile counts take less)
+{
+    Workspace dry;
+    bounds_carve(dry, n, num_sms);
+    return dry.used;
+}
+
+constexpr int kKeepTiles = 24;   // 1 KB of keep bits a tile, eight blocks per SM
+
+__global__ void __launch_bounds__(kBdNT, 8) k_keep_all(const fp_point* __restrict__ pts, uint64_t n, uint64_t first,
+                                                       KeepMultiple mult, KeepScratch s, uint32_t* bar,
+                                                       fp_point* __restrict__ out, uint64_t out_cap,
+                                                       uint64_t* __restrict__ out_count, uint32_t* err)
+{
+    constexpr int kWarps = kBdNT / 32, ROWS = kKeepRows;
+    extern __shared__ uint32_t s_words[];   // [tiles of the block][kWarps][32]
+    __shared__ uint32_t s_tot[kKeepTiles][kWarps];
+    __shared__ uint64_t s_sum[kWarps], s_all[kWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint64_t t0 = blockIdx.x * s.per, t1 = min(s.ntiles, t0 + s.per);
+    const int nt = (int)(t1 - t0);
+    for (int t = 0; t < nt; ++t) {
+        const uint32_t word = keep_word<ROWS>(((t0 + t) * kWarps + warp) * (32 * ROWS) + lane, n, first, mult);
+        s_words[(t * kWarps + warp) * 32 + lane] = word;
+        const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, __popc(word));
+        if (lane == 0) s_tot[t][warp] = total;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t run = 0;
+        for (int t = 0; t < nt; ++t)
+            for (int w = 0; w < kWarps; ++w) {   // kept points of the segment before the tile's warp
+                const uint32_t v = s_tot[t][w];
+                s_tot[t][w] = run;
+                run += v;
+            }
+        s.seg[blockIdx.x] = run;
+    }
+    if (!grid_barrier(bar, 1, err)) return;
+    uint64_t sum = 0, rest = 0;
+    for (uint32_t q = threadIdx.x; q < gridDim.x; q += kBdNT) {
+        const uint32_t v = s.seg[q];
+        if (q < blockIdx.x) sum += v;
+        else rest += v;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+        rest += __shfl_xor_sync(0xFFFFFFFFu, rest, o);
+    }
+    if (lane == 0) { s_sum[warp] = sum; s_all[warp] = sum + rest; }
+    __syncthreads();
+    uint64_t base = 0, all = 0;
+    for (int w = 0; w < kWarps; ++w) { base += s_sum[w]; all += s_all[w]; }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *out_count = all;
+        if (all > out_cap) raise(err, FP_ERR_CAPACITY, 0);
+    }
+    for (int t = 0; t < nt; ++t) {
+        const uint32_t word = s_words[(t * kWarps + warp) * 32 + lane];
+        uint32_t inc = __popc(word);
+#pragma unroll
+        for (int o = 1; o < ROWS; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        const uint64_t at = base + s_tot[t][warp];
+        const uint32_t ex = inc - __popc(word);
+        const uint64_t i0 = ((t0 + t) * kWarps + warp) * (32 * ROWS) + lane;
+#pragma unroll 8
+        for (int r = 0; r < ROWS; ++r) {
+            const uint32_t bal = __shfl_sync(0xFFFFFFFFu, word, r);
+            const uint32_t rx = __shfl_sync(0xFFFFFFFFu, ex, r);
+            if ((bal >> lane) & 1u) {
+                const uint64_t pos = at + rx + __popc(bal & lanemask_lt());
+                if (pos < out_cap) st_point(out, pos, ld_point(pts, i0 + 32 * r));
+            }
+        }
+    }
+}
+
+// the carve of the previews without extents
+static KeepScratch keep_carve(const Workspace& ws, uint64_t n, int rows, bool cell_min)
+{
+    KeepScratch s;
+    const uint64_t tile = (uint64_t)kBdNT * rows;
+    s.ntiles = (n + tile - 1) / tile;
+    s.per = std::max<uint64_t>(1, (s.ntiles + kKeepSegs - 1) / kKeepSegs);
+    s.words = cell_min ? ws.take<uint32_t>(s.ntiles * (tile / 32)) : nullptr;
+    s.before = ws.take<uint32_t>(s.ntiles);
+    s.seg = ws.take<uint32_t>(kKeepSegs);
+    return s;
+}
+
+static size_t keep_bytes(uint64_t n, int rows, bool cell_min)
+{
+    Workspace dry;
+    keep_carve(dry, n, rows, cell_min);
+    return dry.used;
+}
+
+template <bool CELL_MIN, int ROWS>
+static void keep_launch(const fp_point* pts, uint64_t n, uint64_t first, uint32_t modulus, fp_point* out,
+                        uint64_t out_cap, uint64_t* out_count, const uint64_t* cell_min, const fp_cube* cube,
+                        int level, const Workspace& ws, cudaStream_t st)
+{
+    const KeepScratch s = keep_carve(ws, n, ROWS, CELL_MIN);
+    const uint32_t nseg = (uint32_t)((s.ntiles + s.per - 1) / s.per);
+    k_keep<CELL_MIN, ROWS><<<nseg, kBdNT, 0, st>>>(pts, n, first, KeepMultiple::of(modulus), s, cell_min, cube, level);
+    k_keep_write<CELL_MIN, ROWS><<<(unsigned)s.ntiles, kBdNT, 0, st>>>(pts, n, first, KeepMultiple::of(modulus), s, nseg, out,
+                                                                       out_cap, out_count, ws.err);
 }
 
 cudaError_t launch_bounds_decimate(const fp_point* pts, uint64_t n, fp_cube* cube, bool bounds, bool decim,
                                    uint64_t first, uint32_t modulus, fp_point* out, uint64_t out_cap,
                                    uint64_t* out_count, const Workspace& ws, cudaStream_t st)
 {
-    uint64_t ntiles = (n + kBdTile - 1) / kBdTile;
-    int grid = (int)std::min<uint64_t>(ntiles ? ntiles : 1, (uint64_t)ws.num_sms * 8);
-    int32_t* partial = ws.take<int32_t>(6 * (size_t)grid);
-    uint64_t* status = ws.take<uint64_t>(ntiles ? ntiles : 1);
-    uint32_t* counter = ws.take<uint32_t>(4);
-    cudaError_t e = cudaMemsetAsync(counter, 0, 4 * sizeof(uint32_t), st);
-    if (e) return e;
-    if (decim && ntiles) {
-        e = cudaMemsetAsync(status, 0, ntiles * sizeof(uint64_t), st);
-        if (e) return e;
-    }
+    cudaError_t e;
     if (decim && n == 0) k_zero_count<<<1, 1, 0, st>>>(out_count);
-    if (n) {
+    if (!bounds) {
         KTimerScope kt(FP_KERNEL_BOUNDS_DECIMATE, st);
-        if (bounds) {   // points by bulk copy into shared memory
-            auto kern = decim ? k_bounds_bulk<true> : k_bounds_bulk<false>;
-            if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBdBulkSmem)))
-                return e;
-            kern<<<grid, kBdNT, kBdBulkSmem, st>>>(pts, n, first, modulus, out, out_cap, out_count, partial, status,
-                                                  counter, ntiles, ws.err);
-        } else
-            k_bounds_decimate<false, KEEP_MODULUS><<<grid, kBdNT, 0, st>>>(
-                pts, n, first, modulus, out, out_cap, out_count, partial, status, counter, ntiles, ws.err, nullptr,
-                nullptr, 0);
+        // 8192-point tiles; 2048-point ones while those leave SMs without a block
+        if (n == 0) return cudaGetLastError();
+        // 8192-point tiles, as many blocks as are resident; from four tiles an SM on (fewer leave most of the
+        // GPU without work: the two launches with 2048-point tiles then) up to kKeepTiles a block
+        KeepScratch s = keep_carve(ws, n, kKeepRows, false);
+        uint32_t* bar = ws.take<uint32_t>(1);
+        int per_sm = 0;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_keep_all, kBdNT, kKeepTiles * kBdNT * 4)))
+            return e;
+        const uint64_t blocks = std::min<uint64_t>((uint64_t)std::max(per_sm, 1) * ws.num_sms, kKeepSegs);
+        s.per = (s.ntiles + blocks - 1) / blocks;
+        if (s.ntiles >= (uint64_t)ws.num_sms * 4 && s.per <= (uint64_t)kKeepTiles) {
+            if ((e = cudaMemsetAsync(bar, 0, sizeof(uint32_t), st))) return e;
+            return coop_launch(k_keep_all, (unsigned)((s.ntiles + s.per - 1) / s.per), kBdNT, s.per * kBdNT * 4, st, pts, n,
+                               first, KeepMultiple::of(modulus), s, bar, out, out_cap, out_count, ws.err);
+        }
+        ws.used = 0;
+        if (s.ntiles >= (uint64_t)ws.num_sms * 4)
+            keep_launch<false, kKeepRows>(pts, n, first, modulus, out, out_cap, out_count, nullptr, nullptr, 0, ws, st);
+        else
+            keep_launch<false, kKeepRowsCell>(pts, n, first, modulus, out, out_cap, out_count, nullptr, nullptr, 0, ws, st);
+        return cudaGetLastError();
     }
-    if (bounds) k_bounds_final<<<1, 256, 0, st>>>(partial, n ? grid : 0, n, cube);
+    const BoundsScratch b = bounds_carve(ws, n, ws.num_sms);
+    const int grid = (int)std::min<uint64_t>(b.ntiles ? b.ntiles : 1, (uint64_t)ws.num_sms * 8);
+    if (n) {
+        if (decim) e = cudaMemsetAsync(b.status, 0, (b.ntiles + 1) * sizeof(uint64_t), st);
+        else e = cudaMemsetAsync(b.counter, 0, sizeof(uint32_t), st);
+        if (e) return e;
+        KTimerScope kt(FP_KERNEL_BOUNDS_DECIMATE, st);
+        auto kern = decim ? k_bounds_bulk<true> : k_bounds_bulk<false>;   // points by bulk copy into shared memory
+        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBdBulkSmem))) return e;
+        kern<<<grid, kBdNT, kBdBulkSmem, st>>>(pts, n, first, KeepMultiple::of(decim ? modulus : 1), out, out_cap, out_count,
+                                               b.partial, b.status, b.counter, b.ntiles, ws.err);
+    }
+    k_bounds_final<<<1, 256, 0, st>>>(b.partial, n ? grid : 0, n, cube);
     return cudaGetLastError();
 }
 
@@ -607,26 +728,44 @@ cudaError_t launch_bounds_decimate(const fp_point* pts, uint64_t n, fp_cube* cub
 // smallest splitmix64(first + i) is kept (a uniformly random point of the cell,
 // the same on every run).  Pass 1 takes each cell's smallest hash; pass 2 is
 // the preview compaction with "hash == its cell's smallest" as the keep rule.
+constexpr int kMinIPT = 4;
+
 __global__ void __launch_bounds__(256) k_cell_min_hash(const fp_point* __restrict__ pts, uint64_t n, uint64_t first,
                                                        const fp_cube* cube_p, int level,
                                                        unsigned long long* cell_min)
 {
     const CubeDev cube = load_cube(cube_p);
-    const int csh = 3 * (kKeyLevels - level);
+    const float scale = scale_at(cube, level);
     // a cell's running minimum only falls: a hash not below any value read for
     // it (however stale) cannot be the minimum, and the atomic is skipped --
     // in a cell of c points in random order about ln c atomics remain
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-        const int4 q = ld_point_cs(pts, i);
-        unsigned long long* slot = &cell_min[key21(q.x, q.y, q.z, cube) >> csh];
-        const unsigned long long h = splitmix64(first + i);
-        if (h < __ldcg(slot)) atomicMin(slot, h);
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += stride * kMinIPT) {
+        int4 q[kMinIPT];
+#pragma unroll
+        for (int u = 0; u < kMinIPT; ++u)   // points, then minima, all in flight together
+            if (i0 + u * stride < n) q[u] = ld_point_cs(pts, i0 + u * stride);
+        unsigned long long* slot[kMinIPT];
+        unsigned long long seen[kMinIPT];
+#pragma unroll
+        for (int u = 0; u < kMinIPT; ++u)
+            if (i0 + u * stride < n) {
+                slot[u] = &cell_min[key_small(q[u].x, q[u].y, q[u].z, cube, scale, level)];
+                seen[u] = __ldcg(slot[u]);
+            }
+#pragma unroll
+        for (int u = 0; u < kMinIPT; ++u)
+            if (i0 + u * stride < n) {
+                const unsigned long long h = splitmix64(first + i0 + u * stride);
+                if (h < seen[u]) atomicMin(slot[u], h);
+            }
     }
 }
 
 size_t spatial_ws_bytes(uint64_t n, int level, int num_sms)
 {
-    return Workspace::bytes_for({sizeof(uint64_t) << (3 * level)}) + bounds_ws_bytes(n, num_sms);
+    (void)num_sms;
+    return Workspace::bytes_for({sizeof(uint64_t) << (3 * level)}) + keep_bytes(n, kKeepRowsCell, true);
 }
 
 cudaError_t launch_preview_spatial(const fp_point* pts, uint64_t n, const fp_cube* cube, int level, uint64_t first,
@@ -635,24 +774,15 @@ cudaError_t launch_preview_spatial(const fp_point* pts, uint64_t n, const fp_cub
 {
     const uint64_t cells = 1ull << (3 * level);
     uint64_t* cell_min = ws.take<uint64_t>(cells);
-    uint64_t ntiles = (n + kBdTile - 1) / kBdTile;
-    int grid = (int)std::min<uint64_t>(ntiles ? ntiles : 1, (uint64_t)ws.num_sms * 8);
-    int32_t* partial = ws.take<int32_t>(6 * (size_t)grid);
-    uint64_t* status = ws.take<uint64_t>(ntiles ? ntiles : 1);
-    uint32_t* counter = ws.take<uint32_t>(4);
     cudaError_t e;
-    if ((e = cudaMemsetAsync(counter, 0, 4 * sizeof(uint32_t), st))) return e;
     if (n == 0) {
         k_zero_count<<<1, 1, 0, st>>>(out_count);
         return cudaGetLastError();
     }
-    if ((e = cudaMemsetAsync(status, 0, ntiles * sizeof(uint64_t), st))) return e;
     if ((e = cudaMemsetAsync(cell_min, 0xFF, cells * sizeof(uint64_t), st))) return e;
     const int gm = (int)std::min<uint64_t>((n + 255) / 256, (uint64_t)ws.num_sms * 8);
     k_cell_min_hash<<<gm, 256, 0, st>>>(pts, n, first, cube, level, reinterpret_cast<unsigned long long*>(cell_min));
-    k_bounds_decimate<false, KEEP_CELL_MIN><<<grid, kBdNT, 0, st>>>(pts, n, first, 1, out, out_cap, out_count, partial,
-                                                                    status, counter, ntiles, ws.err, cell_min, cube,
-                                                                    level);
+    keep_launch<true, kKeepRowsCell>(pts, n, first, 1, out, out_cap, out_count, cell_min, cube, level, ws, st);
     return cudaGetLastError();
 }
 

@@ -262,28 +262,6 @@ FP_DEV void open_node(const RoundArgs& a, int round, const OpenNode& node)
     }
 }
 
-// barrier number `k` (from 1) of the grid, every block of which is resident
-// (cooperative launch); false when the bounded wait ran out
-FP_DEV bool grid_barrier(uint32_t* word, uint32_t k, uint32_t* err)
-{
-    __shared__ int s_ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(word, 1u);
-        const uint32_t target = k * gridDim.x;
-        uint32_t spins = 0;
-        s_ok = 1;
-        while (ld_volatile(word) < target) {
-            if (++spins > (1u << 22)) { raise(err, FP_ERR_TIMEOUT); s_ok = 0; break; }
-            __nanosleep(64);
-        }
-        __threadfence();
-    }
-    __syncthreads();
-    return s_ok != 0;
-}
-
 struct RoundSmem {
     uint32_t h[kRoundNT], st[kRoundNT], mn[kRoundNT];   // per cell three levels down: count, start, smallest index
     uint32_t c2[64], m2[64], m1[8];
@@ -1923,17 +1901,9 @@ cudaError_t launch_octree_impl(const fp_point* sorted, const uint32_t* perm, uin
         KTimerScope kt(FP_KERNEL_SPLIT_ROUNDS, st);
         int per_sm = 0;
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rounds, kRoundNT, 0))) return e;
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3((unsigned)std::min<uint64_t>((N + kRoundTile - 1) / kRoundTile,
-                                                        (uint64_t)ws.num_sms * std::max(per_sm, 1)));
-        cfg.blockDim = dim3(kRoundNT);
-        cfg.stream = st;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeCooperative;   // its blocks wait for one another
-        at[0].val.cooperative = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        if ((e = cudaLaunchKernelEx(&cfg, k_rounds, ra))) return e;
+        const unsigned grid = (unsigned)std::min<uint64_t>((N + kRoundTile - 1) / kRoundTile,
+                                                           (uint64_t)ws.num_sms * std::max(per_sm, 1));
+        if ((e = coop_launch(k_rounds, grid, kRoundNT, 0, st, ra))) return e;
     }
     // 4. lambda of every record: owner level and leaf level
     {
