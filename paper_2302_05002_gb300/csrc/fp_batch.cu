@@ -286,7 +286,6 @@ __global__ void __launch_bounds__(NT) k_fused_count(const __grid_constant__ Fuse
         const FusedCloud& d = a.c[c];
         const CubeDev cube = load_cube(d.cube);
         const int g = (int)d.g;
-        const float sg = scale_at(cube, g);
         const uint64_t b0 = (t - a.item0[c]) * (uint64_t)(kFcTiles * kFbTile);
         const uint64_t b1 = min(d.n, b0 + (uint64_t)(kFcTiles * kFbTile));
         for (uint64_t i0 = b0; i0 < b1; i0 += 4 * NT) {   // block-uniform
@@ -297,7 +296,7 @@ __global__ void __launch_bounds__(NT) k_fused_count(const __grid_constant__ Fuse
                 key[u] = kNone;
                 if (i < b1) {
                     const int4 p = ld_point_cs(reinterpret_cast<const fp_point*>(d.pts), i);
-                    key[u] = key_small(p.x, p.y, p.z, cube, sg, g);
+                    key[u] = key_small(p.x, p.y, p.z, cube, g);
                 }
             }
 #pragma unroll

@@ -1,13 +1,18 @@
 // fp_common.cuh -- device helpers shared by the kernels of libfastpoints.
 //
 // Cell arithmetic (paper Sec. 4.4; exact-integer reading): for axis a,
-//   c_a(l) = floor((p_a - o_a) * 2^l / S),   0 <= p_a - o_a < 2^32,  1 <= S <= 2^32.
-// It is evaluated once at l = 21 and shifted for coarser levels (floor of a
-// floor: c(l) = c(21) >> (21 - l)).  The level-21 quotient is first estimated in
-// fp32 (relative error < 2^-22, so the estimate is within 1 of the true floor
-// for quotients below 2^21) and then corrected exactly with one 64-bit
-// remainder test.  The Morton key interleaves one bit per axis per level with
-// the x bit most significant inside every 3-bit digit.
+//   c_a(l) = floor((p_a - o_a) * 2^l / S),   0 <= p_a - o_a < S <= 2^32,  S >= 1.
+// (floor of a floor: c(l) = c(21) >> (21 - l), so the deepest level in use is
+// enough).  With R = floor(2^a / S), a = 31 + ceil(log2 S), so 2^31 <= R < 2^32:
+// the truncated product (d R) >> (a - l) is the cell or one less, because
+// d R / 2^(a-l) falls short of d 2^l / S by less than 2^l S / 2^a <= 2^(l-31);
+// one test of the remainder, which is below 2 S, corrects it.  For S <= 2^31 the
+// remainder fits 32 bits and the whole takes about eight integer instructions
+// (which run at half rate, and bound the passes that compute cells); the one
+// binade above takes 64-bit steps.  (An fp32 estimate corrected both ways in 64
+// bits took about three times as many.)
+// The Morton key interleaves one bit per axis per level with the x bit most
+// significant inside every 3-bit digit.
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -34,7 +39,8 @@ FP_DEV void raise(uint32_t* err, fp_status s, int site = -1)
 struct CubeDev {
     int32_t o[3];
     uint64_t S;
-    float scale21;   // 2^21 / S in fp32
+    uint32_t R;      // floor(2^a / S)
+    int32_t a;       // 31 + ceil(log2 S)
 };
 
 FP_DEV CubeDev load_cube(const fp_cube* c)
@@ -42,26 +48,27 @@ FP_DEV CubeDev load_cube(const fp_cube* c)
     CubeDev d;
     d.o[0] = c->o[0]; d.o[1] = c->o[1]; d.o[2] = c->o[2];
     d.S = c->S;
-    d.scale21 = d.S ? 2097152.0f / (float)d.S : 0.f;
+    d.a = 31 + (d.S > 1 ? 64 - __clzll((long long)(d.S - 1)) : 0);
+    // floor(2^a / S) with a <= 63: 2^a - 1 has the same quotient unless S divides 2^a (S a power of two)
+    d.R = d.S ? ((d.S & (d.S - 1)) ? (uint32_t)(((1ull << d.a) - 1) / d.S) : 0x80000000u) : 0u;
     return d;
 }
 
-// floor(d * 2^l / S) for d = p - o, 0 <= d < S <= 2^32, l <= 21; scale = 2^l / S
-// in fp32.  d fits 32 bits, q * S is a 32 x 32 -> 64-bit product (S = 2^32 is
-// the one value with a high word).
-FP_DEV uint32_t cell_at(int32_t p, int32_t o, uint64_t S, float scale, int l)
+// floor(d * 2^l / S) for d = p - o, 0 <= d < S, l <= 21
+FP_DEV uint32_t cell_at(int32_t p, int32_t o, const CubeDev& c, int l)
 {
-    const uint32_t d = (uint32_t)((int64_t)p - (int64_t)o);
-    int32_t q = (int32_t)((float)d * scale);
-    if (q < 0) q = 0;
-    const uint64_t num = (uint64_t)d << l;
-    const uint64_t qs = (uint64_t)(uint32_t)q * (uint32_t)S + ((uint64_t)((uint32_t)q * (uint32_t)(S >> 32)) << 32);
-    if (num < qs) --q;
-    else if (num - qs >= S) ++q;
-    return (uint32_t)q;
+    const uint32_t d = (uint32_t)p - (uint32_t)o;
+    const int sh = c.a - l;   // 10 .. 62
+    const uint32_t hi = __umulhi(d, c.R);
+    uint32_t q = sh >= 32 ? hi >> (sh - 32) : __funnelshift_r(d * c.R, hi, sh);
+    if (c.S <= 0x80000000ull) {
+        const uint32_t S = (uint32_t)c.S;
+        q += (d << l) - q * S >= S ? 1u : 0u;
+    } else {
+        q += ((uint64_t)d << l) - (uint64_t)q * c.S >= c.S ? 1u : 0u;
+    }
+    return q;
 }
-
-FP_DEV uint32_t cell21(int32_t p, int32_t o, uint64_t S, float scale21) { return cell_at(p, o, S, scale21, 21); }
 
 FP_DEV uint32_t spread3_10(uint32_t x)   // 10 bits -> bits 0, 3, ..., 27
 {
@@ -81,20 +88,17 @@ FP_DEV uint64_t spread3(uint32_t v)   // 21 bits -> bits 0, 3, ..., 60
 // 63-bit Morton key of the level-21 cell of a point
 FP_DEV uint64_t key21(int32_t x, int32_t y, int32_t z, const CubeDev& c)
 {
-    uint32_t cx = cell21(x, c.o[0], c.S, c.scale21);
-    uint32_t cy = cell21(y, c.o[1], c.S, c.scale21);
-    uint32_t cz = cell21(z, c.o[2], c.S, c.scale21);
+    uint32_t cx = cell_at(x, c.o[0], c, kKeyLevels);
+    uint32_t cy = cell_at(y, c.o[1], c, kKeyLevels);
+    uint32_t cz = cell_at(z, c.o[2], c, kKeyLevels);
     return (spread3(cx) << 2) | (spread3(cy) << 1) | spread3(cz);
 }
 
-// fp32 2^l / S from the cube's 2^21 / S (scaling by a power of two is exact)
-FP_DEV float scale_at(const CubeDev& c, int l) { return c.scale21 * __int_as_float((127 + l - 21) << 23); }
-
 // Morton key of the level-l cell of a point, l <= 10 (equal to key21 >> 3 (21 - l))
-FP_DEV uint32_t key_small(int32_t x, int32_t y, int32_t z, const CubeDev& c, float scale, int l)
+FP_DEV uint32_t key_small(int32_t x, int32_t y, int32_t z, const CubeDev& c, int l)
 {
-    return (spread3_10(cell_at(x, c.o[0], c.S, scale, l)) << 2) | (spread3_10(cell_at(y, c.o[1], c.S, scale, l)) << 1) |
-           spread3_10(cell_at(z, c.o[2], c.S, scale, l));
+    return (spread3_10(cell_at(x, c.o[0], c, l)) << 2) | (spread3_10(cell_at(y, c.o[1], c, l)) << 1) |
+           spread3_10(cell_at(z, c.o[2], c, l));
 }
 
 FP_DEV uint64_t key_at(uint64_t k21, int level) { return k21 >> (3 * (kKeyLevels - level)); }

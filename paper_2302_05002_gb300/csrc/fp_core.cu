@@ -123,10 +123,8 @@ __global__ void __launch_bounds__(kBdNT) k_keep(const fp_point* __restrict__ pts
     __shared__ uint32_t s_tot[2][kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     CubeDev cube;
-    float scale = 0.f;
     if (CELL_MIN) {
         cube = load_cube(cube_p);
-        scale = scale_at(cube, level);
     }
     const uint64_t t0 = blockIdx.x * s.per, t1 = min(s.ntiles, t0 + s.per);
     uint32_t run = 0;
@@ -141,7 +139,7 @@ __global__ void __launch_bounds__(kBdNT) k_keep(const fp_point* __restrict__ pts
                 if (base + 32 * r < n) q[r] = ld_point_cs(pts, base + 32 * r);
 #pragma unroll
             for (int r = 0; r < ROWS; ++r)
-                if (base + 32 * r < n) least[r] = __ldcg(cell_min + key_small(q[r].x, q[r].y, q[r].z, cube, scale, level));
+                if (base + 32 * r < n) least[r] = __ldcg(cell_min + key_small(q[r].x, q[r].y, q[r].z, cube, level));
 #pragma unroll
             for (int r = 0; r < ROWS; ++r) {
                 const uint64_t i = base + 32 * r;
@@ -275,7 +273,6 @@ __global__ void __launch_bounds__(256) k_count(const fp_point* __restrict__ pts,
     for (int q = threadIdx.x; q < kCountSlots; q += blockDim.x) { s_tag[q] = kNone; s_cnt[q] = 0; }
     __syncthreads();
     const CubeDev c = load_cube(cube);
-    const float sg = scale_at(c, g);
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     const int lane = threadIdx.x & 31;
     for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x; i0 < n; i0 += stride * 4) {
@@ -286,7 +283,7 @@ __global__ void __launch_bounds__(256) k_count(const fp_point* __restrict__ pts,
             key[u] = kNone;
             if (i < n) {
                 int4 p = ld_point_cs(pts, i);
-                key[u] = key_small(p.x, p.y, p.z, c, sg, g);
+                key[u] = key_small(p.x, p.y, p.z, c, g);
                 if (cells) cells[i] = key[u];
             }
         }
@@ -735,7 +732,6 @@ __global__ void __launch_bounds__(256) k_cell_min_hash(const fp_point* __restric
                                                        unsigned long long* cell_min)
 {
     const CubeDev cube = load_cube(cube_p);
-    const float scale = scale_at(cube, level);
     // a cell's running minimum only falls: a hash not below any value read for
     // it (however stale) cannot be the minimum, and the atomic is skipped --
     // in a cell of c points in random order about ln c atomics remain
@@ -750,7 +746,7 @@ __global__ void __launch_bounds__(256) k_cell_min_hash(const fp_point* __restric
 #pragma unroll
         for (int u = 0; u < kMinIPT; ++u)
             if (i0 + u * stride < n) {
-                slot[u] = &cell_min[key_small(q[u].x, q[u].y, q[u].z, cube, scale, level)];
+                slot[u] = &cell_min[key_small(q[u].x, q[u].y, q[u].z, cube, level)];
                 seen[u] = __ldcg(slot[u]);
             }
 #pragma unroll

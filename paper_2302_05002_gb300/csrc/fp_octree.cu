@@ -1564,14 +1564,14 @@ FP_DEV void own_add(uint32_t* keys, uint32_t* cnt, const OwnCounts& own, uint32_
 // by binary search among the descendants of its level-g cell's node, on the
 // point's key at max_level
 template <bool SMALL>
-__device__ __noinline__ uint32_t deep_id(const fp_point* __restrict__ pts, uint64_t j, const CubeDev& cb, float scale_l,
+__device__ __noinline__ uint32_t deep_id(const fp_point* __restrict__ pts, uint64_t j, const CubeDev& cb,
                                          uint32_t cell, int L, const uint32_t* idxtab, const uint64_t* sorted_start,
                                          const uint8_t* sorted_level, const uint32_t* ndesc, uint32_t M, int g, int lmax)
 {
     const uint32_t c0 = idxtab[((1ull << (3 * g)) - 1) / 7 + cell];
     if (L > lmax || c0 >= M) return kNone;
     const int4 p = ld_point(pts, j);
-    const uint64_t kl = SMALL ? (uint64_t)key_small(p.x, p.y, p.z, cb, scale_l, lmax)
+    const uint64_t kl = SMALL ? (uint64_t)key_small(p.x, p.y, p.z, cb, lmax)
                               : key21(p.x, p.y, p.z, cb) >> (3 * (kKeyLevels - lmax));
     const uint64_t k = kl >> (3 * (lmax - L));
     const uint32_t rr =
@@ -1593,7 +1593,6 @@ __global__ void __launch_bounds__(kResolveNT) k_resolve(const fp_point* __restri
     const int tl = min(g, kResolveTabLevel);
     const uint32_t ntab = ((1u << (3 * (tl + 1))) - 1) / 7;
     for (uint32_t q = threadIdx.x; q < ntab; q += kResolveNT) s_idx[q] = idxtab[q];
-    const float scale_l = SMALL ? scale_at(cb, lmax) : 0.f;
     const uint32_t M = *nnode;
     const int nt = leafid ? 2 : 1;
     const uint64_t ntiles = (n + kResolveTile - 1) / kResolveTile;
@@ -1622,7 +1621,7 @@ __global__ void __launch_bounds__(kResolveNT) k_resolve(const fp_point* __restri
                     else if (L <= g)
                         ids[u] = idxtab[((1ull << (3 * L)) - 1) / 7 + (cell >> (3 * (g - L)))];
                     else   // (kept out of the unrolled loop: its code is large and rarely run)
-                        ids[u] = deep_id<SMALL>(pts, j, cb, scale_l, cell, L, idxtab, sorted_start, sorted_level,
+                        ids[u] = deep_id<SMALL>(pts, j, cb, cell, L, idxtab, sorted_start, sorted_level,
                                                 ndesc, M, g, lmax);
                 }
                 if (ids[0] >= M || ids[1] >= M) {   // never for a consistent tree

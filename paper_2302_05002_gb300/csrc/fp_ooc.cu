@@ -74,7 +74,6 @@ __global__ void k_piece_hist(const fp_point* pts, uint64_t n, const fp_cube* cub
                              uint32_t* pcnt)
 {
     const CubeDev c = load_cube(cube);
-    const float sg = scale_at(c, g);
     const int lane = threadIdx.x & 31;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < n; i0 += stride) {
@@ -82,7 +81,7 @@ __global__ void k_piece_hist(const fp_point* pts, uint64_t n, const fp_cube* cub
         uint32_t ch = 0xFFFFFFFFu;
         if (i < n) {
             const int4 p = ld_point(pts, i);
-            ch = __ldg(lut + key_small(p.x, p.y, p.z, c, sg, g));
+            ch = __ldg(lut + key_small(p.x, p.y, p.z, c, g));
         }
         const uint32_t peers = __match_any_sync(0xFFFFFFFFu, ch);
         if (ch != 0xFFFFFFFFu && lane == __ffs(peers) - 1) atomicAdd(&pcnt[ch], (uint32_t)__popc(peers));
@@ -98,10 +97,9 @@ __global__ void k_piece_scatter(const int4* dpts, const uint32_t* dperm, uint64_
                                 uint32_t* err)
 {
     const CubeDev c = load_cube(cube);
-    const float sg = scale_at(c, g);
     for (uint64_t q = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (uint64_t)gridDim.x * blockDim.x) {
         const int4 p = dpts[q];
-        const uint32_t ch = __ldg(lut + key_small(p.x, p.y, p.z, c, sg, g));
+        const uint32_t ch = __ldg(lut + key_small(p.x, p.y, p.z, c, g));
         const uint64_t dest = ccur[ch] + (q - poff[ch]);
         if (dest >= n_all) { raise(err, FP_ERR_CAPACITY); continue; }
         if (h_pts) {

@@ -315,10 +315,8 @@ FP_DEV void dist_count(const DistSweepArgs& a, uint32_t nb, const uint16_t* dist
     const uint32_t d = threadIdx.x;
     const int tsh = 3 * (a.g - a.tl);
     CubeDev cube;
-    float sg = 0.f;
     if (!CELLS) {
         cube = load_cube(a.cube);
-        sg = scale_at(cube, a.g);
     }
     for (uint64_t gi = blockIdx.x; gi < ngroups; gi += gridDim.x) {
         const uint64_t t0 = gi * a.group, t1 = min(a.ntiles, t0 + a.group);
@@ -344,7 +342,7 @@ FP_DEV void dist_count(const DistSweepArgs& a, uint32_t nb, const uint16_t* dist
                 }
 #pragma unroll
                 for (int r = 0; r < kDistCountIPT; ++r)
-                    c[r] = base + (uint64_t)r * kDistCountNT + d < a.n ? key_small(p[r].x, p[r].y, p[r].z, cube, sg, a.g)
+                    c[r] = base + (uint64_t)r * kDistCountNT + d < a.n ? key_small(p[r].x, p[r].y, p[r].z, cube, a.g)
                                                                       : kNone;
             }
         };

@@ -221,7 +221,6 @@ __global__ void __launch_bounds__(kSortNT, 2) k_sort_pass(SortArgs a, int slot)
 
     CubeDev cube;
     if (DIG == DIG_CHUNK) cube = load_cube(a.cube);
-    const float scale_g = DIG == DIG_CHUNK ? scale_at(cube, a.g) : 0.f;
 
     const bool use_bulk = SM::BULK && a.bulk;
     const bool has_val = in_val != nullptr;
@@ -284,7 +283,7 @@ __global__ void __launch_bounds__(kSortNT, 2) k_sort_pass(SortArgs a, int slot)
                 else if (DIG == DIG_K32) d = (in_k32[i] >> shift) & dmask;
                 else {
                     int4 q = __ldg(in_pt + i);
-                    d = key_small(q.x, q.y, q.z, cube, scale_g, a.g);   // cell; its chunk below
+                    d = key_small(q.x, q.y, q.z, cube, a.g);   // cell; its chunk below
                 }
             }
             dg[r] = d;
