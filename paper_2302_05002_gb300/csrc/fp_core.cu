@@ -747,7 +747,7 @@ __global__ void __launch_bounds__(256) k_cell_min_hash(const fp_point* __restric
         for (int u = 0; u < kMinIPT; ++u)
             if (i0 + u * stride < n) {
                 slot[u] = &cell_min[key_small(q[u].x, q[u].y, q[u].z, cube, level)];
-                seen[u] = __ldcg(slot[u]);
+                seen[u] = *slot[u];   // (through L1: an SM's own atomics drop its stale line; 0.62 -> 0.54 ms at 10^8)
             }
 #pragma unroll
         for (int u = 0; u < kMinIPT; ++u)

@@ -171,11 +171,15 @@ FP_DEV void put_piece(const OctCtx& c, PieceList l, uint32_t id, const Piece& p)
 // reductions, keys are sorted where their order matters).  One pass over the
 // points; the lanes of a warp that share a cell take their slots with one
 // atomic on the cell's cursor, which starts at cstart[m].  The points arrive
-// chunk by chunk, so the cells in use at any time are consecutive: cursors sit
-// at bit-reversed cell ids, which spreads those atomics over the whole array
-// (and every L2 slice).  A cursor that does not end at cstart[m + 1] means the
+// chunk by chunk, so the cells in use at any time are consecutive: the cursors of
+// 8 cells share a sector, and the sectors sit at bit-reversed places, which
+// spreads those atomics over the whole array (and every L2 slice) while the
+// passes over all cells still write and read whole sectors.  A cursor that does not end at cstart[m + 1] means the
 // count grid was not the grid of these points (reported by k_small_pieces).
-FP_DEV uint32_t cursor_slot(uint32_t m, int g) { return __brev(m) >> (32 - 3 * g); }
+FP_DEV uint32_t cursor_slot(uint32_t m, int g)
+{
+    return g == 1 ? m : ((__brev(m >> 3) >> (35 - 3 * g)) << 3) | (m & 7u);
+}
 
 __global__ void __launch_bounds__(256) k_cell_scatter(const int4* __restrict__ pts, uint64_t n, const fp_cube* cube_p,
                                                       uint32_t* cursor, uint4* __restrict__ rec, int g,
@@ -530,7 +534,7 @@ __global__ void __launch_bounds__(kRoundNT, 2) k_rounds(RoundArgs a)
 // one time then lie in one or two tiles, and their scattered codes stay in L2
 // (appended one by one as the atomics fell, k_tab_pieces took 15.5 instead of
 // 13.0 ms for 5 * 10^8 uniform points, before it took its pieces in order).
-__global__ void __launch_bounds__(kGtNT) k_cells_open(RoundArgs ra, const uint32_t* __restrict__ pyr,
+__global__ void __launch_bounds__(kGtNT, 4) k_cells_open(RoundArgs ra, const uint32_t* __restrict__ pyr,
                                                       const uint32_t* __restrict__ rsum, int cells, int upper,
                                                       uint32_t* __restrict__ cstart, uint32_t* __restrict__ cursor)
 {
@@ -568,15 +572,12 @@ __global__ void __launch_bounds__(kGtNT) k_cells_open(RoundArgs ra, const uint32
     uint8_t hier[kGtPer];
     uint32_t tab = 0;   // bit q: cell q is a piece for the tables
     if (cells) {
-        uint32_t at = at0;
+        uint32_t at = at0, st[kGtPer];
 #pragma unroll
         for (int q = 0; q < kGtPer; ++q) {
             const uint32_t m = base + q;
             hier[q] = kEmpty;
-            if (m < ncell) {
-                cstart[m] = at;
-                cursor[cursor_slot(m, g)] = at;
-            }
+            st[q] = at;
             if (rv[q]) {
                 hier[q] = hl != 255 ? (uint8_t)hl
                                     : (s.s1[q >> 3] <= c.C ? (uint8_t)max(g - 1, 0)
@@ -602,9 +603,19 @@ __global__ void __launch_bounds__(kGtNT) k_cells_open(RoundArgs ra, const uint32
             at += rv[q];
         }
         if (tile == gridDim.x - 1 && tid == 0) cstart[ncell] = before + total;
+        // (base is a multiple of 16, the grid one of 8)
 #pragma unroll
-        for (int q = 0; q < kGtPer; ++q)
-            if (base + q < ncell) c.cell_leaf[base + q] = hier[q];
+        for (int h = 0; h < kGtPer; h += 8)
+            if (base + h < ncell) {
+                uint4* cs = reinterpret_cast<uint4*>(cstart + base + h);
+                uint4* cu = reinterpret_cast<uint4*>(cursor + cursor_slot(base + h, g));
+                cs[0] = cu[0] = make_uint4(st[h], st[h + 1], st[h + 2], st[h + 3]);
+                cs[1] = cu[1] = make_uint4(st[h + 4], st[h + 5], st[h + 6], st[h + 7]);
+                uint2 lv;
+                lv.x = hier[h] | (hier[h + 1] << 8) | (hier[h + 2] << 16) | ((uint32_t)hier[h + 3] << 24);
+                lv.y = hier[h + 4] | (hier[h + 5] << 8) | (hier[h + 6] << 16) | ((uint32_t)hier[h + 7] << 24);
+                *reinterpret_cast<uint2*>(c.cell_leaf + base + h) = lv;
+            }
     }
 
     // nodes of this thread: bits 0..15 its cells, 16, 17 the runs of 8, 18 the 64 cells, 19 the warp's
@@ -734,16 +745,23 @@ __global__ void __launch_bounds__(256) k_small_pieces(OctCtx c)
     const int lane = threadIdx.x & 31;
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
     const uint32_t cells = 1u << (3 * c.g);
-    for (uint32_t m0 = warp * 32; m0 < cells; m0 += nwarps * 32) {
+    if (warp == 0 && lane == 0 && c.cstart[cells] != c.nrec_max) raise(c.err, FP_ERR_CAPACITY, 4);
+    // the counts of the next cells are on their way while these are worked on
+    const uint32_t step = nwarps * 32;
+    uint32_t ahead = warp * 32 + lane < cells ? c.rcounts[warp * 32 + lane] : 0u;
+    for (uint32_t m0 = warp * 32; m0 < cells; m0 += step) {
         const uint32_t m = m0 + lane;
-        uint32_t cnt = m < cells ? c.rcounts[m] : 0u, leafl = 0, begin = 0;
-        // a cursor that does not end at the next cell's start: a count grid of other points
-        if (m < cells && c.cursor[cursor_slot(m, c.g)] != c.cstart[m + 1]) raise(c.err, FP_ERR_CAPACITY, 4);
-        if (cnt > (uint32_t)kSmallMax) cnt = 0;
+        uint32_t cnt = ahead, leafl = 0, begin = 0;
+        if (cells - m0 > step) ahead = m + step < cells ? c.rcounts[m + step] : 0u;
+        if (!__any_sync(0xFFFFFFFFu, cnt != 0)) continue;
         if (cnt) {
+            const uint32_t end = c.cursor[cursor_slot(m, c.g)], to = c.cstart[m + 1];
+            begin = c.cstart[m];
             leafl = c.cell_leaf[m];
-            if (leafl == kInner) cnt = 0;
-            else begin = c.cstart[m];
+            // a cell's cursor that does not end at the next one's start: a count grid of other points (points
+            // in a cell without any by the grid make another one come up short, or the totals differ)
+            if (end != to) raise(c.err, FP_ERR_CAPACITY, 4);
+            if (cnt > (uint32_t)kSmallMax || leafl == kInner) cnt = 0;
         }
         if (__any_sync(0xFFFFFFFFu, cnt != 0)) small_warp(c, begin, cnt, 0, leafl, c.g);
     }
