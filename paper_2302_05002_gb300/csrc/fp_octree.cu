@@ -528,137 +528,169 @@ __global__ void __launch_bounds__(kRoundNT, 2) k_rounds(RoundArgs a)
 // hierarchy ends at or above g, kInner if the cell's node is inner, kEmpty
 // without a record.  Cells with at most kPieceMax records become pieces
 // (k_small_pieces finds the smallest by itself); larger ones open the split
-// tree.  With `upper`: the nodes at levels <= g, each by the thread of its first
-// cell.  Pieces for the tables, nearly all of them on large clouds, and nodes are
-// appended with one atomic per tile, the pieces in cell order: those in work at
-// one time then lie in one or two tiles, and their scattered codes stay in L2
-// (appended one by one as the atomics fell, k_tab_pieces took 15.5 instead of
-// 13.0 ms for 5 * 10^8 uniform points, before it took its pieces in order).
-__global__ void __launch_bounds__(kGtNT, 4) k_cells_open(RoundArgs ra, const uint32_t* __restrict__ pyr,
-                                                      const uint32_t* __restrict__ rsum, int cells, int upper,
-                                                      uint32_t* __restrict__ cstart, uint32_t* __restrict__ cursor)
-{
-    const OctCtx& c = ra.c;
-    __shared__ GridTop top;
-    __shared__ uint32_t s_warp[kGtNT / 32], s_base[2];
-    const int g = c.g, tid = threadIdx.x;
-    const uint32_t ncell = 1u << (3 * g), tile = blockIdx.x, base = tile * kGtCells + tid * kGtPer;
-    uint32_t v[kGtPer], rv[kGtPer];
-    grid_load16(c.counts, base, ncell, v);
-    const GridSums s = grid_sums(v, s_warp);
-    const int up = grid_top(top, pyr, g, s.s4);
-    uint32_t before = 0;
-    for (uint32_t i = tid; i < tile; i += kGtNT) before += rsum[i];
-    before = block_sum(before, s_warp);
-    if (c.rcounts == c.counts) {
-#pragma unroll
-        for (int q = 0; q < kGtPer; ++q) rv[q] = v[q];
-    } else {
-        grid_load16(c.rcounts, base, ncell, rv);
-    }
-    uint32_t mine = 0;
-#pragma unroll
-    for (int q = 0; q < kGtPer; ++q) mine += rv[q];
-    uint32_t total;
-    const uint32_t at0 = before + block_exclusive_scan<kGtNT, uint32_t>(mine, s_warp, total);
+// tree.  With `upper`: the nodes at levels <= g.  The tile's counts, starts and
+// coarser sums go through shared memory, and the cells are taken 256 at a time in
+// one rolled loop each for the decisions and the appends (unrolled over a
+// thread's 16 cells the code overran the instruction cache, the top stall: 29 us
+// for the 2^21 cells of a cloud of 10^6 points, OPENUS now).  Pieces for the
+// tables, nearly all of them on large clouds, and nodes are appended with one
+// atomic per tile, the pieces in cell order: those in work at one time then lie
+// in one or two tiles, and their scattered codes stay in L2 (appended one by one
+// as the atomics fell, k_tab_pieces took 15.5 instead of 13.0 ms for 5 * 10^8
+// uniform points, before it took its pieces in order).
+struct OpenSmem {
+    uint32_t v[kGtCells], st[kGtCells];   // points (hierarchy) and start of every cell
+    uint32_t s1[kGtCells / 8], s2[kGtCells / 64], s3[kGtCells / 512];
+    uint32_t at[kGtPer][kGtNT / 32];      // appends before a warp's 32 cells: pieces | nodes << 16
+    GridTop top;
+    uint32_t warp[kGtNT / 32], base[2];
+};
 
-    // leaf level of the nodes around this thread's cells, down to the 64-cell one (255: all inner)
-    int hl = 255;
-    if (s.s2 <= c.C) hl = g - 2;
-    if (s.s3 <= c.C) hl = g - 3;
-    for (int a = 0; a <= up; ++a)
-        if (top.at(a, tile) <= c.C) hl = g - 4 - a;
-    if (hl < 0) hl = 0;   // (a grid of fewer than 4096 cells)
-    uint8_t hier[kGtPer];
-    uint32_t tab = 0;   // bit q: cell q is a piece for the tables
-    if (cells) {
-        uint32_t at = at0, st[kGtPer];
+__global__ void __launch_bounds__(kGtNT, 4) k_cells_open(RoundArgs ra, const uint32_t* __restrict__ pyr,
+                                                         const uint32_t* __restrict__ rsum, int cells, int upper,
+                                                         uint32_t* __restrict__ cstart, uint32_t* __restrict__ cursor)
+{
+    __shared__ OpenSmem S;
+    const OctCtx& c = ra.c;
+    const int g = c.g, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t ncell = 1u << (3 * g), tile = blockIdx.x, base = tile * kGtCells + tid * kGtPer;
+    const bool same = c.rcounts == c.counts;
+    uint32_t before = 0;
+    uint32_t s4;
+    {
+        uint32_t v[kGtPer];
+        grid_load16(c.counts, base, ncell, v);
+        const GridSums s = grid_sums(v, S.warp);
+        s4 = s.s4;
 #pragma unroll
-        for (int q = 0; q < kGtPer; ++q) {
-            const uint32_t m = base + q;
-            hier[q] = kEmpty;
-            st[q] = at;
-            if (rv[q]) {
-                hier[q] = hl != 255 ? (uint8_t)hl
-                                    : (s.s1[q >> 3] <= c.C ? (uint8_t)max(g - 1, 0)
-                                                           : (v[q] <= c.C || g == c.lmax ? (uint8_t)g : kInner));
-                if (rv[q] > (uint32_t)kPieceMax) {
+        for (int q = 0; q < kGtPer; q += 4)
+            *reinterpret_cast<uint4*>(&S.v[tid * kGtPer + q]) = make_uint4(v[q], v[q + 1], v[q + 2], v[q + 3]);
+        S.s1[2 * tid] = s.s1[0];
+        S.s1[2 * tid + 1] = s.s1[1];
+        if ((tid & 3) == 0) S.s2[tid >> 2] = s.s2;
+        if (lane == 0) S.s3[warp] = s.s3;
+        for (uint32_t i = tid; i < tile; i += kGtNT) before += rsum[i];
+        before = block_sum(before, S.warp);
+        if (!same) grid_load16(c.rcounts, base, ncell, v);
+        uint32_t mine = 0;
+#pragma unroll
+        for (int q = 0; q < kGtPer; ++q) mine += v[q];
+        uint32_t total;
+        uint32_t at = before + block_exclusive_scan<kGtNT, uint32_t>(mine, S.warp, total);
+#pragma unroll
+        for (int q = 0; q < kGtPer; ++q) { S.st[tid * kGtPer + q] = at; at += v[q]; }
+        if (cells && tile == gridDim.x - 1 && tid == 0) cstart[ncell] = before + total;
+        before += total;   // the end of the tile
+    }
+    const int up = grid_top(S.top, pyr, g, s4);   // (its barriers publish the arrays above)
+    int ht = 255;                                 // leaf level at or above the tile's node
+    for (int a = 0; a <= up; ++a)
+        if (S.top.at(a, tile) <= c.C) ht = max(g - 4 - a, 0);   // (a grid of fewer than 4096 cells: its root)
+    auto rcount = [&](uint32_t i) {   // records of cell i of the tile
+        return same ? S.v[i] : (i + 1 < (uint32_t)kGtCells ? S.st[i + 1] : before) - S.st[i];
+    };
+    auto leaf_of = [&](uint32_t i) -> uint8_t {
+        if (ht != 255) return (uint8_t)ht;
+        if (S.s3[i >> 9] <= c.C) return (uint8_t)max(g - 3, 0);
+        if (S.s2[i >> 6] <= c.C) return (uint8_t)max(g - 2, 0);
+        if (S.s1[i >> 3] <= c.C) return (uint8_t)max(g - 1, 0);
+        return S.v[i] <= c.C || g == c.lmax ? (uint8_t)g : kInner;
+    };
+    // nodes whose first cell is i: levels g, g - 1 (i a multiple of 8), g - 2 (64), g - 3 (512), g - 4 and above (0)
+    auto exists = [&](int L, uint32_t cnt, uint32_t parent) { return L >= 0 && cnt && (L == 0 || parent > c.C); };
+    auto node_mask = [&](uint32_t i) {
+        uint32_t f = 0;
+        if (exists(g, S.v[i], S.s1[i >> 3])) f |= 1u;
+        if ((i & 7) == 0 && exists(g - 1, S.s1[i >> 3], S.s2[i >> 6])) f |= 2u;
+        if ((i & 63) == 0 && exists(g - 2, S.s2[i >> 6], S.s3[i >> 9])) f |= 4u;
+        if ((i & 511) == 0 && exists(g - 3, S.s3[i >> 9], s4)) f |= 8u;
+        if (i == 0)
+            for (int a = 0; a <= up; ++a)
+                if ((tile & ((1u << (3 * a)) - 1)) == 0 &&
+                    exists(g - 4 - a, S.top.at(a, tile), a < up ? S.top.at(a + 1, tile) : 0u))
+                    f |= 16u << a;
+        return f;
+    };
+    const uint32_t in_tile = min((uint32_t)kGtCells, ncell);
+    uint32_t tab = 0;   // bit r: cell r * 256 + tid is a piece for the tables
+#pragma unroll 1
+    for (int r = 0; r < kGtPer; ++r) {
+        const uint32_t i = r * kGtNT + tid, m = tile * kGtCells + i;
+        const bool valid = i < in_tile;
+        const uint32_t n = valid ? rcount(i) : 0u;
+        uint8_t hier = kEmpty;
+        bool t = false;
+        if (cells && valid) {
+            const uint32_t at = S.st[i];
+            if (n) {
+                hier = leaf_of(i);
+                if (n > (uint32_t)kPieceMax) {
                     OpenNode o;
                     o.key = m;
                     o.begin = at;
-                    o.count = rv[q];
+                    o.count = n;
                     o.q = (uint8_t)g;
-                    o.hier = hier[q];
+                    o.hier = hier;
                     o.A = (uint8_t)g;
                     o.buf = 0;
                     o.tile0 = o.pad2 = o.pad3 = 0;
                     open_node(ra, 0, o);
                 } else {
-                    const PieceList l = piece_list(c, rv[q], g, hier[q]);
-                    if (l == LIST_TAB) tab |= 1u << q;
-                    else if (l == LIST_GEN)
-                        put_piece(c, l, atomicAdd(c.n[l], 1u), make_piece(at, rv[q], g, hier[q], (uint8_t)g, g, 0));
+                    const PieceList l = piece_list(c, n, g, hier);
+                    t = l == LIST_TAB;
+                    if (l == LIST_GEN)
+                        put_piece(c, l, atomicAdd(c.n[l], 1u), make_piece(at, n, g, hier, (uint8_t)g, g, 0));
                 }
             }
-            at += rv[q];
+            cstart[m] = at;
+            cursor[cursor_slot(m, g)] = at;
+            c.cell_leaf[m] = hier;
         }
-        if (tile == gridDim.x - 1 && tid == 0) cstart[ncell] = before + total;
-        // (base is a multiple of 16, the grid one of 8)
-#pragma unroll
-        for (int h = 0; h < kGtPer; h += 8)
-            if (base + h < ncell) {
-                uint4* cs = reinterpret_cast<uint4*>(cstart + base + h);
-                uint4* cu = reinterpret_cast<uint4*>(cursor + cursor_slot(base + h, g));
-                cs[0] = cu[0] = make_uint4(st[h], st[h + 1], st[h + 2], st[h + 3]);
-                cs[1] = cu[1] = make_uint4(st[h + 4], st[h + 5], st[h + 6], st[h + 7]);
-                uint2 lv;
-                lv.x = hier[h] | (hier[h + 1] << 8) | (hier[h + 2] << 16) | ((uint32_t)hier[h + 3] << 24);
-                lv.y = hier[h + 4] | (hier[h + 5] << 8) | (hier[h + 6] << 16) | ((uint32_t)hier[h + 7] << 24);
-                *reinterpret_cast<uint2*>(c.cell_leaf + base + h) = lv;
-            }
-    }
-
-    // nodes of this thread: bits 0..15 its cells, 16, 17 the runs of 8, 18 the 64 cells, 19 the warp's
-    // 512, 20 the tile, 20 + a the node a levels above it
-    auto exists = [&](int L, uint32_t cnt, uint32_t parent) { return L >= 0 && cnt && (L == 0 || parent > c.C); };
-    uint32_t nf = 0;
-    if (upper && base < ncell) {
-#pragma unroll
-        for (int q = 0; q < kGtPer; ++q)
-            if (base + q < ncell && exists(g, v[q], s.s1[q >> 3])) nf |= 1u << q;
-        if (exists(g - 1, s.s1[0], s.s2)) nf |= 1u << 16;
-        if (base + 8 < ncell && exists(g - 1, s.s1[1], s.s2)) nf |= 1u << 17;
-        if ((tid & 3) == 0 && exists(g - 2, s.s2, s.s3)) nf |= 1u << 18;
-        if ((tid & 31) == 0 && exists(g - 3, s.s3, s.s4)) nf |= 1u << 19;
-        if (tid == 0)
-            for (int a = 0; a <= up; ++a)
-                if ((tile & ((1u << (3 * a)) - 1)) == 0 &&
-                    exists(g - 4 - a, top.at(a, tile), a < up ? top.at(a + 1, tile) : 0u))
-                    nf |= 1u << (20 + a);
-    }
-    // both appends: one scan (tables in the low half, nodes in the high half: at most 5 * 4096 each)
-    const uint32_t ex = block_exclusive_scan<kGtNT, uint32_t>(__popc(tab) | (__popc(nf) << 16), s_warp, total);
-    if (tid == 0) {
-        s_base[0] = (total & 0xFFFFu) ? atomicAdd(c.n[LIST_TAB], total & 0xFFFFu) : 0u;
-        s_base[1] = (total >> 16) ? atomicAdd(c.nnode, total >> 16) : 0u;
+        const uint32_t nodes = upper && valid ? __popc(node_mask(i)) : 0u;
+        if (t) tab |= 1u << r;
+        const uint32_t sum = __reduce_add_sync(0xFFFFFFFFu, (t ? 1u : 0u) | (nodes << 16));
+        if (lane == 0) S.at[r][warp] = sum;
     }
     __syncthreads();
-    uint32_t pi = s_base[0] + (ex & 0xFFFFu), ni = s_base[1] + (ex >> 16), at = at0;
-#pragma unroll
-    for (int q = 0; q < kGtPer; ++q) {
-        if ((tab >> q) & 1u) {
-            put_piece(c, LIST_TAB, pi++, make_piece(at, rv[q], g, hier[q], (uint8_t)g, g, 0));
+    {   // the 128 runs of 32 cells in order; one atomic each for the tile's pieces and nodes
+        uint32_t* at = &S.at[0][0];
+        const uint32_t v = tid < kGtPer * (kGtNT / 32) ? at[tid] : 0u;
+        uint32_t total;
+        const uint32_t ex = block_exclusive_scan<kGtNT, uint32_t>(v, S.warp, total);
+        if (tid < kGtPer * (kGtNT / 32)) at[tid] = ex;
+        if (tid == 0) {
+            S.base[0] = (total & 0xFFFFu) ? atomicAdd(c.n[LIST_TAB], total & 0xFFFFu) : 0u;
+            S.base[1] = (total >> 16) ? atomicAdd(c.nnode, total >> 16) : 0u;
         }
-        if ((nf >> q) & 1u) put_node(c, ni++, base + q, g, v[q], at, v[q] <= c.C || g == c.lmax);
-        if (q == 7 && ((nf >> 17) & 1u)) put_node(c, ni++, (base >> 3) + 1, g - 1, s.s1[1], at + rv[7], s.s1[1] <= c.C);
-        at += rv[q];
+        __syncthreads();
+        if (total == 0) return;
     }
-    if ((nf >> 16) & 1u) put_node(c, ni++, base >> 3, g - 1, s.s1[0], at0, s.s1[0] <= c.C);
-    if ((nf >> 18) & 1u) put_node(c, ni++, base >> 6, g - 2, s.s2, at0, s.s2 <= c.C);
-    if ((nf >> 19) & 1u) put_node(c, ni++, base >> 9, g - 3, s.s3, at0, s.s3 <= c.C);
-    for (int a = 0; a <= up; ++a)
-        if ((nf >> (20 + a)) & 1u)
-            put_node(c, ni++, tile >> (3 * a), g - 4 - a, top.at(a, tile), at0, top.at(a, tile) <= c.C);
+#pragma unroll 1
+    for (int r = 0; r < kGtPer; ++r) {
+        const uint32_t i = r * kGtNT + tid, m = tile * kGtCells + i;
+        const bool t = (tab >> r) & 1u;
+        const uint32_t f = upper && i < in_tile ? node_mask(i) : 0u;
+        const uint32_t mine = (t ? 1u : 0u) | ((uint32_t)__popc(f) << 16);
+        if (!__any_sync(0xFFFFFFFFu, mine != 0)) continue;
+        uint32_t inc = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        const uint32_t ex = S.at[r][warp] + inc - mine, at = i < in_tile ? S.st[i] : 0u;
+        if (t)
+            put_piece(c, LIST_TAB, S.base[0] + (ex & 0xFFFFu), make_piece(at, rcount(i), g, leaf_of(i), (uint8_t)g, g, 0));
+        uint32_t ni = S.base[1] + (ex >> 16);
+#pragma unroll 1
+        for (uint32_t todo = f; todo; todo &= todo - 1) {
+            const int k = __ffs(todo) - 1;   // levels above the cell
+            const int lev = g - k;
+            const uint32_t cnt = k == 0 ? S.v[i] : (k == 1 ? S.s1[i >> 3] : (k == 2 ? S.s2[i >> 6] : (k == 3 ? S.s3[i >> 9]
+                                                                                                   : S.top.at(k - 4, tile))));
+            put_node(c, ni++, m >> (3 * k), lev, cnt, at, cnt <= c.C || lev == c.lmax);
+        }
+    }
 }
 
 // ------------------------------------------------------------ pieces
@@ -696,39 +728,50 @@ FP_DEV void put_lambda(const OctCtx& c, uint32_t jj, int lambda, int leafl, uint
     else raise(c.err, FP_ERR_CAPACITY, 17);
 }
 
-// The points of up to 32 small pieces, one piece per lane (cnt 0: none), spread
-// over the lanes of the warp one record each: lambda is one more than the
-// deepest level shared with any point of smaller index in the piece (every pair
-// of the piece; its records are a few consecutive words, read through L1).
-FP_DEV void small_warp(const OctCtx& c, uint32_t begin, uint32_t cnt, uint32_t buf, uint32_t leafl, uint32_t A)
+// The points of up to 64 small pieces, two neighbouring ones per lane (cnt 0:
+// none), spread over the lanes of the warp one record each: lambda is one more
+// than the deepest level shared with any point of smaller index in the piece
+// (every pair of the piece; its records are a few consecutive words, read
+// through L1).
+struct SmallPiece {
+    uint32_t begin, cnt, what;   // what: record buffer | leaf level << 8 | first-min level << 16
+};
+
+FP_DEV void small_warp(const OctCtx& c, SmallPiece a, SmallPiece b)
 {
     const int lane = threadIdx.x & 31;
-    if ((uint64_t)begin + cnt > c.nrec_max) { raise(c.err, FP_ERR_CAPACITY, 18); cnt = 0; }
-    uint32_t inc = cnt;
+    if ((uint64_t)a.begin + a.cnt > c.nrec_max || (uint64_t)b.begin + b.cnt > c.nrec_max) {
+        raise(c.err, FP_ERR_CAPACITY, 18);
+        a.cnt = b.cnt = 0;
+    }
+    uint32_t inc = a.cnt + b.cnt;
     for (int o = 1; o < 32; o <<= 1) {
         const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
         if (lane >= o) inc += y;
     }
     const uint32_t total = __shfl_sync(0xFFFFFFFFu, inc, 31);
-    const uint32_t what = buf | (leafl << 8) | (A << 16);
+    const uint32_t counts = a.cnt | (b.cnt << 16);
     for (uint32_t r0 = 0; r0 < total; r0 += 32) {
         const uint32_t r = r0 + lane;
         int o = 0;   // lanes whose pieces end at or before r
 #pragma unroll
-        for (int b = 16; b > 0; b >>= 1)
-            if (__shfl_sync(0xFFFFFFFFu, inc, (o + b - 1) & 31) <= r) o += b;
+        for (int s = 16; s > 0; s >>= 1)
+            if (__shfl_sync(0xFFFFFFFFu, inc, (o + s - 1) & 31) <= r) o += s;
         o &= 31;
-        const uint32_t w = __shfl_sync(0xFFFFFFFFu, what, o);
-        const uint32_t cn = __shfl_sync(0xFFFFFFFFu, cnt, o);
-        const uint32_t b0 = __shfl_sync(0xFFFFFFFFu, begin, o);
-        const uint32_t at = b0 + r - (__shfl_sync(0xFFFFFFFFu, inc, o) - cn);
+        const uint32_t cc = __shfl_sync(0xFFFFFFFFu, counts, o);
+        const uint32_t ca = cc & 0xFFFFu, cb = cc >> 16;
+        const uint32_t k0 = r - (__shfl_sync(0xFFFFFFFFu, inc, o) - ca - cb);   // place in the lane's two pieces
+        const bool second = k0 >= ca;
+        const uint32_t ba = __shfl_sync(0xFFFFFFFFu, a.begin, o), bb = __shfl_sync(0xFFFFFFFFu, b.begin, o);
+        const uint32_t wa = __shfl_sync(0xFFFFFFFFu, a.what, o), wb = __shfl_sync(0xFFFFFFFFu, b.what, o);
         if (r >= total) continue;   // (no shuffle below)
-        const uint4* rec = c.recs[w & 1u];
-        const uint4 me = rec[at];
+        const uint32_t w = second ? wb : wa, cn = second ? cb : ca;
+        const uint4* rec = c.recs[w & 1u] + (second ? bb : ba);
+        const uint4 me = rec[second ? k0 - ca : k0];
         const uint64_t k = rec_key(me);
         uint64_t near = ~0ull;   // smallest key difference to a smaller index: the deepest shared level
         for (uint32_t t = 0; t < cn; ++t) {
-            const uint4 other = rec[b0 + t];
+            const uint4 other = rec[t];
             const uint64_t x = rec_key(other) ^ k;
             if (other.z < me.z && x < near) near = x;
         }
@@ -738,38 +781,48 @@ FP_DEV void small_warp(const OctCtx& c, uint32_t begin, uint32_t cnt, uint32_t b
     }
 }
 
-// level-g cells of 1 .. kSmallMax points (not inner), one cell per lane, then the
+// level-g cells of 1 .. kSmallMax points (not inner), two cells per lane, then the
 // small pieces of the split rounds
 __global__ void __launch_bounds__(256) k_small_pieces(OctCtx c)
 {
     const int lane = threadIdx.x & 31;
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
-    const uint32_t cells = 1u << (3 * c.g);
+    const uint32_t cells = 1u << (3 * c.g);   // (a multiple of 8)
     if (warp == 0 && lane == 0 && c.cstart[cells] != c.nrec_max) raise(c.err, FP_ERR_CAPACITY, 4);
     // the counts of the next cells are on their way while these are worked on
-    const uint32_t step = nwarps * 32;
-    uint32_t ahead = warp * 32 + lane < cells ? c.rcounts[warp * 32 + lane] : 0u;
-    for (uint32_t m0 = warp * 32; m0 < cells; m0 += step) {
-        const uint32_t m = m0 + lane;
-        uint32_t cnt = ahead, leafl = 0, begin = 0;
-        if (cells - m0 > step) ahead = m + step < cells ? c.rcounts[m + step] : 0u;
-        if (!__any_sync(0xFFFFFFFFu, cnt != 0)) continue;
-        if (cnt) {
-            const uint32_t end = c.cursor[cursor_slot(m, c.g)], to = c.cstart[m + 1];
-            begin = c.cstart[m];
-            leafl = c.cell_leaf[m];
+    const uint32_t step = nwarps * 64;
+    auto load = [&](uint32_t m) {
+        return m < cells ? make_uint2(c.rcounts[m], c.rcounts[m + 1]) : make_uint2(0u, 0u);
+    };
+    uint2 ahead = load(warp * 64 + 2 * lane);
+    for (uint32_t m0 = warp * 64; m0 < cells; m0 += step) {
+        const uint32_t m = m0 + 2 * lane;
+        const uint2 n = ahead;
+        if (cells - m0 > step) ahead = load(m + step);
+        if (!__any_sync(0xFFFFFFFFu, (n.x | n.y) != 0)) continue;
+        SmallPiece a{0u, 0u, 0u}, b{0u, 0u, 0u};
+        if (n.x | n.y) {
+            const uint2 end = *reinterpret_cast<const uint2*>(c.cursor + cursor_slot(m, c.g));
+            const uint2 st = *reinterpret_cast<const uint2*>(c.cstart + m);
+            const uint32_t to = c.cstart[m + 2];
+            const uint32_t leaf = *reinterpret_cast<const uint16_t*>(c.cell_leaf + m);
             // a cell's cursor that does not end at the next one's start: a count grid of other points (points
             // in a cell without any by the grid make another one come up short, or the totals differ)
-            if (end != to) raise(c.err, FP_ERR_CAPACITY, 4);
-            if (cnt > (uint32_t)kSmallMax || leafl == kInner) cnt = 0;
+            if ((n.x && end.x != st.y) || (n.y && end.y != to)) raise(c.err, FP_ERR_CAPACITY, 4);
+            const uint32_t la = leaf & 255u, lb = leaf >> 8;
+            if (n.x <= (uint32_t)kSmallMax && la != kInner) a = SmallPiece{st.x, n.x, (la << 8) | ((uint32_t)c.g << 16)};
+            if (n.y <= (uint32_t)kSmallMax && lb != kInner) b = SmallPiece{st.y, n.y, (lb << 8) | ((uint32_t)c.g << 16)};
         }
-        if (__any_sync(0xFFFFFFFFu, cnt != 0)) small_warp(c, begin, cnt, 0, leafl, c.g);
+        if (__any_sync(0xFFFFFFFFu, (a.cnt | b.cnt) != 0)) small_warp(c, a, b);
     }
     const uint32_t ns = min(*c.n[LIST_SMALL], c.piece_cap);
     for (uint32_t p0 = warp * 32; p0 < ns; p0 += nwarps * 32) {
-        Piece p{};
-        if (p0 + lane < ns) p = c.list[LIST_SMALL][p0 + lane];
-        small_warp(c, p.begin, p.count, p.buf, p.hier, p.A);
+        SmallPiece a{0u, 0u, 0u};
+        if (p0 + lane < ns) {
+            const Piece p = c.list[LIST_SMALL][p0 + lane];
+            a = SmallPiece{p.begin, p.count, (uint32_t)p.buf | ((uint32_t)p.hier << 8) | ((uint32_t)p.A << 16)};
+        }
+        small_warp(c, a, SmallPiece{0u, 0u, 0u});
     }
 }
 
