@@ -598,12 +598,15 @@ __global__ void __launch_bounds__(kGtNT, 4) k_cells_open(RoundArgs ra, const uin
     };
     // nodes whose first cell is i: levels g, g - 1 (i a multiple of 8), g - 2 (64), g - 3 (512), g - 4 and above (0)
     auto exists = [&](int L, uint32_t cnt, uint32_t parent) { return L >= 0 && cnt && (L == 0 || parent > c.C); };
+    const bool below = s4 > c.C || g <= 4;   // nodes below the tile's
     auto node_mask = [&](uint32_t i) {
         uint32_t f = 0;
-        if (exists(g, S.v[i], S.s1[i >> 3])) f |= 1u;
-        if ((i & 7) == 0 && exists(g - 1, S.s1[i >> 3], S.s2[i >> 6])) f |= 2u;
-        if ((i & 63) == 0 && exists(g - 2, S.s2[i >> 6], S.s3[i >> 9])) f |= 4u;
-        if ((i & 511) == 0 && exists(g - 3, S.s3[i >> 9], s4)) f |= 8u;
+        if (below) {
+            if (exists(g, S.v[i], S.s1[i >> 3])) f |= 1u;
+            if ((i & 7) == 0 && exists(g - 1, S.s1[i >> 3], S.s2[i >> 6])) f |= 2u;
+            if ((i & 63) == 0 && exists(g - 2, S.s2[i >> 6], S.s3[i >> 9])) f |= 4u;
+            if ((i & 511) == 0 && exists(g - 3, S.s3[i >> 9], s4)) f |= 8u;
+        }
         if (i == 0)
             for (int a = 0; a <= up; ++a)
                 if ((tile & ((1u << (3 * a)) - 1)) == 0 &&
@@ -770,10 +773,15 @@ FP_DEV void small_warp(const OctCtx& c, SmallPiece a, SmallPiece b)
         const uint4 me = rec[second ? k0 - ca : k0];
         const uint64_t k = rec_key(me);
         uint64_t near = ~0ull;   // smallest key difference to a smaller index: the deepest shared level
-        for (uint32_t t = 0; t < cn; ++t) {
-            const uint4 other = rec[t];
-            const uint64_t x = rec_key(other) ^ k;
-            if (other.z < me.z && x < near) near = x;
+        for (uint32_t t = 0; t < cn; t += 4) {   // four loads in flight (the last record again beyond the end)
+            uint4 other[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) other[u] = rec[min(t + u, cn - 1)];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const uint64_t x = rec_key(other[u]) ^ k;
+                if (other[u].z < me.z && x < near) near = x;
+            }
         }
         int lambda = (int)(w >> 16);   // the piece minimum: from the split tree
         if (near != ~0ull) lambda = (near == 0 ? kKeyLevels : (__clzll((long long)near) - 1) / 3) + 1;
@@ -816,10 +824,12 @@ __global__ void __launch_bounds__(256) k_small_pieces(OctCtx c)
         if (__any_sync(0xFFFFFFFFu, (a.cnt | b.cnt) != 0)) small_warp(c, a, b);
     }
     const uint32_t ns = min(*c.n[LIST_SMALL], c.piece_cap);
-    for (uint32_t p0 = warp * 32; p0 < ns; p0 += nwarps * 32) {
+    // spread over the warps (32 pieces in a row kept a few warps busy for 40 us after the others)
+    for (uint64_t p0 = warp; p0 < ns; p0 += 32ull * nwarps) {
         SmallPiece a{0u, 0u, 0u};
-        if (p0 + lane < ns) {
-            const Piece p = c.list[LIST_SMALL][p0 + lane];
+        const uint64_t at = p0 + (uint64_t)lane * nwarps;
+        if (at < ns) {
+            const Piece p = c.list[LIST_SMALL][at];
             a = SmallPiece{p.begin, p.count, (uint32_t)p.buf | ((uint32_t)p.hier << 8) | ((uint32_t)p.A << 16)};
         }
         small_warp(c, a, SmallPiece{0u, 0u, 0u});
