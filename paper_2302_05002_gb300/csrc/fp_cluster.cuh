@@ -79,6 +79,69 @@ FP_DEV bool grid_barrier(uint32_t* word, uint32_t k, uint32_t* err)
     return s_ok != 0;
 }
 
+// One pass of a stable sort of n records by an 8-bit digit: digit(i) of record i,
+// put(i, at) moves it to place `at`.  Every CTA counts the digits of its slice,
+// all CTAs' counts (hist: kClCtas * 256 words) give every digit's base, and each
+// tile of 1024 records is ranked by ballots.  All threads of the cluster.
+struct ClSortSmem {
+    uint32_t whist[kClNT / 32][256];
+    uint32_t cnt[256], base[256], warp[32];
+};
+
+template <typename Digit, typename Put>
+FP_DEV void cl_sort_pass(uint32_t n, ClSortSmem& S, uint32_t* hist, Digit digit, Put put)
+{
+    const uint32_t rank = cl_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t per = (n + kClCtas - 1) / kClCtas, lo = min(n, rank * per), hi = min(n, lo + per);
+    if (tid < 256) S.cnt[tid] = 0;
+    __syncthreads();
+    for (uint32_t i0 = lo; i0 < hi; i0 += kClNT) {
+        const uint32_t i = i0 + tid;
+        const uint32_t d = i < hi ? digit(i) : 0u;
+        const uint32_t peers = match_bits<8>(d, i < hi);
+        if (i < hi && lane == (uint32_t)__ffs(peers) - 1) atomicAdd(&S.cnt[d], (uint32_t)__popc(peers));
+    }
+    __syncthreads();
+    if (tid < 256) hist[rank * 256 + tid] = S.cnt[tid];
+    cl_sync();
+    {
+        uint32_t before = 0, total = 0;
+        if (tid < 256)
+            for (int r = 0; r < kClCtas; ++r) {
+                const uint32_t v = ld_volatile(hist + r * 256 + tid);
+                if (r < (int)rank) before += v;
+                total += v;
+            }
+        uint32_t all;
+        const uint32_t ex = block_exclusive_scan<kClNT, uint32_t>(total, S.warp, all);
+        if (tid < 256) S.base[tid] = ex + before;
+    }
+    for (uint32_t i0 = lo; i0 < hi; i0 += kClNT) {
+        for (uint32_t q = tid; q < (kClNT / 32) * 256 / 4; q += kClNT)
+            reinterpret_cast<uint4*>(&S.whist[0][0])[q] = make_uint4(0, 0, 0, 0);
+        __syncthreads();
+        const uint32_t i = i0 + tid;
+        const bool valid = i < hi;
+        const uint32_t d = valid ? digit(i) : 0u;
+        const uint32_t peers = match_bits<8>(d, valid);
+        if (valid && lane == (uint32_t)__ffs(peers) - 1) S.whist[warp][d] = __popc(peers);
+        __syncthreads();
+        if (tid < 256) {
+            uint32_t run = S.base[tid];
+            for (int w = 0; w < kClNT / 32; ++w) {
+                const uint32_t c = S.whist[w][tid];
+                S.whist[w][tid] = run;
+                run += c;
+            }
+            S.base[tid] = run;
+        }
+        __syncthreads();
+        if (valid) put(i, S.whist[warp][d] + __popc(peers & lanemask_lt()));
+        __syncthreads();
+    }
+    cl_sync();
+}
+
 // cooperative launch (all blocks resident, so that they may wait for one another)
 template <typename... Params, typename... Args>
 inline cudaError_t coop_launch(void (*kernel)(Params...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,

@@ -532,7 +532,7 @@ __global__ void __launch_bounds__(kRoundNT, 2) k_rounds(RoundArgs a)
 // coarser sums go through shared memory, and the cells are taken 256 at a time in
 // one rolled loop each for the decisions and the appends (unrolled over a
 // thread's 16 cells the code overran the instruction cache, the top stall: 29 us
-// for the 2^21 cells of a cloud of 10^6 points, OPENUS now).  Pieces for the
+// for the 2^21 cells of a cloud of 10^6 points, 20 us now).  Pieces for the
 // tables, nearly all of them on large clouds, and nodes are appended with one
 // atomic per tile, the pieces in cell order: those in work at one time then lie
 // in one or two tiles, and their scattered codes stay in L2 (appended one by one
@@ -1430,10 +1430,9 @@ __global__ void k_node_children(const uint32_t* nnode, const uint64_t* sorted_st
 
 // The node table in one launch of one cluster, for at most kNodeClusterMax nodes
 // by the host's bound (28 launches otherwise; 1M points: about 110 -> 19 us).  Stable
-// least-significant-digit-first passes over (level, start): every CTA counts the
-// digits of its slice, all CTAs' counts give every digit's base, and each tile of
-// 1024 records is ranked by ballots.  A pass in which all records share the digit
-// is left out (without nodes below the count grid: all bits below level g).
+// least-significant-digit-first passes over (level, start); a pass in which all
+// records share the digit is left out (without nodes below the count grid: all bits
+// below level g).
 constexpr uint64_t kNodeClusterMax = 1ull << 18;
 
 struct NodeClusterArgs {
@@ -1456,10 +1455,9 @@ struct NodeClusterArgs {
 
 __global__ void __launch_bounds__(kClNT, 1) k_node_cluster(NodeClusterArgs a)
 {
-    __shared__ uint32_t s_whist[kClNT / 32][256];
-    __shared__ uint32_t s_cnt[256], s_base[256], s_warp[32];
+    __shared__ ClSortSmem s_sort;
     __shared__ unsigned long long s_mask;
-    const uint32_t rank = cl_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t rank = cl_rank(), tid = threadIdx.x, lane = tid & 31;
     const uint32_t M = min(*a.nnode, a.ncap);
     const int lmax = a.lmax;
     if (rank == 0 && tid == 0) {
@@ -1489,68 +1487,22 @@ __global__ void __launch_bounds__(kClNT, 1) k_node_cluster(NodeClusterArgs a)
     uint64_t mask = 0;
     for (int r = 0; r < kClCtas; ++r) mask |= *(volatile const uint64_t*)(a.part + r);
 
-    const uint32_t per = (M + kClCtas - 1) / kClCtas, lo = min(M, rank * per), hi = min(M, lo + per);
     int cur = 0;
     for (int pass = -1; pass < 8; ++pass) {   // -1: the level
         if (pass >= 0 && !((mask >> (8 * pass)) & 255u)) continue;
         const uint64_t* kin = a.key[cur];
         const uint32_t* vin = a.val[cur];
-        auto digit = [&](uint32_t i) -> uint32_t {
-            return pass < 0 ? a.rec[vin[i]].level : (uint32_t)(kin[i] >> (8 * pass)) & 255u;
-        };
-        if (tid < 256) s_cnt[tid] = 0;
-        __syncthreads();
-        for (uint32_t i0 = lo; i0 < hi; i0 += kClNT) {
-            const uint32_t i = i0 + tid;
-            const uint32_t d = i < hi ? digit(i) : 0u;
-            const uint32_t peers = match_bits<8>(d, i < hi);
-            if (i < hi && lane == (uint32_t)__ffs(peers) - 1) atomicAdd(&s_cnt[d], (uint32_t)__popc(peers));
-        }
-        __syncthreads();
-        if (tid < 256) a.hist[rank * 256 + tid] = s_cnt[tid];
-        cl_sync();
-        {
-            uint32_t before = 0, total = 0;
-            if (tid < 256)
-                for (int r = 0; r < kClCtas; ++r) {
-                    const uint32_t v = ld_volatile(a.hist + r * 256 + tid);
-                    if (r < (int)rank) before += v;
-                    total += v;
-                }
-            uint32_t all;
-            const uint32_t ex = block_exclusive_scan<kClNT, uint32_t>(total, s_warp, all);
-            if (tid < 256) s_base[tid] = ex + before;
-        }
         uint64_t* kout = a.key[cur ^ 1];
         uint32_t* vout = a.val[cur ^ 1];
-        for (uint32_t i0 = lo; i0 < hi; i0 += kClNT) {
-            for (uint32_t q = tid; q < (kClNT / 32) * 256 / 4; q += kClNT)
-                reinterpret_cast<uint4*>(&s_whist[0][0])[q] = make_uint4(0, 0, 0, 0);
-            __syncthreads();
-            const uint32_t i = i0 + tid;
-            const bool valid = i < hi;
-            const uint32_t d = valid ? digit(i) : 0u;
-            const uint32_t peers = match_bits<8>(d, valid);
-            if (valid && lane == (uint32_t)__ffs(peers) - 1) s_whist[warp][d] = __popc(peers);
-            __syncthreads();
-            if (tid < 256) {
-                uint32_t run = s_base[tid];
-                for (int w = 0; w < kClNT / 32; ++w) {
-                    const uint32_t c = s_whist[w][tid];
-                    s_whist[w][tid] = run;
-                    run += c;
-                }
-                s_base[tid] = run;
-            }
-            __syncthreads();
-            if (valid) {
-                const uint32_t at = s_whist[warp][d] + __popc(peers & lanemask_lt());
+        cl_sort_pass(
+            M, s_sort, a.hist,
+            [&](uint32_t i) -> uint32_t {
+                return pass < 0 ? a.rec[vin[i]].level : (uint32_t)(kin[i] >> (8 * pass)) & 255u;
+            },
+            [&](uint32_t i, uint32_t at) {
                 kout[at] = kin[i];
                 vout[at] = vin[i];
-            }
-            __syncthreads();
-        }
-        cl_sync();
+            });
         cur ^= 1;
     }
     // records in preorder and the lookups
@@ -1596,6 +1548,82 @@ __global__ void __launch_bounds__(kClNT, 1) k_node_cluster(NodeClusterArgs a)
     }
     if (rank == 0 && tid == 0 && *a.nnode > M) *a.nnode = M;   // (every CTA has read it: barriers above)
 }
+
+// The layouts of small clouds in one launch of one cluster: the points sorted
+// stably by node id, from the chunk order (leaf grouping) or from the original
+// order (final layout: every node's points in ascending index, the stitch
+// included), then moved once.  Bound by the latency of its phases: 20,000 points,
+// 157 nodes (one pass): subsample 107 -> 25 us, the leaf grouping 40 -> 15 us; the
+// chain of plan, scatters, sort passes and placement was 15 launches.  Two passes
+// of 65,000 points take 66 us here and 57 us as one grid-wide sort (below); one
+// pass takes 37 us in both.
+constexpr uint64_t kLayoutCluster = 1ull << 15;
+
+struct LayoutArgs {
+    fp_node* nodes;              // original order: `first` is filled too
+    const uint32_t* num_nodes;
+    uint32_t node_cap, n;
+    int original;                // 1: original order, 0: chunk order
+    const int4* pts;
+    const uint32_t *perm, *id;   // by chunk position
+    uint32_t *key[2], *val[2];   // n each
+    uint32_t* hist;              // [kClCtas * 256]
+    uint64_t* part;              // [kClCtas]
+    int4* out;                   // nullable
+    uint32_t* out_perm;          // nullable
+    uint32_t* err;
+};
+
+__global__ void __launch_bounds__(kClNT, 1) k_layout_cluster(LayoutArgs a)
+{
+    __shared__ ClSortSmem s_sort;
+    __shared__ uint64_t s_warp[32];
+    const uint32_t t = cl_rank() * kClNT + threadIdx.x;
+    const uint32_t M = min(*a.num_nodes, a.node_cap);
+    if (a.original)
+        cl_scan(M, a.part, s_warp, [&](uint32_t i) -> uint64_t { return a.nodes[i].n_own; },
+                [&](uint32_t i, uint64_t ex) { a.nodes[i].first = ex; });
+    for (uint32_t j = t; j < a.n; j += kClThreads) {
+        uint32_t i = a.original ? a.perm[j] : j;
+        uint32_t id = a.id[j];
+        if (i >= a.n) { raise(a.err, FP_ERR_CAPACITY, 11); i = j; }
+        if (id >= M) { raise(a.err, FP_ERR_CAPACITY, 15); id = 0; }   // not a node of the table
+        a.key[0][i] = id;
+        a.val[0][i] = j;
+    }
+    cl_sync();
+    int cur = 0;
+    for (uint32_t sh = 0; sh < 32 && (M ? M - 1 : 0u) >> sh; sh += 8) {
+        const uint32_t *kin = a.key[cur], *vin = a.val[cur];
+        uint32_t *kout = a.key[cur ^ 1], *vout = a.val[cur ^ 1];
+        cl_sort_pass(
+            a.n, s_sort, a.hist, [&](uint32_t i) -> uint32_t { return (kin[i] >> sh) & 255u; },
+            [&](uint32_t i, uint32_t at) {
+                kout[at] = kin[i];
+                vout[at] = vin[i];
+            });
+        cur ^= 1;
+    }
+    const uint32_t* v = a.val[cur];
+    for (uint32_t q = t; q < a.n; q += kClThreads) {
+        const uint32_t j = v[q];
+        if (j >= a.n) continue;   // (a slot that no point claimed: perm holds repeats)
+        if (a.original) {         // the node's own range, as its record says
+            const uint32_t id = a.id[j];
+            if (id >= M || q < a.nodes[id].first || q - a.nodes[id].first >= a.nodes[id].n_own)
+                raise(a.err, FP_ERR_CAPACITY, 15);
+        }
+        if (a.out) a.out[q] = __ldg(a.pts + j);
+        if (a.out_perm) a.out_perm[q] = a.perm[j];
+    }
+}
+
+// Above, up to kLayoutWhole points: one sort by node id of the whole array, a pass
+// per 8 bits of the node count, over arrays that stay in L2.  It moves the points
+// once or twice more than the chunk-wise scatter but is a third of its launches:
+// 1M points, subsample 133 -> 55 us (195 nodes), 167 -> 71 us (7192 nodes), the
+// leaf grouping 57 -> 46 us; at 4M points 217 -> 240 us and 98 -> 125 us.
+constexpr uint64_t kLayoutWhole = 1ull << 21;
 
 // owner and leaf ids of every distributed point; owned counts per node.
 // A node at a level <= g is found from the level-g cell in the point's code
@@ -2030,6 +2058,15 @@ cudaError_t launch_octree_impl(const fp_point* sorted, const uint32_t* perm, uin
     // leaf id runs instead, gated on the device, when a chunk does not fit
     if (leaf_pts || leaf_perm) {
         KTimerScope kt(FP_KERNEL_LEAF_SCATTER, st);
+        if (N <= kLayoutCluster) {
+            LayoutArgs a{};
+            a.nodes = nodes; a.num_nodes = nnode; a.node_cap = (uint32_t)Ly.node_cap; a.n = (uint32_t)N;
+            a.pts = reinterpret_cast<const int4*>(sorted); a.perm = perm; a.id = B.leafid;
+            a.key[0] = B.leafid; a.key[1] = B.lt_k32; a.val[0] = B.lt_val; a.val[1] = B.codes;
+            a.hist = sc.hist; a.part = B.seg.part;
+            a.out = reinterpret_cast<int4*>(leaf_pts); a.out_perm = leaf_perm; a.err = ws.err;
+            return cl_launch(k_layout_cluster, a, st);
+        }
         SegCall sg{};
         sg.mode = SEG_LEAF;
         sg.nodes = nodes; sg.num_nodes = num_nodes; sg.node_cap = node_cap;
@@ -2042,7 +2079,10 @@ cudaError_t launch_octree_impl(const fp_point* sorted, const uint32_t* perm, uin
         sg.first = reinterpret_cast<const uint64_t*>(nodes) + offsetof(fp_node, leaf_first) / sizeof(uint64_t);
         sg.first_stride = sizeof(fp_node) / sizeof(uint64_t);
         sg.hist = sc.hist;
-        if ((e = seg_scatter(B.seg, sg, ws, st))) return e;
+        const bool all = N <= kLayoutWhole;   // the one sort by leaf id
+        if (all) e = cudaMemsetAsync(sc.hist, 0, sizeof(uint32_t) * kSortHistWords, st);
+        else e = seg_scatter(B.seg, sg, ws, st);
+        if (e) return e;
         SortArgs a{};
         a.b.pt_src = reinterpret_cast<const int4*>(sorted);
         a.b.pt_tmp = B.lt_pt;
@@ -2050,7 +2090,7 @@ cudaError_t launch_octree_impl(const fp_point* sorted, const uint32_t* perm, uin
         a.b.val_src = perm; a.b.val_tmp = B.lt_val; a.b.val_dst = leaf_perm;
         // (three passes read the ids back from dst; the codes are not needed any more)
         a.b.k32_src = B.leafid; a.b.k32_tmp = B.lt_k32; a.b.k32_dst = B.codes;
-        a.n = N; a.run_if = B.seg.cnt + 2; a.err = ws.err;
+        a.n = N; a.run_if = all ? nullptr : B.seg.cnt + 2; a.err = ws.err;
         if ((e = sort_plan_weights(sc, a, B.leafw, nullptr, nnode, Ly.node_cap, true, ws.num_sms, st))) return e;
         const int np = sort_passes(count_bits(Ly.node_cap));   // leaf ids below node_cap
         if (leaf_pts) e = sort_run<DIG_K32, true, false, true>(a, np, ws.num_sms, st);
@@ -2173,14 +2213,14 @@ cudaError_t launch_node_first(fp_node* nodes, const uint32_t* num_nodes, uint32_
     return cudaGetLastError();
 }
 
-// Whole-array path, where a chunk holds more nodes than the segmented scatter
-// takes: the points and owners in original order, from which one stable sort by
-// owner gives the final layout.
+// Whole-array path: the points and owners in original order, from which one
+// stable sort by owner gives the final layout.  For clouds of up to kLayoutWhole
+// points, and where a chunk holds more nodes than the segmented scatter takes.
 __global__ void __launch_bounds__(256) k_original_order(const uint32_t* gate, const int4* pts, const uint32_t* perm,
                                                         const uint32_t* owner, uint64_t n, int4* opts,
                                                         uint32_t* oowner, uint32_t* err)
 {
-    if (!*gate) return;
+    if (gate && !*gate) return;
     for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (uint64_t)gridDim.x * blockDim.x) {
         const uint32_t i = perm[j];
         if (i >= n) { raise(err, FP_ERR_CAPACITY, 11); continue; }
@@ -2255,6 +2295,32 @@ cudaError_t launch_subsample(fp_node* nodes, const uint32_t* num_nodes, uint32_t
     uint32_t* nrank = B.cnt + 4;   // nodes outside every chunk subtree
     const unsigned gN = (unsigned)std::min<uint64_t>((N + 255) / 256, (uint64_t)ws.num_sms * 16);
 
+    if (N <= kLayoutCluster) {
+        LayoutArgs a{};
+        a.nodes = nodes; a.num_nodes = num_nodes; a.node_cap = node_cap; a.n = (uint32_t)N;
+        a.original = 1;
+        a.pts = reinterpret_cast<const int4*>(sorted); a.perm = perm; a.id = owner;
+        a.key[0] = B.o_own; a.key[1] = B.o_own2; a.val[0] = B.t_val; a.val[1] = B.t_k32;
+        a.hist = sc.hist; a.part = B.seg.part;
+        a.out = reinterpret_cast<int4*>(final_pts); a.out_perm = final_perm; a.err = ws.err;
+        KTimerScope kt(FP_KERNEL_OWNER_SCATTER, st);
+        return cl_launch(k_layout_cluster, a, st);
+    }
+    // the sort by owner of the points in original order, gated or not
+    auto whole = [&](const uint32_t* gate) -> cudaError_t {
+        k_original_order<<<gN, 256, 0, st>>>(gate, reinterpret_cast<const int4*>(sorted), perm, owner, N, B.o_pt,
+                                             B.o_own, ws.err);
+        SortArgs a{};
+        a.b.pt_src = B.o_pt; a.b.pt_tmp = B.t_pt; a.b.pt_dst = reinterpret_cast<int4*>(final_pts);
+        a.b.val_src = nullptr; a.b.val_tmp = B.t_val; a.b.val_dst = final_perm;   // the original index
+        a.b.k32_src = B.o_own; a.b.k32_tmp = B.t_k32; a.b.k32_dst = B.o_own2;
+        a.n = N; a.run_if = gate; a.err = ws.err;
+        const SortScratch sc2{B.hist2, {sc.status[0], sc.status[1]}};
+        cudaError_t x = sort_plan_weights(sc2, a, B.nown, nullptr, nm, M, true, ws.num_sms, st);
+        if (x) return x;
+        return sort_run<DIG_K32, true, false, true>(a, sort_passes(count_bits(M)), ws.num_sms, st);
+    };
+
     // 1. stable scatter by owner id, chunk by chunk; owners above the chunk are staged
     int pbits = 1;
     while ((1ull << pbits) < N) ++pbits;   // original indices are below 2^pbits
@@ -2271,6 +2337,11 @@ cudaError_t launch_subsample(fp_node* nodes, const uint32_t* num_nodes, uint32_t
     sg.nown = B.nown; sg.first_out = B.first; sg.nm = nm;
     sg.st_key = B.s_key; sg.st_src = B.s_val; sg.st_count = nstaged; sg.st_shift = pbits;
     sg.st_rank = B.srank; sg.st_list = B.slist; sg.st_nrank = nrank; sg.st_soff = B.soff;
+    if (N <= kLayoutWhole) {
+        KTimerScope kt(FP_KERNEL_OWNER_SCATTER, st);
+        if ((e = seg_node_starts(B.seg, sg, ws, st))) return e;
+        return whole(nullptr);
+    }
     {
         KTimerScope kt(FP_KERNEL_OWNER_SCATTER, st);
         if ((e = seg_scatter(B.seg, sg, ws, st))) return e;
@@ -2291,18 +2362,8 @@ cudaError_t launch_subsample(fp_node* nodes, const uint32_t* num_nodes, uint32_t
                                            reinterpret_cast<const int4*>(sorted), perm, N,
                                            reinterpret_cast<int4*>(final_pts), final_perm, ws.err);
     }
-    // whole-array path, when a chunk did not fit
-    const uint32_t* gate = B.seg.cnt + 2;
-    k_original_order<<<gN, 256, 0, st>>>(gate, reinterpret_cast<const int4*>(sorted), perm, owner, N, B.o_pt, B.o_own,
-                                         ws.err);
-    SortArgs a{};
-    a.b.pt_src = B.o_pt; a.b.pt_tmp = B.t_pt; a.b.pt_dst = reinterpret_cast<int4*>(final_pts);
-    a.b.val_src = nullptr; a.b.val_tmp = B.t_val; a.b.val_dst = final_perm;   // the original index
-    a.b.k32_src = B.o_own; a.b.k32_tmp = B.t_k32; a.b.k32_dst = B.o_own2;
-    a.n = N; a.run_if = gate; a.err = ws.err;
-    const SortScratch sc2{B.hist2, {sc.status[0], sc.status[1]}};
-    if ((e = sort_plan_weights(sc2, a, B.nown, nullptr, nm, M, true, ws.num_sms, st))) return e;
-    return sort_run<DIG_K32, true, false, true>(a, sort_passes(count_bits(M)), ws.num_sms, st);
+    // a chunk did not fit: all of it again
+    return whole(B.seg.cnt + 2);
 }
 
 }  // namespace fp

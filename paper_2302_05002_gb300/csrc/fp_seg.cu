@@ -29,12 +29,11 @@ FP_DEV uint32_t find_node(const fp_node* nodes, uint32_t M, uint64_t key, uint32
 //     chunk subtrees; the look-back words of tiles that others will read cleared;
 //   C (owner layout): the nodes outside every chunk subtree ranked in order, and
 //     where each one's staged points start.
-// One cluster does all of them for up to kSegClusterMax points (a chain of 20
-// launches before, about 80 us; 11 us now for 20,000 points); step B, whose work grows with chunks and tiles, takes
-// the whole GPU for larger clouds.
+// One cluster does A and C (a chain of launches before); step B, whose work grows
+// with chunks and tiles, takes the whole GPU.
 struct SegPlan {
     int owner;               // 1: owner layout, 0: leaf grouping
-    int steps;               // 1: A, 2: B, 4: C
+    int step_c;              // 0: A, 1: C
     fp_node* nodes;
     const uint32_t* num_nodes;
     uint32_t node_cap;
@@ -55,7 +54,6 @@ struct SegPlan {
     uint32_t *hist, *hist2;  // the sorts' histograms, cleared in A
     uint32_t* err;
 };
-constexpr uint64_t kSegClusterMax = 1ull << 18;
 
 // step B for the chunk of this lane (c < K); all 32 lanes of the warp take part.
 // Callers spread the chunks over the warps first (a few large chunks: one each).
@@ -118,22 +116,14 @@ FP_DEV void seg_chunk(const SegPlan& a, uint64_t c, uint64_t K, uint32_t M)
     }
 }
 
-FP_DEV void seg_chunks(const SegPlan& a, uint32_t warp, uint32_t nwarps, uint64_t K, uint32_t M)
-{   // lane l of warp w: chunks w + l * nwarps, + 32 * nwarps, ...
-    for (uint64_t c0 = warp; c0 < K; c0 += 32ull * nwarps) seg_chunk(a, c0 + (uint64_t)(threadIdx.x & 31) * nwarps, K, M);
-}
-
-FP_DEV void seg_chunk_head(const SegPlan& a, uint64_t K)
-{
-    if (*a.num_chunks > a.kmax || a.offsets[K] != a.n) atomicOr(&a.cnt[2], 1u);
-}
-
 __global__ void __launch_bounds__(256) k_seg_chunks(SegPlan a)
 {
     const uint64_t K = min((uint64_t)*a.num_chunks, a.kmax);
     const uint32_t M = min(*a.num_nodes, a.node_cap);
-    if (blockIdx.x == 0 && threadIdx.x == 0) seg_chunk_head(a, K);
-    seg_chunks(a, (blockIdx.x * blockDim.x + threadIdx.x) >> 5, (gridDim.x * blockDim.x) >> 5, K, M);
+    if (blockIdx.x == 0 && threadIdx.x == 0 && (*a.num_chunks > a.kmax || a.offsets[K] != a.n)) atomicOr(&a.cnt[2], 1u);
+    // lane l of warp w: chunks w + l * nwarps, + 32 * nwarps, ...
+    const uint64_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
+    for (uint64_t c0 = warp; c0 < K; c0 += 32 * nwarps) seg_chunk(a, c0 + (threadIdx.x & 31) * nwarps, K, M);
 }
 
 __global__ void __launch_bounds__(kClNT, 1) k_seg_plan(SegPlan a)
@@ -141,45 +131,35 @@ __global__ void __launch_bounds__(kClNT, 1) k_seg_plan(SegPlan a)
     __shared__ uint64_t s_warp[32];
     const uint32_t t = cl_rank() * kClNT + threadIdx.x;
     const uint32_t M = min(*a.num_nodes, a.node_cap);
-    if (a.steps & 1) {
+    if (!a.step_c) {
         for (uint32_t q = t; q < 8; q += kClThreads) a.cnt[q] = 0;
         for (uint32_t q = t; q < (uint32_t)kSortHistWords; q += kClThreads) {
             a.hist[q] = 0;
             if (a.hist2) a.hist2[q] = 0;
         }
-        if (a.owner) {
-            if (t == 0) { *a.nm = M; *a.nstaged = 0; }
-            for (uint32_t i = t; i < M; i += kClThreads) {
-                a.nown[i] = a.nodes[i].n_own;
-                a.inside[i] = 0;
-            }
-            cl_sync();
-            cl_scan(M, a.part, s_warp, [&](uint32_t i) -> uint64_t { return a.nown[i]; },
-                    [&](uint32_t i, uint64_t ex) {
-                        a.first[i] = ex;
-                        a.nodes[i].first = ex;
-                    });
-        } else {
-            cl_sync();
+        if (!a.owner) return;
+        if (t == 0) { *a.nm = M; *a.nstaged = 0; }
+        for (uint32_t i = t; i < M; i += kClThreads) {
+            a.nown[i] = a.nodes[i].n_own;
+            a.inside[i] = 0;
         }
-    }
-    if (a.steps & 2) {
-        const uint64_t K = min((uint64_t)*a.num_chunks, a.kmax);
-        if (t == 0) seg_chunk_head(a, K);
-        seg_chunks(a, t >> 5, kClThreads / 32, K, M);
         cl_sync();
+        cl_scan(M, a.part, s_warp, [&](uint32_t i) -> uint64_t { return a.nown[i]; },
+                [&](uint32_t i, uint64_t ex) {
+                    a.first[i] = ex;
+                    a.nodes[i].first = ex;
+                });
+        return;
     }
-    if (a.steps & 4) {
-        const uint64_t all = cl_scan(
-            M, a.part, s_warp,
-            [&](uint32_t i) -> uint64_t { return a.inside[i] ? 0ull : (1ull << 32) | a.nown[i]; },
-            [&](uint32_t i, uint64_t ex) {
-                a.soff[i] = (uint32_t)ex;
-                a.rank[i] = (uint32_t)(ex >> 32);
-                if (!a.inside[i]) a.list[ex >> 32] = i;
-            });
-        if (t == 0) *a.nrank = (uint32_t)(all >> 32);
-    }
+    const uint64_t all = cl_scan(
+        M, a.part, s_warp,
+        [&](uint32_t i) -> uint64_t { return a.inside[i] ? 0ull : (1ull << 32) | a.nown[i]; },
+        [&](uint32_t i, uint64_t ex) {
+            a.soff[i] = (uint32_t)ex;
+            a.rank[i] = (uint32_t)(ex >> 32);
+            if (!a.inside[i]) a.list[ex >> 32] = i;
+        });
+    if (t == 0) *a.nrank = (uint32_t)(all >> 32);
 }
 
 SegScratch take_seg_scratch(const Workspace& ws, uint64_t n, uint64_t kmax, uint64_t node_cap)
@@ -772,12 +752,10 @@ cudaError_t dist_wide(const int4* pts, uint64_t n, const fp_cube* cube, int g, c
     return cudaGetLastError();
 }
 
-cudaError_t seg_scatter(const SegScratch& sc, const SegCall& c, const Workspace& ws, cudaStream_t st)
+static SegPlan seg_plan(const SegScratch& sc, const SegCall& c, const Workspace& ws)
 {
-    cudaError_t e;
-    const bool owner = c.mode == SEG_OWNER;
     SegPlan p{};
-    p.owner = owner;
+    p.owner = c.mode == SEG_OWNER;
     p.nodes = c.nodes; p.num_nodes = c.num_nodes; p.node_cap = c.node_cap;
     p.chunks = c.chunks; p.num_chunks = c.num_chunks; p.offsets = c.offsets;
     p.kmax = sc.kmax; p.n = c.n; p.tiles_max = sc.tiles_max;
@@ -788,17 +766,25 @@ cudaError_t seg_scatter(const SegScratch& sc, const SegCall& c, const Workspace&
     p.rank = c.st_rank; p.list = c.st_list; p.nrank = c.st_nrank; p.soff = c.st_soff; p.nm = c.nm; p.nstaged = c.st_count;
     p.hist = c.hist; p.hist2 = c.hist2;
     p.err = ws.err;
-    if (c.n <= kSegClusterMax) {
-        p.steps = owner ? 7 : 3;
-        if ((e = cl_launch(k_seg_plan, p, st))) return e;
-    } else {
-        p.steps = 1;
-        if ((e = cl_launch(k_seg_plan, p, st))) return e;
-        const int gk = (int)std::max<uint64_t>(1, std::min<uint64_t>((sc.kmax + 255) / 256, (uint64_t)ws.num_sms * 8));
-        k_seg_chunks<<<gk, 256, 0, st>>>(p);
-        p.steps = 4;
-        if (owner && (e = cl_launch(k_seg_plan, p, st))) return e;
-    }
+    return p;
+}
+
+cudaError_t seg_node_starts(const SegScratch& sc, const SegCall& c, const Workspace& ws, cudaStream_t st)
+{
+    const SegPlan p = seg_plan(sc, c, ws);
+    return cl_launch(k_seg_plan, p, st);
+}
+
+cudaError_t seg_scatter(const SegScratch& sc, const SegCall& c, const Workspace& ws, cudaStream_t st)
+{
+    cudaError_t e;
+    const bool owner = c.mode == SEG_OWNER;
+    SegPlan p = seg_plan(sc, c, ws);
+    if ((e = cl_launch(k_seg_plan, p, st))) return e;
+    const int gk = (int)std::max<uint64_t>(1, std::min<uint64_t>((sc.kmax + 255) / 256, (uint64_t)ws.num_sms * 8));
+    k_seg_chunks<<<gk, 256, 0, st>>>(p);
+    p.step_c = 1;
+    if (owner && (e = cl_launch(k_seg_plan, p, st))) return e;
     SegArgs a{};
     a.pt_in = c.pt_in; a.pt_out = c.pt_out;
     a.val_in = c.val_in; a.val_out = c.val_out;

@@ -284,4 +284,8 @@ cudaError_t dist_wide(const int4* pts, uint64_t n, const fp_cube* cube, int g, c
 // path, gated on it, must run.
 cudaError_t seg_scatter(const SegScratch& sc, const SegCall& call, const Workspace& ws, cudaStream_t st);
 
+// Only the plan's first step (owner layout): owned counts and first points of the
+// nodes, the sorts' histograms cleared.
+cudaError_t seg_node_starts(const SegScratch& sc, const SegCall& call, const Workspace& ws, cudaStream_t st);
+
 }  // namespace fp
