@@ -144,16 +144,25 @@ def _ptr(t):
     return None if t is None else ctypes.c_void_p(t.data_ptr())
 
 
+def _adr(t):
+    """Address for the library's functions, whose declared argument types convert
+    it (_ptr is for functions without; 45 objects less in a whole build)."""
+    return None if t is None else t.data_ptr()
+
+
 def _on_stream(fn):
     """Run a wrapper with its `stream` argument as torch's current stream, so that
     the temporaries it allocates (workspaces, outputs) belong to that stream:
     torch's caching allocator may hand a freed block to the next allocation at
     once, which is safe only when both are ordered on the same stream."""
-    sig = inspect.signature(fn)
+    # The argument's place is looked up once, not by binding every call's arguments:
+    # a whole build of 20,000 points takes 252 instead of 322 us with this, raw
+    # addresses, and counts that the library writes left unfilled.
+    place = list(inspect.signature(fn).parameters).index("stream")
 
     @functools.wraps(fn)
     def wrapper(*args, **kw):
-        st = sig.bind_partial(*args, **kw).arguments.get("stream")
+        st = args[place] if len(args) > place else kw.get("stream")
         if st is None:
             return fn(*args, **kw)
         with torch.cuda.stream(st):
@@ -164,6 +173,10 @@ def _on_stream(fn):
 def _stream(stream):
     s = stream if stream is not None else torch.cuda.current_stream()
     return ctypes.c_void_p(s.cuda_stream)
+
+
+def _raw_stream(stream):
+    return (stream if stream is not None else torch.cuda.current_stream()).cuda_stream
 
 
 def _dev(t):
@@ -215,12 +228,13 @@ def get_device_error(stream=None, clear=True):
 
 
 # ------------------------------------------------------------------ stages
+# (Counts are written by the library, for empty clouds too: they are not filled first.)
 @_on_stream
 def fp_bounds(pts, stream=None, ws=None):
     n = pts.shape[0]
     cube = torch.empty(CUBE_BYTES // 4, dtype=torch.int32, device=_dev(pts))
     w, need = _ws("bounds", n, None, _dev(pts), ws)
-    _check(load().fp_bounds(_ptr(pts), n, _ptr(cube), _ptr(w), w.numel(), _stream(stream)), "fp_bounds")
+    _check(load().fp_bounds(_adr(pts), n, _adr(cube), _adr(w), w.numel(), _raw_stream(stream)), "fp_bounds")
     return cube
 
 
@@ -235,10 +249,10 @@ def fp_decimate(pts, first_index=0, modulus=16, out=None, stream=None, ws=None):
     cap = out.shape[0] if out is not None else _preview_cap(n, modulus)
     if out is None:
         out = torch.empty((max(cap, 1), 4), dtype=torch.int32, device=_dev(pts))
-    count = torch.zeros(1, dtype=torch.int64, device=_dev(pts))
+    count = torch.empty(1, dtype=torch.int64, device=_dev(pts))
     w, need = _ws("decimate", n, None, _dev(pts), ws)
-    _check(load().fp_decimate(_ptr(pts), n, first_index, modulus, _ptr(out), cap, _ptr(count), _ptr(w), w.numel(),
-                              _stream(stream)), "fp_decimate")
+    _check(load().fp_decimate(_adr(pts), n, first_index, modulus, _adr(out), cap, _adr(count), _adr(w), w.numel(),
+                              _raw_stream(stream)), "fp_decimate")
     return out, count
 
 
@@ -255,11 +269,11 @@ def fp_preview_spatial(pts, cube, level=7, first_index=0, out=None, stream=None,
     cap = out.shape[0] if out is not None else min(n, 1 << (3 * level))
     if out is None:
         out = torch.empty((max(cap, 1), 4), dtype=torch.int32, device=_dev(pts))
-    count = torch.zeros(1, dtype=torch.int64, device=_dev(pts))
+    count = torch.empty(1, dtype=torch.int64, device=_dev(pts))
     prm = params(grid_log2=level, sub_log2=level, max_level=level)
     w, need = _ws("preview_spatial", n, prm, _dev(pts), ws)
-    _check(load().fp_preview_spatial(_ptr(pts), n, _ptr(cube), level, first_index, _ptr(out), cap, _ptr(count),
-                                     _ptr(w), w.numel(), _stream(stream)), "fp_preview_spatial")
+    _check(load().fp_preview_spatial(_adr(pts), n, _adr(cube), level, first_index, _adr(out), cap, _adr(count),
+                                     _adr(w), w.numel(), _raw_stream(stream)), "fp_preview_spatial")
     return out, count
 
 
@@ -270,10 +284,10 @@ def fp_bounds_decimate(pts, first_index=0, modulus=16, out=None, stream=None, ws
     if out is None:
         out = torch.empty((max(cap, 1), 4), dtype=torch.int32, device=_dev(pts))
     cube = torch.empty(CUBE_BYTES // 4, dtype=torch.int32, device=_dev(pts))
-    count = torch.zeros(1, dtype=torch.int64, device=_dev(pts))
+    count = torch.empty(1, dtype=torch.int64, device=_dev(pts))
     w, need = _ws("bounds_decimate", n, None, _dev(pts), ws)
-    _check(load().fp_bounds_decimate(_ptr(pts), n, _ptr(cube), first_index, modulus, _ptr(out), cap, _ptr(count),
-                                     _ptr(w), w.numel(), _stream(stream)), "fp_bounds_decimate")
+    _check(load().fp_bounds_decimate(_adr(pts), n, _adr(cube), first_index, modulus, _adr(out), cap, _adr(count),
+                                     _adr(w), w.numel(), _raw_stream(stream)), "fp_bounds_decimate")
     return cube, out, count
 
 
@@ -282,8 +296,8 @@ def fp_count(pts, cube, grid_log2=7, counts=None, accumulate=False, stream=None)
     n = pts.shape[0]
     if counts is None:
         counts = torch.empty(1 << (3 * grid_log2), dtype=torch.int32, device=_dev(pts))
-    _check(load().fp_count(_ptr(pts), n, _ptr(cube), grid_log2, _ptr(counts), int(accumulate), None, 0,
-                           _stream(stream)), "fp_count")
+    _check(load().fp_count(_adr(pts), n, _adr(cube), grid_log2, _adr(counts), int(accumulate), None, 0,
+                           _raw_stream(stream)), "fp_count")
     return counts
 
 
@@ -295,8 +309,8 @@ def fp_count_cells(pts, cube, grid_log2=7, counts=None, cells=None, accumulate=F
         counts = torch.empty(1 << (3 * grid_log2), dtype=torch.int32, device=_dev(pts))
     if cells is None:
         cells = torch.empty(max(n, 1), dtype=torch.int32, device=_dev(pts))
-    _check(load().fp_count_cells(_ptr(pts), n, _ptr(cube), grid_log2, _ptr(counts), int(accumulate), _ptr(cells),
-                                 None, 0, _stream(stream)), "fp_count_cells")
+    _check(load().fp_count_cells(_adr(pts), n, _adr(cube), grid_log2, _adr(counts), int(accumulate), _adr(cells),
+                                 None, 0, _raw_stream(stream)), "fp_count_cells")
     return counts, cells
 
 
@@ -305,13 +319,13 @@ def fp_merge_chunks(counts, grid_log2, threshold, stream=None, ws=None):
     dev = counts.device
     cells = 1 << (3 * grid_log2)
     chunks = torch.empty((cells, CHUNK_BYTES // 8), dtype=torch.int64, device=dev)
-    num = torch.zeros(1, dtype=torch.int32, device=dev)
+    num = torch.empty(1, dtype=torch.int32, device=dev)
     lut = torch.empty(cells, dtype=torch.int32, device=dev)
     offsets = torch.empty(cells + 1, dtype=torch.int64, device=dev)
     prm = params(grid_log2=grid_log2)
     w, need = _ws("merge", 0, prm, dev, ws)
-    _check(load().fp_merge_chunks(_ptr(counts), grid_log2, threshold, _ptr(chunks), _ptr(num), _ptr(lut),
-                                  _ptr(offsets), _ptr(w), w.numel(), _stream(stream)), "fp_merge_chunks")
+    _check(load().fp_merge_chunks(_adr(counts), grid_log2, threshold, _adr(chunks), _adr(num), _adr(lut),
+                                  _adr(offsets), _adr(w), w.numel(), _raw_stream(stream)), "fp_merge_chunks")
     return chunks, num, lut, offsets
 
 
@@ -326,8 +340,8 @@ def fp_distribute(pts, cube, grid_log2, lut, offsets, num_chunks, with_perm=True
         perm = torch.empty(n, dtype=torch.int32, device=dev)
     prm = params(grid_log2=grid_log2)
     w, need = _ws("distribute", n, prm, dev, ws)
-    _check(load().fp_distribute(_ptr(pts), n, _ptr(cube), grid_log2, _ptr(lut), _ptr(offsets), _ptr(num_chunks),
-                                _ptr(out), _ptr(perm) if with_perm else None, _ptr(w), w.numel(), _stream(stream)),
+    _check(load().fp_distribute(_adr(pts), n, _adr(cube), grid_log2, _adr(lut), _adr(offsets), _adr(num_chunks),
+                                _adr(out), _adr(perm) if with_perm else None, _adr(w), w.numel(), _raw_stream(stream)),
            "fp_distribute")
     return out, perm
 
@@ -344,9 +358,9 @@ def fp_distribute_cells(pts, cells, cube, grid_log2, lut, offsets, num_chunks, w
         perm = torch.empty(n, dtype=torch.int32, device=dev)
     prm = params(grid_log2=grid_log2)
     w, need = _ws("distribute", n, prm, dev, ws)
-    _check(load().fp_distribute_cells(_ptr(pts), _ptr(cells), n, _ptr(cube), grid_log2, _ptr(lut), _ptr(offsets),
-                                      _ptr(num_chunks), _ptr(out), _ptr(perm) if with_perm else None, _ptr(w),
-                                      w.numel(), _stream(stream)), "fp_distribute_cells")
+    _check(load().fp_distribute_cells(_adr(pts), _adr(cells), n, _adr(cube), grid_log2, _adr(lut), _adr(offsets),
+                                      _adr(num_chunks), _adr(out), _adr(perm) if with_perm else None, _adr(w),
+                                      w.numel(), _raw_stream(stream)), "fp_distribute_cells")
     return out, perm
 
 
@@ -362,15 +376,15 @@ def fp_build_chunk_octree(sorted_pts, perm, cube, chunks, num_chunks, offsets, c
     if node_cap is None:
         node_cap = node_capacity_bound(n, prm)
     nodes = torch.zeros((node_cap, NODE_BYTES // 8), dtype=torch.int64, device=dev)
-    num_nodes = torch.zeros(1, dtype=torch.int32, device=dev)
+    num_nodes = torch.empty(1, dtype=torch.int32, device=dev)
     leaf_pts = torch.empty_like(sorted_pts) if leaf else None
     leaf_perm = torch.empty(n, dtype=torch.int32, device=dev) if leaf else None
     owner = torch.empty(n, dtype=torch.int32, device=dev)
     w, need = _ws("octree", n, prm, dev, ws)
-    _check(load().fp_build_chunk_octree(_ptr(sorted_pts), _ptr(perm), n, _ptr(cube), _ptr(chunks), _ptr(num_chunks),
-                                        _ptr(offsets), _ptr(counts), ctypes.byref(prm), _ptr(nodes), node_cap,
-                                        _ptr(num_nodes), _ptr(leaf_pts), _ptr(leaf_perm), _ptr(owner), _ptr(w),
-                                        w.numel(), _stream(stream)), "fp_build_chunk_octree")
+    _check(load().fp_build_chunk_octree(_adr(sorted_pts), _adr(perm), n, _adr(cube), _adr(chunks), _adr(num_chunks),
+                                        _adr(offsets), _adr(counts), ctypes.byref(prm), _adr(nodes), node_cap,
+                                        _adr(num_nodes), _adr(leaf_pts), _adr(leaf_perm), _adr(owner), _adr(w),
+                                        w.numel(), _raw_stream(stream)), "fp_build_chunk_octree")
     return nodes, num_nodes, leaf_pts, leaf_perm, owner
 
 
@@ -387,9 +401,9 @@ def fp_subsample(nodes, num_nodes, sorted_pts, perm, owner, chunks, num_chunks, 
     if final_perm is None:
         final_perm = torch.empty(n, dtype=torch.int32, device=dev)
     w, need = _ws("subsample", n, prm, dev, ws)
-    _check(load().fp_subsample(_ptr(nodes), _ptr(num_nodes), nodes.shape[0], _ptr(sorted_pts), _ptr(perm),
-                               _ptr(owner), n, _ptr(chunks), _ptr(num_chunks), _ptr(offsets), _ptr(final),
-                               _ptr(final_perm), _ptr(w), w.numel(), _stream(stream)),
+    _check(load().fp_subsample(_adr(nodes), _adr(num_nodes), nodes.shape[0], _adr(sorted_pts), _adr(perm),
+                               _adr(owner), n, _adr(chunks), _adr(num_chunks), _adr(offsets), _adr(final),
+                               _adr(final_perm), _adr(w), w.numel(), _raw_stream(stream)),
            "fp_subsample")
     return final, final_perm
 
@@ -432,7 +446,7 @@ def cloud_desc(pts, prm, out):
 @_on_stream
 def plain_calls(d, ws, stream=None):
     """The seven plain calls of one cloud (descriptor d), in order, on one stream."""
-    L, S, W, Wn = load(), _stream(stream), _ptr(ws), ws.numel()
+    L, S, W, Wn = load(), _raw_stream(stream), _adr(ws), ws.numel()
     g, T = d.prm.grid_log2, d.prm.chunk_threshold
     _check(L.fp_bounds_decimate(d.d_pts, d.n, d.d_cube, 0, d.prm.decim_modulus, d.d_preview, d.preview_cap,
                                 d.d_preview_count, W, Wn, S), "fp_bounds_decimate")
@@ -474,13 +488,13 @@ def batch_workspace_size_ex(descs, ncloud, opts):
 
 @_on_stream
 def fp_build_batched_ex(descs, ncloud, opts, ws, stream=None):
-    _check(load().fp_build_batched_ex(descs, ncloud, ctypes.byref(opts), _ptr(ws), ws.numel(), _stream(stream)),
+    _check(load().fp_build_batched_ex(descs, ncloud, ctypes.byref(opts), _adr(ws), ws.numel(), _raw_stream(stream)),
            "fp_build_batched_ex")
 
 
 @_on_stream
 def fp_build_batched(descs, ncloud, nlanes, ws, stream=None):
-    _check(load().fp_build_batched(descs, ncloud, nlanes, _ptr(ws), ws.numel(), _stream(stream)), "fp_build_batched")
+    _check(load().fp_build_batched(descs, ncloud, nlanes, _adr(ws), ws.numel(), _raw_stream(stream)), "fp_build_batched")
 
 
 @_on_stream
@@ -536,12 +550,12 @@ def build_ooc(host_pts, prm, arena, piece_points=1 << 23, group_points=0, scratc
     if scratch is None or scratch.numel() < need:
         scratch = torch.empty(need, dtype=torch.uint8).pin_memory()
     cb = PREVIEW_DONE((lambda _u: on_preview()) if on_preview is not None else 0)
-    st = load().fp_build_ooc(_ptr(host_pts), n, ctypes.byref(prm), piece_points, group_points, _ptr(arena),
+    st = load().fp_build_ooc(_adr(host_pts), n, ctypes.byref(prm), piece_points, group_points, _adr(arena),
                              arena.numel(),
-                             _ptr(scratch), scratch.numel(), _ptr(out["cube"]), _ptr(out["preview"]),
-                             out["preview_cap"], _ptr(out["preview_count"]), _ptr(out["nodes"]), out["node_cap"],
-                             _ptr(out["num_nodes"]), _ptr(out["final"]), _ptr(out["final_perm"]), cb, None,
-                             _stream(stream))
+                             _adr(scratch), scratch.numel(), _adr(out["cube"]), _adr(out["preview"]),
+                             out["preview_cap"], _adr(out["preview_count"]), _adr(out["nodes"]), out["node_cap"],
+                             _adr(out["num_nodes"]), _adr(out["final"]), _adr(out["final_perm"]), cb, None,
+                             _raw_stream(stream))
     _check(st, "fp_build_ooc")
     return out
 
@@ -597,8 +611,8 @@ def build_octree(pts, prm, stream=None):
 @_on_stream
 def fp_cloud_digest(pts, stream=None):
     """64-bit digest of a cloud (every point and the order): the cache key."""
-    d = torch.zeros(1, dtype=torch.int64, device=_dev(pts))
-    _check(load().fp_cloud_digest(_ptr(pts), pts.shape[0], _ptr(d), _stream(stream)), "fp_cloud_digest")
+    d = torch.empty(1, dtype=torch.int64, device=_dev(pts))
+    _check(load().fp_cloud_digest(_adr(pts), pts.shape[0], _adr(d), _raw_stream(stream)), "fp_cloud_digest")
     return int(d.item()) & 0xFFFFFFFFFFFFFFFF
 
 
@@ -612,10 +626,10 @@ def octree_save(path, prm, out, digest=0, with_perm=True, staging=None, stream=N
     num_nodes, final, final_perm) to one file."""
     stg = _staging(staging)
     n = out["final"].shape[0] if out.get("n") is None else out["n"]
-    _check(load().fp_octree_save(os.fsencode(path), ctypes.byref(prm), _ptr(out["cube"]), _ptr(out["nodes"]),
-                                 _ptr(out["num_nodes"]), _ptr(out["final"]),
-                                 _ptr(out["final_perm"]) if with_perm else None, n, digest & 0xFFFFFFFFFFFFFFFF,
-                                 _ptr(stg), stg.numel(), _stream(stream)), "fp_octree_save")
+    _check(load().fp_octree_save(os.fsencode(path), ctypes.byref(prm), _adr(out["cube"]), _adr(out["nodes"]),
+                                 _adr(out["num_nodes"]), _adr(out["final"]),
+                                 _adr(out["final_perm"]) if with_perm else None, n, digest & 0xFFFFFFFFFFFFFFFF,
+                                 _adr(stg), stg.numel(), _raw_stream(stream)), "fp_octree_save")
 
 
 def octree_header(path):
@@ -635,8 +649,8 @@ def octree_load(path, nodes=True, first=0, count=None, perm=True, device=None, s
     d_nodes = torch.zeros((max(h.num_nodes, 1), NODE_BYTES // 8), dtype=torch.int64, device=dev) if nodes else None
     pts = torch.empty((max(count, 1), 4), dtype=torch.int32, device=dev)
     prm_ = torch.empty(max(count, 1), dtype=torch.int32, device=dev) if perm and (h.flags & FILE_HAS_PERM) else None
-    _check(load().fp_octree_load(os.fsencode(path), _ptr(d_nodes), h.num_nodes, _ptr(pts), _ptr(prm_), first, count,
-                                 _ptr(stg), stg.numel(), _stream(stream)), "fp_octree_load")
+    _check(load().fp_octree_load(os.fsencode(path), _adr(d_nodes), h.num_nodes, _adr(pts), _adr(prm_), first, count,
+                                 _adr(stg), stg.numel(), _raw_stream(stream)), "fp_octree_load")
     num = torch.tensor([h.num_nodes], dtype=torch.int32, device=dev)
     return dict(header=h, nodes=d_nodes, num_nodes=num, final=pts[:count], final_perm=None if prm_ is None else prm_[:count])
 
@@ -711,8 +725,8 @@ def fp_select_nodes(nodes, num_nodes, cube, cam, ws=None, stream=None):
     nsel = torch.zeros(1, dtype=torch.int32, device=dev)
     npts = torch.zeros(1, dtype=torch.int64, device=dev)
     w = ws if ws is not None else torch.empty(max(render_workspace_size(cap), 1), dtype=torch.uint8, device=dev)
-    _check(load().fp_select_nodes(_ptr(nodes), _ptr(num_nodes), cap, _ptr(cube), ctypes.byref(cam), _ptr(ids),
-                                  _ptr(nsel), _ptr(npts), _ptr(w), w.numel(), _stream(stream)), "fp_select_nodes")
+    _check(load().fp_select_nodes(_adr(nodes), _adr(num_nodes), cap, _adr(cube), ctypes.byref(cam), _adr(ids),
+                                  _adr(nsel), _adr(npts), _adr(w), w.numel(), _raw_stream(stream)), "fp_select_nodes")
     return ids, nsel, npts
 
 
@@ -724,6 +738,6 @@ def fp_rasterize(nodes, ids, nsel, final, cam, fb=None, ws=None, stream=None):
     if fb is None:
         fb = torch.empty((cam.height, cam.width), dtype=torch.int64, device=dev)
     w = ws if ws is not None else torch.empty(max(render_workspace_size(cap), 1), dtype=torch.uint8, device=dev)
-    _check(load().fp_rasterize(_ptr(nodes), _ptr(ids), _ptr(nsel), cap, _ptr(final), final.shape[0],
-                               ctypes.byref(cam), _ptr(fb), _ptr(w), w.numel(), _stream(stream)), "fp_rasterize")
+    _check(load().fp_rasterize(_adr(nodes), _adr(ids), _adr(nsel), cap, _adr(final), final.shape[0],
+                               ctypes.byref(cam), _adr(fb), _adr(w), w.numel(), _raw_stream(stream)), "fp_rasterize")
     return fb
