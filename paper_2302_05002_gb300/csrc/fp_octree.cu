@@ -531,15 +531,18 @@ __global__ void __launch_bounds__(kRoundNT, 2) k_rounds(RoundArgs a)
 // tree.  With `upper`: the nodes at levels <= g.  The tile's counts, starts and
 // coarser sums go through shared memory, and the cells are taken 256 at a time in
 // one rolled loop each for the decisions and the appends (unrolled over a
-// thread's 16 cells the code overran the instruction cache, the top stall: 29 us
-// for the 2^21 cells of a cloud of 10^6 points, 20 us now).  Pieces for the
+// thread's 16 cells the code overran the instruction cache).  The decisions are
+// selects over the five counts around a cell, read together: as a chain of
+// branches a round of 256 cells took 900 cycles, and the few tiles that hold a
+// small cloud's points kept the whole kernel waiting: the 2^21 cells of 20,000
+// points 24 -> 17 us (21 us for 10^6 points, every tile alike, then and now).  Pieces for the
 // tables, nearly all of them on large clouds, and nodes are appended with one
 // atomic per tile, the pieces in cell order: those in work at one time then lie
 // in one or two tiles, and their scattered codes stay in L2 (appended one by one
 // as the atomics fell, k_tab_pieces took 15.5 instead of 13.0 ms for 5 * 10^8
 // uniform points, before it took its pieces in order).
 struct OpenSmem {
-    uint32_t v[kGtCells], st[kGtCells];   // points (hierarchy) and start of every cell
+    uint32_t v[kGtCells], st[kGtCells + 4];   // points (hierarchy) and start of every cell; the end
     uint32_t s1[kGtCells / 8], s2[kGtCells / 64], s3[kGtCells / 512];
     uint32_t at[kGtPer][kGtNT / 32];      // appends before a warp's 32 cells: pieces | nodes << 16
     GridTop top;
@@ -578,80 +581,94 @@ __global__ void __launch_bounds__(kGtNT, 4) k_cells_open(RoundArgs ra, const uin
         uint32_t total;
         uint32_t at = before + block_exclusive_scan<kGtNT, uint32_t>(mine, S.warp, total);
 #pragma unroll
-        for (int q = 0; q < kGtPer; ++q) { S.st[tid * kGtPer + q] = at; at += v[q]; }
+        for (int q = 0; q < kGtPer; q += 4) {
+            const uint4 w = make_uint4(at, at + v[q], at + v[q] + v[q + 1], at + v[q] + v[q + 1] + v[q + 2]);
+            *reinterpret_cast<uint4*>(&S.st[tid * kGtPer + q]) = w;
+            at = w.w + v[q + 3];
+        }
+        if (tid == kGtNT - 1) S.st[kGtCells] = at;
         if (cells && tile == gridDim.x - 1 && tid == 0) cstart[ncell] = before + total;
-        before += total;   // the end of the tile
     }
     const int up = grid_top(S.top, pyr, g, s4);   // (its barriers publish the arrays above)
     int ht = 255;                                 // leaf level at or above the tile's node
     for (int a = 0; a <= up; ++a)
         if (S.top.at(a, tile) <= c.C) ht = max(g - 4 - a, 0);   // (a grid of fewer than 4096 cells: its root)
-    auto rcount = [&](uint32_t i) {   // records of cell i of the tile
-        return same ? S.v[i] : (i + 1 < (uint32_t)kGtCells ? S.st[i + 1] : before) - S.st[i];
+    const uint32_t C = (uint32_t)min((unsigned long long)c.C, 0xFFFFFFFFull);
+    const bool lowest = g == c.lmax;
+    uint32_t topf = 0;                            // nodes at levels <= g - 4 whose first cell is the tile's first
+    if (tid == 0)
+        for (int a = 0; a <= up; ++a)
+            if (g - 4 - a >= 0 && (tile & ((1u << (3 * a)) - 1)) == 0 && S.top.at(a, tile) &&
+                (g - 4 - a == 0 || (a < up && S.top.at(a + 1, tile) > C)))
+                topf |= 16u << a;
+    // Cell i of the tile: its records, its leaf level or kInner, and the nodes whose first cell it is, bit k for
+    // level g - k: a node exists when it holds points and is the root or its parent holds more than C.
+    struct Look { uint32_t at, n, f; uint8_t hier; };
+    auto look = [&](uint32_t i) {
+        const uint32_t v = S.v[i], a1 = S.s1[i >> 3], a2 = S.s2[i >> 6], a3 = S.s3[i >> 9];
+        Look o;
+        o.at = S.st[i];
+        o.n = S.st[i + 1] - o.at;
+        int h = v <= C || lowest ? g : (int)kInner;
+        h = a1 <= C ? max(g - 1, 0) : h;
+        h = a2 <= C ? max(g - 2, 0) : h;
+        h = a3 <= C ? max(g - 3, 0) : h;
+        h = ht != 255 ? ht : h;
+        o.hier = (uint8_t)h;
+        uint32_t f = v && a1 > C ? 1u : 0u;
+        f |= (i & 7) == 0 && a1 && (g == 1 || a2 > C) ? 2u : 0u;
+        f |= (i & 63) == 0 && g >= 2 && a2 && (g == 2 || a3 > C) ? 4u : 0u;
+        f |= (i & 511) == 0 && g >= 3 && a3 && (g == 3 || s4 > C) ? 8u : 0u;
+        o.f = upper ? (i == 0 ? f | topf : f) : 0u;
+        return o;
     };
-    auto leaf_of = [&](uint32_t i) -> uint8_t {
-        if (ht != 255) return (uint8_t)ht;
-        if (S.s3[i >> 9] <= c.C) return (uint8_t)max(g - 3, 0);
-        if (S.s2[i >> 6] <= c.C) return (uint8_t)max(g - 2, 0);
-        if (S.s1[i >> 3] <= c.C) return (uint8_t)max(g - 1, 0);
-        return S.v[i] <= c.C || g == c.lmax ? (uint8_t)g : kInner;
-    };
-    // nodes whose first cell is i: levels g, g - 1 (i a multiple of 8), g - 2 (64), g - 3 (512), g - 4 and above (0)
-    auto exists = [&](int L, uint32_t cnt, uint32_t parent) { return L >= 0 && cnt && (L == 0 || parent > c.C); };
-    const bool below = s4 > c.C || g <= 4;   // nodes below the tile's
-    auto node_mask = [&](uint32_t i) {
-        uint32_t f = 0;
-        if (below) {
-            if (exists(g, S.v[i], S.s1[i >> 3])) f |= 1u;
-            if ((i & 7) == 0 && exists(g - 1, S.s1[i >> 3], S.s2[i >> 6])) f |= 2u;
-            if ((i & 63) == 0 && exists(g - 2, S.s2[i >> 6], S.s3[i >> 9])) f |= 4u;
-            if ((i & 511) == 0 && exists(g - 3, S.s3[i >> 9], s4)) f |= 8u;
-        }
-        if (i == 0)
-            for (int a = 0; a <= up; ++a)
-                if ((tile & ((1u << (3 * a)) - 1)) == 0 &&
-                    exists(g - 4 - a, S.top.at(a, tile), a < up ? S.top.at(a + 1, tile) : 0u))
-                    f |= 16u << a;
-        return f;
+    // 64 cells without a point that no node of a coarser level starts with either (the
+    // same for the whole warp): nothing to decide (LiDAR clouds fill a few percent of
+    // the cells).
+    auto idle = [&](uint32_t i) {
+        return i >= 64 && S.s2[i >> 6] == 0 && ((i & 511) >= 64 || S.s3[i >> 9] == 0);
     };
     const uint32_t in_tile = min((uint32_t)kGtCells, ncell);
-    uint32_t tab = 0;   // bit r: cell r * 256 + tid is a piece for the tables
+    uint32_t busy = 0;   // bit r (the same for the warp): the warp's cells of round r append pieces or nodes
+    auto is_tab = [&](const Look& o) { return cells && o.n && piece_list(c, o.n, g, o.hier) == LIST_TAB; };
 #pragma unroll 1
     for (int r = 0; r < kGtPer; ++r) {
         const uint32_t i = r * kGtNT + tid, m = tile * kGtCells + i;
-        const bool valid = i < in_tile;
-        const uint32_t n = valid ? rcount(i) : 0u;
-        uint8_t hier = kEmpty;
-        bool t = false;
-        if (cells && valid) {
-            const uint32_t at = S.st[i];
-            if (n) {
-                hier = leaf_of(i);
-                if (n > (uint32_t)kPieceMax) {
-                    OpenNode o;
-                    o.key = m;
-                    o.begin = at;
-                    o.count = n;
-                    o.q = (uint8_t)g;
-                    o.hier = hier;
-                    o.A = (uint8_t)g;
-                    o.buf = 0;
-                    o.tile0 = o.pad2 = o.pad3 = 0;
-                    open_node(ra, 0, o);
-                } else {
-                    const PieceList l = piece_list(c, n, g, hier);
-                    t = l == LIST_TAB;
-                    if (l == LIST_GEN)
-                        put_piece(c, l, atomicAdd(c.n[l], 1u), make_piece(at, n, g, hier, (uint8_t)g, g, 0));
+        const bool write = cells && i < in_tile;
+        uint32_t sum = 0;
+        if (idle(i)) {
+            if (write) {
+                cstart[m] = S.st[i];
+                cursor[cursor_slot(m, g)] = S.st[i];
+                c.cell_leaf[m] = kEmpty;
+            }
+        } else {
+            const Look o = look(i);
+            const PieceList l = piece_list(c, o.n, g, o.hier);
+            if (write) {
+                cstart[m] = o.at;
+                cursor[cursor_slot(m, g)] = o.at;
+                c.cell_leaf[m] = o.n ? o.hier : kEmpty;
+                if (o.n && (l == LIST_GEN || l == LIST_DUP)) {
+                    if (l == LIST_GEN) {
+                        put_piece(c, l, atomicAdd(c.n[l], 1u), make_piece(o.at, o.n, g, o.hier, (uint8_t)g, g, 0));
+                    } else {   // more than kPieceMax records
+                        OpenNode b;
+                        b.key = m;
+                        b.begin = o.at;
+                        b.count = o.n;
+                        b.q = (uint8_t)g;
+                        b.hier = o.hier;
+                        b.A = (uint8_t)g;
+                        b.buf = 0;
+                        b.tile0 = b.pad2 = b.pad3 = 0;
+                        open_node(ra, 0, b);
+                    }
                 }
             }
-            cstart[m] = at;
-            cursor[cursor_slot(m, g)] = at;
-            c.cell_leaf[m] = hier;
+            sum = __reduce_add_sync(0xFFFFFFFFu, (is_tab(o) ? 1u : 0u) | ((uint32_t)__popc(o.f) << 16));
+            if (sum) busy |= 1u << r;
         }
-        const uint32_t nodes = upper && valid ? __popc(node_mask(i)) : 0u;
-        if (t) tab |= 1u << r;
-        const uint32_t sum = __reduce_add_sync(0xFFFFFFFFu, (t ? 1u : 0u) | (nodes << 16));
         if (lane == 0) S.at[r][warp] = sum;
     }
     __syncthreads();
@@ -669,29 +686,29 @@ __global__ void __launch_bounds__(kGtNT, 4) k_cells_open(RoundArgs ra, const uin
         if (total == 0) return;
     }
 #pragma unroll 1
-    for (int r = 0; r < kGtPer; ++r) {
+    for (; busy; busy &= busy - 1) {
+        const int r = __ffs(busy) - 1;
         const uint32_t i = r * kGtNT + tid, m = tile * kGtCells + i;
-        const bool t = (tab >> r) & 1u;
-        const uint32_t f = upper && i < in_tile ? node_mask(i) : 0u;
-        const uint32_t mine = (t ? 1u : 0u) | ((uint32_t)__popc(f) << 16);
-        if (!__any_sync(0xFFFFFFFFu, mine != 0)) continue;
+        const Look o = look(i);
+        const bool t = is_tab(o);
+        const uint32_t mine = (t ? 1u : 0u) | ((uint32_t)__popc(o.f) << 16);
         uint32_t inc = mine;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
-            if (lane >= o) inc += y;
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+            if (lane >= d) inc += y;
         }
-        const uint32_t ex = S.at[r][warp] + inc - mine, at = i < in_tile ? S.st[i] : 0u;
+        const uint32_t ex = S.at[r][warp] + inc - mine;
         if (t)
-            put_piece(c, LIST_TAB, S.base[0] + (ex & 0xFFFFu), make_piece(at, rcount(i), g, leaf_of(i), (uint8_t)g, g, 0));
+            put_piece(c, LIST_TAB, S.base[0] + (ex & 0xFFFFu), make_piece(o.at, o.n, g, o.hier, (uint8_t)g, g, 0));
         uint32_t ni = S.base[1] + (ex >> 16);
 #pragma unroll 1
-        for (uint32_t todo = f; todo; todo &= todo - 1) {
+        for (uint32_t todo = o.f; todo; todo &= todo - 1) {
             const int k = __ffs(todo) - 1;   // levels above the cell
             const int lev = g - k;
             const uint32_t cnt = k == 0 ? S.v[i] : (k == 1 ? S.s1[i >> 3] : (k == 2 ? S.s2[i >> 6] : (k == 3 ? S.s3[i >> 9]
                                                                                                    : S.top.at(k - 4, tile))));
-            put_node(c, ni++, m >> (3 * k), lev, cnt, at, cnt <= c.C || lev == c.lmax);
+            put_node(c, ni++, m >> (3 * k), lev, cnt, o.at, cnt <= C || lev == c.lmax);
         }
     }
 }
@@ -1631,15 +1648,17 @@ constexpr uint64_t kLayoutWhole = 1ull << 21;
 // level-g ancestor, whose ids are consecutive in preorder: the search runs over
 // that subtree only, with the point's key at max_level (32-bit for max_level
 // <= 10) -- only then is the point itself read.  leafid (nullable): the leaf id.
-// Owned counts are summed per tile of kResolveTile consecutive points in a
+// Owned counts are summed per tile of consecutive points in a
 // shared-memory table keyed by node id (open addressing, bounded probes; a point
 // that finds no slot adds to the global count directly), then flushed with one
 // global atomic per node of the tile: consecutive points lie in one chunk, whose
 // owners are few, and the nodes above the chunks (the root owns a point of every
 // occupied level-s cell) are not hit by an atomic per point.
+// Tiles of 4096 points, of 1024 for clouds of up to kResolveSmall points, whose few
+// large tiles left most SMs idle: 20,000 points 11 -> 6 us (5 blocks before); 500,000 points 9 -> 6 us.
 constexpr int kResolveNT = 256;
-constexpr int kResolveIPT = 16;
-constexpr int kResolveTile = kResolveNT * kResolveIPT;
+constexpr int kResolveIPT = 16, kResolveIPTSmall = 4;
+constexpr uint64_t kResolveSmall = 1ull << 19;
 constexpr int kOwnSlots = 1024;   // power of two
 constexpr int kOwnProbes = 32;
 constexpr int kResolveTabLevel = 4;   // node ids of the levels 0..4 in shared memory
@@ -1688,7 +1707,7 @@ __device__ __noinline__ uint32_t deep_id(const fp_point* __restrict__ pts, uint6
     return rr != kNone ? c0 + rr : kNone;
 }
 
-template <bool SMALL>
+template <bool SMALL, int kResolveIPT>
 __global__ void __launch_bounds__(kResolveNT) k_resolve(const fp_point* __restrict__ pts, uint64_t n,
                                                         const fp_cube* cube, const uint32_t* codes,
                                                         const uint32_t* idxtab, const uint64_t* sorted_start,
@@ -1704,6 +1723,7 @@ __global__ void __launch_bounds__(kResolveNT) k_resolve(const fp_point* __restri
     for (uint32_t q = threadIdx.x; q < ntab; q += kResolveNT) s_idx[q] = idxtab[q];
     const uint32_t M = *nnode;
     const int nt = leafid ? 2 : 1;
+    constexpr uint64_t kResolveTile = (uint64_t)kResolveNT * kResolveIPT;
     const uint64_t ntiles = (n + kResolveTile - 1) / kResolveTile;
     for (int q = threadIdx.x; q < kOwnSlots; q += kResolveNT) { s_key[q] = kNone; s_cnt[q] = 0; }
     for (uint64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
@@ -1753,6 +1773,20 @@ __global__ void __launch_bounds__(kResolveNT) k_resolve(const fp_point* __restri
             }
         }
     }
+}
+
+typedef void (*ResolveKernel)(const fp_point*, uint64_t, const fp_cube*, const uint32_t*, const uint32_t*,
+                              const uint64_t*, const uint8_t*, const uint32_t*, const uint32_t*, uint32_t*, uint32_t*,
+                              OwnCounts, int, int, uint32_t*);
+
+// the variant for n points, and its grid
+static ResolveKernel resolve_kernel(uint64_t n, int lmax, int num_sms, int& grid)
+{
+    const bool few = n <= kResolveSmall;
+    const uint64_t tile = (uint64_t)kResolveNT * (few ? kResolveIPTSmall : kResolveIPT);
+    grid = (int)std::max<uint64_t>(1, std::min<uint64_t>((n + tile - 1) / tile, (uint64_t)num_sms * 8));
+    if (lmax <= 10) return few ? k_resolve<true, kResolveIPTSmall> : k_resolve<true, kResolveIPT>;
+    return few ? k_resolve<false, kResolveIPTSmall> : k_resolve<false, kResolveIPT>;
 }
 
 __global__ void k_write_nown(fp_node* nodes, const uint32_t* nnode, uint32_t node_cap, const uint32_t* n_own)
@@ -2042,9 +2076,8 @@ cudaError_t launch_octree_impl(const fp_point* sorted, const uint32_t* perm, uin
     }
     // 6. owner and leaf ids per distributed point, owned counts
     {
-        const int grid = (int)std::max<uint64_t>(
-            1, std::min<uint64_t>((N + kResolveTile - 1) / kResolveTile, (uint64_t)ws.num_sms * 8));
-        auto kres = lmax <= 10 ? k_resolve<true> : k_resolve<false>;
+        int grid;
+        const ResolveKernel kres = resolve_kernel(N, lmax, ws.num_sms, grid);
         // counted in the node records (zeroed with the table)
         const OwnCounts own{reinterpret_cast<uint32_t*>(nodes) + offsetof(fp_node, n_own) / sizeof(uint32_t),
                             sizeof(fp_node) / sizeof(uint32_t), node_cap};
@@ -2159,9 +2192,8 @@ cudaError_t launch_octree_resolve(const fp_point* pts, uint64_t n, const fp_cube
                                   uint32_t* owner, const Workspace& ws, cudaStream_t st)
 {
     if (n == 0) return cudaSuccess;
-    const int grid = (int)std::max<uint64_t>(
-        1, std::min<uint64_t>((n + kResolveTile - 1) / kResolveTile, (uint64_t)ws.num_sms * 8));
-    auto kres = prm.max_level <= 10 ? k_resolve<true> : k_resolve<false>;
+    int grid;
+    const ResolveKernel kres = resolve_kernel(n, (int)prm.max_level, ws.num_sms, grid);
     kres<<<grid, kResolveNT, 0, st>>>(pts, n, cube, codes, T.idxtab, T.starts, T.slevel, T.ndesc, T.nnode, owner, nullptr,
                                OwnCounts{T.nown, 1u, 0xFFFFFFFFu}, (int)prm.grid_log2, (int)prm.max_level, ws.err);
     return cudaGetLastError();

@@ -268,6 +268,16 @@ struct SegCall {
     uint32_t *st_rank, *st_list, *st_nrank, *st_soff;
 };
 
+// distribution of up to kDistCluster points in one launch (tmp: n words each;
+// hist: kClCtas * 256 words).  At 32,768 points 27 us and 45 us by the sweep with 37
+// chunks (one pass), 38 and 51 us with 1268 (two); its time grows with the points,
+// 1 us per 2000, and would meet the sweep's near 65,000.
+constexpr uint64_t kDistCluster = 1ull << 15;
+cudaError_t dist_cluster(const int4* pts, uint64_t n, const fp_cube* cube, int g, const uint32_t* lut,
+                         const uint64_t* offsets, const uint32_t* num_chunks, int4* out, uint32_t* perm,
+                         const uint32_t* cells, uint32_t* const tmp[4], uint32_t* hist, uint32_t* err, cudaStream_t st);
+
+
 // Distribution of n points into up to 4096 chunks by the counting pass and a
 // double-buffered sweep (fp_seg.cu); the points' cells given or computed.
 // chunk_tmp: n chunk ids, 16-byte aligned.  *run_sort is set to 1, and hist

@@ -4,7 +4,7 @@
 // a node of the global tree, Fig. "octree") is a stable scatter of the points by
 // chunk id, looked up from the point's level-g cell (lut).  Up to 4096 chunks the
 // count and sweep of fp_seg.cu; more take two or three least-significant-digit-
-// first passes, chosen on the device.
+// first passes, chosen on the device.  Small clouds take one launch (k_dist_cluster).
 #include "fp_seg.cuh"
 
 namespace fp {
@@ -139,6 +139,12 @@ cudaError_t launch_distribute(const fp_point* pts, uint64_t n, const fp_cube* cu
     uint32_t* run_sort = ws.take<uint32_t>(1);
     Workspace rest = ws;
     KTimerScope kt(FP_KERNEL_DISTRIBUTE, st);
+    if (n <= kDistCluster) {
+        uint32_t* const w = reinterpret_cast<uint32_t*>(pt_tmp);   // four words a point
+        uint32_t* const tmp[4] = {w, w + n, w + 2 * n, w + 3 * n};
+        return dist_cluster(reinterpret_cast<const int4*>(pts), n, cube, g, lut, offsets, num_chunks,
+                            reinterpret_cast<int4*>(out), perm, cells, tmp, sc.hist, ws.err, st);
+    }
     // Up to 4096 chunks: the count, scan and double-buffered sweep (every point's
     // chunk kept in val_tmp, which the radix passes below then do not use), from
     // the cells or from the points.  More: the radix passes, which compute the
