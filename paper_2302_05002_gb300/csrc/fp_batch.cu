@@ -55,7 +55,8 @@ constexpr int kFusedMax = 256;
 constexpr int kFbNT = 256;
 constexpr int kFbIPT = 16;
 constexpr int kFbTile = kFbNT * kFbIPT;   // 4096 points per preview tile (the layout does not depend on it)
-constexpr int kFcTiles = 16;              // count work item: 16 tiles (65,536 points)
+constexpr int kFcTiles = 4;               // count work item: 4 tiles (16,384 points); of 16 tiles, 3 or 4 items
+                                          // an SM: 48 clouds, 32M points 434 -> 294 us
 
 struct FusedCloud {
     const int4* pts;
@@ -89,32 +90,50 @@ FP_DEV uint32_t fused_cloud(const uint64_t* first, uint32_t ncloud, uint64_t t)
     return a;
 }
 
-// zero every count grid and preview count, open every cube's extents
-__global__ void k_fused_init(const __grid_constant__ FusedArgs a)
+// zero every count grid, preview count, look-back word and work counter, open
+// every cube's extents: kFiParts blocks per cloud (one each wrote at 1.9 TB/s:
+// 48 clouds 214 -> 61 us)
+constexpr uint32_t kFiParts = 32;
+
+__global__ void __launch_bounds__(256) k_fused_init(const __grid_constant__ FusedArgs a, uint64_t* status,
+                                                    uint32_t* counter)
 {
-    for (uint32_t c = blockIdx.x; c < a.ncloud; c += gridDim.x) {
-        const FusedCloud& d = a.c[c];
-        const uint64_t cells = 1ull << (3 * d.g);
-        for (uint64_t m = threadIdx.x; m < cells; m += blockDim.x) d.counts[m] = 0;
-        if (threadIdx.x == 0) {
-            *d.prev_cnt = 0;
-            for (int k = 0; k < 3; ++k) { d.cube->o[k] = INT32_MAX; d.cube->mx[k] = INT32_MIN; }
-            d.cube->S = 0;
-        }
+    const uint32_t part = blockIdx.x % kFiParts;
+    const FusedCloud& d = a.c[blockIdx.x / kFiParts];
+    const uint64_t cells = 1ull << (3 * d.g);   // (a multiple of 8)
+    const uint64_t t = part * 256 + threadIdx.x;
+    if ((reinterpret_cast<uintptr_t>(d.counts) & 15u) == 0) {
+        for (uint64_t m = t; m < cells / 4; m += kFiParts * 256)
+            reinterpret_cast<uint4*>(d.counts)[m] = make_uint4(0u, 0u, 0u, 0u);
+    } else {
+        for (uint64_t m = t; m < cells; m += kFiParts * 256) d.counts[m] = 0;
+    }
+    const uint64_t ntiles = a.tile0[a.ncloud];
+    for (uint64_t m = (uint64_t)blockIdx.x * 256 + threadIdx.x; m < ntiles; m += (uint64_t)gridDim.x * 256) status[m] = 0;
+    if (blockIdx.x == 0 && threadIdx.x < 4) counter[threadIdx.x] = 0;
+    if (t == 0) {
+        *d.prev_cnt = 0;
+        for (int k = 0; k < 3; ++k) { d.cube->o[k] = INT32_MAX; d.cube->mx[k] = INT32_MIN; }
+        d.cube->S = 0;
     }
 }
 
 // bounds + preview of every tile of every cloud: per-axis extents folded into
 // the cloud's cube by atomics; kept points compacted in index order by a
-// decoupled look-back that stops at the cloud's first tile
-__global__ void __launch_bounds__(kFbNT, 2) k_fused_bounds_decimate(const __grid_constant__ FusedArgs a,
+// decoupled look-back that stops at the cloud's first tile.  A tile's points go
+// through registers eight at a time and the kept ones are read again (one in
+// `modulus`, from L2): held until the tile's place was known they took half the
+// register file, two blocks an SM, and one thread walked the look-back words: 32M
+// points of 48 clouds 231 -> 161 us.
+__global__ void __launch_bounds__(kFbNT, 4) k_fused_bounds_decimate(const __grid_constant__ FusedArgs a,
                                                                     uint64_t* status, uint32_t* counter,
                                                                     uint32_t* err)
 {
+    constexpr int kBatch = 8, kWarps = kFbNT / 32;
     __shared__ uint32_t s_item[2];
-    __shared__ uint32_t s_cnt[kFbIPT][kFbNT / 32];
+    __shared__ uint32_t s_cnt[kFbIPT][kWarps];
     __shared__ uint64_t s_base;
-    __shared__ int32_t s_red[6][kFbNT / 32];
+    __shared__ int32_t s_red[6][kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint64_t ntiles = a.tile0[a.ncloud];
     for (;;) {
@@ -126,41 +145,37 @@ __global__ void __launch_bounds__(kFbNT, 2) k_fused_bounds_decimate(const __grid
         __syncthreads();
         const uint64_t t = s_item[0];
         const uint32_t c = s_item[1];
-        __syncthreads();
         if (t >= ntiles) break;
         const FusedCloud& d = a.c[c];
-        const uint64_t t0 = a.tile0[c], tl = t - t0, nt = a.tile0[c + 1] - t0;
-        constexpr uint64_t kFlagAgg = 1ull << 62, kFlagInc = 2ull << 62, kValMask = (1ull << 62) - 1;
+        const uint64_t t0 = a.tile0[c], tl = t - t0, nt = a.tile0[c + 1] - t0, n = d.n;
         const uint64_t base = tl * kFbTile;
-        int4 pv[kFbIPT];
-#pragma unroll
-        for (int r = 0; r < kFbIPT; ++r) {   // all loads in flight together
-            const uint64_t i = base + (uint64_t)r * kFbNT + threadIdx.x;
-            pv[r] = i < d.n ? ld_point_cs(reinterpret_cast<const fp_point*>(d.pts), i) : make_int4(0, 0, 0, 0);
-        }
+        const KeepMultiple keep = d.mult;
         uint32_t keepmask = 0;
+        int32_t lo[3] = {INT32_MAX, INT32_MAX, INT32_MAX}, hi[3] = {INT32_MIN, INT32_MIN, INT32_MIN};
+#pragma unroll 1
+        for (int r0 = 0; r0 < kFbIPT; r0 += kBatch) {
+            int4 p[kBatch];
 #pragma unroll
-        for (int r = 0; r < kFbIPT; ++r) {
-            const uint64_t i = base + (uint64_t)r * kFbNT + threadIdx.x;
-            bool k = false;
-            if (i < d.n) {
-                k = d.mult(i);
+            for (int r = 0; r < kBatch; ++r) {   // all loads in flight together
+                const uint64_t i = base + (uint64_t)(r0 + r) * kFbNT + threadIdx.x;
+                p[r] = __ldg(d.pts + (i < n ? i : base));   // (a point of the tile again beyond the end)
             }
-            const uint32_t bal = __ballot_sync(0xFFFFFFFFu, k);
-            if (lane == 0) s_cnt[r][warp] = __popc(bal);
-            keepmask |= (uint32_t)k << r;
+#pragma unroll
+            for (int r = 0; r < kBatch; ++r) {
+                const uint64_t i = base + (uint64_t)(r0 + r) * kFbNT + threadIdx.x;
+                const bool k = i < n && keep(i);
+                const uint32_t bal = __ballot_sync(0xFFFFFFFFu, k);
+                if (lane == 0) s_cnt[r0 + r][warp] = __popc(bal);
+                keepmask |= (uint32_t)k << (r0 + r);
+            }
+#pragma unroll
+            for (int r = 0; r < kBatch; ++r) {
+                lo[0] = min(lo[0], p[r].x); hi[0] = max(hi[0], p[r].x);
+                lo[1] = min(lo[1], p[r].y); hi[1] = max(hi[1], p[r].y);
+                lo[2] = min(lo[2], p[r].z); hi[2] = max(hi[2], p[r].z);
+            }
         }
         // extents of the tile, folded into the cloud's cube
-        int32_t lo[3] = {INT32_MAX, INT32_MAX, INT32_MAX}, hi[3] = {INT32_MIN, INT32_MIN, INT32_MIN};
-#pragma unroll
-        for (int r = 0; r < kFbIPT; ++r) {
-            const uint64_t i = base + (uint64_t)r * kFbNT + threadIdx.x;
-            if (i < d.n) {
-                lo[0] = min(lo[0], pv[r].x); hi[0] = max(hi[0], pv[r].x);
-                lo[1] = min(lo[1], pv[r].y); hi[1] = max(hi[1], pv[r].y);
-                lo[2] = min(lo[2], pv[r].z); hi[2] = max(hi[2], pv[r].z);
-            }
-        }
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             lo[k] = __reduce_min_sync(0xFFFFFFFFu, lo[k]);
@@ -169,22 +184,21 @@ __global__ void __launch_bounds__(kFbNT, 2) k_fused_bounds_decimate(const __grid
         if (lane == 0)
             for (int k = 0; k < 3; ++k) { s_red[k][warp] = lo[k]; s_red[3 + k][warp] = hi[k]; }
         __syncthreads();
-        if (threadIdx.x < 6) {
-            const int k = threadIdx.x;
-            int32_t v = s_red[k][0];
-            for (int w = 1; w < kFbNT / 32; ++w) v = k < 3 ? min(v, s_red[k][w]) : max(v, s_red[k][w]);
-            if (k < 3) atomicMin(&d.cube->o[k], v);
-            else atomicMax(&d.cube->mx[k - 3], v);
+        if (threadIdx.x >= kFbNT - 32 && lane < 6) {   // the last warp (the first one looks back)
+            int32_t v = s_red[lane][0];
+            for (int w = 1; w < kWarps; ++w) v = lane < 3 ? min(v, s_red[lane][w]) : max(v, s_red[lane][w]);
+            if (lane < 3) atomicMin(&d.cube->o[lane], v);
+            else atomicMax(&d.cube->mx[lane - 3], v);
         }
         // exclusive scan of the keep counts over (r, warp) order = index order, then the look-back
         if (threadIdx.x < 32) {
-            constexpr int per = kFbIPT * (kFbNT / 32) / 32;
+            constexpr int per = kFbIPT * kWarps / 32;
             uint32_t v[per];
             uint32_t s = 0;
 #pragma unroll
             for (int q = 0; q < per; ++q) {
                 const int e = lane * per + q;
-                v[q] = s_cnt[e / (kFbNT / 32)][e % (kFbNT / 32)];
+                v[q] = s_cnt[e / kWarps][e % kWarps];
                 s += v[q];
             }
             uint32_t x = s;
@@ -198,47 +212,23 @@ __global__ void __launch_bounds__(kFbNT, 2) k_fused_bounds_decimate(const __grid
 #pragma unroll
             for (int q = 0; q < per; ++q) {
                 const int e = lane * per + q;
-                s_cnt[e / (kFbNT / 32)][e % (kFbNT / 32)] = ex;
+                s_cnt[e / kWarps][e % kWarps] = ex;
                 ex += v[q];
             }
-            if (lane == 0) {
-                uint64_t excl = 0;
-                if (tl == 0) {
-                    atomicExch((unsigned long long*)&status[t], (unsigned long long)(kFlagInc | total));
-                } else {
-                    atomicExch((unsigned long long*)&status[t], (unsigned long long)(kFlagAgg | total));
-                    int64_t q = (int64_t)t - 1;
-                    uint32_t spins = 0;
-                    while (q >= (int64_t)t0) {
-                        const uint64_t s2 = ld_volatile64(&status[q]);
-                        if ((s2 >> 62) == 0) {
-                            if (++spins > kSpinLimit) { raise(err, FP_ERR_TIMEOUT); break; }
-                            continue;
-                        }
-                        excl += s2 & kValMask;
-                        if ((s2 >> 62) == 2) break;
-                        --q;
-                    }
-                    atomicExch((unsigned long long*)&status[t], (unsigned long long)(kFlagInc | (excl + total)));
-                }
-                s_base = excl;
-                if (tl == nt - 1) {
-                    *d.prev_cnt = excl + total;
-                    if (excl + total > d.prev_cap) raise(err, FP_ERR_CAPACITY, 0);
-                }
-            }
+            const uint64_t excl = preview_base(status + t0, tl, nt, total, d.prev_cap, d.prev_cnt, err);
+            if (lane == 0) s_base = excl;
         }
         __syncthreads();
-#pragma unroll
+#pragma unroll 4
         for (int r = 0; r < kFbIPT; ++r) {
             const bool kept = (keepmask >> r) & 1u;
             const uint32_t bal = __ballot_sync(0xFFFFFFFFu, kept);
             if (kept) {
                 const uint64_t pos = s_base + s_cnt[r][warp] + __popc(bal & lanemask_lt());
-                if (pos < d.prev_cap) d.prev[pos] = pv[r];
+                if (pos < d.prev_cap) d.prev[pos] = __ldg(d.pts + base + (uint64_t)r * kFbNT + threadIdx.x);
             }
         }
-        __syncthreads();
+        // (the next tile's first barrier is passed after these reads; its counts are written behind it)
     }
 }
 
@@ -448,11 +438,9 @@ fp_status fused_first(const fp_cloud_desc* c, uint32_t g0, uint32_t g1, const fp
     w.base = ws;
     uint64_t* status = w.take<uint64_t>(tiles ? tiles : 1);
     uint32_t* counter = w.take<uint32_t>(4);
-    if (cudaMemsetAsync(status, 0, 8 * (tiles ? tiles : 1), st) != cudaSuccess) return FP_ERR_CUDA;
-    if (cudaMemsetAsync(counter, 0, 16, st) != cudaSuccess) return FP_ERR_CUDA;
-    k_fused_init<<<(int)std::min<uint32_t>(a.ncloud, 1024u), 256, 0, st>>>(a);
+    k_fused_init<<<a.ncloud * kFiParts, 256, 0, st>>>(a, status, counter);
     if (tiles) {
-        const int gb = (int)std::max<uint64_t>(1, std::min<uint64_t>(tiles, (uint64_t)num_sms * 2));
+        const int gb = (int)std::max<uint64_t>(1, std::min<uint64_t>(tiles, (uint64_t)num_sms * 4));
         k_fused_bounds_decimate<<<gb, kFbNT, 0, st>>>(a, status, counter, err);
     }
     k_fused_cube<<<1, 256, 0, st>>>(a);
