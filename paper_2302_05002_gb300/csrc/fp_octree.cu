@@ -529,22 +529,26 @@ __global__ void __launch_bounds__(kRoundNT, 2) k_rounds(RoundArgs a)
 // without a record.  Cells with at most kPieceMax records become pieces
 // (k_small_pieces finds the smallest by itself); larger ones open the split
 // tree.  With `upper`: the nodes at levels <= g.  The tile's counts, starts and
-// coarser sums go through shared memory, and the cells are taken 256 at a time in
-// one rolled loop each for the decisions and the appends (unrolled over a
-// thread's 16 cells the code overran the instruction cache).  The decisions are
-// selects over the five counts around a cell, read together: as a chain of
-// branches a round of 256 cells took 900 cycles, and the few tiles that hold a
-// small cloud's points kept the whole kernel waiting: the 2^21 cells of 20,000
-// points 24 -> 17 us (21 us for 10^6 points, every tile alike, then and now).  Pieces for the
-// tables, nearly all of them on large clouds, and nodes are appended with one
-// atomic per tile, the pieces in cell order: those in work at one time then lie
-// in one or two tiles, and their scattered codes stay in L2 (appended one by one
-// as the atomics fell, k_tab_pieces took 15.5 instead of 13.0 ms for 5 * 10^8
-// uniform points, before it took its pieces in order).
-struct OpenSmem {
+// coarser sums go through shared memory, and the cells are taken 1024 at a time,
+// four neighbours per thread, in one rolled loop each for the decisions and the
+// appends (unrolled over a thread's 16 cells the code overran the instruction
+// cache).  The decisions are selects over the counts around the four cells, read
+// together, and the four starts, cursors and leaf levels are stored as one vector
+// each: bound by instructions (120 a cell of its own at one cell per thread and
+// round; as a chain of branches a round took 900 cycles of latency on top, and the
+// few tiles that hold a small cloud's points kept the whole kernel waiting).  The
+// 2^21 cells of 10^6 points: 29 -> 21 -> 15 us, of 20,000 points: 24 -> 14 us.
+// Pieces for the tables, nearly all of them on large clouds, and nodes are appended
+// with one atomic per tile, the pieces in cell order: those in work at one time
+// then lie in one or two tiles, and their scattered codes stay in L2 (appended one
+// by one as the atomics fell, k_tab_pieces took 15.5 instead of 13.0 ms for
+// 5 * 10^8 uniform points, before it took its pieces in order).
+constexpr int kOpenRounds = kGtPer / 4;
+
+struct __align__(16) OpenSmem {
     uint32_t v[kGtCells], st[kGtCells + 4];   // points (hierarchy) and start of every cell; the end
     uint32_t s1[kGtCells / 8], s2[kGtCells / 64], s3[kGtCells / 512];
-    uint32_t at[kGtPer][kGtNT / 32];      // appends before a warp's 32 cells: pieces | nodes << 16
+    uint32_t at[kOpenRounds][kGtNT / 32]; // appends before a warp's 128 cells: pieces | nodes << 16
     GridTop top;
     uint32_t warp[kGtNT / 32], base[2];
 };
@@ -601,64 +605,89 @@ __global__ void __launch_bounds__(kGtNT, 4) k_cells_open(RoundArgs ra, const uin
             if (g - 4 - a >= 0 && (tile & ((1u << (3 * a)) - 1)) == 0 && S.top.at(a, tile) &&
                 (g - 4 - a == 0 || (a < up && S.top.at(a + 1, tile) > C)))
                 topf |= 16u << a;
-    // Cell i of the tile: its records, its leaf level or kInner, and the nodes whose first cell it is, bit k for
-    // level g - k: a node exists when it holds points and is the root or its parent holds more than C.
-    struct Look { uint32_t at, n, f; uint8_t hier; };
+    const bool tab_g = piece_depth(c, g, (uint8_t)g) <= kHashMaxD;   // table pieces whose leaf is the cell
+    // Cells i .. i + 3 of the tile (i a multiple of 4): their starts and the end, their leaf levels or kInner, the
+    // ones that are table pieces, and the nodes whose first cell is one of them: bit k < 8 for level g - k at cell
+    // i, bits 8 .. 10 for level g at the others.  A node exists when it holds points and is the root or its parent
+    // holds more than C.
+    struct Look {
+        uint4 v, st;
+        uint32_t end, hier, tab, f;   // hier: a byte per cell
+    };
     auto look = [&](uint32_t i) {
-        const uint32_t v = S.v[i], a1 = S.s1[i >> 3], a2 = S.s2[i >> 6], a3 = S.s3[i >> 9];
+        const uint32_t a1 = S.s1[i >> 3], a2 = S.s2[i >> 6], a3 = S.s3[i >> 9];
         Look o;
-        o.at = S.st[i];
-        o.n = S.st[i + 1] - o.at;
-        int h = v <= C || lowest ? g : (int)kInner;
+        o.v = *reinterpret_cast<const uint4*>(&S.v[i]);
+        o.st = *reinterpret_cast<const uint4*>(&S.st[i]);
+        o.end = S.st[i + 4];
+        int h = -1;   // leaf level above the cells
         h = a1 <= C ? max(g - 1, 0) : h;
         h = a2 <= C ? max(g - 2, 0) : h;
         h = a3 <= C ? max(g - 3, 0) : h;
         h = ht != 255 ? ht : h;
-        o.hier = (uint8_t)h;
-        uint32_t f = v && a1 > C ? 1u : 0u;
-        f |= (i & 7) == 0 && a1 && (g == 1 || a2 > C) ? 2u : 0u;
-        f |= (i & 63) == 0 && g >= 2 && a2 && (g == 2 || a3 > C) ? 4u : 0u;
-        f |= (i & 511) == 0 && g >= 3 && a3 && (g == 3 || s4 > C) ? 8u : 0u;
-        o.f = upper ? (i == 0 ? f | topf : f) : 0u;
+        const bool tab_h = h >= 0 && piece_depth(c, g, (uint8_t)h) <= kHashMaxD;
+        o.hier = o.tab = o.f = 0;
+        auto cell = [&](int q, uint32_t v, uint32_t n) {
+            const bool own = v <= C || lowest;   // (h < 0) the cell is a leaf
+            const uint32_t hq = h >= 0 ? (uint32_t)h : (own ? (uint32_t)g : (uint32_t)kInner);
+            o.hier |= (n ? hq : (uint32_t)kEmpty) << (8 * q);
+            if (n > (uint32_t)kSmallMax && n <= (uint32_t)kPieceMax && (h >= 0 ? tab_h : own && tab_g)) o.tab |= 1u << q;
+            if (v && a1 > C) o.f |= q ? 128u << q : 1u;
+        };
+        cell(0, o.v.x, o.st.y - o.st.x);
+        cell(1, o.v.y, o.st.z - o.st.y);
+        cell(2, o.v.z, o.st.w - o.st.z);
+        cell(3, o.v.w, o.end - o.st.w);
+        o.f |= (i & 7) == 0 && a1 && (g == 1 || a2 > C) ? 2u : 0u;
+        o.f |= (i & 63) == 0 && g >= 2 && a2 && (g == 2 || a3 > C) ? 4u : 0u;
+        o.f |= (i & 511) == 0 && g >= 3 && a3 && (g == 3 || s4 > C) ? 8u : 0u;
+        o.f |= i == 0 ? topf : 0u;
+        o.f = upper ? o.f : 0u;
+        o.tab = cells ? o.tab : 0u;
         return o;
     };
-    // 64 cells without a point that no node of a coarser level starts with either (the
-    // same for the whole warp): nothing to decide (LiDAR clouds fill a few percent of
-    // the cells).
+    auto start_of = [](const Look& o, int q) { return q == 0 ? o.st.x : (q == 1 ? o.st.y : (q == 2 ? o.st.z : o.st.w)); };
+    auto end_of = [](const Look& o, int q) { return q == 0 ? o.st.y : (q == 1 ? o.st.z : (q == 2 ? o.st.w : o.end)); };
+    auto hier_of = [](const Look& o, int q) { return (uint8_t)(o.hier >> (8 * q)); };
+    // 64 cells without a point that no node of a coarser level starts with either:
+    // nothing to decide (LiDAR clouds fill a few percent of the cells)
     auto idle = [&](uint32_t i) {
         return i >= 64 && S.s2[i >> 6] == 0 && ((i & 511) >= 64 || S.s3[i >> 9] == 0);
     };
     const uint32_t in_tile = min((uint32_t)kGtCells, ncell);
     uint32_t busy = 0;   // bit r (the same for the warp): the warp's cells of round r append pieces or nodes
-    auto is_tab = [&](const Look& o) { return cells && o.n && piece_list(c, o.n, g, o.hier) == LIST_TAB; };
 #pragma unroll 1
-    for (int r = 0; r < kGtPer; ++r) {
-        const uint32_t i = r * kGtNT + tid, m = tile * kGtCells + i;
+    for (int r = 0; r < kOpenRounds; ++r) {
+        const uint32_t i = (r * kGtNT + tid) * 4, m = tile * kGtCells + i;
         const bool write = cells && i < in_tile;
         uint32_t sum = 0;
-        if (idle(i)) {
+        if (__all_sync(0xFFFFFFFFu, idle(i))) {
             if (write) {
-                cstart[m] = S.st[i];
-                cursor[cursor_slot(m, g)] = S.st[i];
-                c.cell_leaf[m] = kEmpty;
+                const uint4 st = *reinterpret_cast<const uint4*>(&S.st[i]);
+                *reinterpret_cast<uint4*>(cstart + m) = st;
+                *reinterpret_cast<uint4*>(cursor + cursor_slot(m, g)) = st;
+                *reinterpret_cast<uint32_t*>(c.cell_leaf + m) = kEmpty * 0x01010101u;
             }
         } else {
             const Look o = look(i);
-            const PieceList l = piece_list(c, o.n, g, o.hier);
             if (write) {
-                cstart[m] = o.at;
-                cursor[cursor_slot(m, g)] = o.at;
-                c.cell_leaf[m] = o.n ? o.hier : kEmpty;
-                if (o.n && (l == LIST_GEN || l == LIST_DUP)) {
-                    if (l == LIST_GEN) {
-                        put_piece(c, l, atomicAdd(c.n[l], 1u), make_piece(o.at, o.n, g, o.hier, (uint8_t)g, g, 0));
-                    } else {   // more than kPieceMax records
+                *reinterpret_cast<uint4*>(cstart + m) = o.st;
+                *reinterpret_cast<uint4*>(cursor + cursor_slot(m, g)) = o.st;
+                *reinterpret_cast<uint32_t*>(c.cell_leaf + m) = o.hier;
+#pragma unroll 1
+                for (int q = 0; q < 4; ++q) {   // what is neither empty, small nor for the tables
+                    const uint32_t at = start_of(o, q), n = end_of(o, q) - at;
+                    const uint8_t h = hier_of(o, q);
+                    if (n == 0 || ((o.tab >> q) & 1u) || (n <= (uint32_t)kSmallMax && h != kInner)) continue;
+                    if (n <= (uint32_t)kPieceMax) {
+                        put_piece(c, LIST_GEN, atomicAdd(c.n[LIST_GEN], 1u), make_piece(at, n, g, h, (uint8_t)g, g, 0));
+                    } else {
                         OpenNode b;
-                        b.key = m;
-                        b.begin = o.at;
-                        b.count = o.n;
+                        b.key = m + q;
+                        b.begin = at;
+                        b.count = n;
                         b.q = (uint8_t)g;
-                        b.hier = o.hier;
+                        b.hier = h;
                         b.A = (uint8_t)g;
                         b.buf = 0;
                         b.tile0 = b.pad2 = b.pad3 = 0;
@@ -666,18 +695,18 @@ __global__ void __launch_bounds__(kGtNT, 4) k_cells_open(RoundArgs ra, const uin
                     }
                 }
             }
-            sum = __reduce_add_sync(0xFFFFFFFFu, (is_tab(o) ? 1u : 0u) | ((uint32_t)__popc(o.f) << 16));
+            sum = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)__popc(o.tab) | ((uint32_t)__popc(o.f) << 16));
             if (sum) busy |= 1u << r;
         }
         if (lane == 0) S.at[r][warp] = sum;
     }
     __syncthreads();
-    {   // the 128 runs of 32 cells in order; one atomic each for the tile's pieces and nodes
+    {   // the 32 runs of 128 cells in order; one atomic each for the tile's pieces and nodes
         uint32_t* at = &S.at[0][0];
-        const uint32_t v = tid < kGtPer * (kGtNT / 32) ? at[tid] : 0u;
+        const uint32_t v = tid < kOpenRounds * (kGtNT / 32) ? at[tid] : 0u;
         uint32_t total;
         const uint32_t ex = block_exclusive_scan<kGtNT, uint32_t>(v, S.warp, total);
-        if (tid < kGtPer * (kGtNT / 32)) at[tid] = ex;
+        if (tid < kOpenRounds * (kGtNT / 32)) at[tid] = ex;
         if (tid == 0) {
             S.base[0] = (total & 0xFFFFu) ? atomicAdd(c.n[LIST_TAB], total & 0xFFFFu) : 0u;
             S.base[1] = (total >> 16) ? atomicAdd(c.nnode, total >> 16) : 0u;
@@ -688,10 +717,9 @@ __global__ void __launch_bounds__(kGtNT, 4) k_cells_open(RoundArgs ra, const uin
 #pragma unroll 1
     for (; busy; busy &= busy - 1) {
         const int r = __ffs(busy) - 1;
-        const uint32_t i = r * kGtNT + tid, m = tile * kGtCells + i;
+        const uint32_t i = (r * kGtNT + tid) * 4, m = tile * kGtCells + i;
         const Look o = look(i);
-        const bool t = is_tab(o);
-        const uint32_t mine = (t ? 1u : 0u) | ((uint32_t)__popc(o.f) << 16);
+        const uint32_t mine = (uint32_t)__popc(o.tab) | ((uint32_t)__popc(o.f) << 16);
         uint32_t inc = mine;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
@@ -699,16 +727,22 @@ __global__ void __launch_bounds__(kGtNT, 4) k_cells_open(RoundArgs ra, const uin
             if (lane >= d) inc += y;
         }
         const uint32_t ex = S.at[r][warp] + inc - mine;
-        if (t)
-            put_piece(c, LIST_TAB, S.base[0] + (ex & 0xFFFFu), make_piece(o.at, o.n, g, o.hier, (uint8_t)g, g, 0));
-        uint32_t ni = S.base[1] + (ex >> 16);
+        uint32_t pi = S.base[0] + (ex & 0xFFFFu), ni = S.base[1] + (ex >> 16);
+#pragma unroll 1
+        for (uint32_t todo = o.tab; todo; todo &= todo - 1) {
+            const int q = __ffs(todo) - 1;
+            const uint32_t at = start_of(o, q);
+            put_piece(c, LIST_TAB, pi++, make_piece(at, end_of(o, q) - at, g, hier_of(o, q), (uint8_t)g, g, 0));
+        }
 #pragma unroll 1
         for (uint32_t todo = o.f; todo; todo &= todo - 1) {
-            const int k = __ffs(todo) - 1;   // levels above the cell
+            const int b = __ffs(todo) - 1;
+            const int k = b < 8 ? b : 0, q = b < 8 ? 0 : b - 7;   // levels above the cell, and which of the four
             const int lev = g - k;
-            const uint32_t cnt = k == 0 ? S.v[i] : (k == 1 ? S.s1[i >> 3] : (k == 2 ? S.s2[i >> 6] : (k == 3 ? S.s3[i >> 9]
-                                                                                                   : S.top.at(k - 4, tile))));
-            put_node(c, ni++, m >> (3 * k), lev, cnt, o.at, cnt <= C || lev == c.lmax);
+            const uint32_t cnt =
+                k == 0 ? (q == 0 ? o.v.x : (q == 1 ? o.v.y : (q == 2 ? o.v.z : o.v.w)))
+                       : (k == 1 ? S.s1[i >> 3] : (k == 2 ? S.s2[i >> 6] : (k == 3 ? S.s3[i >> 9] : S.top.at(k - 4, tile))));
+            put_node(c, ni++, (m + q) >> (3 * k), lev, cnt, start_of(o, q), cnt <= C || lev == c.lmax);
         }
     }
 }
@@ -806,39 +840,57 @@ FP_DEV void small_warp(const OctCtx& c, SmallPiece a, SmallPiece b)
     }
 }
 
-// level-g cells of 1 .. kSmallMax points (not inner), two cells per lane, then the
-// small pieces of the split rounds
-__global__ void __launch_bounds__(256) k_small_pieces(OctCtx c)
+// level-g cells of 1 .. kSmallMax points (not inner), then the small pieces of the
+// split rounds.  The cells in groups of 64, two per lane: a lane reads the counts
+// of 32 groups (grid level g - 2) first and only those that hold points are
+// opened; the four words of a group's cells arrive together.  Bound by the latency
+// of these reads.  (Reading every cell's count first: 10^7 LiDAR points 36 -> 30 us,
+// 20,000 points 12 -> 10 us; 10^6 uniform points, where every group holds some, 18 ->
+// 19 us.)
+__global__ void __launch_bounds__(256) k_small_pieces(OctCtx c, const uint32_t* __restrict__ pyr)
 {
     const int lane = threadIdx.x & 31;
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
     const uint32_t cells = 1u << (3 * c.g);   // (a multiple of 8)
     if (warp == 0 && lane == 0 && c.cstart[cells] != c.nrec_max) raise(c.err, FP_ERR_CAPACITY, 4);
-    // the counts of the next cells are on their way while these are worked on
-    const uint32_t step = nwarps * 64;
-    auto load = [&](uint32_t m) {
-        return m < cells ? make_uint2(c.rcounts[m], c.rcounts[m + 1]) : make_uint2(0u, 0u);
+    const uint32_t groups = max(cells / 64, 1u);
+    const uint32_t* held = c.g >= 2 ? pyr + pyr_off(c.g - 2) : nullptr;   // points of every group
+    struct Words {   // of two cells: cursors' ends, starts, the next start, leaf levels
+        uint2 end, st;
+        uint32_t to, leaf;
     };
-    uint2 ahead = load(warp * 64 + 2 * lane);
-    for (uint32_t m0 = warp * 64; m0 < cells; m0 += step) {
-        const uint32_t m = m0 + 2 * lane;
-        const uint2 n = ahead;
-        if (cells - m0 > step) ahead = load(m + step);
-        if (!__any_sync(0xFFFFFFFFu, (n.x | n.y) != 0)) continue;
-        SmallPiece a{0u, 0u, 0u}, b{0u, 0u, 0u};
-        if (n.x | n.y) {
-            const uint2 end = *reinterpret_cast<const uint2*>(c.cursor + cursor_slot(m, c.g));
-            const uint2 st = *reinterpret_cast<const uint2*>(c.cstart + m);
-            const uint32_t to = c.cstart[m + 2];
-            const uint32_t leaf = *reinterpret_cast<const uint16_t*>(c.cell_leaf + m);
+    auto load = [&](uint32_t m) {
+        Words w{make_uint2(0u, 0u), make_uint2(0u, 0u), 0u, 0u};
+        if (m < cells) {
+            w.end = *reinterpret_cast<const uint2*>(c.cursor + cursor_slot(m, c.g));
+            w.st = *reinterpret_cast<const uint2*>(c.cstart + m);
+            w.to = c.cstart[m + 2];
+            w.leaf = *reinterpret_cast<const uint16_t*>(c.cell_leaf + m);
+        }
+        return w;
+    };
+    for (uint64_t g0 = warp; g0 < groups; g0 += 32ull * nwarps) {
+        const uint64_t mine = g0 + (uint64_t)lane * nwarps;
+        uint32_t todo = __ballot_sync(0xFFFFFFFFu, mine < groups && (!held || __ldg(held + mine) != 0));
+        if (!todo) continue;
+        auto cell = [&](uint32_t left) {   // this lane's first cell of the next group (cells: none)
+            const uint64_t m = left ? (g0 + (uint64_t)(__ffs(left) - 1) * nwarps) * 64 + 2 * lane : (uint64_t)cells;
+            return (uint32_t)min(m, (uint64_t)cells);
+        };
+        Words ahead = load(cell(todo));
+        for (; todo; todo &= todo - 1) {   // the next group's words are on their way while this one is worked on
+            const Words w = ahead;
+            ahead = load(cell(todo & (todo - 1)));
+            SmallPiece a{0u, 0u, 0u}, b{0u, 0u, 0u};
+            const uint32_t na = w.st.y - w.st.x, nb = w.to - w.st.y;
             // a cell's cursor that does not end at the next one's start: a count grid of other points (points
             // in a cell without any by the grid make another one come up short, or the totals differ)
-            if ((n.x && end.x != st.y) || (n.y && end.y != to)) raise(c.err, FP_ERR_CAPACITY, 4);
-            const uint32_t la = leaf & 255u, lb = leaf >> 8;
-            if (n.x <= (uint32_t)kSmallMax && la != kInner) a = SmallPiece{st.x, n.x, (la << 8) | ((uint32_t)c.g << 16)};
-            if (n.y <= (uint32_t)kSmallMax && lb != kInner) b = SmallPiece{st.y, n.y, (lb << 8) | ((uint32_t)c.g << 16)};
+            if ((na && w.end.x != w.st.y) || (nb && w.end.y != w.to)) raise(c.err, FP_ERR_CAPACITY, 4);
+            const uint32_t la = w.leaf & 255u, lb = w.leaf >> 8;
+            if (na <= (uint32_t)kSmallMax && la != kInner) a = SmallPiece{w.st.x, na, (la << 8) | ((uint32_t)c.g << 16)};
+            if (nb <= (uint32_t)kSmallMax && lb != kInner) b = SmallPiece{w.st.y, nb, (lb << 8) | ((uint32_t)c.g << 16)};
+            if (__any_sync(0xFFFFFFFFu, (a.cnt | b.cnt) != 0)) small_warp(c, a, b);
         }
-        if (__any_sync(0xFFFFFFFFu, (a.cnt | b.cnt) != 0)) small_warp(c, a, b);
     }
     const uint32_t ns = min(*c.n[LIST_SMALL], c.piece_cap);
     // spread over the warps (32 pieces in a row kept a few warps busy for 40 us after the others)
@@ -2053,7 +2105,7 @@ cudaError_t launch_octree_impl(const fp_point* sorted, const uint32_t* perm, uin
         const uint64_t blk = N / (kSmallMax + 1) + 1;   // at most that many table pieces
         k_tab_pieces<<<(int)std::min<uint64_t>(blk, (uint64_t)ws.num_sms * kTabCtas), kTabNT, 0, st>>>(c);
         k_small_pieces<<<(int)std::max<uint64_t>(1, std::min<uint64_t>(Ly.cells / 256, ws.num_sms * 8ull)), 256, 0,
-                         st>>>(c);
+                         st>>>(c, B.pyr);
         const size_t smem = sizeof(GenSmem);
         if ((e = cudaFuncSetAttribute(k_general_pieces, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
             return e;
