@@ -722,8 +722,8 @@ def fp_select_nodes(nodes, num_nodes, cube, cam, ws=None, stream=None):
     cap = nodes.shape[0]
     dev = nodes.device
     ids = torch.empty(max(cap, 1), dtype=torch.int32, device=dev)
-    nsel = torch.zeros(1, dtype=torch.int32, device=dev)
-    npts = torch.zeros(1, dtype=torch.int64, device=dev)
+    nsel = torch.empty(1, dtype=torch.int32, device=dev)
+    npts = torch.empty(1, dtype=torch.int64, device=dev)
     w = ws if ws is not None else torch.empty(max(render_workspace_size(cap), 1), dtype=torch.uint8, device=dev)
     _check(load().fp_select_nodes(_adr(nodes), _adr(num_nodes), cap, _adr(cube), ctypes.byref(cam), _adr(ids),
                                   _adr(nsel), _adr(npts), _adr(w), w.numel(), _raw_stream(stream)), "fp_select_nodes")
