@@ -69,23 +69,45 @@ __global__ void k_preview_append(const int4* prev, const uint64_t* cnt, int4* ou
 
 __global__ void k_add_u64(uint64_t* run, const uint64_t* cnt) { *run += *cnt; }
 
-// points of a piece per chunk (warp-aggregated)
-__global__ void k_piece_hist(const fp_point* pts, uint64_t n, const fp_cube* cube, int g, const uint32_t* lut,
-                             uint32_t* pcnt)
+// Points of a piece per chunk: equal chunks of a warp added at once, per block in
+// shared memory for up to kHistChunks chunks (K; more go to the global counts
+// directly, which a scan's few dense chunks turn into a queue: 2M points 298 ->
+// 26 us).
+constexpr uint32_t kHistChunks = 4096;
+
+__global__ void __launch_bounds__(256) k_piece_hist(const fp_point* pts, uint64_t n, const fp_cube* cube, int g,
+                                                    const uint32_t* lut, uint32_t* pcnt, uint32_t K)
 {
+    __shared__ uint32_t s_cnt[kHistChunks];
+    const bool local = K <= kHistChunks;
+    if (local)
+        for (uint32_t q = threadIdx.x; q < K; q += 256) s_cnt[q] = 0;
+    __syncthreads();
     const CubeDev c = load_cube(cube);
     const int lane = threadIdx.x & 31;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < n; i0 += stride) {
-        const uint64_t i = i0 + lane;
-        uint32_t ch = 0xFFFFFFFFu;
-        if (i < n) {
-            const int4 p = ld_point(pts, i);
-            ch = __ldg(lut + key_small(p.x, p.y, p.z, c, g));
+    for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < n; i0 += 4 * stride) {
+        uint32_t ch[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const uint64_t i = i0 + u * stride + lane;
+            ch[u] = 0xFFFFFFFFu;
+            if (i < n) {
+                const int4 p = ld_point(pts, i);
+                ch[u] = __ldg(lut + key_small(p.x, p.y, p.z, c, g));
+            }
         }
-        const uint32_t peers = __match_any_sync(0xFFFFFFFFu, ch);
-        if (ch != 0xFFFFFFFFu && lane == __ffs(peers) - 1) atomicAdd(&pcnt[ch], (uint32_t)__popc(peers));
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const uint32_t peers = __match_any_sync(0xFFFFFFFFu, ch[u]);
+            if (ch[u] < K && lane == __ffs(peers) - 1)
+                atomicAdd((local ? s_cnt : pcnt) + ch[u], (uint32_t)__popc(peers));
+        }
     }
+    __syncthreads();
+    if (local)
+        for (uint32_t q = threadIdx.x; q < K; q += 256)
+            if (s_cnt[q]) atomicAdd(&pcnt[q], s_cnt[q]);
 }
 
 // a piece scattered stably by chunk: its run of chunk c lands at the chunk's cursor
@@ -410,16 +432,18 @@ struct Piecer {   // double-buffered host -> device copies of the pieces on a si
     uint64_t pieces() const { return (n + P - 1) / P; }
     int4* dst(uint64_t k) const { return raw ? raw + k * P : buf[k & 1]; }
     uint64_t size(uint64_t k) const { return std::min(P, n - k * P); }
-    // enqueue the copy of piece k (after the work that read its buffer), compute stream waits for it
+    // enqueue the copy of piece k (after the work that read its buffer)
     cudaError_t fetch(uint64_t k)
     {
         const int b = (int)(k & 1);
         cudaError_t e;
         if ((e = cudaStreamWaitEvent(cs, consumed[b], 0))) return e;
         if ((e = cudaMemcpyAsync(dst(k), h + k * P, size(k) * sizeof(fp_point), cudaMemcpyHostToDevice, cs))) return e;
-        if ((e = cudaEventRecord(copied[b], cs))) return e;
-        return cudaStreamWaitEvent(st, copied[b], 0);
+        return cudaEventRecord(copied[b], cs);
     }
+    // the compute stream waits for piece k, when its work is enqueued (waiting as soon
+    // as the copy was enqueued held the piece before it back too: nothing overlapped)
+    cudaError_t arrived(uint64_t k) { return cudaStreamWaitEvent(st, copied[k & 1], 0); }
     cudaError_t done(uint64_t k) { return cudaEventRecord(consumed[k & 1], st); }
     // a pass over the device copy made by an earlier pass (raw set): no copies
     template <typename F>
@@ -439,6 +463,7 @@ struct Piecer {   // double-buffered host -> device copies of the pieces on a si
         if (np && (e = fetch(0))) return e;
         for (uint64_t k = 0; k < np; ++k) {
             if (k + 1 < np && (e = fetch(k + 1))) return e;   // the next copy overlaps this piece's work
+            if ((e = arrived(k))) return e;
             if ((e = body(k, reinterpret_cast<const fp_point*>(dst(k)), size(k)))) return e;
             if ((e = done(k))) return e;
         }
@@ -592,7 +617,8 @@ fp_status build(const fp_point* h_pts, uint64_t n, const fp_params& prm, uint64_
     auto distribute_piece = [&](uint64_t k, const fp_point* p, uint64_t np) -> cudaError_t {
         cudaError_t x;
         if ((x = cudaMemsetAsync(F.pcnt, 0, (size_t)K * sizeof(uint32_t), st))) return x;
-        k_piece_hist<<<grid_for(np, base.num_sms), 256, 0, st>>>(p, np, F.cube, g, F.lut, F.pcnt);
+        k_piece_hist<<<std::min<unsigned>(grid_for((np + 3) / 4, base.num_sms), base.num_sms * 4u), 256, 0, st>>>(
+            p, np, F.cube, g, F.lut, F.pcnt, K);
         if ((x = scan_exclusive<uint32_t, uint64_t>(F.pcnt, F.poff, K, nullptr, F.tiles64, F.poff + K,
                                                     (uint64_t*)nullptr, st)))
             return x;
