@@ -21,7 +21,11 @@
 // fewer); when the arena also holds a raw copy of the cloud, pass 1 leaves it
 // there and passes 2 and 3 read it on the device.  The pinned host scratch is the out-of-core store between passes:
 // the distributed points and original indices of every group, the two levels
-// and the owner of every point, and the staged records.
+// and the owner of every point, and the staged records.  What fits the piece
+// buffers, which are dead after pass 3, stays on the device instead: a second set
+// of group buffers (the next group crosses the link while one is worked on), the
+// levels, then owners, of the whole cloud, the staged records.  12M points, pieces
+// of 2M: 14.2 -> 9.6 ms.
 #include <algorithm>
 #include <vector>
 #include "fp_sort.cuh"
@@ -183,40 +187,60 @@ __global__ void k_run_starts(const uint64_t* key, uint64_t S, int shift, uint32_
 
 // A group's points sorted by owner: points of nodes inside the group's chunks go
 // to their final positions (index order inside an owner is the distributed
-// order); points of nodes above the chunks are staged with key (owner, index)
-// and their position in the store of group points.
+// order); points of nodes above the chunks are staged: key (owner, index) and
+// the point, in any order (on the device, or in the host store: there over the
+// points of groups already read, as no more are staged than have been).
 __global__ void k_group_place(const uint64_t* key, const uint32_t* src, uint64_t n, const uint32_t* soff,
                               const fp_node* nodes, uint32_t M, uint64_t T, int g, const uint64_t* first,
-                              const int4* pts, const uint32_t* perm, uint64_t group_base, int4* h_final,
-                              uint32_t* h_final_perm, uint64_t n_all, uint64_t* h_st_key, uint32_t* h_st_src,
-                              int4* h_st_pt, uint64_t* st_run, uint64_t st_cap, int pbits, uint32_t* err)
+                              const int4* pts, const uint32_t* perm, int4* h_final, uint32_t* h_final_perm,
+                              uint64_t n_all, uint64_t* st_key, int4* st_pt, uint64_t* st_run, uint64_t st_cap,
+                              int pbits, uint32_t* err)
 {
-    for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (uint64_t)gridDim.x * blockDim.x) {
-        const uint32_t X = (uint32_t)key[t];
-        const uint32_t j = src[t];
-        if (X >= M) { raise(err, FP_ERR_CAPACITY); continue; }
-        const bool above = nodes[X].count > T && (int)nodes[X].level < g;
+    const int lane = threadIdx.x & 31;
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t t0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); t0 < n; t0 += stride) {
+        const uint64_t t = t0 + lane;
+        uint32_t X = 0, j = 0;
+        bool here = t < n, above = false;
+        if (here) {
+            X = (uint32_t)key[t];
+            j = src[t];
+            if (X >= M) { raise(err, FP_ERR_CAPACITY); here = false; }
+            else above = nodes[X].count > T && (int)nodes[X].level < g;
+        }
+        // the warp's staged points take their places with one atomic
+        const uint32_t st = __ballot_sync(0xFFFFFFFFu, here && above);
+        uint64_t o = 0;
+        if (st && lane == __ffs(st) - 1) o = atomicAdd((unsigned long long*)st_run, (unsigned long long)__popc(st));
+        if (st) o = __shfl_sync(0xFFFFFFFFu, (unsigned long long)o, __ffs(st) - 1) + __popc(st & lanemask_lt());
+        if (!here) continue;
         if (!above) {
             const uint64_t f = first[X] + (t - soff[X]);
             if (f >= n_all) { raise(err, FP_ERR_CAPACITY); continue; }
             h_final[f] = pts[j];
             h_final_perm[f] = perm[j];
         } else {
-            const uint64_t o = atomicAdd((unsigned long long*)st_run, 1ull);
             if (o >= st_cap) { raise(err, FP_ERR_CAPACITY); continue; }
-            h_st_key[o] = ((uint64_t)X << pbits) | perm[j];
-            h_st_src[o] = (uint32_t)(group_base + j);
-            if (h_st_pt) h_st_pt[o] = pts[j];   // the point itself (no host store of the cloud)
+            st_key[o] = ((uint64_t)X << pbits) | perm[j];
+            st_pt[o] = pts[j];
         }
     }
 }
 
-// staged records sorted by (owner, index): position first[owner] + rank.  The
-// point comes from the host store, or (staged_pts) from its staged copy, the
-// index from the key.
+// points owned by nodes above the chunks: what k_group_place stages
+__global__ void k_staged_count(const fp_node* nodes, const uint32_t* num, uint32_t cap, uint64_t T, int g, uint64_t* out)
+{
+    const uint32_t M = min(*num, cap);
+    uint64_t s = 0;
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < M; i += gridDim.x * blockDim.x)
+        if (nodes[i].count > T && (int)nodes[i].level < g) s += nodes[i].n_own;
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+    if ((threadIdx.x & 31) == 0 && s) atomicAdd((unsigned long long*)out, (unsigned long long)s);
+}
+
+// staged records sorted by (owner, index): position first[owner] + rank
 __global__ void k_stitch_final(const uint64_t* key, const uint32_t* val, uint64_t S, int pbits, const uint32_t* soff,
-                               const uint64_t* first, const uint32_t* h_st_src, const int4* h_pts,
-                               const uint32_t* h_perm, int staged_pts, int4* h_final, uint32_t* h_final_perm,
+                               const uint64_t* first, const int4* st_pt, int4* h_final, uint32_t* h_final_perm,
                                uint64_t n_all, uint32_t M, uint32_t* err)
 {
     const uint64_t imask = (1ull << pbits) - 1;
@@ -224,10 +248,10 @@ __global__ void k_stitch_final(const uint64_t* key, const uint32_t* val, uint64_
         const uint64_t X = key[t] >> pbits;
         if (X >= M) { raise(err, FP_ERR_CAPACITY); continue; }
         const uint64_t f = first[X] + (t - soff[X]);
-        const uint32_t j = staged_pts ? val[t] : h_st_src[val[t]];
-        if (f >= n_all || j >= n_all) { raise(err, FP_ERR_CAPACITY); continue; }
-        h_final[f] = h_pts[j];
-        h_final_perm[f] = staged_pts ? (uint32_t)(key[t] & imask) : h_perm[j];
+        const uint32_t j = val[t];
+        if (f >= n_all || j >= S) { raise(err, FP_ERR_CAPACITY); continue; }
+        h_final[f] = st_pt[j];
+        h_final_perm[f] = (uint32_t)(key[t] & imask);
     }
 }
 
@@ -238,7 +262,6 @@ struct HostStore {
     uint32_t* codes;    // n: owner level, leaf level, level-g cell (code_make)
     uint32_t* owner;    // n: owner id
     uint64_t* st_key;   // n: staged (owner, index)
-    uint32_t* st_src;   // n: staged record's position in pts
 };
 
 HostStore host_carve(void* base, uint64_t n)
@@ -252,14 +275,13 @@ HostStore host_carve(void* base, uint64_t n)
     h.codes = w.take<uint32_t>(N);
     h.owner = w.take<uint32_t>(N);
     h.st_key = w.take<uint64_t>(N);
-    h.st_src = w.take<uint32_t>(N);
     return h;
 }
 
 size_t host_bytes(uint64_t n)
 {   // the pieces host_carve takes, in its order
     const uint64_t N = n ? n : 1;
-    return Workspace::bytes_for({16 * N, 4 * N, 4 * N, 4 * N, 8 * N, 4 * N});
+    return Workspace::bytes_for({16 * N, 4 * N, 4 * N, 4 * N, 8 * N});
 }
 
 uint64_t preview_piece_cap(uint64_t p, uint32_t m)
@@ -639,6 +661,60 @@ fp_status build(const fp_point* h_pts, uint64_t n, const fp_params& prm, uint64_
     ws.bytes = B.ws_bytes;
     ws.used = 0;
 
+    // ---- The groups are read three times (levels; owners; final positions).  The
+    // piece buffers and pass 3's tables are dead from here on: they hold a second
+    // set of group buffers, so that the next group (of this pass or the next one)
+    // crosses the link while one is worked on, and the codes, then owners, of the
+    // whole cloud, which otherwise go to the host store and back twice.
+    Workspace dead = base;
+    dead.base = reinterpret_cast<char*>(F.piece[0]);
+    dead.bytes = (size_t)(reinterpret_cast<char*>(F.ccur + cells) - dead.base);
+    dead.used = 0;
+    auto fits = [&](size_t bytes) { return dead.used + Workspace::bytes_for({bytes}) + 256 <= dead.bytes; };
+    int4* gpts[2] = {B.pts, B.pts};
+    uint32_t* gperm[2] = {B.perm, B.perm};
+    bool ahead = false;
+    if (!resident && fits(20 * (size_t)G + 512)) {
+        gpts[1] = dead.take<int4>(G);
+        gperm[1] = dead.take<uint32_t>(G);
+        ahead = true;
+    }
+    uint32_t* all_codes = fits(4 * (size_t)n) ? dead.take<uint32_t>(n) : nullptr;
+    const size_t ngroups = groups.size(), nloads = 3 * ngroups;
+    // load l: group l % ngroups for pass l / ngroups (the indices for the last pass only)
+    auto load = [&](size_t l, cudaStream_t on) -> cudaError_t {
+        const uint64_t b0 = off[groups[l % ngroups].first], ng = off[groups[l % ngroups].second] - b0;
+        const int b = ahead ? (int)(l & 1) : 0;
+        cudaError_t x;
+        if (ahead && (x = cudaStreamWaitEvent(on, io.consumed[b], 0))) return x;
+        if ((x = cudaMemcpyAsync(gpts[b], H.pts + b0, ng * 16, cudaMemcpyHostToDevice, on))) return x;
+        if (l >= 2 * ngroups && (x = cudaMemcpyAsync(gperm[b], H.perm + b0, ng * 4, cudaMemcpyHostToDevice, on))) return x;
+        return ahead ? cudaEventRecord(io.copied[b], on) : cudaSuccess;
+    };
+    if (ahead) {   // the store is written and the buffers are free once pass 3 is done
+        for (int b = 0; b < 2; ++b)
+            if ((e = cudaEventRecord(io.consumed[b], st))) return cu(e);
+        if (nloads && (e = load(0, io.cs))) return cu(e);
+    }
+    // B.pts and B.perm: the group of load l, there when the compute stream gets to what follows
+    auto enter = [&](size_t l) -> cudaError_t {
+        const uint64_t b0 = off[groups[l % ngroups].first];
+        if (resident) {
+            B.pts = res_pts + b0;
+            B.perm = res_perm + b0;
+            return cudaSuccess;
+        }
+        const int b = ahead ? (int)(l & 1) : 0;
+        B.pts = gpts[b];
+        B.perm = gperm[b];
+        if (!ahead) return load(l, st);
+        cudaError_t x;
+        if (l + 1 < nloads && (x = load(l + 1, io.cs))) return x;
+        return cudaStreamWaitEvent(st, io.copied[b], 0);
+    };
+    auto leave = [&](size_t l) -> cudaError_t { return ahead ? cudaEventRecord(io.consumed[l & 1], st) : cudaSuccess; };
+    size_t at = 0;
+
     // ---- per group: its points from the store; levels and nodes below level g
     if ((e = cudaMemsetAsync(F.num_deep, 0, sizeof(uint32_t), st))) return cu(e);
     const unsigned gc = grid_for(cells, base.num_sms);
@@ -646,20 +722,16 @@ fp_status build(const fp_point* h_pts, uint64_t n, const fp_params& prm, uint64_
         const uint64_t b0 = off[c0], ng = off[c1] - off[c0];
         k_group_tables<<<gc, 256, 0, st>>>(F.counts, F.lut, cells, c0, c1, F.rcounts, F.lut_local);
         k_group_offsets<<<gc, 256, 0, st>>>(F.offsets, c0, c1 - c0, F.off_local, F.kdev);
-        if (resident) {
-            B.pts = res_pts + b0;
-            B.perm = res_perm + b0;
-        } else {
-            if ((e = cudaMemcpyAsync(B.pts, H.pts + b0, ng * 16, cudaMemcpyHostToDevice, st))) return cu(e);
-            if ((e = cudaMemcpyAsync(B.perm, H.perm + b0, ng * 4, cudaMemcpyHostToDevice, st))) return cu(e);
-        }
-        OctGroup grp{F.rcounts, (uint32_t)b0, B.codes, F.recs, node_cap, F.num_deep};
+        if ((e = enter(at))) return cu(e);
+        uint32_t* codes = all_codes ? all_codes + b0 : B.codes;
+        OctGroup grp{F.rcounts, (uint32_t)b0, codes, F.recs, node_cap, F.num_deep};
         ws.used = 0;
         if ((e = launch_octree_impl(reinterpret_cast<const fp_point*>(B.pts), B.perm, ng, F.cube, F.chunks + c0,
                                     F.kdev, F.off_local, F.counts, prm, nullptr, 0, nullptr, nullptr, nullptr,
                                     nullptr, &grp, ws, st)))
             return cu(e);
-        if ((e = cudaMemcpyAsync(H.codes + b0, B.codes, ng * 4, cudaMemcpyDeviceToHost, st))) return cu(e);
+        if (!all_codes && (e = cudaMemcpyAsync(H.codes + b0, codes, ng * 4, cudaMemcpyDeviceToHost, st))) return cu(e);
+        if ((e = leave(at++))) return cu(e);
     }
 
     // ---- node table of the whole cloud
@@ -668,22 +740,34 @@ fp_status build(const fp_point* h_pts, uint64_t n, const fp_params& prm, uint64_
                                  st)))
         return cu(e);
 
-    // ---- pass 4 per group: owner ids, owned counts
+    // ---- pass 4 per group: owner ids (over the codes where those stay on the device), owned counts
     for (auto [c0, c1] : groups) {
         const uint64_t b0 = off[c0], ng = off[c1] - off[c0];
-        if (resident) B.pts = res_pts + b0;
-        else if ((e = cudaMemcpyAsync(B.pts, H.pts + b0, ng * 16, cudaMemcpyHostToDevice, st))) return cu(e);
-        if ((e = cudaMemcpyAsync(B.codes, H.codes + b0, ng * 4, cudaMemcpyHostToDevice, st))) return cu(e);
-        if ((e = launch_octree_resolve(reinterpret_cast<const fp_point*>(B.pts), ng, F.cube, B.codes, F.T, prm,
-                                       B.owner, ws, st)))
+        if ((e = enter(at))) return cu(e);
+        uint32_t* codes = all_codes ? all_codes + b0 : B.codes;
+        uint32_t* owner = all_codes ? codes : B.owner;
+        if (!all_codes && (e = cudaMemcpyAsync(codes, H.codes + b0, ng * 4, cudaMemcpyHostToDevice, st))) return cu(e);
+        if ((e = launch_octree_resolve(reinterpret_cast<const fp_point*>(B.pts), ng, F.cube, codes, F.T, prm, owner, ws,
+                                       st)))
             return cu(e);
-        if ((e = cudaMemcpyAsync(H.owner + b0, B.owner, ng * 4, cudaMemcpyDeviceToHost, st))) return cu(e);
+        if (!all_codes && (e = cudaMemcpyAsync(H.owner + b0, owner, ng * 4, cudaMemcpyDeviceToHost, st))) return cu(e);
+        if ((e = leave(at++))) return cu(e);
     }
     if ((e = launch_node_first(F.nodes, F.num_nodes, node_cap, F.T.nown, F.first, F.nm, F.tiles64, st))) return cu(e);
     uint32_t M = 0;
+    uint64_t S = 0;   // points of nodes above the chunks
+    if ((e = cudaMemsetAsync(F.st_run, 0, sizeof(uint64_t), st))) return cu(e);
+    k_staged_count<<<grid_for(node_cap, base.num_sms), 256, 0, st>>>(F.nodes, F.num_nodes, node_cap, prm.chunk_threshold,
+                                                                     g, F.st_run);
     if ((e = cudaMemcpyAsync(&M, F.num_nodes, sizeof(M), cudaMemcpyDeviceToHost, st))) return cu(e);
+    if ((e = cudaMemcpyAsync(&S, F.st_run, sizeof(S), cudaMemcpyDeviceToHost, st))) return cu(e);
     if ((e = cudaStreamSynchronize(st))) return cu(e);
     if (M > node_cap) return FP_ERR_INVALID;
+    if (S > n) return FP_ERR_INVALID;
+    // staged on the device where the dead buffers have room, else in the host store
+    const bool st_dev = fits(24 * (size_t)(S ? S : 1) + 512);
+    uint64_t* st_key = st_dev ? dead.take<uint64_t>(S ? S : 1) : H.st_key;
+    int4* st_pt = st_dev ? dead.take<int4>(S ? S : 1) : H.pts;
     int pbits = 1;
     while ((1ull << pbits) < n) ++pbits;
     int mbits = 1;
@@ -696,15 +780,10 @@ fp_status build(const fp_point* h_pts, uint64_t n, const fp_params& prm, uint64_
     const size_t ws_after_sc = ws.used;
     for (auto [c0, c1] : groups) {
         const uint64_t b0 = off[c0], ng = off[c1] - off[c0];
-        if (resident) {
-            B.pts = res_pts + b0;
-            B.perm = res_perm + b0;
-        } else {
-            if ((e = cudaMemcpyAsync(B.pts, H.pts + b0, ng * 16, cudaMemcpyHostToDevice, st))) return cu(e);
-            if ((e = cudaMemcpyAsync(B.perm, H.perm + b0, ng * 4, cudaMemcpyHostToDevice, st))) return cu(e);
-        }
-        if ((e = cudaMemcpyAsync(B.owner, H.owner + b0, ng * 4, cudaMemcpyHostToDevice, st))) return cu(e);
-        k_owner_keys<<<grid_for(ng, base.num_sms), 256, 0, st>>>(B.owner, ng, B.key);
+        if ((e = enter(at))) return cu(e);
+        const uint32_t* owner = all_codes ? all_codes + b0 : B.owner;
+        if (!all_codes && (e = cudaMemcpyAsync(B.owner, H.owner + b0, ng * 4, cudaMemcpyHostToDevice, st))) return cu(e);
+        k_owner_keys<<<grid_for(ng, base.num_sms), 256, 0, st>>>(owner, ng, B.key);
         ws.used = ws_after_sc;
         SortArgs a{};
         a.b.k64_src = B.key; a.b.k64_tmp = B.key2; a.b.k64_dst = B.key3;
@@ -714,30 +793,35 @@ fp_status build(const fp_point* h_pts, uint64_t n, const fp_params& prm, uint64_
         if ((e = sort_run<DIG_K64, false, true, false>(a, sort_passes(mbits), base.num_sms, st))) return cu(e);
         k_run_starts<<<grid_for(ng, base.num_sms), 256, 0, st>>>(B.key3, ng, 0, F.soff, M);
         k_group_place<<<grid_for(ng, base.num_sms), 256, 0, st>>>(
-            B.key3, B.val3, ng, F.soff, F.nodes, M, prm.chunk_threshold, g, F.first, B.pts, B.perm, b0,
-            reinterpret_cast<int4*>(h_final), h_final_perm, n, H.st_key, H.st_src, resident ? H.pts : nullptr,
-            F.st_run, n, pbits, base.err);
+            B.key3, B.val3, ng, F.soff, F.nodes, M, prm.chunk_threshold, g, F.first, B.pts, B.perm,
+            reinterpret_cast<int4*>(h_final), h_final_perm, n, st_key, st_pt, F.st_run, S, pbits, base.err);
         if ((e = cudaGetLastError())) return cu(e);
+        if ((e = leave(at++))) return cu(e);
     }
 
     // ---- the staged points: sorted by (owner, index), placed after their owners' earlier points
-    uint64_t S = 0;
-    if ((e = cudaMemcpyAsync(&S, F.st_run, sizeof(S), cudaMemcpyDeviceToHost, st))) return cu(e);
-    if ((e = cudaStreamSynchronize(st))) return cu(e);
     if (S) {   // the sort of the staged records reuses the whole group region
         Workspace wf = base;
         // (the resident cloud is dead by now: the staged points were copied out with their records)
         wf.base = resident ? reinterpret_cast<char*>(res_pts) : B.region;
         wf.bytes = group_bytes(G, P, prm, node_cap, base.num_sms, resident) + (resident ? resident_bytes(n) : 0);
         wf.used = 0;
-        uint64_t* k1 = wf.take<uint64_t>(S);
+        uint64_t* k1 = st_dev ? st_key : wf.take<uint64_t>(S);
         uint64_t* k2 = wf.take<uint64_t>(S);
         uint64_t* k3 = wf.take<uint64_t>(S);
         uint32_t* v2 = wf.take<uint32_t>(S);
         uint32_t* v3 = wf.take<uint32_t>(S);
         const SortScratch sf = take_sort_scratch(wf, S);
         if (wf.used > wf.bytes) return FP_ERR_WORKSPACE;
-        if ((e = cudaMemcpyAsync(k1, H.st_key, S * 8, cudaMemcpyHostToDevice, st))) return cu(e);
+        if (!st_dev) {
+            if ((e = cudaMemcpyAsync(k1, st_key, S * 8, cudaMemcpyHostToDevice, st))) return cu(e);
+            // their points too where there is room (else read from the host one by one)
+            if (wf.used + Workspace::bytes_for({16 * (size_t)S}) + 256 <= wf.bytes) {
+                int4* p = wf.take<int4>(S);
+                if ((e = cudaMemcpyAsync(p, st_pt, S * 16, cudaMemcpyHostToDevice, st))) return cu(e);
+                st_pt = p;
+            }
+        }
         SortArgs a{};
         a.b.k64_src = k1; a.b.k64_tmp = k2; a.b.k64_dst = k3;
         a.b.val_src = nullptr; a.b.val_tmp = v2; a.b.val_dst = v3;
@@ -745,10 +829,9 @@ fp_status build(const fp_point* h_pts, uint64_t n, const fp_params& prm, uint64_
         if ((e = sort_plan_keys(sf, a, 0, (uint32_t)(pbits + mbits), nullptr, false, base.num_sms, st))) return cu(e);
         if ((e = sort_run<DIG_K64, false, true, false>(a, sort_passes(pbits + mbits), base.num_sms, st))) return cu(e);
         k_run_starts<<<grid_for(S, base.num_sms), 256, 0, st>>>(k3, S, pbits, F.soff, M);
-        k_stitch_final<<<grid_for(S, base.num_sms), 256, 0, st>>>(k3, v3, S, pbits, F.soff, F.first, H.st_src, H.pts,
-                                                                  H.perm, resident ? 1 : 0,
-                                                                  reinterpret_cast<int4*>(h_final),
-                                                                  h_final_perm, n, M, base.err);
+        k_stitch_final<<<grid_for(S, base.num_sms), 256, 0, st>>>(k3, v3, S, pbits, F.soff, F.first, st_pt,
+                                                                  reinterpret_cast<int4*>(h_final), h_final_perm, n, M,
+                                                                  base.err);
         if ((e = cudaGetLastError())) return cu(e);
     }
     if ((e = cudaMemcpyAsync(h_nodes, F.nodes, (size_t)M * sizeof(fp_node), cudaMemcpyDeviceToHost, st))) return cu(e);
