@@ -25,25 +25,25 @@ constexpr int kBdIPT = 8;
 constexpr int kBdTile = kBdNT * kBdIPT;   // 2048 points per tile
 
 // The previews that need no extents, without a look-back.  Keep rule: the index
-// hash is a multiple of the modulus (the uniform preview: only the kept points
-// are read), or it is the smallest of the point's cell (the spatial one).  A
-// block takes a segment of consecutive tiles; a warp takes ROWS rows of 32
+// hash is a multiple of the modulus (the uniform preview), or it is the smallest
+// of the point's cell (the spatial one, whose keep bits k_cell_mark sets first).
+// Only the kept points are read.  A block takes a segment of consecutive tiles; a warp takes ROWS rows of 32
 // points, lane r holds row r's keep bits.  When every block has counted its
 // segment, a tile's output starts at the totals of the earlier segments plus its
 // place in its own.
 //   k_keep_all: both halves in one cooperative launch, the keep bits in shared
 //     memory across the barrier (the uniform rule, up to kKeepTiles tiles a block);
-//   k_keep, k_keep_write: in two launches (the spatial rule, its bits stored, and
-//     larger pieces, whose bits are computed again).
-// Both halves are bound by the hash's integer instructions (10 us for 8M points).
-// (In one launch with a look-back, all tiles of a wave publish at about the same
-// time and the last walks back over all of them: 38 us for 8M points, 25 us now,
-// and 880 us for the spatial pass over 10^8, 820 us now.)
+//   k_keep, k_keep_write: in two launches (the spatial rule, and larger pieces,
+//     whose bits are computed again).
+// Both halves of the uniform rule are bound by the hash's integer instructions (10
+// us for 8M points).  (In one launch with a look-back, all tiles of a wave publish
+// at about the same time and the last walks back over all of them: 38 us for 8M
+// points, 25 us now.)
 constexpr int kKeepSegs = 2048;
-constexpr int kKeepRows = 32, kKeepRowsCell = 8;   // rows per warp and tile
+constexpr int kKeepRows = 32, kKeepRowsSmall = 8;   // rows per warp and tile
 
 struct KeepScratch {
-    uint32_t* words;      // spatial rule: keep bits, tile by tile, warp by warp, row by row
+    uint32_t* words;      // spatial rule: keep bits, bit i & 31 of word i / 32 for point i
     uint32_t* before;     // per tile: kept points of its segment before it
     uint32_t* seg;        // per segment: kept points
     uint64_t ntiles, per; // tiles, tiles per segment
@@ -64,42 +64,18 @@ FP_DEV uint32_t keep_word(uint64_t i, uint64_t n, uint64_t first, const KeepMult
     return word;
 }
 
-template <bool CELL_MIN, int ROWS>
-__global__ void __launch_bounds__(kBdNT) k_keep(const fp_point* __restrict__ pts, uint64_t n, uint64_t first,
-                                                KeepMultiple mult, KeepScratch s, const uint64_t* __restrict__ cell_min,
-                                                const fp_cube* cube_p, int level)
+template <bool BITS, int ROWS>
+__global__ void __launch_bounds__(kBdNT) k_keep(uint64_t n, uint64_t first, KeepMultiple mult, KeepScratch s)
 {
     constexpr int kWarps = kBdNT / 32;
     __shared__ uint32_t s_tot[2][kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    CubeDev cube;
-    if (CELL_MIN) {
-        cube = load_cube(cube_p);
-    }
     const uint64_t t0 = blockIdx.x * s.per, t1 = min(s.ntiles, t0 + s.per);
     uint32_t run = 0;
     for (uint64_t tile = t0; tile < t1; ++tile) {
-        const uint64_t base = (tile * kWarps + warp) * (32 * ROWS) + lane;
-        uint32_t word = 0;
-        if (CELL_MIN) {
-            int4 q[ROWS];
-            uint64_t least[ROWS];
-#pragma unroll
-            for (int r = 0; r < ROWS; ++r)   // points, then minima, all in flight together
-                if (base + 32 * r < n) q[r] = ld_point_cs(pts, base + 32 * r);
-#pragma unroll
-            for (int r = 0; r < ROWS; ++r)
-                if (base + 32 * r < n) least[r] = __ldcg(cell_min + key_small(q[r].x, q[r].y, q[r].z, cube, level));
-#pragma unroll
-            for (int r = 0; r < ROWS; ++r) {
-                const uint64_t i = base + 32 * r;
-                const uint32_t bal = __ballot_sync(0xFFFFFFFFu, i < n && least[r] == splitmix64(first + i));
-                if (lane == r) word = bal;
-            }
-            if (lane < ROWS) s.words[(tile * kWarps + warp) * ROWS + lane] = word;
-        } else {
-            word = keep_word<ROWS>(base, n, first, mult);
-        }
+        const uint64_t w0 = (tile * kWarps + warp) * ROWS;
+        const uint32_t word = BITS ? (lane < ROWS ? s.words[w0 + lane] : 0u)
+                                   : keep_word<ROWS>(w0 * 32 + lane, n, first, mult);
         const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, __popc(word));
         uint32_t* tot = s_tot[(tile - t0) & 1];   // (two sets: one barrier a tile)
         if (lane == 0) tot[warp] = total;
@@ -111,7 +87,7 @@ __global__ void __launch_bounds__(kBdNT) k_keep(const fp_point* __restrict__ pts
     if (threadIdx.x == 0) s.seg[blockIdx.x] = run;
 }
 
-template <bool CELL_MIN, int ROWS>
+template <bool BITS, int ROWS>
 __global__ void __launch_bounds__(kBdNT) k_keep_write(const fp_point* __restrict__ pts, uint64_t n, uint64_t first,
                                                       KeepMultiple mult, KeepScratch s, uint32_t nseg,
                                                       fp_point* __restrict__ out, uint64_t out_cap,
@@ -124,8 +100,8 @@ __global__ void __launch_bounds__(kBdNT) k_keep_write(const fp_point* __restrict
     const uint64_t tile = blockIdx.x;
     const uint32_t g = (uint32_t)(tile / s.per);
     const uint64_t w0 = (tile * kWarps + warp) * ROWS;
-    const uint32_t word = CELL_MIN ? (lane < ROWS ? s.words[w0 + lane] : 0u)
-                                   : keep_word<ROWS>(w0 * 32 + lane, n, first, mult);
+    const uint32_t word = BITS ? (lane < ROWS ? s.words[w0 + lane] : 0u)
+                               : keep_word<ROWS>(w0 * 32 + lane, n, first, mult);
     uint64_t sum = 0, rest = 0;
     for (uint32_t q = threadIdx.x; q < nseg; q += kBdNT) {
         const uint32_t v = s.seg[q];
@@ -590,35 +566,33 @@ __global__ void __launch_bounds__(kBdNT, 8) k_keep_all(const fp_point* __restric
 }
 
 // the carve of the previews without extents
-static KeepScratch keep_carve(const Workspace& ws, uint64_t n, int rows, bool cell_min)
+static KeepScratch keep_carve(const Workspace& ws, uint64_t n, int rows, bool bits)
 {
     KeepScratch s;
     const uint64_t tile = (uint64_t)kBdNT * rows;
     s.ntiles = (n + tile - 1) / tile;
     s.per = std::max<uint64_t>(1, (s.ntiles + kKeepSegs - 1) / kKeepSegs);
-    s.words = cell_min ? ws.take<uint32_t>(s.ntiles * (tile / 32)) : nullptr;
+    s.words = bits ? ws.take<uint32_t>(s.ntiles * (tile / 32)) : nullptr;
     s.before = ws.take<uint32_t>(s.ntiles);
     s.seg = ws.take<uint32_t>(kKeepSegs);
     return s;
 }
 
-static size_t keep_bytes(uint64_t n, int rows, bool cell_min)
+static size_t keep_bytes(uint64_t n, int rows, bool bits)
 {
     Workspace dry;
-    keep_carve(dry, n, rows, cell_min);
+    keep_carve(dry, n, rows, bits);
     return dry.used;
 }
 
-template <bool CELL_MIN, int ROWS>
-static void keep_launch(const fp_point* pts, uint64_t n, uint64_t first, uint32_t modulus, fp_point* out,
-                        uint64_t out_cap, uint64_t* out_count, const uint64_t* cell_min, const fp_cube* cube,
-                        int level, const Workspace& ws, cudaStream_t st)
+template <bool BITS, int ROWS>
+static void keep_launch(const KeepScratch& s, const fp_point* pts, uint64_t n, uint64_t first, uint32_t modulus,
+                        fp_point* out, uint64_t out_cap, uint64_t* out_count, const Workspace& ws, cudaStream_t st)
 {
-    const KeepScratch s = keep_carve(ws, n, ROWS, CELL_MIN);
     const uint32_t nseg = (uint32_t)((s.ntiles + s.per - 1) / s.per);
-    k_keep<CELL_MIN, ROWS><<<nseg, kBdNT, 0, st>>>(pts, n, first, KeepMultiple::of(modulus), s, cell_min, cube, level);
-    k_keep_write<CELL_MIN, ROWS><<<(unsigned)s.ntiles, kBdNT, 0, st>>>(pts, n, first, KeepMultiple::of(modulus), s, nseg, out,
-                                                                       out_cap, out_count, ws.err);
+    k_keep<BITS, ROWS><<<nseg, kBdNT, 0, st>>>(n, first, KeepMultiple::of(modulus), s);
+    k_keep_write<BITS, ROWS><<<(unsigned)s.ntiles, kBdNT, 0, st>>>(pts, n, first, KeepMultiple::of(modulus), s, nseg, out,
+                                                                   out_cap, out_count, ws.err);
 }
 
 cudaError_t launch_bounds_decimate(const fp_point* pts, uint64_t n, fp_cube* cube, bool bounds, bool decim,
@@ -647,9 +621,11 @@ cudaError_t launch_bounds_decimate(const fp_point* pts, uint64_t n, fp_cube* cub
         }
         ws.used = 0;
         if (s.ntiles >= (uint64_t)ws.num_sms * 4)
-            keep_launch<false, kKeepRows>(pts, n, first, modulus, out, out_cap, out_count, nullptr, nullptr, 0, ws, st);
+            keep_launch<false, kKeepRows>(keep_carve(ws, n, kKeepRows, false), pts, n, first, modulus, out, out_cap,
+                                          out_count, ws, st);
         else
-            keep_launch<false, kKeepRowsCell>(pts, n, first, modulus, out, out_cap, out_count, nullptr, nullptr, 0, ws, st);
+            keep_launch<false, kKeepRowsSmall>(keep_carve(ws, n, kKeepRowsSmall, false), pts, n, first, modulus, out,
+                                               out_cap, out_count, ws, st);
         return cudaGetLastError();
     }
     const BoundsScratch b = bounds_carve(ws, n, ws.num_sms);
@@ -673,8 +649,11 @@ cudaError_t launch_bounds_decimate(const fp_point* pts, uint64_t n, fp_cube* cub
 // proposes for clouds whose file order makes the uniform one uneven, Sec. 6):
 // of the points of every occupied cell of the 2^level grid, the one with the
 // smallest splitmix64(first + i) is kept (a uniformly random point of the cell,
-// the same on every run).  Pass 1 takes each cell's smallest hash; pass 2 is
-// the preview compaction with "hash == its cell's smallest" as the keep rule.
+// the same on every run).  One pass over the points takes each cell's smallest
+// hash; the hash is a bijection, so the index of the point it is from follows from
+// it, and the points of all cells are compacted in index order as the uniform
+// preview's are.  (A second pass over the points, comparing each one's hash with
+// its cell's smallest: 10^8 points, 800 us; 75 us now.)
 constexpr int kMinIPT = 4;
 
 __global__ void __launch_bounds__(256) k_cell_min_hash(const fp_point* __restrict__ pts, uint64_t n, uint64_t first,
@@ -711,7 +690,43 @@ __global__ void __launch_bounds__(256) k_cell_min_hash(const fp_point* __restric
 size_t spatial_ws_bytes(uint64_t n, int level, int num_sms)
 {
     (void)num_sms;
-    return Workspace::bytes_for({sizeof(uint64_t) << (3 * level)}) + keep_bytes(n, kKeepRowsCell, true);
+    return Workspace::bytes_for({sizeof(uint64_t) << (3 * level)}) + keep_bytes(n, kKeepRows, true);
+}
+
+constexpr uint64_t inverse64(uint64_t d)   // d odd, modulo 2^64: three bits right, doubled by every step
+{
+    uint64_t x = d;
+    for (int i = 0; i < 5; ++i) x *= 2 - d * x;
+    return x;
+}
+
+// the v with splitmix64(v) = z: every step of the hash undone
+FP_DEV uint64_t splitmix64_inverse(uint64_t z)
+{
+    constexpr uint64_t m1 = inverse64(0xBF58476D1CE4E5B9ull), m2 = inverse64(0x94D049BB133111EBull);
+    z = (z ^ (z >> 31) ^ (z >> 62)) * m2;
+    z = (z ^ (z >> 27) ^ (z >> 54)) * m1;
+    return (z ^ (z >> 30) ^ (z >> 60)) - 0x9E3779B97F4A7C15ull;
+}
+
+// keep bits of the points whose hashes the cells' smallest are.  A cell of ~0 is
+// empty, or holds only the one point whose hash that is: thread 0 looks at it.
+__global__ void __launch_bounds__(256) k_cell_mark(const uint64_t* __restrict__ cell_min, uint32_t cells,
+                                                   const fp_point* pts, uint64_t n, uint64_t first,
+                                                   const fp_cube* cube_p, int level, uint32_t* words)
+{
+    const uint32_t m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (m >= cells) return;
+    const uint64_t h = cell_min[m], i = splitmix64_inverse(h) - first;
+    if (h != ~0ull && i < n) atomicOr(&words[i >> 5], 1u << (i & 31));
+    if (m == 0) {
+        const uint64_t last = splitmix64_inverse(~0ull) - first;
+        if (last < n) {
+            const CubeDev cube = load_cube(cube_p);
+            const int4 p = ld_point(pts, last);
+            if (cell_min[key_small(p.x, p.y, p.z, cube, level)] == ~0ull) atomicOr(&words[last >> 5], 1u << (last & 31));
+        }
+    }
 }
 
 cudaError_t launch_preview_spatial(const fp_point* pts, uint64_t n, const fp_cube* cube, int level, uint64_t first,
@@ -728,7 +743,11 @@ cudaError_t launch_preview_spatial(const fp_point* pts, uint64_t n, const fp_cub
     if ((e = cudaMemsetAsync(cell_min, 0xFF, cells * sizeof(uint64_t), st))) return e;
     const int gm = (int)std::min<uint64_t>((n + 255) / 256, (uint64_t)ws.num_sms * 8);
     k_cell_min_hash<<<gm, 256, 0, st>>>(pts, n, first, cube, level, reinterpret_cast<unsigned long long*>(cell_min));
-    keep_launch<true, kKeepRowsCell>(pts, n, first, 1, out, out_cap, out_count, cell_min, cube, level, ws, st);
+    const KeepScratch s = keep_carve(ws, n, kKeepRows, true);
+    if ((e = cudaMemsetAsync(s.words, 0, s.ntiles * kBdNT * kKeepRows / 8, st))) return e;
+    k_cell_mark<<<(unsigned)((cells + 255) / 256), 256, 0, st>>>(cell_min, (uint32_t)cells, pts, n, first, cube, level,
+                                                                 s.words);
+    keep_launch<true, kKeepRows>(s, pts, n, first, 1, out, out_cap, out_count, ws, st);
     return cudaGetLastError();
 }
 

@@ -67,3 +67,32 @@ def test_decimate_beyond_the_cooperative_path(gpu_lib):
     assert fp.get_device_error() == 0
     k = int(ca.item())
     assert k == int(cb.item()) and torch.equal(a[:k], b[:k])
+
+
+# around the tile of 8192 points; grids of 8 cells and of 2^21; LiDAR's empty cells
+@pytest.mark.parametrize("n", [1, 31, 33, 8191, 8192, 8193, 100_003])
+@pytest.mark.parametrize("level", [1, 4, 7])
+def test_spatial_sizes(gpu_lib, n, level):
+    fp = gpu_lib
+    pts_np = synth.lidar(n, 72)
+    cube, pts = oracle.bounds(pts_np), dev_points(pts_np)
+    out, count = fp.fp_preview_spatial(pts, fp.fp_bounds(pts), level, (1 << 33) + n)
+    want, _ = oracle.preview_spatial(pts_np, cube, level, (1 << 33) + n)
+    assert int(count.item()) == len(want)
+    assert_points_equal(out, want, count=len(want))
+
+
+# the one index whose hash is the largest value (it marks empty cells on the device): alone in its cell, or not
+@pytest.mark.parametrize("alone", [False, True])
+def test_spatial_largest_hash(gpu_lib, alone):
+    fp = gpu_lib
+    first = (0x31628AF67B2131AB - 5) % (1 << 64)
+    pts_np = synth.uniform(64, 73, bits=10)
+    pts_np["x"][5] = 4000 if alone else pts_np["x"][6]
+    if not alone:
+        pts_np["y"][5], pts_np["z"][5] = pts_np["y"][6], pts_np["z"][6]
+    pts = dev_points(pts_np)
+    out, count = fp.fp_preview_spatial(pts, fp.fp_bounds(pts), 3, first)
+    want, _ = oracle.preview_spatial(pts_np, oracle.bounds(pts_np), 3, first)
+    assert int(count.item()) == len(want)
+    assert_points_equal(out, want, count=len(want))
