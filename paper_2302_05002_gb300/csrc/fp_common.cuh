@@ -204,6 +204,12 @@ FP_DEV uint32_t match_bits(uint32_t v, bool valid)
 // the line at p on its way to L2
 FP_DEV void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
+// size bytes at p (16-byte aligned, size a multiple of 16) on their way to L2
+FP_DEV void bulk_prefetch_l2(const void* p, uint32_t size)
+{
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(size) : "memory");
+}
+
 // volatile load for inter-block flags
 FP_DEV uint32_t ld_volatile(const uint32_t* p) { return *(const volatile uint32_t*)p; }
 
