@@ -876,6 +876,7 @@ cudaError_t seg_scatter(const SegScratch& sc, const SegCall& c, const Workspace&
     a.stitch = owner ? 1 : 0;
     a.st_key = c.st_key; a.st_src = c.st_src; a.st_count = c.st_count; a.st_cap = c.n; a.st_shift = c.st_shift;
     a.st_rank = c.st_rank;
+    a.st_nrank = c.st_nrank; a.st_code = c.st_code; a.st_inv = c.st_inv;
     a.n = c.n;
     a.d_fail = sc.cnt + 2;
     a.err = ws.err;

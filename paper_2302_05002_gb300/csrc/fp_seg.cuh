@@ -58,8 +58,14 @@ struct SegArgs {
     uint64_t n;                           // bound of the output positions
 
     const uint32_t* d_fail;
+    // up to kStitchRanks nodes outside every chunk subtree: staged points marked by
+    // original index instead (rank + 1, and the position they are at)
+    const uint32_t* st_nrank;
+    uint8_t* st_code;
+    uint32_t* st_inv;
     uint32_t* err;
 };
+constexpr uint32_t kStitchRanks = 254;   // (rank + 1 in a byte, for an inconsistent table's ranks too)
 
 template <bool CPT, int MAXB>
 struct SegSmem {
@@ -103,6 +109,7 @@ __global__ void __launch_bounds__(kSortNT, (seg_ctas<CPT, MAXB>())) k_seg_pass(S
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint64_t ntiles = min((uint64_t)*a.d_ntiles, a.ntiles_max);
     constexpr int kStride = 1 << MAXB;
+    const bool marked = a.stitch && a.st_code && *a.st_nrank <= kStitchRanks;
 
     // the next tile is claimed while the current one is worked on (tiles only
     // wait on earlier tiles of their chunk, so a reserved tile cannot deadlock)
@@ -199,7 +206,7 @@ __global__ void __launch_bounds__(kSortNT, (seg_ctas<CPT, MAXB>())) k_seg_pass(S
         for (int d = threadIdx.x; d < nb; d += kSortNT) {
             if (d == sdig) {
                 const uint32_t k = s_cnt[d];
-                const uint32_t at = k ? atomicAdd(a.st_count, k) : 0u;
+                const uint32_t at = k && !marked ? atomicAdd(a.st_count, k) : 0u;
                 s_gbase[d] = (uint64_t)at - s_off[d];
                 continue;
             }
@@ -218,9 +225,16 @@ __global__ void __launch_bounds__(kSortNT, (seg_ctas<CPT, MAXB>())) k_seg_pass(S
             const int d = s_dig[q];
             const uint64_t o = s_gbase[d] + q;
             if (d == sdig) {
-                if (o >= a.st_cap) { raise(a.err, FP_ERR_CAPACITY, 14); continue; }
                 const uint64_t src = base + s_pos[q];
                 const uint32_t id = a.id_in[src];
+                if (marked) {
+                    const uint32_t i = s_val[q];
+                    if (i >= a.n) { raise(a.err, FP_ERR_CAPACITY, 14); continue; }
+                    a.st_code[i] = (uint8_t)(a.st_rank[id] + 1);
+                    a.st_inv[i] = (uint32_t)src;
+                    continue;
+                }
+                if (o >= a.st_cap) { raise(a.err, FP_ERR_CAPACITY, 14); continue; }
                 a.st_key[o] = ((uint64_t)a.st_rank[id] << a.st_shift) | s_val[q];
                 a.st_src[o] = (uint32_t)src;
             } else {
@@ -266,6 +280,8 @@ struct SegCall {
     // st_soff[node] = staged points of the nodes before it
     uint64_t* st_key; uint32_t* st_src; uint32_t* st_count; int st_shift;
     uint32_t *st_rank, *st_list, *st_nrank, *st_soff;
+    uint8_t* st_code;         // n bytes, zero, and n words: marks of up to kStitchRanks nodes' points instead
+    uint32_t* st_inv;
 };
 
 // distribution of up to kDistCluster points in one launch (tmp: n words each;
