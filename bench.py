@@ -55,8 +55,8 @@ FIXED_BYTES = {"merge": 3 * 4 * (1 << 21)}
 # launches of a kernel, from one ncu capture of the workload, valid while the
 # sources that kernel is built from hash to the recorded value (a changed
 # kernel reports null)
-_COMMON = ["fp_common.cuh", "fp_internal.cuh", "fp_scan.cuh"]   # (fp_api.cu: argument checks, no kernel)
-_OCT = _COMMON + ["fp_sort.cuh", "fp_seg.cuh", "fp_octree.cu"]
+_COMMON = ["fp_common.cuh", "fp_internal.cuh", "fp_cluster.cuh", "fp_grid.cuh"]   # (fp_api.cu: argument checks)
+_OCT = _COMMON + ["fp_scan.cuh", "fp_sort.cuh", "fp_seg.cuh", "fp_octree.cu"]
 KERNEL_FILES = {
     "bounds_decimate": _COMMON + ["fp_core.cu"],
     "count": _COMMON + ["fp_core.cu"],

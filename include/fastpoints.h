@@ -152,17 +152,17 @@ fp_status fp_get_device_error_sites(cudaStream_t stream, uint32_t* h_sites);
 fp_status fp_debug_withhold_publish(uint32_t tile, uint32_t spin_limit);
 
 /* Kernel timing for profiling.  The library's main kernels, by stage:
- *   FP_KERNEL_BOUNDS_DECIMATE  k_bounds_decimate (fp_bounds, fp_decimate, fp_bounds_decimate)
- *   FP_KERNEL_COUNT            k_count (fp_count)
+ *   FP_KERNEL_BOUNDS_DECIMATE  the bounds and preview pass (fp_bounds, fp_decimate, fp_bounds_decimate)
+ *   FP_KERNEL_COUNT            the count pass (fp_count, fp_count_cells)
  *   FP_KERNEL_DISTRIBUTE       the stable scatter of fp_distribute (every launch of it)
  *   FP_KERNEL_CELL_GROUP       k_cell_scatter: points grouped by count-grid cell (fp_build_chunk_octree)
  *   FP_KERNEL_SPLIT_ROUNDS     the split rounds of cells larger than one shared-memory piece
- *   FP_KERNEL_UNITS            k_units: LOD level and leaf level of every point
+ *   FP_KERNEL_UNITS            LOD level and leaf level of every point, piece by piece (three launches)
  *   FP_KERNEL_NODE_TABLE       node records sorted into preorder
  *   FP_KERNEL_RESOLVE          k_resolve: owner node and leaf node of every point
  *   FP_KERNEL_LEAF_SCATTER     the leaf-grouped layout (when requested)
  *   FP_KERNEL_OWNER_SCATTER    the final layout scatter of fp_subsample
- *   FP_KERNEL_STITCH           the merge of points kept above the chunks (sort and placement)
+ *   FP_KERNEL_STITCH           the merge of points kept above the chunks (clouds of more than 2^21 points)
  * fp_time_kernel(k, start, stop) arms kernel k for the calling process: every
  * later call that launches it records `start` on its stream before the first
  * launch of k and `stop` after the last one (cudaEventElapsedTime then gives

@@ -101,8 +101,6 @@ FP_DEV uint32_t key_small(int32_t x, int32_t y, int32_t z, const CubeDev& c, int
            spread3_10(cell_at(z, c.o[2], c, l));
 }
 
-FP_DEV uint64_t key_at(uint64_t k21, int level) { return k21 >> (3 * (kKeyLevels - level)); }
-
 // per-point code of the octree stage: LOD owner level (5 bits), leaf level (5
 // bits) and the Morton key of the point's level-g cell (3 g <= 21 bits)
 FP_DEV uint32_t code_make(int own, int leaf, uint32_t cell)
