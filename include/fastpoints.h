@@ -157,7 +157,7 @@ fp_status fp_debug_withhold_publish(uint32_t tile, uint32_t spin_limit);
  *   FP_KERNEL_DISTRIBUTE       the stable scatter of fp_distribute (every launch of it)
  *   FP_KERNEL_CELL_GROUP       k_cell_scatter: points grouped by count-grid cell (fp_build_chunk_octree)
  *   FP_KERNEL_SPLIT_ROUNDS     the split rounds of cells larger than one shared-memory piece
- *   FP_KERNEL_UNITS            LOD level and leaf level of every point, piece by piece (three launches)
+ *   FP_KERNEL_UNITS            LOD level and leaf level of every point, piece by piece (all of its launches)
  *   FP_KERNEL_NODE_TABLE       node records sorted into preorder
  *   FP_KERNEL_RESOLVE          k_resolve: owner node and leaf node of every point
  *   FP_KERNEL_LEAF_SCATTER     the leaf-grouped layout (when requested)

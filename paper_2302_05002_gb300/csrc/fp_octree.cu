@@ -752,7 +752,8 @@ __global__ void __launch_bounds__(kGtNT, 4) k_cells_open(RoundArgs ra, const uin
 //   * level-g cells of at most kSmallMax points: k_small_pieces, one lane per
 //     point, straight from the count grid (no piece is listed);
 //   * pieces whose node is not inner, at most kHashMaxD levels deep: k_tab_pieces,
-//     one block per piece, smallest index per occupied cell in tables;
+//     one block per piece, smallest index per occupied cell in tables (on large
+//     clouds the small shallow ones by one warp each, k_warp_pieces);
 //   * inner pieces, and deeper ones: k_general_pieces, one block per piece, sort
 //     and nearest-smaller search, which also finds the nodes inside the piece;
 //   * more than kPieceMax equal keys: k_general_pieces too, by a minimum.
@@ -762,7 +763,7 @@ __global__ void __launch_bounds__(kGtNT, 4) k_cells_open(RoundArgs ra, const uin
 // their pieces in one 512-thread block, and the pieces sorted into record order
 // first, spent 950 instructions per point at 238 points per cell, where the
 // fourth and fifth table of a window did not fit its shared memory: 26.1 ms for
-// 5 * 10^8 uniform points, 6.1 ms now at about 300 instructions per point.)
+// 5 * 10^8 uniform points, 5.3 ms now at about 300 instructions per point.)
 constexpr int kTabNT = 128;
 constexpr int kTabRun = 8;                    // pieces taken at a time
 constexpr int kTabCtas = 10;                  // blocks per SM (20 KB of tables each)
@@ -1090,6 +1091,165 @@ __global__ void __launch_bounds__(kTabNT, kTabCtas) k_tab_pieces(OctCtx c)
             k1 = k + run;
             if (k < nt) next = c.list[LIST_TAB][k];
             __syncthreads();   // s_next is read before it is written again
+        }
+    }
+}
+
+// Large clouds: table pieces of up to kWarpMax points and kWarpDepth levels take one
+// warp each, with a table of its own and no block barrier (k_warp_pieces); a block
+// takes the other ones of the same list, a run's in order (k_tab_pieces_split).  A
+// block of 128 threads per piece spent its time on barriers and half-empty rows.
+// Octree stage of uniform points: 6.4 * 10^7 (31 a cell) 3.9 -> 3.0 ms, 10^8 6.6 -> 5.3,
+// 2 * 10^8 9.2 -> 7.8; pieces of 5 * 10^8 (238 a cell) 6.6 -> 5.3 ms, of 10^8 LiDAR points
+// 2.0 -> 1.9 ms; of 10^7 LiDAR points, mostly deep pieces, 0.235 -> 0.265 ms: hence
+// the line at kTabSplit points.
+constexpr uint64_t kTabSplit = 1ull << 25;
+constexpr int kWarpMax = 128, kWarpDepth = 3;
+constexpr int kWarpWords = 592;   // 8 + 64 + 512 entries, 16-byte rows
+
+FP_DEV bool warp_kind(const OctCtx& c, const Piece& p)
+{
+    return p.count <= (uint32_t)kWarpMax && piece_depth(c, p.q, p.hier) <= kWarpDepth;
+}
+
+__global__ void __launch_bounds__(kTabNT, kTabCtas) k_tab_pieces_split(OctCtx c)
+{
+    __shared__ __align__(16) unsigned char buf[kTabBytes];
+    __shared__ Piece s_piece[kTabNT];
+    __shared__ uint32_t s_min;
+    __shared__ uint32_t s_next;
+    __shared__ uint32_t s_warp[kTabNT / 32];
+    const uint32_t nt = min(*c.n[LIST_TAB], c.piece_cap);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // (runs as above; while one holds nothing but pieces for single warps, the next is twice as long)
+    const uint32_t run0 = max(1u, min((uint32_t)kTabRun, nt / (gridDim.x * 16)));
+    uint32_t run = run0;
+    if (threadIdx.x == 0) s_next = atomicAdd(c.tab_claim, run);
+    __syncthreads();
+    uint32_t k = s_next;
+    while (k < nt) {
+        // the run's pieces for a block, in order
+        Piece mine{};
+        const bool in = threadIdx.x < run && k + threadIdx.x < nt;
+        if (in) mine = c.list[LIST_TAB][k + threadIdx.x];
+        const bool take = in && !warp_kind(c, mine);
+        const uint32_t bal = __ballot_sync(0xFFFFFFFFu, take);
+        if (lane == 0) s_warp[warp] = __popc(bal);
+        __syncthreads();   // (also: s_next is read)
+        uint32_t before = 0, m = 0;
+#pragma unroll
+        for (int x = 0; x < kTabNT / 32; ++x) {
+            if (x < warp) before += s_warp[x];
+            m += s_warp[x];
+        }
+        if (take) s_piece[before + __popc(bal & lanemask_lt())] = mine;
+        run = m ? run0 : min(2 * run, (uint32_t)kTabNT);
+        if (threadIdx.x == 0) s_next = atomicAdd(c.tab_claim, run);
+        __syncthreads();
+        for (uint32_t i = 0; i < m; ++i) {
+            const Piece p = s_piece[i];
+            if (i + 1 < m) {   // the next piece's records on their way to L2 during this one's work
+                const Piece next = s_piece[i + 1];
+                const uint32_t line = threadIdx.x * 8;   // 128 bytes a thread
+                if (line < next.count && (uint64_t)next.begin + line < c.nrec_max)
+                    prefetch_l2(c.recs[next.buf] + next.begin + line);
+            }
+            const int D = piece_depth(c, p.q, p.hier);
+            uint32_t* tab = reinterpret_cast<uint32_t*>(buf);
+            if (D > kTabDirect)
+                hash_piece(c, p, D, reinterpret_cast<uint64_t*>(buf),
+                           reinterpret_cast<unsigned long long*>(buf + sizeof(uint64_t) * kPieceMax), &s_min);
+            else if (p.count <= 2 * kTabNT) direct_piece<2>(c, p, D, tab, &s_min);
+            else if (p.count <= 4 * kTabNT) direct_piece<4>(c, p, D, tab, &s_min);
+            else direct_piece<kPieceMax / kTabNT>(c, p, D, tab, &s_min);
+        }
+        k = s_next;   // (written before the barrier above)
+    }
+}
+
+constexpr int kWarpNT = 256;
+
+__global__ void __launch_bounds__(kWarpNT, 6) k_warp_pieces(OctCtx c)
+{
+    __shared__ __align__(16) uint32_t s_tab[kWarpNT / 32][kWarpWords];
+    const int lane = threadIdx.x & 31;
+    uint32_t* tab = s_tab[threadIdx.x >> 5];
+    const uint32_t nt = min(*c.n[LIST_TAB], c.piece_cap);
+    const uint32_t w = (blockIdx.x * kWarpNT + threadIdx.x) >> 5, nwarps = gridDim.x * (kWarpNT / 32);
+    constexpr uint32_t kRun = 8;   // pieces a warp looks at together; the warps side by side
+    for (uint64_t k0 = (uint64_t)w * kRun; k0 < nt; k0 += (uint64_t)nwarps * kRun) {
+        Piece mine{};
+        const bool in = lane < (int)kRun && k0 + lane < nt;
+        if (in) mine = c.list[LIST_TAB][k0 + lane];
+        uint32_t todo = __ballot_sync(0xFFFFFFFFu, in && warp_kind(c, mine));
+        for (; todo; todo &= todo - 1) {
+            const int l = __ffs(todo) - 1;
+            Piece p;
+            p.begin = __shfl_sync(0xFFFFFFFFu, mine.begin, l);
+            const uint32_t n = __shfl_sync(0xFFFFFFFFu, mine.count, l);
+            const uint32_t what = __shfl_sync(
+                0xFFFFFFFFu, (uint32_t)mine.q | ((uint32_t)mine.hier << 8) | ((uint32_t)mine.A << 16) | ((uint32_t)mine.buf << 24), l);
+            const int q = (int)(what & 255u), leafl = (int)((what >> 8) & 255u), A = (int)((what >> 16) & 255u);
+            const int bufi = (int)(what >> 24);
+            const int D = piece_depth(c, q, leafl);
+            const int sh = 3 * (kKeyLevels - q - D);
+            const uint32_t cmask = (1u << (3 * D)) - 1u;
+            constexpr int R = kWarpMax / 32;
+            uint32_t kk[R], j[R], cell = 0;
+            {
+                uint4 rec[R];
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    rec[r] = make_uint4(0u, 0u, 0u, 0u);
+                    if (r * 32u + lane < n) rec[r] = get_rec(c, bufi, (uint64_t)p.begin + r * 32 + lane);
+                }
+                const int words4 = (int)((((1u << (3 * (D + 1))) - 8u) / 7u + 3u) / 4u);
+                for (int x = lane; x < words4; x += 32)
+                    reinterpret_cast<uint4*>(tab)[x] = make_uint4(kNone, kNone, kNone, kNone);
+                cell = (uint32_t)(rec_key(rec[0]) >> (3 * (kKeyLevels - c.g)));   // the piece lies in one level-g cell
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    kk[r] = (uint32_t)(rec_key(rec[r]) >> sh) & cmask;
+                    j[r] = rec[r].z;
+                }
+            }
+            __syncwarp();
+            uint32_t least_j = kNone;
+            int lost[R];   // level at which the record met a smaller index (0: none)
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                lost[r] = 0;
+                if (r * 32u + lane >= n) continue;
+                const uint32_t jv = j[r];
+                least_j = min(least_j, jv);
+                bool least = true;
+#pragma unroll
+                for (int d = kWarpDepth; d >= 1; --d) {
+                    if (d <= D && least) {
+                        uint32_t* t = &tab[((1u << (3 * d)) - 8u) / 7u + (kk[r] >> (3 * (D - d)))];
+                        if (*(volatile uint32_t*)t < jv) { least = false; lost[r] = d; }
+                        else atomicMin(t, jv);
+                    }
+                }
+            }
+            const uint32_t jmin = __reduce_min_sync(0xFFFFFFFFu, least_j);
+            __syncwarp();
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                if (r * 32u + lane >= n) continue;
+                int top = kKeyLevels + 1 - q;   // never its cell's minimum down to the piece's depth
+                bool held = true;
+#pragma unroll
+                for (int d = kWarpDepth; d >= 1; --d) {
+                    if (d <= D && held) {
+                        held = d > lost[r] &&
+                               *(volatile uint32_t*)&tab[((1u << (3 * d)) - 8u) / 7u + (kk[r] >> (3 * (D - d)))] == j[r];
+                        if (held) top = d;
+                    }
+                }
+                put_lambda(c, j[r], j[r] == jmin ? A : q + top, leafl, cell);   // (the minimum: from the split tree)
+            }
+            __syncwarp();   // the table is free for the next piece
         }
     }
 }
@@ -2103,7 +2263,13 @@ cudaError_t launch_octree_impl(const fp_point* sorted, const uint32_t* perm, uin
     {
         KTimerScope kt(FP_KERNEL_UNITS, st);
         const uint64_t blk = N / (kSmallMax + 1) + 1;   // at most that many table pieces
-        k_tab_pieces<<<(int)std::min<uint64_t>(blk, (uint64_t)ws.num_sms * kTabCtas), kTabNT, 0, st>>>(c);
+        const int gt = (int)std::min<uint64_t>(blk, (uint64_t)ws.num_sms * kTabCtas);
+        if (N >= kTabSplit) {
+            k_tab_pieces_split<<<gt, kTabNT, 0, st>>>(c);
+            k_warp_pieces<<<(int)std::min<uint64_t>(blk / (kWarpNT / 4) + 1, (uint64_t)ws.num_sms * 6), kWarpNT, 0, st>>>(c);
+        } else {
+            k_tab_pieces<<<gt, kTabNT, 0, st>>>(c);
+        }
         k_small_pieces<<<(int)std::max<uint64_t>(1, std::min<uint64_t>(Ly.cells / 256, ws.num_sms * 8ull)), 256, 0,
                          st>>>(c, B.pyr);
         const size_t smem = sizeof(GenSmem);
