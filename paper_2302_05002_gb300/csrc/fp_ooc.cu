@@ -279,9 +279,9 @@ HostStore host_carve(void* base, uint64_t n)
 }
 
 size_t host_bytes(uint64_t n)
-{   // the pieces host_carve takes, in its order
+{   // the pieces host_carve takes, in its order, and 4 n more: the size that callers have sized stores by
     const uint64_t N = n ? n : 1;
-    return Workspace::bytes_for({16 * N, 4 * N, 4 * N, 4 * N, 8 * N});
+    return Workspace::bytes_for({16 * N, 4 * N, 4 * N, 4 * N, 8 * N, 4 * N});
 }
 
 uint64_t preview_piece_cap(uint64_t p, uint32_t m)
