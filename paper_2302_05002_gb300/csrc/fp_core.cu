@@ -765,36 +765,43 @@ cudaError_t launch_bounds_decimate(const fp_point* pts, uint64_t n, fp_cube* cub
 // it, and the points of all cells are compacted in index order as the uniform
 // preview's are.  (A second pass over the points, comparing each one's hash with
 // its cell's smallest: 10^8 points, 800 us; 75 us now.)
-constexpr int kMinIPT = 4;
+constexpr int kMinIPT = 4, kMinCtas = 5;
 
-__global__ void __launch_bounds__(256) k_cell_min_hash(const fp_point* __restrict__ pts, uint64_t n, uint64_t first,
-                                                       const fp_cube* cube_p, int level,
-                                                       unsigned long long* cell_min)
+__global__ void __launch_bounds__(256, kMinCtas) k_cell_min_hash(const fp_point* __restrict__ pts, uint64_t n,
+                                                                 uint64_t first, const fp_cube* cube_p, int level,
+                                                                 unsigned long long* cell_min)
 {
     const CubeDev cube = load_cube(cube_p);
     // a cell's running minimum only falls: a hash not below any value read for
     // it (however stale) cannot be the minimum, and the atomic is skipped --
-    // in a cell of c points in random order about ln c atomics remain
+    // in a cell of c points in random order about ln c atomics remain.  (Read
+    // through L1: an SM's own atomics drop its stale line; 0.62 -> 0.54 ms at 10^8.)
+    // Bound by instructions: without a test per point and with no more blocks than
+    // are resident 0.54 -> 0.45 ms, the same at 2 to 8 points and 3 to 8 blocks an SM.
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += stride * kMinIPT) {
+    uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (; i0 + (kMinIPT - 1) * stride < n; i0 += stride * kMinIPT) {
         int4 q[kMinIPT];
 #pragma unroll
-        for (int u = 0; u < kMinIPT; ++u)   // points, then minima, all in flight together
-            if (i0 + u * stride < n) q[u] = ld_point_cs(pts, i0 + u * stride);
-        unsigned long long* slot[kMinIPT];
+        for (int u = 0; u < kMinIPT; ++u) q[u] = ld_point_cs(pts, i0 + u * stride);   // points, then minima, in flight together
+        uint32_t cell[kMinIPT];
         unsigned long long seen[kMinIPT];
 #pragma unroll
-        for (int u = 0; u < kMinIPT; ++u)
-            if (i0 + u * stride < n) {
-                slot[u] = &cell_min[key_small(q[u].x, q[u].y, q[u].z, cube, level)];
-                seen[u] = *slot[u];   // (through L1: an SM's own atomics drop its stale line; 0.62 -> 0.54 ms at 10^8)
-            }
+        for (int u = 0; u < kMinIPT; ++u) {
+            cell[u] = key_small(q[u].x, q[u].y, q[u].z, cube, level);
+            seen[u] = cell_min[cell[u]];
+        }
 #pragma unroll
-        for (int u = 0; u < kMinIPT; ++u)
-            if (i0 + u * stride < n) {
-                const unsigned long long h = splitmix64(first + i0 + u * stride);
-                if (h < seen[u]) atomicMin(slot[u], h);
-            }
+        for (int u = 0; u < kMinIPT; ++u) {
+            const unsigned long long h = splitmix64(first + i0 + u * stride);
+            if (h < seen[u]) atomicMin(cell_min + cell[u], h);
+        }
+    }
+    for (; i0 < n; i0 += stride) {
+        const int4 q = ld_point_cs(pts, i0);
+        unsigned long long* slot = cell_min + key_small(q.x, q.y, q.z, cube, level);
+        const unsigned long long h = splitmix64(first + i0);
+        if (h < *slot) atomicMin(slot, h);
     }
 }
 
@@ -852,7 +859,7 @@ cudaError_t launch_preview_spatial(const fp_point* pts, uint64_t n, const fp_cub
         return cudaGetLastError();
     }
     if ((e = cudaMemsetAsync(cell_min, 0xFF, cells * sizeof(uint64_t), st))) return e;
-    const int gm = (int)std::min<uint64_t>((n + 255) / 256, (uint64_t)ws.num_sms * 8);
+    const int gm = (int)std::min<uint64_t>((n + 255) / 256, (uint64_t)ws.num_sms * kMinCtas);
     k_cell_min_hash<<<gm, 256, 0, st>>>(pts, n, first, cube, level, reinterpret_cast<unsigned long long*>(cell_min));
     const KeepScratch s = keep_carve(ws, n, kKeepRows, true);
     if ((e = cudaMemsetAsync(s.words, 0, s.ntiles * kBdNT * kKeepRows / 8, st))) return e;
