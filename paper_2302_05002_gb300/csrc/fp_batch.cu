@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(NT) k_fused_count(const __grid_constant__ Fuse
                 key[u] = kNone;
                 if (i < b1) {
                     const int4 p = ld_point_cs(reinterpret_cast<const fp_point*>(d.pts), i);
-                    key[u] = key_small(p.x, p.y, p.z, cube, g);
+                    key[u] = key_cell(p.x, p.y, p.z, cube, g);
                 }
             }
 #pragma unroll

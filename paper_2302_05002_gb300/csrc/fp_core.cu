@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(256) k_count(const fp_point* __restrict__ pts,
             key[u] = kNone;
             if (i < n) {
                 int4 p = ld_point_cs(pts, i);
-                key[u] = key_small(p.x, p.y, p.z, c, g);
+                key[u] = key_cell(p.x, p.y, p.z, c, g);
                 if (cells) cells[i] = key[u];
             }
         }
@@ -247,8 +247,8 @@ __global__ void __launch_bounds__(256) k_count(const fp_point* __restrict__ pts,
 // says that one does; the count below), the first cell that comes.  A block whose
 // first points rarely find their cell (a uniform cloud) goes past the table.  The
 // next points are loaded while these are counted.  With the cells written: 10^8
-// LiDAR points in random order 1562 -> 546 us, scan by scan 1761 -> 937 us; 10^7
-// 168 -> 89 and 127 -> 96 us; uniform, 10^8 710 -> 685 us, 10^7 79 -> 86 us, 4 * 10^6
+// LiDAR points in random order 1562 -> 518 us, scan by scan 1761 -> 934 us; 10^7
+// 168 -> 87 and 127 -> 95 us; uniform, 10^8 710 -> 692 us, 10^7 79 -> 85 us, 4 * 10^6
 // 32 -> 42 us (half the warps in flight and the trial), so smaller clouds keep the
 // 1024-slot table of k_count.
 constexpr uint64_t kCountTable = 1ull << 23;             // from this many points on
@@ -308,7 +308,7 @@ __global__ void __launch_bounds__(kCtNT, 1) k_count_table(const fp_point* __rest
             const uint64_t i = i0 + u * stride + threadIdx.x;
             key[u] = kNone;
             if (i < n) {
-                key[u] = key_small(p[u].x, p[u].y, p[u].z, c, g);
+                key[u] = key_cell(p[u].x, p[u].y, p[u].z, c, g);
                 if (cells) cells[i] = key[u];
             }
         }
@@ -777,7 +777,8 @@ __global__ void __launch_bounds__(256, kMinCtas) k_cell_min_hash(const fp_point*
     // in a cell of c points in random order about ln c atomics remain.  (Read
     // through L1: an SM's own atomics drop its stale line; 0.62 -> 0.54 ms at 10^8.)
     // Bound by instructions: without a test per point and with no more blocks than
-    // are resident 0.54 -> 0.45 ms, the same at 2 to 8 points and 3 to 8 blocks an SM.
+    // are resident 0.54 -> 0.45 ms, the same at 2 to 8 points and 3 to 8 blocks an SM;
+    // 0.42 ms with the shorter cell arithmetic.
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     for (; i0 + (kMinIPT - 1) * stride < n; i0 += stride * kMinIPT) {
@@ -788,7 +789,7 @@ __global__ void __launch_bounds__(256, kMinCtas) k_cell_min_hash(const fp_point*
         unsigned long long seen[kMinIPT];
 #pragma unroll
         for (int u = 0; u < kMinIPT; ++u) {
-            cell[u] = key_small(q[u].x, q[u].y, q[u].z, cube, level);
+            cell[u] = key_cell(q[u].x, q[u].y, q[u].z, cube, level);
             seen[u] = cell_min[cell[u]];
         }
 #pragma unroll
@@ -799,7 +800,7 @@ __global__ void __launch_bounds__(256, kMinCtas) k_cell_min_hash(const fp_point*
     }
     for (; i0 < n; i0 += stride) {
         const int4 q = ld_point_cs(pts, i0);
-        unsigned long long* slot = cell_min + key_small(q.x, q.y, q.z, cube, level);
+        unsigned long long* slot = cell_min + key_cell(q.x, q.y, q.z, cube, level);
         const unsigned long long h = splitmix64(first + i0);
         if (h < *slot) atomicMin(slot, h);
     }
@@ -842,7 +843,7 @@ __global__ void __launch_bounds__(256) k_cell_mark(const uint64_t* __restrict__ 
         if (last < n) {
             const CubeDev cube = load_cube(cube_p);
             const int4 p = ld_point(pts, last);
-            if (cell_min[key_small(p.x, p.y, p.z, cube, level)] == ~0ull) atomicOr(&words[last >> 5], 1u << (last & 31));
+            if (cell_min[key_cell(p.x, p.y, p.z, cube, level)] == ~0ull) atomicOr(&words[last >> 5], 1u << (last & 31));
         }
     }
 }

@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(256) k_piece_hist(const fp_point* pts, uint64_
             ch[u] = 0xFFFFFFFFu;
             if (i < n) {
                 const int4 p = ld_point(pts, i);
-                ch[u] = __ldg(lut + key_small(p.x, p.y, p.z, c, g));
+                ch[u] = __ldg(lut + key_cell(p.x, p.y, p.z, c, g));
             }
         }
 #pragma unroll
@@ -125,7 +125,7 @@ __global__ void k_piece_scatter(const int4* dpts, const uint32_t* dperm, uint64_
     const CubeDev c = load_cube(cube);
     for (uint64_t q = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (uint64_t)gridDim.x * blockDim.x) {
         const int4 p = dpts[q];
-        const uint32_t ch = __ldg(lut + key_small(p.x, p.y, p.z, c, g));
+        const uint32_t ch = __ldg(lut + key_cell(p.x, p.y, p.z, c, g));
         const uint64_t dest = ccur[ch] + (q - poff[ch]);
         if (dest >= n_all) { raise(err, FP_ERR_CAPACITY); continue; }
         if (h_pts) {

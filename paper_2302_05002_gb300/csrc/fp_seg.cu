@@ -321,7 +321,7 @@ FP_DEV void dist_count(const DistSweepArgs& a, uint32_t nb, const uint16_t* dist
                 }
 #pragma unroll
                 for (int r = 0; r < kDistCountIPT; ++r)
-                    c[r] = base + (uint64_t)r * kDistCountNT + d < a.n ? key_small(p[r].x, p[r].y, p[r].z, cube, a.g)
+                    c[r] = base + (uint64_t)r * kDistCountNT + d < a.n ? key_cell(p[r].x, p[r].y, p[r].z, cube, a.g)
                                                                       : kNone;
             }
         };
@@ -762,7 +762,7 @@ __global__ void __launch_bounds__(kClNT, 1) k_dist_cluster(DistClusterArgs a)
             if (m >= a.ncell) { raise(a.err, FP_ERR_CAPACITY, 19); m = 0; }
         } else {
             const int4 p = __ldg(a.pts + i);
-            m = key_small(p.x, p.y, p.z, cube, a.g);
+            m = key_cell(p.x, p.y, p.z, cube, a.g);
         }
         uint32_t c = __ldg(a.lut + m);
         if (c >= K) { raise(a.err, FP_ERR_CAPACITY, 13); c = K ? K - 1 : 0; }   // not a chunk

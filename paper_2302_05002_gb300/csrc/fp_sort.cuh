@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(kSortNT, 2) k_sort_pass(SortArgs a, int slot)
                 else if (DIG == DIG_K32) d = (in_k32[i] >> shift) & dmask;
                 else {
                     int4 q = __ldg(in_pt + i);
-                    d = key_small(q.x, q.y, q.z, cube, a.g);   // cell; its chunk below
+                    d = key_cell(q.x, q.y, q.z, cube, a.g);   // cell; its chunk below
                 }
             }
             dg[r] = d;
