@@ -68,10 +68,10 @@ KERNEL_FILES = {
 # pass and sweep; the table and scan launches move under 20 MB), with the hash of the
 # kernel's sources at the capture (profiles/kernels_uniform100M.md); uniform-1B has the
 # same per-point structure (512 chunks, the same node levels) and ten times the points
-_T100 = {"bounds_decimate": (1.698e9, "51ee5eecfb9411cf"), "count": (1.974e9, "51ee5eecfb9411cf"),
-         "distribute": (0.613e9 + 3.955e9, "f8a054bc46db0a7b"),
-         "cell_group": (4.556e9, "270bd362a21f9dcb"), "units": (2.752e9, "270bd362a21f9dcb"),
-         "resolve": (0.840e9, "270bd362a21f9dcb"), "owner_scatter": (3.806e9, "2d260d891fe956b0")}
+_T100 = {"bounds_decimate": (1.697e9, "b6a2dbecdf70285a"), "count": (1.974e9, "b6a2dbecdf70285a"),
+         "distribute": (0.613e9 + 3.958e9, "c299010c4a85751c"),
+         "cell_group": (4.535e9, "e24cb5430d20a1bb"), "units": (2.741e9, "e24cb5430d20a1bb"),
+         "resolve": (0.839e9, "e24cb5430d20a1bb"), "owner_scatter": (3.807e9, "a96e07133017ba54")}
 NCU_TRAFFIC = {}
 for _k, (_b, _h) in _T100.items():
     NCU_TRAFFIC[("uniform-100M", _k)] = (_b, _h)
