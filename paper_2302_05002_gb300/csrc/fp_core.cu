@@ -256,7 +256,7 @@ constexpr int kCtNT = 1024, kCtIPT = 4;
 constexpr int kCtBits = 15, kCtSlots = 1 << kCtBits;
 constexpr int kCtLow = 21 - kCtBits;                    // bits of the hash below the slot
 constexpr uint32_t kCtMul = 0x9E3779B1u & 0x1FFFFFu;    // odd: a bijection of 21 bits
-constexpr int kCtProbe = 2;                             // rounds of kCtNT * kCtIPT points before the table is judged
+constexpr int kCtProbe = 2;                             // rounds of kCtNT * kCtIPT points before the table is kept or given up
 constexpr uint32_t kCtFull = 1u << 23;                  // points of a block between two flushes (counts stay below 2^24)
 
 constexpr uint32_t inverse21(uint32_t d)
