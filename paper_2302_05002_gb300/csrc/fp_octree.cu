@@ -1066,11 +1066,12 @@ __global__ void __launch_bounds__(kTabNT, kTabCtas) k_tab_pieces(OctCtx c)
     if (threadIdx.x == 0) s_next = atomicAdd(c.tab_claim, run);
     __syncthreads();
     uint32_t k = s_next, k1 = k + run;
+    __syncthreads();   // every warp has read s_next before thread 0 writes it (at once, where run is 1)
     Piece next{};
     if (k < nt) next = c.list[LIST_TAB][k];
     while (k < nt) {
         const Piece p = next;
-        if (k + 1 == k1) {   // (every block barrier of a piece lies between this write and the read below)
+        if (k + 1 == k1) {   // (a barrier before this write, the piece's own ones before the read below)
             if (threadIdx.x == 0) s_next = atomicAdd(c.tab_claim, run);
         } else if (k + 1 < nt) {   // the next piece's records on their way to L2 during this one's work
             next = c.list[LIST_TAB][k + 1];
