@@ -118,6 +118,15 @@ FP_DEV uint32_t key_cell(int32_t x, int32_t y, int32_t z, const CubeDev& c, int 
            spread3_8(cell_at(z, c.o[2], c, l));
 }
 
+// key_cell of a point that may lie outside the cube, whose cells repeat there with
+// the cube's side: always below 8^l (exact up to 2^(31 - l) sides away)
+FP_DEV uint32_t key_cell_any(int32_t x, int32_t y, int32_t z, const CubeDev& c, int l)
+{
+    const uint32_t m = (1u << l) - 1u;
+    return spread3_8(cell_at(x, c.o[0], c, l) & m) * 4u + spread3_8(cell_at(y, c.o[1], c, l) & m) * 2u +
+           spread3_8(cell_at(z, c.o[2], c, l) & m);
+}
+
 // per-point code of the octree stage: LOD owner level (5 bits), leaf level (5
 // bits) and the Morton key of the point's level-g cell (3 g <= 21 bits)
 FP_DEV uint32_t code_make(int own, int leaf, uint32_t cell)

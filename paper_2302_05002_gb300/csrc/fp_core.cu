@@ -764,7 +764,8 @@ cudaError_t launch_bounds_decimate(const fp_point* pts, uint64_t n, fp_cube* cub
 // hash; the hash is a bijection, so the index of the point it is from follows from
 // it, and the points of all cells are compacted in index order as the uniform
 // preview's are.  (A second pass over the points, comparing each one's hash with
-// its cell's smallest: 10^8 points, 800 us; 75 us now.)
+// its cell's smallest: 10^8 points, 800 us; 75 us now.)  The cube is the caller's and
+// may be another cloud's: points outside it fall into the cells that repeat there.
 constexpr int kMinIPT = 4, kMinCtas = 5;
 
 __global__ void __launch_bounds__(256, kMinCtas) k_cell_min_hash(const fp_point* __restrict__ pts, uint64_t n,
@@ -789,7 +790,7 @@ __global__ void __launch_bounds__(256, kMinCtas) k_cell_min_hash(const fp_point*
         unsigned long long seen[kMinIPT];
 #pragma unroll
         for (int u = 0; u < kMinIPT; ++u) {
-            cell[u] = key_cell(q[u].x, q[u].y, q[u].z, cube, level);
+            cell[u] = key_cell_any(q[u].x, q[u].y, q[u].z, cube, level);
             seen[u] = cell_min[cell[u]];
         }
 #pragma unroll
@@ -800,7 +801,7 @@ __global__ void __launch_bounds__(256, kMinCtas) k_cell_min_hash(const fp_point*
     }
     for (; i0 < n; i0 += stride) {
         const int4 q = ld_point_cs(pts, i0);
-        unsigned long long* slot = cell_min + key_cell(q.x, q.y, q.z, cube, level);
+        unsigned long long* slot = cell_min + key_cell_any(q.x, q.y, q.z, cube, level);
         const unsigned long long h = splitmix64(first + i0);
         if (h < *slot) atomicMin(slot, h);
     }
@@ -843,7 +844,8 @@ __global__ void __launch_bounds__(256) k_cell_mark(const uint64_t* __restrict__ 
         if (last < n) {
             const CubeDev cube = load_cube(cube_p);
             const int4 p = ld_point(pts, last);
-            if (cell_min[key_cell(p.x, p.y, p.z, cube, level)] == ~0ull) atomicOr(&words[last >> 5], 1u << (last & 31));
+            if (cell_min[key_cell_any(p.x, p.y, p.z, cube, level)] == ~0ull)
+                atomicOr(&words[last >> 5], 1u << (last & 31));
         }
     }
 }
