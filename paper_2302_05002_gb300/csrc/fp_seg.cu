@@ -759,11 +759,11 @@ __global__ void __launch_bounds__(kClNT, 1) k_dist_cluster(DistClusterArgs a)
         uint32_t m;
         if (a.cells) {
             m = __ldg(a.cells + i);
-            if (m >= a.ncell) { raise(a.err, FP_ERR_CAPACITY, 19); m = 0; }
         } else {
             const int4 p = __ldg(a.pts + i);
             m = key_cell(p.x, p.y, p.z, cube, a.g);
         }
+        if (m >= a.ncell) { raise(a.err, FP_ERR_CAPACITY, 19); m = 0; }   // not a cell of the grid
         uint32_t c = __ldg(a.lut + m);
         if (c >= K) { raise(a.err, FP_ERR_CAPACITY, 13); c = K ? K - 1 : 0; }   // not a chunk
         a.key[0][i] = c;

@@ -284,6 +284,7 @@ __global__ void __launch_bounds__(kSortNT, 2) k_sort_pass(SortArgs a, int slot)
                 else {
                     int4 q = __ldg(in_pt + i);
                     d = key_cell(q.x, q.y, q.z, cube, a.g);   // cell; its chunk below
+                    if (d >> (3 * a.g)) { raise(a.err, FP_ERR_CAPACITY, 19); d = 0; }   // a point outside the cube
                 }
             }
             dg[r] = d;

@@ -59,3 +59,25 @@ def test_expected_is_the_oracles_inside(gpu_lib):
     cube = oracle.bounds(pts)
     want, _ = oracle.preview_spatial(pts, cube, 5, 7)
     assert np.array_equal(pts[expected(pts, np.atleast_1d(cube), 5, 7)], want)
+
+
+# one cluster, the sweeps, the radix passes
+@pytest.mark.parametrize("n", [1000, 1 << 15, (1 << 15) + 1, 100_003])
+@pytest.mark.parametrize("K", [8, 4097])
+def test_distribute_outside_the_cube(gpu_lib, n, K):
+    """Points of another cloud than the grid's: reported, and every read stays in the tables."""
+    fp, g = gpu_lib, 5
+    pts = synth.uniform(n, 95)
+    inner = synth.uniform(1000, 96)
+    for a in "xyz":
+        inner[a] = inner[a] // 64 + (1 << 18)
+    dev, cube = dev_points(pts), fp.fp_bounds(dev_points(inner))
+    lut = (torch.arange(1 << (3 * g), dtype=torch.int64, device="cuda") * K >> (3 * g)).to(torch.int32)
+    offsets = (torch.arange(K + 1, dtype=torch.int64, device="cuda") * n // K)
+    num = torch.tensor([K], dtype=torch.int32, device="cuda")
+    fp.get_device_error(clear=True)
+    fp.fp_distribute(dev, cube, g, lut, offsets, num)
+    torch.cuda.synchronize()
+    sites = fp.get_device_error_sites()
+    assert fp.get_device_error(clear=True) & (1 << 9)
+    assert sites >> 19 & 1
