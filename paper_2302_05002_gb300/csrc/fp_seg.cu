@@ -782,12 +782,25 @@ __global__ void __launch_bounds__(kClNT, 1) k_dist_cluster(DistClusterArgs a)
             });
         cur ^= 1;
     }
+    const uint32_t* key = a.key[cur];
     for (uint32_t q = t; q < a.n; q += kClThreads) {
-        const uint32_t c = a.key[cur][q], j = a.val[cur][q];
-        if (c >= K || q < a.offsets[c] || q >= a.offsets[c + 1])
-            raise(a.err, FP_ERR_CAPACITY, 15);   // offsets not those of these points
-        a.out[q] = __ldg(a.pts + j);
-        if (a.perm) a.perm[q] = j;
+        const uint32_t c = key[q], j = a.val[cur][q];
+        if (c >= K) continue;   // (no chunks)
+        const uint64_t start = a.offsets[c];
+        uint64_t o = q;
+        // starts in chunk order are the sorted places; else place q - (the chunk's first) behind the start
+        if (start > q || key[start] != c || (start && key[start - 1] == c)) {
+            uint32_t x = 0, y = q;
+            while (x < y) {
+                const uint32_t m = (x + y) >> 1;
+                if (key[m] < c) x = m + 1;
+                else y = m;
+            }
+            o = start + (q - x);
+        }
+        if (o >= a.n) { raise(a.err, FP_ERR_CAPACITY, 15); continue; }   // offsets not those of these points
+        a.out[o] = __ldg(a.pts + j);
+        if (a.perm) a.perm[o] = j;
     }
 }
 
