@@ -2052,9 +2052,9 @@ uint64_t node_capacity_bound(uint64_t n, const fp_params& p) { return oct_layout
 // node, and the inner nodes of a level hold more than C points each
 static uint64_t node_bound(uint64_t n, const fp_params& p)
 {
+    const uint64_t inner = n > p.node_capacity ? n / (p.node_capacity + 1) : 0;   // (a capacity of 2^64 - 1 is one)
     uint64_t b = 1;
-    for (uint32_t l = 0; l < p.max_level; ++l)
-        b += 8 * std::min(l < 20 ? 1ull << (3 * l) : ~0ull, (unsigned long long)(n / (p.node_capacity + 1)));
+    for (uint32_t l = 0; l < p.max_level; ++l) b += 8 * std::min<uint64_t>(l < 20 ? 1ull << (3 * l) : ~0ull, inner);
     return b;
 }
 
