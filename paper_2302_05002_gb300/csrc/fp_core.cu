@@ -244,19 +244,24 @@ __global__ void __launch_bounds__(256) k_count(const fp_point* __restrict__ pts,
 // uniform ones 143 * 10^9): most of their hits stay on chip instead.  A slot is one
 // word, found by a bijective hash of the cell: its upper bits are the slot, its
 // lower ones tell which of the slot's cells owns it (bits 24 .. 30, with a bit that
-// says that one does; the count below), the first cell that comes.  A block whose
-// first points rarely find their cell (a uniform cloud) goes past the table.  The
-// next points are loaded while these are counted.  With the cells written: 10^8
-// LiDAR points in random order 1562 -> 518 us, scan by scan 1761 -> 934 us; 10^7
-// 168 -> 87 and 127 -> 95 us; uniform, 10^8 710 -> 692 us, 10^7 79 -> 85 us, 4 * 10^6
-// 32 -> 42 us (half the warps in flight and the trial), so smaller clouds keep the
-// 1024-slot table of k_count.
+// says that one does; the count below), the first cell that comes.  A block tries
+// the table with its first points and goes past it when less than an eighth of them
+// brought an add that it took, which is where neighbouring lanes share cells (points
+// in cell order: few adds, to cells that no other block is at), unless one cell alone
+// holds an eighth: then every block is at the same few counters.  The next points are
+// loaded while these are counted.  With the cells written: 10^8 LiDAR points in random
+// order 1562 -> 518 us, scan by scan 1761 -> 934 us; 10^7 168 -> 87 and 127 -> 95 us;
+// uniform, 10^8 710 -> 692 us (707 past the table), 4 * 10^6 32 -> 42 us (half the warps
+// in flight and the trial), so smaller clouds keep the 1024-slot table of k_count.  In
+// cell order, 10^8: 666 -> 469 us (518 with the table); 5 * 10^7 points in one cell 336 ->
+// 264 us (1280 past the table), 95 in 100 of them 334 -> 276 us.
 constexpr uint64_t kCountTable = 1ull << 23;             // from this many points on
 constexpr int kCtNT = 1024, kCtIPT = 4;
 constexpr int kCtBits = 15, kCtSlots = 1 << kCtBits;
 constexpr int kCtLow = 21 - kCtBits;                    // bits of the hash below the slot
 constexpr uint32_t kCtMul = 0x9E3779B1u & 0x1FFFFFu;    // odd: a bijection of 21 bits
 constexpr int kCtProbe = 2;                             // rounds of kCtNT * kCtIPT points before the table is kept or given up
+constexpr uint32_t kCtTrial = kCtProbe * kCtNT * kCtIPT / 8;   // an eighth of these points
 constexpr uint32_t kCtFull = 1u << 23;                  // points of a block between two flushes (counts stay below 2^24)
 
 constexpr uint32_t inverse21(uint32_t d)
@@ -271,10 +276,10 @@ __global__ void __launch_bounds__(kCtNT, 1) k_count_table(const fp_point* __rest
                                                           uint32_t* __restrict__ counts, uint32_t* __restrict__ cells)
 {
     extern __shared__ uint32_t s_slot[];
-    __shared__ uint32_t s_hits;
+    __shared__ uint32_t s_hits, s_hot;
     const int lane = threadIdx.x & 31;
     for (int q = threadIdx.x; q < kCtSlots; q += kCtNT) s_slot[q] = 0;
-    if (threadIdx.x == 0) s_hits = 0;
+    if (threadIdx.x == 0) s_hits = s_hot = 0;
     __syncthreads();
     const CubeDev c = load_cube(cube);
     auto flush = [&]() {
@@ -284,6 +289,7 @@ __global__ void __launch_bounds__(kCtNT, 1) k_count_table(const fp_point* __rest
             if (w & 0xFFFFFFu) {
                 const uint32_t h = ((uint32_t)q << kCtLow) | ((w >> 24) & ((1u << kCtLow) - 1));
                 atomicAdd(&counts[(h * inverse21(kCtMul)) & 0x1FFFFFu], w & 0xFFFFFFu);
+                if ((w & 0xFFFFFFu) >= kCtTrial) s_hot = 1;
                 s_slot[q] = w & 0xFF000000u;
             }
         }
@@ -340,7 +346,7 @@ __global__ void __launch_bounds__(kCtNT, 1) k_count_table(const fp_point* __rest
             hits = __reduce_add_sync(0xFFFFFFFFu, hits);
             if (lane == 0) atomicAdd(&s_hits, hits);
             flush();   // (its barriers publish the sum)
-            table = s_hits >= kCtProbe * (uint32_t)(kCtNT * kCtIPT) / 8;
+            table = s_hits >= kCtTrial || s_hot;
             held = 0;
         }
         held += kCtNT * kCtIPT;
