@@ -55,40 +55,42 @@ struct SegPlan {
     uint32_t* err;
 };
 
-// step B for the chunk of this lane (c < K); all 32 lanes of the warp take part.
-// Callers spread the chunks over the warps first (a few large chunks: one each).
+// chunk c's node and digits; false: it does not fit the scatter
+FP_DEV bool seg_digits(const SegPlan& a, uint64_t c, uint32_t M, uint32_t& id, uint32_t& nb)
+{
+    const fp_chunk ch = a.chunks[c];
+    id = find_node(a.nodes, M, ch.key, ch.level);
+    if (id == kNone) return false;   // not in the table
+    const uint32_t nd = a.nodes[id].n_desc;
+    const uint64_t b = (uint64_t)nd + (a.owner ? 2 : 1);
+    nb = (uint32_t)b;
+    return (uint64_t)id + nd < M && b <= (1u << kSegMaxBits);
+}
+
+FP_DEV int seg_variant(uint32_t nb) { return nb <= (1u << kSegSmallBits) ? 0 : 1; }
+
+// step B for the chunk of this lane (c < K): its node, digits and tiles; all 32
+// lanes of the warp take part.  Callers spread the chunks over the warps first (a
+// few large chunks: one each).
 FP_DEV void seg_chunk(const SegPlan& a, uint64_t c, uint64_t K, uint32_t M)
 {
     const int lane = threadIdx.x & 31;
-    uint32_t id = 0, nd = 0, ntl = 0, at = 0, nb = 1;
-    uint64_t beg = 0;
-    int v = 0;
+    uint32_t id = 0, ntl = 0, at = 0, nb = 1;
     if (c < K) {
-        beg = a.offsets[c];
-        const uint64_t end = a.offsets[c + 1], cn = end - beg;
-        bool ok = true;
-        if (end > a.n || end < beg) ok = false;   // offsets not a partition of [0, n)
+        const uint64_t beg = a.offsets[c], end = a.offsets[c + 1], cn = end - beg;
+        bool ok = end <= a.n && end >= beg;   // else: offsets not a partition of [0, n)
         if (ok && cn) {
-            const fp_chunk ch = a.chunks[c];
-            id = find_node(a.nodes, M, ch.key, ch.level);
-            if (id == kNone) ok = false;          // not in the table: the whole-array path runs
+            ok = seg_digits(a, c, M, id, nb);
             if (ok) {
-                nd = a.nodes[id].n_desc;
-                const uint64_t b = (uint64_t)nd + (a.owner ? 2 : 1);
-                if ((uint64_t)id + nd >= M || b > (1u << kSegMaxBits)) ok = false;
-                else nb = (uint32_t)b;
-            }
-            if (ok) {
-                v = nb <= (1u << kSegSmallBits) ? 0 : 1;
                 ntl = (uint32_t)((cn + kSortTile - 1) / kSortTile);
-                at = atomicAdd(&a.cnt[v], ntl);
+                at = atomicAdd(&a.cnt[seg_variant(nb)], ntl);
                 if ((uint64_t)at + ntl > a.tiles_max) {
                     raise(a.err, FP_ERR_CAPACITY, 12);
                     ok = false;
                 }
             }
         }
-        if (!ok) {
+        if (!ok) {   // the whole-array path runs
             atomicOr(&a.cnt[2], 1u);
             id = 0; nb = 1; ntl = 0;
         }
@@ -100,22 +102,48 @@ FP_DEV void seg_chunk(const SegPlan& a, uint64_t c, uint64_t K, uint32_t M)
         const int l = __ffs(todo) - 1;
         const uint32_t nt = __shfl_sync(0xFFFFFFFFu, ntl, l), t0 = __shfl_sync(0xFFFFFFFFu, at, l);
         const uint32_t b = __shfl_sync(0xFFFFFFFFu, nb, l), x0 = __shfl_sync(0xFFFFFFFFu, id, l);
-        const uint32_t vv = __shfl_sync(0xFFFFFFFFu, (uint32_t)v, l);
         const uint32_t cc = __shfl_sync(0xFFFFFFFFu, (uint32_t)c, l);
-        const uint64_t base = __shfl_sync(0xFFFFFFFFu, (unsigned long long)beg, l);
-        SegTile* tl = a.tiles[vv];
-        uint32_t* st = a.status[vv];
-        const int sb = vv ? kSegMaxBits : kSegSmallBits;
+        SegTile* tl = a.tiles[seg_variant(b)];
         for (uint32_t i = lane; i < nt; i += 32) tl[t0 + i] = SegTile{cc, i};
-        for (uint32_t i = 0; i + 1 < nt; ++i) {   // (the last tile publishes nothing)
-            uint32_t* row = st + ((base / kSortTile + i) << sb);
-            for (uint32_t d = lane; d < b; d += 32) row[d] = 0;
-        }
         if (a.owner)
             for (uint32_t x = lane; x < b - 1; x += 32) a.inside[x0 + x] = 1;   // the chunk's node and n_desc below it
     }
 }
 
+// step B: the look-back words of rows r0 + lane (lane < per) cleared, by the whole
+// warp.  A row is written and read back where it holds the start of a tile that is
+// not its chunk's last: of the last chunk that starts in or before the row.
+FP_DEV void seg_rows(const SegPlan& a, uint64_t r0, uint32_t per, uint64_t rows, uint64_t K, uint32_t M)
+{
+    const int lane = threadIdx.x & 31;
+    const uint64_t r = r0 + lane;
+    uint32_t nb = 0;
+    if (lane < (int)per && r < rows) {
+        const uint64_t last = (r + 1) * kSortTile - 1;
+        uint64_t x = 0, y = K;   // chunks that start at or before `last`
+        while (x < y) {
+            const uint64_t m = (x + y) >> 1;
+            if (a.offsets[m] <= last) x = m + 1;
+            else y = m;
+        }
+        if (x) {
+            const uint64_t beg = a.offsets[x - 1], base = beg + (last - beg) / kSortTile * kSortTile;
+            uint32_t id;
+            if (base + kSortTile < a.offsets[x] && !seg_digits(a, x - 1, M, id, nb)) nb = 0;
+        }
+    }
+    for (uint32_t todo = __ballot_sync(0xFFFFFFFFu, nb != 0); todo; todo &= todo - 1) {
+        const int l = __ffs(todo) - 1;
+        const uint32_t b = __shfl_sync(0xFFFFFFFFu, nb, l);
+        const int v = seg_variant(b);
+        uint32_t* row = a.status[v] + ((r0 + l) << (v ? kSegMaxBits : kSegSmallBits));
+        for (uint32_t d = lane; d < b; d += 32) row[d] = 0;
+    }
+}
+
+// The chunks go over the warps from the first one, the rows from the last.  (The rows
+// of a chunk cleared by the chunk's warp: subsample of 10^8 points in one chunk, 133 MB
+// of look-back words, 8.5 instead of 2.9 ms.)
 __global__ void __launch_bounds__(256) k_seg_chunks(SegPlan a)
 {
     const uint64_t K = min((uint64_t)*a.num_chunks, a.kmax);
@@ -124,6 +152,8 @@ __global__ void __launch_bounds__(256) k_seg_chunks(SegPlan a)
     // lane l of warp w: chunks w + l * nwarps, + 32 * nwarps, ...
     const uint64_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
     for (uint64_t c0 = warp; c0 < K; c0 += 32 * nwarps) seg_chunk(a, c0 + (threadIdx.x & 31) * nwarps, K, M);
+    const uint64_t rows = a.n / kSortTile + 1, per = min((uint64_t)32, (rows + nwarps - 1) / nwarps);
+    for (uint64_t r0 = (nwarps - 1 - warp) * per; r0 < rows; r0 += nwarps * per) seg_rows(a, r0, (uint32_t)per, rows, K, M);
 }
 
 __global__ void __launch_bounds__(kClNT, 1) k_seg_plan(SegPlan a)
@@ -875,7 +905,8 @@ cudaError_t seg_scatter(const SegScratch& sc, const SegCall& c, const Workspace&
     const bool owner = c.mode == SEG_OWNER;
     SegPlan p = seg_plan(sc, c, ws);
     if ((e = cl_launch(k_seg_plan, p, st))) return e;
-    const int gk = (int)std::max<uint64_t>(1, std::min<uint64_t>((sc.kmax + 255) / 256, (uint64_t)ws.num_sms * 8));
+    const int gk = (int)std::min<uint64_t>(std::max<uint64_t>((sc.kmax + 255) / 256, (sc.rows + 7) / 8),
+                                           (uint64_t)ws.num_sms * 8);   // (a thread a chunk, a warp a row)
     k_seg_chunks<<<gk, 256, 0, st>>>(p);
     p.step_c = 1;
     if (owner && (e = cl_launch(k_seg_plan, p, st))) return e;
