@@ -30,14 +30,24 @@ FP_DEV void cl_sync()
 // Exclusive prefix sums over i in [0, n) of value(i) (a pair packed into 64
 // bits, each half below 2^32 in all), handed to store(i, prefix); returns the
 // total.  part: kClCtas words of global memory.  All threads of the cluster.
+// Rows of 1024 values, eight in flight a thread: with more than some 10^4 values
+// the time is the latency of these loads on 8 SMs (one in flight: 1.5 times as long).
+constexpr int kClRows = 8;
+struct ClScanSmem {
+    uint64_t row[kClRows][kClNT / 32], total, warp[kClNT / 32];
+};
+
 template <typename Value, typename Store>
-FP_DEV uint64_t cl_scan(uint32_t n, uint64_t* part, uint64_t* smem_warp /* 32 words */, Value value, Store store)
+FP_DEV uint64_t cl_scan(uint32_t n, uint64_t* part, ClScanSmem& S, Value value, Store store)
 {
+    constexpr int kWarps = kClNT / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t per = (n + kClCtas - 1) / kClCtas, lo = min(n, cl_rank() * per), hi = min(n, lo + per);
     uint64_t s = 0;
+#pragma unroll 8
     for (uint32_t i = lo + threadIdx.x; i < hi; i += kClNT) s += value(i);
     uint64_t tot;
-    block_exclusive_scan<kClNT, uint64_t>(s, smem_warp, tot);
+    block_exclusive_scan<kClNT, uint64_t>(s, S.warp, tot);
     if (threadIdx.x == 0) part[cl_rank()] = tot;
     cl_sync();
     uint64_t run = 0, all = 0;
@@ -46,12 +56,54 @@ FP_DEV uint64_t cl_scan(uint32_t n, uint64_t* part, uint64_t* smem_warp /* 32 wo
         if (r < (int)cl_rank()) run += v;
         all += v;
     }
-    for (uint32_t i0 = lo; i0 < hi; i0 += kClNT) {
-        const uint32_t i = i0 + threadIdx.x;
-        const uint64_t v = i < hi ? value(i) : 0;
-        const uint64_t ex = run + block_exclusive_scan<kClNT, uint64_t>(v, smem_warp, tot);
-        if (i < hi) store(i, ex);
-        run += tot;
+    for (uint32_t i0 = lo; i0 < hi; i0 += kClNT * kClRows) {
+        uint64_t v[kClRows], ex[kClRows];
+#pragma unroll
+        for (int u = 0; u < kClRows; ++u) {
+            const uint32_t i = i0 + u * kClNT + threadIdx.x;
+            v[u] = i < hi ? value(i) : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < kClRows; ++u) {
+            uint64_t x = v[u];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint64_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+                if (lane >= o) x += y;
+            }
+            if (lane == 31) S.row[u][warp] = x;
+            ex[u] = x - v[u];
+        }
+        __syncthreads();
+        if (warp == 0) {   // the rows' warps in order, eight of them a lane
+            constexpr int kPer = kClRows * kWarps / 32;
+            uint64_t* w = &S.row[0][0] + lane * kPer;
+            uint64_t sum = 0, x;
+#pragma unroll
+            for (int q = 0; q < kPer; ++q) sum += w[q];
+            x = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint64_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+                if (lane >= o) x += y;
+            }
+            if (lane == 31) S.total = x;
+            x -= sum;
+#pragma unroll
+            for (int q = 0; q < kPer; ++q) {
+                const uint64_t y = w[q];
+                w[q] = x;
+                x += y;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < kClRows; ++u) {
+            const uint32_t i = i0 + u * kClNT + threadIdx.x;
+            if (i < hi) store(i, run + S.row[u][warp] + ex[u]);
+        }
+        run += S.total;
+        __syncthreads();
     }
     cl_sync();   // (part may be written again)
     return all;

@@ -1807,11 +1807,11 @@ struct LayoutArgs {
 __global__ void __launch_bounds__(kClNT, 1) k_layout_cluster(LayoutArgs a)
 {
     __shared__ ClSortSmem s_sort;
-    __shared__ uint64_t s_warp[32];
+    __shared__ ClScanSmem s_scan;
     const uint32_t t = cl_rank() * kClNT + threadIdx.x;
     const uint32_t M = min(*a.num_nodes, a.node_cap);
     if (a.original)
-        cl_scan(M, a.part, s_warp, [&](uint32_t i) -> uint64_t { return a.nodes[i].n_own; },
+        cl_scan(M, a.part, s_scan, [&](uint32_t i) -> uint64_t { return a.nodes[i].n_own; },
                 [&](uint32_t i, uint64_t ex) { a.nodes[i].first = ex; });
     for (uint32_t j = t; j < a.n; j += kClThreads) {
         uint32_t i = a.original ? a.perm[j] : j;

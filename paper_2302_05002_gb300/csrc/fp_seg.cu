@@ -29,11 +29,15 @@ FP_DEV uint32_t find_node(const fp_node* nodes, uint32_t M, uint64_t key, uint32
 //     chunk subtrees; the look-back words of tiles that others will read cleared;
 //   C (owner layout): the nodes outside every chunk subtree ranked in order, and
 //     where each one's staged points start.
-// One cluster does A and C (a chain of launches before); step B, whose work grows
-// with chunks and tiles, takes the whole GPU.
+// Three launches: A's sums of segments of the node table (k_seg_nodes); B, with A's
+// prefixes (k_seg_chunks), both on the whole GPU; C by one cluster (k_seg_plan), which
+// reads five bytes a node.  One cluster also does all of A where nothing else is asked
+// for (clouds of up to 2^21 points).  (A by one cluster everywhere: the plan of 2.4 *
+// 10^6 nodes 840 us, 320 us now; of 2257, 25 and 23 us.)
+constexpr uint32_t kSegNodes = 512;   // segments of the node table
 struct SegPlan {
     int owner;               // 1: owner layout, 0: leaf grouping
-    int step_c;              // 0: A, 1: C
+    int step_c;              // k_seg_plan: 0: A, 1: C
     fp_node* nodes;
     const uint32_t* num_nodes;
     uint32_t node_cap;
@@ -54,6 +58,67 @@ struct SegPlan {
     uint32_t *hist, *hist2;  // the sorts' histograms, cleared in A
     uint32_t* err;
 };
+
+// A's scratch words (thread t of nt)
+FP_DEV void seg_clear(const SegPlan& a, uint32_t t, uint32_t nt, uint32_t M)
+{
+    for (uint32_t q = t; q < 8; q += nt) a.cnt[q] = 0;
+    for (uint32_t q = t; q < (uint32_t)kSortHistWords; q += nt) {
+        a.hist[q] = 0;
+        if (a.hist2) a.hist2[q] = 0;
+    }
+    if (a.owner && t == 0) { *a.nm = M; *a.nstaged = 0; }
+}
+
+// nodes of a segment: a multiple of 256, so that its words can be read as vectors
+FP_DEV uint32_t seg_nodes_per(uint32_t M) { return ((M + kSegNodes - 1) / kSegNodes + 255) & ~255u; }
+
+// step A, first half: scratch words, owned counts, and their sum per segment
+__global__ void __launch_bounds__(256) k_seg_nodes(SegPlan a)
+{
+    __shared__ uint64_t s_warp[8];
+    const uint32_t M = min(*a.num_nodes, a.node_cap);
+    seg_clear(a, blockIdx.x * 256 + threadIdx.x, gridDim.x * 256, M);
+    if (!a.owner) return;
+    const uint32_t per = seg_nodes_per(M), lo = min((uint64_t)M, (uint64_t)blockIdx.x * per), hi = min(M, lo + per);
+    uint64_t sum = 0, total;
+#pragma unroll 8
+    for (uint32_t i = lo + threadIdx.x; i < hi; i += 256) {
+        const uint32_t v = a.nodes[i].n_own;
+        a.nown[i] = v;
+        a.inside[i] = 0;
+        sum += v;
+    }
+    block_exclusive_scan<256, uint64_t>(sum, s_warp, total);
+    if (threadIdx.x == 0) a.part[blockIdx.x] = total;
+}
+
+// second half: the first points of the nodes of segment q
+FP_DEV void seg_first(const SegPlan& a, uint32_t q, uint32_t M, uint64_t* smem /* 8 */)
+{
+    const uint32_t per = seg_nodes_per(M), lo = min((uint64_t)M, (uint64_t)q * per), hi = min(M, lo + per);
+    if (lo >= hi) return;   // (the same for the block)
+    uint64_t before = 0, run;
+    for (uint32_t i = threadIdx.x; i < q; i += 256) before += a.part[i];
+    block_exclusive_scan<256, uint64_t>(before, smem, run);
+    for (uint32_t i0 = lo; i0 < hi; i0 += 1024) {
+        const uint32_t i = i0 + 4 * threadIdx.x;
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (i < hi) v = *reinterpret_cast<const uint4*>(a.nown + i);   // (hi is rounded up within the array)
+        const uint32_t w[4] = {v.x, i + 1 < hi ? v.y : 0u, i + 2 < hi ? v.z : 0u, i + 3 < hi ? v.w : 0u};
+        uint64_t total;
+        uint64_t ex = run + block_exclusive_scan<256, uint64_t>((uint64_t)w[0] + w[1] + w[2] + w[3], smem, total);
+        run += total;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (i + u < hi) {
+                a.first[i + u] = ex;
+                a.nodes[i + u].first = ex;
+            }
+            ex += w[u];
+        }
+    }
+}
 
 // chunk c's node and digits; false: it does not fit the scatter
 FP_DEV bool seg_digits(const SegPlan& a, uint64_t c, uint32_t M, uint32_t& id, uint32_t& nb)
@@ -146,6 +211,7 @@ FP_DEV void seg_rows(const SegPlan& a, uint64_t r0, uint32_t per, uint64_t rows,
 // of look-back words, 8.5 instead of 2.9 ms.)
 __global__ void __launch_bounds__(256) k_seg_chunks(SegPlan a)
 {
+    __shared__ uint64_t s_warp[8];
     const uint64_t K = min((uint64_t)*a.num_chunks, a.kmax);
     const uint32_t M = min(*a.num_nodes, a.node_cap);
     if (blockIdx.x == 0 && threadIdx.x == 0 && (*a.num_chunks > a.kmax || a.offsets[K] != a.n)) atomicOr(&a.cnt[2], 1u);
@@ -154,27 +220,21 @@ __global__ void __launch_bounds__(256) k_seg_chunks(SegPlan a)
     for (uint64_t c0 = warp; c0 < K; c0 += 32 * nwarps) seg_chunk(a, c0 + (threadIdx.x & 31) * nwarps, K, M);
     const uint64_t rows = a.n / kSortTile + 1, per = min((uint64_t)32, (rows + nwarps - 1) / nwarps);
     for (uint64_t r0 = (nwarps - 1 - warp) * per; r0 < rows; r0 += nwarps * per) seg_rows(a, r0, (uint32_t)per, rows, K, M);
+    if (a.owner)   // (from the blocks in the middle on)
+        for (uint32_t q = (blockIdx.x + gridDim.x / 2) % gridDim.x; q < kSegNodes; q += gridDim.x) seg_first(a, q, M, s_warp);
 }
 
 __global__ void __launch_bounds__(kClNT, 1) k_seg_plan(SegPlan a)
 {
-    __shared__ uint64_t s_warp[32];
+    __shared__ ClScanSmem s_scan;
     const uint32_t t = cl_rank() * kClNT + threadIdx.x;
     const uint32_t M = min(*a.num_nodes, a.node_cap);
     if (!a.step_c) {
-        for (uint32_t q = t; q < 8; q += kClThreads) a.cnt[q] = 0;
-        for (uint32_t q = t; q < (uint32_t)kSortHistWords; q += kClThreads) {
-            a.hist[q] = 0;
-            if (a.hist2) a.hist2[q] = 0;
-        }
-        if (!a.owner) return;
-        if (t == 0) { *a.nm = M; *a.nstaged = 0; }
-        for (uint32_t i = t; i < M; i += kClThreads) {
-            a.nown[i] = a.nodes[i].n_own;
-            a.inside[i] = 0;
-        }
+        seg_clear(a, t, kClThreads, M);
+#pragma unroll 8
+        for (uint32_t i = t; i < M; i += kClThreads) a.nown[i] = a.nodes[i].n_own;
         cl_sync();
-        cl_scan(M, a.part, s_warp, [&](uint32_t i) -> uint64_t { return a.nown[i]; },
+        cl_scan(M, a.part, s_scan, [&](uint32_t i) -> uint64_t { return a.nown[i]; },
                 [&](uint32_t i, uint64_t ex) {
                     a.first[i] = ex;
                     a.nodes[i].first = ex;
@@ -182,7 +242,7 @@ __global__ void __launch_bounds__(kClNT, 1) k_seg_plan(SegPlan a)
         return;
     }
     const uint64_t all = cl_scan(
-        M, a.part, s_warp,
+        M, a.part, s_scan,
         [&](uint32_t i) -> uint64_t { return a.inside[i] ? 0ull : (1ull << 32) | a.nown[i]; },
         [&](uint32_t i, uint64_t ex) {
             a.soff[i] = (uint32_t)ex;
@@ -207,7 +267,7 @@ SegScratch take_seg_scratch(const Workspace& ws, uint64_t n, uint64_t kmax, uint
     s.status[1] = ws.take<uint32_t>(s.rows << kSegMaxBits);
     s.cnt = ws.take<uint32_t>(8);
     s.inside = ws.take<uint8_t>(s.node_cap);
-    s.part = ws.take<uint64_t>(kClCtas);
+    s.part = ws.take<uint64_t>(std::max<int>(kClCtas, kSegNodes));
     return s;
 }
 
@@ -904,7 +964,7 @@ cudaError_t seg_scatter(const SegScratch& sc, const SegCall& c, const Workspace&
     cudaError_t e;
     const bool owner = c.mode == SEG_OWNER;
     SegPlan p = seg_plan(sc, c, ws);
-    if ((e = cl_launch(k_seg_plan, p, st))) return e;
+    k_seg_nodes<<<owner ? kSegNodes : 1, 256, 0, st>>>(p);
     const int gk = (int)std::min<uint64_t>(std::max<uint64_t>((sc.kmax + 255) / 256, (sc.rows + 7) / 8),
                                            (uint64_t)ws.num_sms * 8);   // (a thread a chunk, a warp a row)
     k_seg_chunks<<<gk, 256, 0, st>>>(p);

@@ -71,3 +71,46 @@ def test_one_chunk_is_no_chain(gpu_lib):
                                                final_perm=final_perm))
     assert fp.get_device_error() == 0
     assert layout < 3 * distribute, (layout, distribute)
+
+
+# a node table of one segment, of a few, of all 512 and of several tiles each
+@pytest.mark.parametrize("C", [1 << 21, 3_000, 100, 1])
+def test_node_tables(gpu_lib, C):
+    fp = gpu_lib
+    pts = synth.uniform(N, 102)
+    prm = (7, 7, 10, 16, max(C, 600), C)
+    r = fp.build_octree(dev_points(pts), fp.params(*prm))
+    torch.cuda.synchronize()
+    assert fp.get_device_error() == 0
+    want = oracle.build_all(pts, oracle.params(*prm))
+    M = int(r["num_nodes"].item())
+    assert_build_matches_oracle(want, nodes=r["nodes"][:M], final=r["final"], final_perm=r["final_perm"])
+
+
+def test_many_nodes_are_no_chain(gpu_lib):
+    """The chunk-wise scatter with 3.2 * 10^6 nodes against the same cloud's with 585: its
+    plan reads the node table on the whole GPU (6.2 times as long; by one cluster 12.6)."""
+    fp, n, ms = gpu_lib, N, []
+    pts = torch.randint(0, 1 << 20, (n, 4), dtype=torch.int32, device="cuda")
+    cube = fp.fp_bounds(pts)
+    counts = fp.fp_count(pts, cube, 7)
+    ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+    for e in ev:
+        e.record()
+    torch.cuda.synchronize()
+    for T, C in ((20_000, 20_000), (600, 1)):
+        prm = fp.params(7, 7, 15, 16, T, C)
+        chunks, num, lut, offsets = fp.fp_merge_chunks(counts, 7, T)
+        dist, perm = fp.fp_distribute(pts, cube, 7, lut, offsets, num)
+        nodes, m, _, _, owner = fp.fp_build_chunk_octree(dist, perm, cube, chunks, num, offsets, counts, prm, leaf=False)
+        ws = torch.empty(fp.workspace_size("subsample", n, prm), dtype=torch.uint8, device="cuda")
+        one = []
+        fp.time_kernel("owner_scatter", ev[0], ev[1])
+        for _ in range(9):
+            fp.fp_subsample(nodes, m, dist, perm, owner, chunks, num, offsets, prm, ws=ws)
+            torch.cuda.synchronize()
+            one.append(ev[0].elapsed_time(ev[1]))
+        fp.time_kernel(0)
+        ms.append(sorted(one)[4])
+    assert fp.get_device_error() == 0
+    assert ms[1] < 9 * ms[0], ms
