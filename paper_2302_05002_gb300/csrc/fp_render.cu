@@ -244,6 +244,7 @@ struct RasterArgs {
     const uint32_t *ids, *num_sel;
     uint32_t cap;
     uint64_t* pstart;    // cap: first drawn point of every drawn node
+    uint64_t* pshift;    // cap: its place among the points, less pstart
     uint64_t* part;      // one word per block
     const int4* fin;
     uint64_t n;
@@ -255,8 +256,11 @@ struct RasterArgs {
 
 // Each block draws a run of consecutive points of the drawn nodes, its warps 128
 // of them in turn: four loads and four projections a lane in flight.  A warp
-// follows the node it is in and holds the next 32 starts, one a lane; only 128
-// points that span more nodes than that are searched each.
+// follows the node it is in and holds the starts of the next 32 and where their
+// points are, one a lane; 128 points that span more nodes are searched among those
+// nodes, and a node further ahead is found by 32 probes at a time.  (Nodes of a few
+// points: with a search of all drawn nodes a chunk, and of each point where they are
+// many, 3 * 10^6 points of 176,581 nodes took 142 us, 86 now.)
 //
 // A node's points fall on few pixels, in random order, about 30 of them on each:
 // a direct-mapped table in shared memory (32 x 32 pixels, pixel and depth in one
@@ -268,7 +272,7 @@ struct RasterArgs {
 // Bound by instructions (about 140 a point) and latency at 32 warps an SM.  A frame
 // of 30M points, 26.6M drawn, selection included: one point in flight a lane, each
 // searched among all drawn nodes, 385 us; runs and four in flight 278 us; with the
-// table 203 us; the next points on their way to L2, 196 us.  Two points a lane and
+// table 203 us; the next points on their way to L2 196, also across nodes 188 us.  Two points a lane and
 // five blocks an SM drew in 200 us instead of 182, three and five in 208.
 constexpr int kRasterPer = 4, kRasterCtas = 4;
 constexpr int kRasterTabX = 32, kRasterTabY = 32;   // powers of two
@@ -301,10 +305,14 @@ __global__ void __launch_bounds__(kRenderNT, kRasterCtas) k_raster(RasterArgs a)
     uint64_t run = pre.before;
     for (uint32_t k0 = lo; k0 < hi; k0 += kRenderNT) {
         const uint32_t k = k0 + tid;
-        const uint64_t v = k < hi ? a.nodes[a.ids[k]].n_own : 0;
+        const fp_node* nd = k < hi ? a.nodes + a.ids[k] : nullptr;
+        const uint64_t v = nd ? nd->n_own : 0, first = nd ? nd->first : 0;
         const uint64_t ex = run + block_exclusive_scan<kRenderNT, uint64_t>(v, s_warp, total);
         run += total;
-        if (k < hi) a.pstart[k] = ex;
+        if (k < hi) {
+            a.pstart[k] = ex;
+            a.pshift[k] = first - ex;
+        }
     }
     if (!grid_barrier(a.bar, 2, a.err)) return;
 
@@ -314,43 +322,45 @@ __global__ void __launch_bounds__(kRenderNT, kRasterCtas) k_raster(RasterArgs a)
     const uint64_t p1 = min(P, ((uint64_t)blockIdx.x + 1) * len);
     uint64_t c = (uint64_t)blockIdx.x * len + (tid >> 5) * kChunk;
     if (c >= p1) return;
-    const uint64_t* ps = a.pstart;
-    auto node_of = [&](uint64_t p, uint32_t x) {   // last start <= p (nodes without points share starts), from x on
-        uint32_t y = S;
+    const uint64_t *ps = a.pstart, *psh = a.pshift;
+    // last start <= p (nodes without points share starts), from x on, by the whole warp:
+    // two reads a lane where it is among the next 1024 nodes, then 32 probes of the rest
+    // at a time
+    auto node_ahead = [&](uint64_t p, uint32_t x) {
+        uint32_t y = min((uint64_t)S, (uint64_t)x + 1024);
         while (x < y) {
-            const uint32_t m = (x + y) >> 1;
-            if (__ldcg(ps + m) <= p) x = m + 1;
-            else y = m;
+            const uint32_t step = (y - x + 31) >> 5, i = x + lane * step;
+            const uint32_t n = __popc(__ballot_sync(0xFFFFFFFFu, i < y && __ldcg(ps + i) <= p));
+            if (!n) break;
+            const uint32_t lo = x + (n - 1) * step, hi = min(y, lo + step);
+            y = hi == y ? (y < S ? S : y) : hi;   // (past the window: the rest)
+            x = lo + 1;
         }
         return x - 1;
     };
-    uint32_t k = node_of(c, 0);
-    uint64_t start = __ldcg(ps + k), first, nxt;   // nxt: start of node k + 1 + lane
+    uint32_t k = node_ahead(c, 0);
+    uint64_t shift, nxt, nsh;   // of node k; start and shift of node k + 1 + lane
     auto enter = [&]() {
-        first = a.nodes[a.ids[k]].first;
-        nxt = k + 1 + lane < S ? __ldcg(ps + k + 1 + lane) : ~0ull;
+        const bool in = k + 1 + lane < S;
+        shift = __ldcg(psh + k);
+        nxt = in ? __ldcg(ps + k + 1 + lane) : ~0ull;
+        nsh = in ? __ldcg(psh + k + 1 + lane) : 0ull;
     };
     enter();
     for (; c < p1; c += kStep) {
         if (const int past = __popc(__ballot_sync(0xFFFFFFFFu, nxt <= c))) {   // this chunk starts in a later node
-            if (past < 32) {
-                k += past;
-                start = __shfl_sync(0xFFFFFFFFu, nxt, past - 1);
-            } else {
-                k = node_of(c, k + 1);
-                start = __ldcg(ps + k);
-            }
+            k = past < 32 ? k + past : node_ahead(c, k + 1);
             enter();
         }
         const uint64_t ce = min(p1, c + kChunk);
+        // the next chunk's lines on their way to L2 (8 points a line; drawn nodes mostly follow one another)
+        if (lane < kChunk / 8 && c + shift + kStep + 8 * lane < a.n) prefetch_l2(a.fin + c + shift + kStep + 8 * lane);
         int4 q[kRasterPer];
         uint32_t ok = 0;   // bit r: point r is there
         if (__shfl_sync(0xFFFFFFFFu, nxt, 0) >= ce) {   // all in one node
-            const uint64_t at = first + (c - start);
+            const uint64_t at = c + shift;
             const uint32_t left = at < a.n ? (uint32_t)min(ce - c, a.n - at) : 0u;   // (a node table of another
             const int4* src = a.fin + at;                                            // point array may pass n)
-            // the next chunk's lines on their way to L2 (8 points a line)
-            if (lane < kChunk / 8 && at + kStep + 8 * lane < a.n) prefetch_l2(src + kStep + 8 * lane);
 #pragma unroll
             for (int r = 0; r < kRasterPer; ++r) {
                 q[r] = make_int4(0, 0, 0, 0);
@@ -361,30 +371,37 @@ __global__ void __launch_bounds__(kRenderNT, kRasterCtas) k_raster(RasterArgs a)
             }
         } else {
             const bool held = __shfl_sync(0xFFFFFFFFu, nxt, 31) >= ce;   // the 32 starts reach beyond the chunk
-#pragma unroll 1
-            for (int r = 0; r < kRasterPer; ++r) {
-                const uint64_t p = c + r * 32 + lane;
-                uint32_t x = k;
-                uint64_t from = start;
-                if (held) {
+            uint64_t at[kRasterPer];
+            if (held) {
+#pragma unroll
+                for (int r = 0; r < kRasterPer; ++r) {
+                    const uint64_t p = c + r * 32 + lane;
                     int o = 0;   // nodes of the 32 that start at or before p
 #pragma unroll
                     for (int d = 16; d > 0; d >>= 1)
                         if (__shfl_sync(0xFFFFFFFFu, nxt, (o + d - 1) & 31) <= p) o += d;
-                    const uint64_t f = __shfl_sync(0xFFFFFFFFu, nxt, (o + 31) & 31);
-                    if (o) { x = k + o; from = f; }
-                } else if (p < ce) {
-                    x = node_of(p, k + 1);
-                    from = __ldcg(ps + x);
+                    const uint64_t f = __shfl_sync(0xFFFFFFFFu, nsh, (o + 31) & 31);
+                    at[r] = p + (o ? f : shift);
                 }
-                int4 v = make_int4(0, 0, 0, 0);
-                if (p < ce) {
-                    const uint64_t at = a.nodes[a.ids[x]].first + (p - from);
-                    if (at < a.n) { v = __ldg(a.fin + at); ok |= 1u << r; }
-                }
+            } else {   // a search each, all in step, among the nodes of the chunk
+                const uint32_t last = node_ahead(ce - 1, k + 1);
+                uint32_t x[kRasterPer];
 #pragma unroll
-                for (int u = 0; u < kRasterPer; ++u)
-                    if (u == r) q[u] = v;
+                for (int r = 0; r < kRasterPer; ++r) x[r] = k;
+                for (uint32_t bit = 0x80000000u >> __clz(last - k); bit; bit >>= 1)
+#pragma unroll
+                    for (int r = 0; r < kRasterPer; ++r)
+                        if (x[r] + bit <= last && __ldcg(ps + x[r] + bit) <= c + r * 32 + lane) x[r] += bit;
+#pragma unroll
+                for (int r = 0; r < kRasterPer; ++r) at[r] = c + r * 32 + lane + __ldcg(psh + x[r]);
+            }
+#pragma unroll
+            for (int r = 0; r < kRasterPer; ++r) {
+                q[r] = make_int4(0, 0, 0, 0);
+                if (c + r * 32 + lane < ce && at[r] < a.n) {
+                    q[r] = __ldg(a.fin + at[r]);
+                    ok |= 1u << r;
+                }
             }
         }
         uint32_t px[kRasterPer];
@@ -421,7 +438,7 @@ __global__ void __launch_bounds__(kRenderNT, kRasterCtas) k_raster(RasterArgs a)
 struct RenderBufs {
     uint8_t* vis;
     uint32_t *diff, *num;
-    uint64_t *pstart, *tiles64;
+    uint64_t *pstart, *pshift, *tiles64;
 };
 
 static RenderBufs render_carve(const Workspace& ws, uint32_t cap)
@@ -432,6 +449,7 @@ static RenderBufs render_carve(const Workspace& ws, uint32_t cap)
     B.diff = ws.take<uint32_t>(M + 1);
     B.num = ws.take<uint32_t>(2);
     B.pstart = ws.take<uint64_t>(M);
+    B.pshift = ws.take<uint64_t>(M);
     B.tiles64 = ws.take<uint64_t>(kScanMaxTiles);
     return B;
 }
@@ -471,7 +489,7 @@ cudaError_t launch_rasterize(const fp_node* nodes, const uint32_t* ids, const ui
     int per_sm = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_raster, kRenderNT, 0))) return e;
     RasterArgs a{};
-    a.nodes = nodes; a.ids = ids; a.num_sel = num_sel; a.cap = cap; a.pstart = B.pstart; a.part = B.tiles64;
+    a.nodes = nodes; a.ids = ids; a.num_sel = num_sel; a.cap = cap; a.pstart = B.pstart; a.pshift = B.pshift; a.part = B.tiles64;
     a.fin = reinterpret_cast<const int4*>(fin); a.n = n; a.cam = cam_dev(cam); a.fb = fb; a.bar = B.num;
     a.err = ws.err;
     const unsigned grid = (unsigned)std::min<uint64_t>(kScanMaxTiles, (uint64_t)num_sms * std::min(std::max(per_sm, 1), kRasterCtas));
