@@ -720,30 +720,30 @@ cudaError_t launch_bounds_decimate(const fp_point* pts, uint64_t n, fp_cube* cub
     if (decim && n == 0) k_zero_count<<<1, 1, 0, st>>>(out_count);
     if (!bounds) {
         KTimerScope kt(FP_KERNEL_BOUNDS_DECIMATE, st);
-        // 8192-point tiles; 2048-point ones while those leave SMs without a block
         if (n == 0) return cudaGetLastError();
-        // 8192-point tiles, as many blocks as are resident; from four tiles an SM on (fewer leave most of the
-        // GPU without work: the two launches with 2048-point tiles then) up to kKeepTiles a block
-        KeepScratch s = keep_carve(ws, n, kKeepRows, false);
+        // tiles of 2048 points in two launches while fewer than four tiles of 8192 an SM would leave most of the GPU
+        // without work; those, as many blocks as are resident, in one launch up to kKeepTiles a block, else in two
+        constexpr uint64_t kTile = (uint64_t)kBdNT * kKeepRows;
+        if ((n + kTile - 1) / kTile < (uint64_t)ws.num_sms * 4) {
+            keep_launch<false, kKeepRowsSmall>(keep_carve(ws, n, kKeepRowsSmall, false), pts, n, first, modulus, out,
+                                               out_cap, out_count, ws, st);
+            return cudaGetLastError();
+        }
+        const KeepScratch two = keep_carve(ws, n, kKeepRows, false);
         uint32_t* bar = ws.take<uint32_t>(1);
         int per_sm = 0;
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_keep_all, kBdNT, kKeepTiles * kBdNT * 4)))
             return e;
         const uint64_t blocks = std::min<uint64_t>((uint64_t)std::max(per_sm, 1) * ws.num_sms, kKeepSegs);
+        KeepScratch s = two;
         s.per = (s.ntiles + blocks - 1) / blocks;
-        if (s.ntiles >= (uint64_t)ws.num_sms * 4 && s.per <= (uint64_t)kKeepTiles) {
-            if ((e = cudaMemsetAsync(bar, 0, sizeof(uint32_t), st))) return e;
-            return coop_launch(k_keep_all, (unsigned)((s.ntiles + s.per - 1) / s.per), kBdNT, s.per * kBdNT * 4, st, pts, n,
-                               first, KeepMultiple::of(modulus), s, bar, out, out_cap, out_count, ws.err);
+        if (s.per > (uint64_t)kKeepTiles) {
+            keep_launch<false, kKeepRows>(two, pts, n, first, modulus, out, out_cap, out_count, ws, st);
+            return cudaGetLastError();
         }
-        ws.used = 0;
-        if (s.ntiles >= (uint64_t)ws.num_sms * 4)
-            keep_launch<false, kKeepRows>(keep_carve(ws, n, kKeepRows, false), pts, n, first, modulus, out, out_cap,
-                                          out_count, ws, st);
-        else
-            keep_launch<false, kKeepRowsSmall>(keep_carve(ws, n, kKeepRowsSmall, false), pts, n, first, modulus, out,
-                                               out_cap, out_count, ws, st);
-        return cudaGetLastError();
+        if ((e = cudaMemsetAsync(bar, 0, sizeof(uint32_t), st))) return e;
+        return coop_launch(k_keep_all, (unsigned)((s.ntiles + s.per - 1) / s.per), kBdNT, s.per * kBdNT * 4, st, pts, n,
+                           first, KeepMultiple::of(modulus), s, bar, out, out_cap, out_count, ws.err);
     }
     const BoundsScratch b = bounds_carve(ws, n, ws.num_sms);
     const int grid = (int)std::min<uint64_t>(b.ntiles ? b.ntiles : 1, (uint64_t)ws.num_sms * 8);
