@@ -190,7 +190,6 @@ __global__ void k_zero_count(uint64_t* out_count) { *out_count = 0; }
 constexpr int kCountSlots = 1024;
 
 // cells (nullable): the level-g Morton cell of every point, for fp_distribute_cells
-template <bool AGG>
 __global__ void __launch_bounds__(256) k_count(const fp_point* __restrict__ pts, uint64_t n,
                                                const fp_cube* __restrict__ cube, int g, uint32_t* __restrict__ counts,
                                                uint32_t* __restrict__ cells)
@@ -219,7 +218,7 @@ __global__ void __launch_bounds__(256) k_count(const fp_point* __restrict__ pts,
             // points) adds directly; otherwise its equal cells are merged first
             const uint32_t knext = __shfl_down_sync(0xFFFFFFFFu, key[u], 1);   // (lane 31: its own)
             const bool twin = lane < 31 && key[u] != kNone && key[u] == knext;
-            if (AGG && __any_sync(0xFFFFFFFFu, twin)) {
+            if (__any_sync(0xFFFFFFFFu, twin)) {
                 uint32_t peers = __match_any_sync(0xFFFFFFFFu, key[u]);
                 if (key[u] != kNone && lane == __ffs(peers) - 1) {
                     const uint32_t slot = (key[u] * 2654435761u) >> 22;   // 10-bit multiplicative hash
@@ -262,7 +261,7 @@ constexpr int kCtLow = 21 - kCtBits;                    // bits of the hash belo
 constexpr uint32_t kCtMul = 0x9E3779B1u & 0x1FFFFFu;    // odd: a bijection of 21 bits
 constexpr int kCtProbe = 2;                             // rounds of kCtNT * kCtIPT points before the table is kept or given up
 constexpr uint32_t kCtTrial = kCtProbe * kCtNT * kCtIPT / 8;   // an eighth of these points
-constexpr uint32_t kCtFull = 1u << 23;                  // points of a block between two flushes (counts stay below 2^24)
+constexpr uint64_t kCtMost = 1ull << 23;                // most points a block takes, so that counts stay below 2^24
 
 constexpr uint32_t inverse21(uint32_t d)
 {
@@ -297,7 +296,7 @@ __global__ void __launch_bounds__(kCtNT, 1) k_count_table(const fp_point* __rest
     };
     const uint64_t stride = (uint64_t)gridDim.x * kCtNT;
     bool table = true;
-    uint32_t round = 0, held = 0, hits = 0;
+    uint32_t round = 0, hits = 0;
     int4 p[kCtIPT];   // the next round's points, on their way while this one is counted
     auto load = [&](uint64_t i0) {
 #pragma unroll
@@ -347,10 +346,7 @@ __global__ void __launch_bounds__(kCtNT, 1) k_count_table(const fp_point* __rest
             if (lane == 0) atomicAdd(&s_hits, hits);
             flush();   // (its barriers publish the sum)
             table = s_hits >= kCtTrial || s_hot;
-            held = 0;
         }
-        held += kCtNT * kCtIPT;
-        if (held >= kCtFull) { flush(); held = 0; }
     }
     flush();
 }
@@ -894,10 +890,11 @@ cudaError_t launch_count(const fp_point* pts, uint64_t n, const fp_cube* cube, i
         const int smem = kCtSlots * (int)sizeof(uint32_t);
         cudaError_t e = cudaFuncSetAttribute(k_count_table, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e) return e;
-        k_count_table<<<ws.num_sms, kCtNT, smem, st>>>(pts, n, cube, g, counts, cells);
+        const unsigned blocks = (unsigned)std::max<uint64_t>(ws.num_sms, n / kCtMost + 1);   // (n < 2^30: 152 are enough)
+        k_count_table<<<blocks, kCtNT, smem, st>>>(pts, n, cube, g, counts, cells);
         return cudaGetLastError();
     }
-    k_count<true><<<grid, 256, 0, st>>>(pts, n, cube, g, counts, cells);
+    k_count<<<grid, 256, 0, st>>>(pts, n, cube, g, counts, cells);
     return cudaGetLastError();
 }
 
