@@ -121,11 +121,33 @@ cudaError_t sort_plan_keys(const SortScratch& sc, SortArgs& a, uint32_t shift0, 
 }
 
 // ------------------------------------------------------------- distribute
+// The tables of the sweep lie where the radix passes' second point buffer does: one
+// or the other runs.
+struct DistBufs {
+    SortScratch sc;
+    int4* pt_tmp;
+    uint32_t *val_tmp, *run_sort;
+    Workspace sweep;   // dist_wide's
+};
+
+static DistBufs dist_bufs(const Workspace& ws, uint64_t n)
+{
+    DistBufs B;
+    B.sc = take_sort_scratch(ws, n);
+    B.sweep = ws;
+    B.pt_tmp = ws.take<int4>(n);
+    ws.used = std::max(ws.used, B.sweep.used + dist_wide_bytes(n));
+    B.val_tmp = ws.take<uint32_t>(n);
+    B.run_sort = ws.take<uint32_t>(1);
+    return B;
+}
+
 size_t distribute_ws_bytes(uint64_t n, int g)
 {
     (void)g;
-    return sort_scratch_bytes(n) + Workspace::bytes_for({16 * (size_t)n, 4 * (size_t)n, sizeof(uint32_t)}) +
-           dist_wide_bytes(n);
+    Workspace dry;
+    dist_bufs(dry, n);
+    return dry.used;
 }
 
 cudaError_t launch_distribute(const fp_point* pts, uint64_t n, const fp_cube* cube, int g, const uint32_t* lut,
@@ -133,11 +155,10 @@ cudaError_t launch_distribute(const fp_point* pts, uint64_t n, const fp_cube* cu
                               const Workspace& ws, cudaStream_t st, const uint32_t* cells)
 {
     if (n == 0) return cudaSuccess;
-    SortScratch sc = take_sort_scratch(ws, n);
-    int4* pt_tmp = ws.take<int4>(n);
-    uint32_t* val_tmp = ws.take<uint32_t>(n);
-    uint32_t* run_sort = ws.take<uint32_t>(1);
-    Workspace rest = ws;
+    const DistBufs B = dist_bufs(ws, n);
+    const SortScratch& sc = B.sc;
+    int4* const pt_tmp = B.pt_tmp;
+    uint32_t *const val_tmp = B.val_tmp, *const run_sort = B.run_sort;
     KTimerScope kt(FP_KERNEL_DISTRIBUTE, st);
     if (n <= kDistCluster) {
         uint32_t* const w = reinterpret_cast<uint32_t*>(pt_tmp);   // four words a point
@@ -150,7 +171,7 @@ cudaError_t launch_distribute(const fp_point* pts, uint64_t n, const fp_cube* cu
     // the cells or from the points.  More: the radix passes, which compute the
     // cells from the points.
     cudaError_t e = dist_wide(reinterpret_cast<const int4*>(pts), n, cube, g, lut, offsets, num_chunks,
-                              reinterpret_cast<int4*>(out), perm, run_sort, sc.hist, rest, st, cells,
+                              reinterpret_cast<int4*>(out), perm, run_sort, sc.hist, B.sweep, st, cells,
                               reinterpret_cast<uint16_t*>(val_tmp));
     if (e) return e;
     SortArgs a{};
