@@ -2470,7 +2470,6 @@ static NodesBufs nodes_carve(const Workspace& ws, const fp_params& p, uint64_t r
     B.rsum = ws.take<uint32_t>(kGtMaxTiles);
     B.nb.nk2 = ws.take<uint64_t>(R); B.nb.nk3 = ws.take<uint64_t>(R); B.nb.nk4 = ws.take<uint64_t>(R);
     B.nb.nl = ws.take<uint32_t>(R); B.nb.nv2 = ws.take<uint32_t>(R); B.nb.nv3 = ws.take<uint32_t>(R);
-    B.nb.leafw = ws.take<uint32_t>(std::max<uint64_t>(R, kScanMaxTiles));
     return B;
 }
 
@@ -2499,6 +2498,7 @@ cudaError_t launch_octree_nodes(const uint32_t* counts, uint64_t n, const fp_par
     k_cells_open<<<grid_tiles(g), kGtNT, 0, st>>>(ra, B.pyr, B.rsum, 0, 1, nullptr, nullptr);
     NodeSortBufs nb = B.nb;
     nb.nk = T.starts; nb.slevel = T.slevel; nb.idxtab = T.idxtab; nb.ndesc = T.ndesc;
+    nb.leafw = T.nown;   // (nobody reads the leaf sizes; cleared below)
     if ((e = node_table(B.sc, recs, T.nnode, (uint32_t)rec_cap, n ? node_bound(n, prm) : rec_cap, nb, nodes, node_cap,
                         num_nodes, g, lmax, ws, st)))
         return e;
