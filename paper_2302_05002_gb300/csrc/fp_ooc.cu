@@ -357,7 +357,6 @@ Fixed fixed_carve(const Workspace& w, uint64_t P, const fp_params& p, uint64_t n
 }
 
 struct Group {   // device buffers of one chunk group (G points), reused group after group
-    char* region;   // the start of the group region
     int4* pts;
     uint32_t *perm, *owner;
     uint32_t* codes;
@@ -384,7 +383,6 @@ Group group_carve(const Workspace& w, uint64_t G, uint64_t P, const fp_params& p
 {
     Group g;
     const uint64_t N = G ? G : 1;
-    g.region = w.base + w.used;
     g.pts = resident ? nullptr : w.take<int4>(N);
     g.perm = resident ? nullptr : w.take<uint32_t>(N);
     g.owner = w.take<uint32_t>(N);
@@ -800,18 +798,22 @@ fp_status build(const fp_point* h_pts, uint64_t n, const fp_params& prm, uint64_
     }
 
     // ---- the staged points: sorted by (owner, index), placed after their owners' earlier points
-    if (S) {   // the sort of the staged records reuses the whole group region
+    if (S) {   // the sort of the staged records has the arena behind the fixed buffers
         Workspace wf = base;
         // (the resident cloud is dead by now: the staged points were copied out with their records)
-        wf.base = resident ? reinterpret_cast<char*>(res_pts) : B.region;
-        wf.bytes = group_bytes(G, P, prm, node_cap, base.num_sms, resident) + (resident ? resident_bytes(n) : 0);
+        wf.base = base.base + after_fixed;
+        wf.bytes = arena_bytes - after_fixed;
         wf.used = 0;
         uint64_t* k1 = st_dev ? st_key : wf.take<uint64_t>(S);
         uint64_t* k2 = wf.take<uint64_t>(S);
         uint64_t* k3 = wf.take<uint64_t>(S);
         uint32_t* v2 = wf.take<uint32_t>(S);
         uint32_t* v3 = wf.take<uint32_t>(S);
-        const SortScratch sf = take_sort_scratch(wf, S);
+        // (the second set of look-back words in the dead piece buffers, where the staged points are not)
+        Workspace wd = dead;
+        if (!st_dev) wd.used = 0;
+        const bool second = wd.used + sort_status_bytes(S) + 256 <= wd.bytes;
+        const SortScratch sf = take_sort_scratch(wf, S, second ? &wd : nullptr);
         if (wf.used > wf.bytes) return FP_ERR_WORKSPACE;
         if (!st_dev) {
             if ((e = cudaMemcpyAsync(k1, st_key, S * 8, cudaMemcpyHostToDevice, st))) return cu(e);

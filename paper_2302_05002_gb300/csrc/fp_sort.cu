@@ -72,20 +72,26 @@ __global__ void __launch_bounds__(1024) k_plan_hist_keys(SortSpec p, uint32_t* s
         if (sh[q]) atomicAdd(&p.hist[q], sh[q]);
 }
 
+size_t sort_status_bytes(uint64_t n)
+{
+    return Workspace::round((sizeof(uint32_t) * std::max<uint64_t>(1, (n + kSortTile - 1) / kSortTile)) << kSortMaxBits);
+}
+
 // (the histogram first: callers clear it together with what lies before it)
 size_t sort_scratch_bytes(uint64_t n)
 {
-    const size_t words = (size_t)std::max<uint64_t>(1, (n + kSortTile - 1) / kSortTile) << kSortMaxBits;
-    return Workspace::bytes_for({sizeof(uint32_t) * kSortHistWords, sizeof(uint32_t) * words, sizeof(uint32_t) * words});
+    Workspace dry;
+    take_sort_scratch(dry, n);
+    return dry.used;
 }
 
-SortScratch take_sort_scratch(const Workspace& ws, uint64_t n)
+SortScratch take_sort_scratch(const Workspace& ws, uint64_t n, const Workspace* second)
 {
-    const size_t words = (size_t)std::max<uint64_t>(1, (n + kSortTile - 1) / kSortTile) << kSortMaxBits;
+    const size_t words = sort_status_bytes(n) / sizeof(uint32_t);
     SortScratch s;
     s.hist = ws.take<uint32_t>(kSortHistWords);
     s.status[0] = ws.take<uint32_t>(words);
-    s.status[1] = ws.take<uint32_t>(words);
+    s.status[1] = (second ? *second : ws).take<uint32_t>(words);
     return s;
 }
 

@@ -405,7 +405,9 @@ struct SortScratch {
     uint32_t* status[2];
 };
 size_t sort_scratch_bytes(uint64_t n);
-SortScratch take_sort_scratch(const Workspace& ws, uint64_t n);
+size_t sort_status_bytes(uint64_t n);   // of one set of look-back words
+// second: where the second set comes from (null: ws too)
+SortScratch take_sort_scratch(const Workspace& ws, uint64_t n, const Workspace* second = nullptr);
 
 // Histogram of a sort; returns its spec in a.spec and the look-back words in
 // a.status.  From weights of ids: record counts per id (weights, or differences
