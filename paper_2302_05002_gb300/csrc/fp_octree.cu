@@ -1867,7 +1867,7 @@ __global__ void __launch_bounds__(kClNT, 1) k_node_cluster(NodeClusterArgs a)
     cl_sync();
     for (uint32_t i = rank * kClNT + tid; i < M; i += kClThreads) {
         const NodeRec r = a.rec[vs[i]];
-        if (r.level == 0) continue;
+        if (r.level == 0 || r.key >> (3 * r.level)) continue;   // (a key beyond its level: not a record of these points)
         uint32_t p;
         if (r.level - 1 <= a.g) p = a.idxtab[((1ull << (3 * (r.level - 1))) - 1) / 7 + (r.key >> 3)];
         else p = node_lookup(ks, a.slevel, M, (r.key >> 3) << (3 * (lmax - r.level + 1)), r.level - 1);
@@ -2052,7 +2052,8 @@ __global__ void __launch_bounds__(kResolveNT) k_resolve(const fp_point* __restri
             const uint64_t j = base + (uint64_t)r * kResolveNT + threadIdx.x;
             uint32_t oid = kNone;
             if (j < n) {
-                const uint32_t cell = code_cell(cw[r]);
+                // (the mask: a point that no piece held, of a count grid of other points, has any code)
+                const uint32_t cell = code_cell(cw[r]) & ((1u << (3 * g)) - 1u);
                 const int ks[2] = {code_own(cw[r]), code_leaf(cw[r])};
                 uint32_t ids[2] = {0u, 0u};
                 for (int u = 0; u < nt; ++u) {
