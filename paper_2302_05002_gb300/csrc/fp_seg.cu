@@ -215,6 +215,15 @@ __global__ void __launch_bounds__(256) k_seg_chunks(SegPlan a)
     const uint64_t K = min((uint64_t)*a.num_chunks, a.kmax);
     const uint32_t M = min(*a.num_nodes, a.node_cap);
     if (blockIdx.x == 0 && threadIdx.x == 0 && (*a.num_chunks > a.kmax || a.offsets[K] != a.n)) atomicOr(&a.cnt[2], 1u);
+    if (blockIdx.x == 0 && a.owner) {   // more owned points than there are: step C counts them in 32 bits
+        uint64_t sum = 0, total;
+        for (uint32_t q = threadIdx.x; q < kSegNodes; q += 256) sum += a.part[q];
+        block_exclusive_scan<256, uint64_t>(sum, s_warp, total);
+        if (threadIdx.x == 0 && total > a.n) {
+            raise(a.err, FP_ERR_CAPACITY, 15);
+            atomicOr(&a.cnt[2], 1u);
+        }
+    }
     // lane l of warp w: chunks w + l * nwarps, + 32 * nwarps, ...
     const uint64_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
     for (uint64_t c0 = warp; c0 < K; c0 += 32 * nwarps) seg_chunk(a, c0 + (threadIdx.x & 31) * nwarps, K, M);
@@ -239,6 +248,10 @@ __global__ void __launch_bounds__(kClNT, 1) k_seg_plan(SegPlan a)
                     a.first[i] = ex;
                     a.nodes[i].first = ex;
                 });
+        return;
+    }
+    if (a.cnt[2]) {   // the whole-array path runs, without ranks
+        if (t == 0) *a.nrank = 0;
         return;
     }
     const uint64_t all = cl_scan(

@@ -52,3 +52,25 @@ def test_a_count_grid_of_other_points(gpu_lib, g, n, wrong):
     torch.cuda.synchronize()
     assert fp.get_device_error(clear=True) & CAPACITY
     rebuild(fp, synth.uniform(5_000, 104), prm)
+
+
+def test_more_owned_points_than_points(gpu_lib):
+    """A node table whose owned counts add up to 2^32 and more (not the table of these points)."""
+    fp = gpu_lib
+    n, prm = (1 << 21) + 5_000, (7, 7, 12, 16, 50_000, 5_000)
+    dev, p = dev_points(synth.uniform(n, 105)), fp.params(*prm)
+    cube = fp.fp_bounds(dev)
+    counts = fp.fp_count(dev, cube, 7)
+    chunks, num, lut, offsets = fp.fp_merge_chunks(counts, 7, prm[4])
+    dist, perm = fp.fp_distribute(dev, cube, 7, lut, offsets, num)
+    nodes, m, _, _, owner = fp.fp_build_chunk_octree(dist, perm, cube, chunks, num, offsets, counts, p, leaf=False)
+    torch.cuda.synchronize()
+    assert fp.get_device_error() == 0
+    words = nodes.view(torch.int32).view(-1, 10)   # n_own is the word behind count
+    M = int(m.item())
+    assert int(words[:M, 7].sum().item()) == n
+    words[:M:3, 7] = -1
+    fp.fp_subsample(nodes, m, dist, perm, owner, chunks, num, offsets, p)
+    torch.cuda.synchronize()
+    assert fp.get_device_error(clear=True) & CAPACITY
+    rebuild(fp, synth.uniform(5_000, 106), prm)
