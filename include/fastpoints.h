@@ -212,8 +212,9 @@ uint32_t fp_preview_modulus(uint64_t n, uint64_t target);
  * 1 <= level <= 7), the one with the smallest splitmix64(first_index + i) is
  * kept; kept points are written to d_out in ascending index, their number to
  * *d_out_count (= the number of occupied cells; beyond out_cap they are not
- * written and FP_ERR_CAPACITY is raised in the device word).  Two passes over
- * the points; the workspace holds an 8^level table of 64-bit minima
+ * written and FP_ERR_CAPACITY is raised in the device word).  The cube need not
+ * hold the points: its cells repeat outside it.  One pass over the points; the
+ * workspace holds an 8^level table of 64-bit minima and a bit per point
  * (fp_workspace_size(FP_STAGE_PREVIEW_SPATIAL, n, prm) with prm->grid_log2 =
  * level).  The whole cloud must be in one call (the minimum is over the cloud). */
 fp_status fp_preview_spatial(const fp_point* d_pts, uint64_t n, const fp_cube* d_cube, uint32_t level,
@@ -286,8 +287,9 @@ fp_status fp_distribute(const fp_point* d_pts, uint64_t n, const fp_cube* d_cube
 /* fp_distribute with the points' level-g cells given (d_cells from
  * fp_count_cells, same cube and grid_log2): the chunk of point i is
  * d_lut[d_cells[i]] instead of being computed from the point.  Both calls: up to
- * 4096 chunks take a counting pass and a double-buffered sweep (no wait between
- * blocks); more chunks the radix passes, which compute the cell.  Every
+ * 2^15 points are sorted in one launch; larger clouds of up to 4096 chunks take a
+ * counting pass and a sweep (no wait between blocks), more chunks the radix
+ * passes, which compute the cell.  Every
  * d_cells[i] must be below 8^grid_log2 (else FP_ERR_CAPACITY, outputs invalid).
  * Outputs identical to fp_distribute's. */
 fp_status fp_distribute_cells(const fp_point* d_pts, const uint32_t* d_cells, uint64_t n, const fp_cube* d_cube,

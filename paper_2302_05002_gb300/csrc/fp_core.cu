@@ -27,16 +27,16 @@ constexpr int kBdTile = kBdNT * kBdIPT;   // 2048 points per tile
 // The previews that need no extents, without a look-back.  Keep rule: the index
 // hash is a multiple of the modulus (the uniform preview), or it is the smallest
 // of the point's cell (the spatial one, whose keep bits k_cell_mark sets first).
-// Only the kept points are read.  A block takes a segment of consecutive tiles; a warp takes ROWS rows of 32
-// points, lane r holds row r's keep bits.  When every block has counted its
-// segment, a tile's output starts at the totals of the earlier segments plus its
-// place in its own.
+// Only the kept points are read.  A block takes a segment of consecutive tiles; a
+// warp takes ROWS rows of 32 points, lane r holds row r's keep bits.  When every
+// block has counted its segment, a tile's output starts at the totals of the earlier
+// segments plus its place in its own.
 //   k_keep_all: both halves in one cooperative launch, the keep bits in shared
 //     memory across the barrier (the uniform rule, up to kKeepTiles tiles a block);
 //   k_keep, k_keep_write: in two launches (the spatial rule, and larger pieces,
 //     whose bits are computed again).
-// Both halves of the uniform rule are bound by the hash's integer instructions (10
-// us for 8M points).  (In one launch with a look-back, all tiles of a wave publish
+// The hash takes 10 us of integer instructions for 8M points; the two launches of the
+// uniform rule compute it twice.  (In one launch with a look-back, all tiles of a wave publish
 // at about the same time and the last walks back over all of them: 38 us for 8M
 // points, 25 us now.)
 constexpr int kKeepSegs = 2048;
@@ -781,7 +781,7 @@ __global__ void __launch_bounds__(256, kMinCtas) k_cell_min_hash(const fp_point*
     // through L1: an SM's own atomics drop its stale line; 0.62 -> 0.54 ms at 10^8.)
     // Bound by instructions: without a test per point and with no more blocks than
     // are resident 0.54 -> 0.45 ms, the same at 2 to 8 points and 3 to 8 blocks an SM;
-    // 0.42 ms with the shorter cell arithmetic.
+    // 0.43 ms with the shorter cell arithmetic (0.42 without the masks of points outside).
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     for (; i0 + (kMinIPT - 1) * stride < n; i0 += stride * kMinIPT) {

@@ -18,14 +18,14 @@
 //   1. group the distributed points by level-g cell (records (key21, j) with j
 //      the position in the chunk array, i.e. index order; any order inside a
 //      cell);
-//   2. cells with more than kPieceMax points are key-sorted and cut into
-//      node-aligned pieces of at most kPieceMax points (split tree, one warp per
-//      open node); the split tree also gives the nodes between level g and the
-//      pieces, and which piece minimum is the minimum of which coarser node;
-//   3. one CTA per window of pieces: sort by key in shared memory, all nearest
-//      smaller values of the index along the key order give each point's
-//      lambda, deep subtrees inside pieces are split by binary search, and each
-//      point gets its owner level and leaf level;
+//   2. cells with more than kPieceMax points are cut into node-aligned pieces of at
+//      most kPieceMax points, three levels a round (split tree, k_rounds); the split
+//      tree also gives the nodes between level g and the pieces, and which piece
+//      minimum is the minimum of which coarser node;
+//   3. lambda piece by piece, by its size and depth: pairs of points, tables of the
+//      smallest index per occupied cell, or a sort by key and nearest smaller
+//      indices; the nodes inside pieces whose node is split further; each point gets
+//      its owner level and leaf level;
 //   4. node records (levels <= g from the count pyramid, deeper ones from steps
 //      2-3) are sorted into preorder; ids are resolved per point;
 //   5. the points are scattered stably by leaf id (leaf-grouped output) and,
@@ -1758,10 +1758,14 @@ __global__ void k_node_children(const uint32_t* nnode, const uint64_t* sorted_st
 }
 
 // The node table in one launch of one cluster, for at most kNodeClusterMax nodes
-// by the host's bound (28 launches otherwise; 1M points: about 110 -> 19 us).  Stable
+// by the host's bound (18 launches otherwise; 1M points: about 110 -> 19 us).  Stable
 // least-significant-digit-first passes over (level, start); a pass in which all
 // records share the digit is left out (without nodes below the count grid: all bits
-// below level g).
+// below level g).  Octree stage with the cluster and with the grid's sorts: 122 nodes
+// 129 and 242 us, 9478 nodes 1.85 and 1.96 ms, 18,295 nodes 215 and 285 us, 60,387
+// nodes 362 and 318 us.  Only the bound is known here, 20 times too high for a usual
+// tree (9018 nodes, bound 2 * 10^5), so the line lies where such trees do; clusters of
+// points made to reach it (137,885 nodes) take 0.26 ms longer than by the sorts.
 constexpr uint64_t kNodeClusterMax = 1ull << 18;
 
 struct NodeClusterArgs {

@@ -293,9 +293,8 @@ cudaError_t dist_cluster(const int4* pts, uint64_t n, const fp_cube* cube, int g
                          const uint64_t* offsets, const uint32_t* num_chunks, int4* out, uint32_t* perm,
                          const uint32_t* cells, uint32_t* const tmp[4], uint32_t* hist, uint32_t* err, cudaStream_t st);
 
-
-// Distribution of n points into up to 4096 chunks by the counting pass and a
-// double-buffered sweep (fp_seg.cu); the points' cells given or computed.
+// Distribution of n points into up to 4096 chunks by the counting pass and the sweep
+// (fp_seg.cu); the points' cells given or computed.
 // chunk_tmp: n chunk ids, 16-byte aligned.  *run_sort is set to 1, and hist
 // (kSortHistWords) cleared, when there are more chunks (the radix passes run
 // instead), else 0.

@@ -172,8 +172,8 @@ cudaError_t launch_distribute(const fp_point* pts, uint64_t n, const fp_cube* cu
         return dist_cluster(reinterpret_cast<const int4*>(pts), n, cube, g, lut, offsets, num_chunks,
                             reinterpret_cast<int4*>(out), perm, cells, tmp, sc.hist, ws.err, st);
     }
-    // Up to 4096 chunks: the count, scan and double-buffered sweep (every point's
-    // chunk kept in val_tmp, which the radix passes below then do not use), from
+    // Up to 4096 chunks: the count, scan and sweep (every point's chunk kept in
+    // val_tmp, which the radix passes below then do not use), from
     // the cells or from the points.  More: the radix passes, which compute the
     // cells from the points.
     cudaError_t e = dist_wide(reinterpret_cast<const int4*>(pts), n, cube, g, lut, offsets, num_chunks,

@@ -5,7 +5,7 @@
 // i.e. a stable scatter by one digit d of a key.  Tiles of 4096 records are
 // claimed in order; each tile
 //   1. computes the digits and ranks every record among the equal digits of its
-//      own warp (match_any), warps own contiguous 256-record slices,
+//      own warp (by ballots), warps own contiguous 256-record slices,
 //   2. publishes its digit histogram, then looks back over earlier tiles for the
 //      per-digit exclusive prefix (decoupled look-back, bounded spin),
 //   3. stages the records in shared memory in digit order and writes each digit
