@@ -66,11 +66,12 @@ FP_DEV uint64_t cl_scan(uint32_t n, uint64_t* part, ClScanSmem& S, Value value, 
 #pragma unroll
         for (int u = 0; u < kClRows; ++u) {
             uint64_t x = v[u];
+            if (i0 + u * kClNT < hi)   // (a small table has one row; the same for the block)
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint64_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-                if (lane >= o) x += y;
-            }
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint64_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+                    if (lane >= o) x += y;
+                }
             if (lane == 31) S.row[u][warp] = x;
             ex[u] = x - v[u];
         }
