@@ -68,10 +68,10 @@ KERNEL_FILES = {
 # pass and sweep; the table and scan launches move under 20 MB), with the hash of the
 # kernel's sources at the capture (profiles/kernels_uniform100M.md); uniform-1B has the
 # same per-point structure (512 chunks, the same node levels) and ten times the points
-_T100 = {"bounds_decimate": (1.697e9, "c7186c53c2890ff3"), "count": (1.974e9, "c7186c53c2890ff3"),
-         "distribute": (0.613e9 + 3.958e9, "c299010c4a85751c"),
-         "cell_group": (4.535e9, "e24cb5430d20a1bb"), "units": (2.741e9, "e24cb5430d20a1bb"),
-         "resolve": (0.839e9, "e24cb5430d20a1bb"), "owner_scatter": (3.807e9, "a96e07133017ba54")}
+_T100 = {"bounds_decimate": (1.697e9, "8686f4b1721e15f2"), "count": (1.974e9, "8686f4b1721e15f2"),
+         "distribute": (0.613e9 + 3.959e9, "d2121aa22ef54a16"),
+         "cell_group": (4.632e9, "bf4dfc8e91c7c195"), "units": (2.758e9, "bf4dfc8e91c7c195"),
+         "resolve": (0.839e9, "bf4dfc8e91c7c195"), "owner_scatter": (3.804e9, "ee7f466c82a91d36")}
 NCU_TRAFFIC = {}
 for _k, (_b, _h) in _T100.items():
     NCU_TRAFFIC[("uniform-100M", _k)] = (_b, _h)
